@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kAuxThreads) init_gradient_kernel(const StepPa
     const long long j = it - static_cast<long long>(q) * p.d;
     float xi[4] = {0.f, 0.f, 0.f, 0.f};
     if (sigma != 0.0)
-      normal_quad(p.seed_lo, p.seed_hi, static_cast<unsigned long long>(p.coord_offset + j), q, p.t_noise, xi);
+      normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j), q, p.t_noise, xi);
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       const int i = 4 * q + w;

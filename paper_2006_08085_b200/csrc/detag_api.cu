@@ -2,6 +2,7 @@
 // (momentum, polynomial of the gossip matrix), workspace layout and kernel launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -17,7 +18,7 @@ namespace {
 size_t align_up(size_t v) { return (v + detag::kWsAlign - 1) / detag::kWsAlign * detag::kWsAlign; }
 
 struct WsLayout {
-  size_t status, result, row_ptr, col_idx, vals, poly, torus, circ_row, wide, partials, total;
+  size_t status, result, row_ptr, col_idx, vals, poly, torus, circ_row, wide, split_blocks, split_exp, split_poly, partials, total;
 };
 
 WsLayout ws_layout(const detag_state* s) {
@@ -40,6 +41,12 @@ WsLayout ws_layout(const detag_state* s) {
   off += align_up(s->circ_row.size() * sizeof(double));
   l.wide = off;
   off += align_up(s->wide_frag.size() * sizeof(double));
+  l.split_blocks = off;
+  off += align_up(s->split.blocks.size());
+  l.split_exp = off;
+  off += align_up(s->split.row_exp.size() * sizeof(int32_t));
+  l.split_poly = off;
+  off += align_up(s->split.poly_t.size() * sizeof(double));
   l.partials = off;
   off += align_up(detag::kMaxPartials * sizeof(double));
   l.total = off;
@@ -63,22 +70,74 @@ int fail_cuda(detag_state* s, int cuda_code, const char* where) {
 // P_K(M) by the matrix form of Algorithm 3: P_{-1} = P_0 = I, P_{r+1} = (1+eta) M P_r - eta P_{r-1}.
 void gossip_polynomial(const detag_state* s, std::vector<double>& out) {
   const int n = s->n;
-  std::vector<double> prev(static_cast<size_t>(n) * n, 0.0), cur, next(static_cast<size_t>(n) * n);
+  std::vector<double> prev(static_cast<size_t>(n) * n, 0.0), cur, next(static_cast<size_t>(n) * n), acc(n);
   for (int i = 0; i < n; ++i) prev[static_cast<size_t>(i) * n + i] = 1.0;
   cur = prev;
   for (int r = 0; r < s->K; ++r) {
     for (int i = 0; i < n; ++i) {
-      for (int j = 0; j < n; ++j) {
-        double acc = 0.0;
-        for (int k = s->row_ptr[i]; k < s->row_ptr[i + 1]; ++k)
-          acc += s->vals[k] * cur[static_cast<size_t>(s->col_idx[k]) * n + j];
-        next[static_cast<size_t>(i) * n + j] = (1.0 + s->eta) * acc - s->eta * prev[static_cast<size_t>(i) * n + j];
+      std::fill(acc.begin(), acc.end(), 0.0);
+      for (int k = s->row_ptr[i]; k < s->row_ptr[i + 1]; ++k) {
+        const double w = s->vals[k];
+        const double* row = &cur[static_cast<size_t>(s->col_idx[k]) * n];
+        for (int j = 0; j < n; ++j) acc[j] += w * row[j];
       }
+      const double* old = &prev[static_cast<size_t>(i) * n];
+      double* out_row = &next[static_cast<size_t>(i) * n];
+      for (int j = 0; j < n; ++j) out_row[j] = (1.0 + s->eta) * acc[j] - s->eta * old[j];
     }
     prev.swap(cur);
     cur.swap(next);
   }
   out = cur;
+}
+
+// Rows 32 further are the same entries 32 columns further: then so is every polynomial of M, and its 32 x 32 blocks
+// depend on their distance only.
+bool block_circulant(const detag_state* s) {
+  constexpr int kBlock = 32;
+  const int n = s->n;
+  if (n % kBlock != 0) return false;
+  std::vector<double> row(n, 0.0);
+  for (int i = 0; i < n; ++i) {
+    const int next = (i + kBlock) % n;
+    if (s->row_ptr[i + 1] - s->row_ptr[i] != s->row_ptr[next + 1] - s->row_ptr[next]) return false;
+    for (int k = s->row_ptr[i]; k < s->row_ptr[i + 1]; ++k) row[s->col_idx[k]] = s->vals[k];
+    bool same = true;
+    for (int k = s->row_ptr[next]; k < s->row_ptr[next + 1]; ++k)
+      same = same && row[(s->col_idx[k] - kBlock + n) % n] == s->vals[k];
+    for (int k = s->row_ptr[i]; k < s->row_ptr[i + 1]; ++k) row[s->col_idx[k]] = 0.0;
+    if (!same) return false;
+  }
+  return true;
+}
+
+// Rows 0 .. 31 of P_K(M), for a matrix whose 32 x 32 blocks depend on their distance only: the recursion of Algorithm 3
+// on those rows alone, P_{r+1} = (1+eta) P_r M - eta P_{r-1} (P_r is a polynomial of M and commutes with it).
+void first_block_row(const detag_state* s, std::vector<double>& out) {
+  constexpr int kRows = 32;
+  const int n = s->n;
+  out.assign(static_cast<size_t>(kRows) * n, 0.0);
+  if (!s->circ_row.empty()) {  // circulant: shifts of the first row, which is known
+    for (int i = 0; i < kRows; ++i)
+      for (int j = 0; j < n; ++j) out[static_cast<size_t>(i) * n + j] = s->circ_row[j >= i ? j - i : j - i + n];
+    return;
+  }
+  std::vector<double> prev(n), cur(n), next(n);
+  for (int i = 0; i < kRows; ++i) {
+    std::fill(prev.begin(), prev.end(), 0.0);
+    prev[i] = 1.0;
+    cur = prev;
+    for (int r = 0; r < s->K; ++r) {
+      std::fill(next.begin(), next.end(), 0.0);
+      for (int k = 0; k < n; ++k)
+        if (cur[k] != 0.0)
+          for (int e = s->row_ptr[k]; e < s->row_ptr[k + 1]; ++e) next[s->col_idx[e]] += cur[k] * s->vals[e];
+      for (int j = 0; j < n; ++j) next[j] = (1.0 + s->eta) * next[j] - s->eta * prev[j];
+      prev.swap(cur);
+      cur.swap(next);
+    }
+    std::copy(cur.begin(), cur.end(), out.begin() + static_cast<size_t>(i) * n);
+  }
 }
 
 // Circulant M (row i = row 0 shifted by i): then P_K(M) is circulant too; its row 0 is computed with the
@@ -98,12 +157,14 @@ void analyse_circulant(detag_state* s) {
   prev[0] = 1.0;
   cur = prev;
   for (int r = 0; r < s->K; ++r) {
-    for (int j = 0; j < n; ++j) {
-      double acc = 0.0;
-      for (int k = s->row_ptr[0]; k < s->row_ptr[1]; ++k)
-        acc += s->vals[k] * cur[((j - s->col_idx[k]) % n + n) % n];
-      next[j] = (1.0 + s->eta) * acc - s->eta * prev[j];
+    std::fill(next.begin(), next.end(), 0.0);
+    for (int k = s->row_ptr[0]; k < s->row_ptr[1]; ++k) {
+      const double w = s->vals[k];
+      const int shift = s->col_idx[k];  // next[j] += w cur[(j - shift) mod n]
+      for (int j = 0; j < shift; ++j) next[j] += w * cur[j - shift + n];
+      for (int j = shift; j < n; ++j) next[j] += w * cur[j - shift];
     }
+    for (int j = 0; j < n; ++j) next[j] = (1.0 + s->eta) * next[j] - s->eta * prev[j];
     prev.swap(cur);
     cur.swap(next);
   }
@@ -232,11 +293,14 @@ StepParams make_params(const detag_state* s) {
   p.torus = s->d_torus;
   p.circ_row = s->d_circ_row;
   p.wide = s->d_wide;
+  p.split = s->d_split;
   p.eta = s->eta;
   p.alpha = s->alpha;
   p.sigma = s->sigma;
-  p.seed_lo = static_cast<uint32_t>(s->seed & 0xffffffffu);
-  p.seed_hi = static_cast<uint32_t>(s->seed >> 32);
+  for (uint32_t round = 0; round < 10; ++round) {
+    p.round_key[2 * round] = static_cast<uint32_t>(s->seed & 0xffffffffu) + round * 0x9E3779B9u;
+    p.round_key[2 * round + 1] = static_cast<uint32_t>(s->seed >> 32) + round * 0xBB67AE85u;
+  }
   p.status = s->d_status;
   p.grad_at_start = s->gradient_point == DETAG_GRADIENT_AT_PHASE_START ? 1 : 0;
   p.mode = step_mode(s);
@@ -303,7 +367,7 @@ int query_device(detag_state* s) {
 }
 
 // Kernel families that take tensor maps.
-enum { kFamilyMma = 1, kFamilyBand = 2, kFamilyTorus = 3, kFamilyRing = 4, kFamilyWide = 5 };
+enum { kFamilyMma = 1, kFamilyBand = 2, kFamilyTorus = 3, kFamilyRing = 4, kFamilyWide = 5, kFamilySplit = 6 };
 
 // Tensor maps for the buffers in `p`: built on first use, then found again by buffer addresses and sizes
 // (detag_step always hits; detag_step_host cycles through its two chunk slots and the ragged last chunk).
@@ -330,6 +394,7 @@ const detag::TensorMapSet* maps_for(detag_state* s, int family, const StepParams
                   : family == kFamilyBand ? detag::build_maps_band(p, &en.maps)
                   : family == kFamilyRing ? detag::build_maps_ring(p, &en.maps)
                   : family == kFamilyWide ? detag::build_maps_wide(p, &en.maps)
+                  : family == kFamilySplit ? detag::build_maps_split(p, &en.maps)
                                           : detag::build_maps_torus(p, &en.maps);
   if (!ok) return nullptr;
   en.family = family;
@@ -357,6 +422,14 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   return DETAG_OK;
 }
 
+// The integer tensor path takes the dense and circulant products with 32 < n <= 256, and, where the choice is the
+// library's, the rounds of such matrices too.
+bool split_ok(const detag_state* s, const StepParams& p, int variant) {
+  if (s->split.blocks.empty() || p.mode == detag::kModeExternal || p.d > 0x7fffffffLL) return false;
+  if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
+  return variant == DETAG_VARIANT_DENSE || variant == DETAG_VARIANT_RING;
+}
+
 // Picks the kernel variant, plans it for the sizes in `p` and launches it.
 int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   int e = 0;
@@ -368,6 +441,17 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     return fail(s, DETAG_ERR_UNBOUND, "the synthetic gradient needs the objective arrays a and c");
   if (p.mode == detag::kModeExternal && !p.g_ext)
     return fail(s, DETAG_ERR_UNBOUND, "caller-written gradients selected but no gradient array given");
+  if (split_ok(s, p, variant)) {
+    const detag::TensorMapSet* maps = maps_for(s, kFamilySplit, p);
+    if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+    const WsLayout l = ws_layout(s);
+    e = detag::launch_step_split(p, *maps, s->split, p.split,
+                                 reinterpret_cast<const int32_t*>(p.split + (l.split_exp - l.split_blocks)),
+                                 reinterpret_cast<const double*>(p.split + (l.split_poly - l.split_blocks)),
+                                 variant == DETAG_VARIANT_CSR, s->sm_count, stream);
+    if (e != 0) return fail_cuda(s, e, "step kernel launch");
+    return DETAG_OK;
+  }
   switch (variant) {
     case DETAG_VARIANT_DENSE: {
       if (p.n > detag::kMaxDenseWorkers) {
@@ -472,16 +556,40 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   s->row_ptr.assign(row_ptr, row_ptr + n + 1);
   s->col_idx.assign(col_idx, col_idx + nnz);
   s->vals.assign(vals, vals + nnz);
+  std::vector<double> poly;
   if (n <= detag::kMaxDenseWorkers) {
     gossip_polynomial(s, s->poly);
   } else if (n <= detag::kMaxWideWorkers) {  // kept as the warp strips of the register-resident kernel only
-    std::vector<double> poly;
     gossip_polynomial(s, poly);
     detag::wide_fragments(n, poly, s->wide_frag);
   }
   analyse_circulant(s);
   analyse_torus(s);
+  if (n > 32 && n <= detag::kMaxSplitWorkers) {
+    const bool blocks = block_circulant(s);
+    if (blocks)
+      first_block_row(s, poly);
+    else if (!s->poly.empty())
+      poly = s->poly;
+    if (!poly.empty()) detag::split_polynomial(n, poly, blocks, s->split);  // else: too many distinct blocks
+  }
   s->map_cache.reserve(8);
+  // the workspace's tables as they are uploaded, the cleared status block in front
+  const WsLayout l = ws_layout(s);
+  s->image.assign(l.partials, 0);
+  auto put = [&](size_t at, const void* src, size_t bytes) {
+    if (bytes != 0) std::memcpy(&s->image[at], src, bytes);
+  };
+  put(l.row_ptr, s->row_ptr.data(), s->row_ptr.size() * sizeof(int32_t));
+  put(l.col_idx, s->col_idx.data(), s->col_idx.size() * sizeof(int32_t));
+  put(l.vals, s->vals.data(), s->vals.size() * sizeof(double));
+  put(l.poly, s->poly.data(), s->poly.size() * sizeof(double));
+  put(l.torus, s->torus_frag.data(), s->torus_frag.size() * sizeof(double));
+  put(l.circ_row, s->circ_row.data(), s->circ_row.size() * sizeof(double));
+  put(l.wide, s->wide_frag.data(), s->wide_frag.size() * sizeof(double));
+  put(l.split_blocks, s->split.blocks.data(), s->split.blocks.size());
+  put(l.split_exp, s->split.row_exp.data(), s->split.row_exp.size() * sizeof(int32_t));
+  put(l.split_poly, s->split.poly_t.data(), s->split.poly_t.size() * sizeof(double));
   *out = s;
   return DETAG_OK;
 }
@@ -518,23 +626,10 @@ int detag_bind(detag_state* s, int64_t ld, float* x, float* y, float* g, const f
   s->d_torus = s->torus_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.torus);
   s->d_circ_row = s->circ_row.empty() ? nullptr : reinterpret_cast<double*>(base + l.circ_row);
   s->d_wide = s->wide_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.wide);
+  s->d_split = s->split.blocks.empty() ? nullptr : base + l.split_blocks;
   s->d_partials = reinterpret_cast<double*>(base + l.partials);
 
-  e = cudaMemset(base, 0, detag::kWsAlign);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(s->d_row_ptr, s->row_ptr.data(), s->row_ptr.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(s->d_col_idx, s->col_idx.data(), s->col_idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(s->d_vals, s->vals.data(), s->vals.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && s->d_poly)
-    e = cudaMemcpy(s->d_poly, s->poly.data(), s->poly.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && s->d_torus)
-    e = cudaMemcpy(s->d_torus, s->torus_frag.data(), s->torus_frag.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && s->d_circ_row)
-    e = cudaMemcpy(s->d_circ_row, s->circ_row.data(), s->circ_row.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && s->d_wide)
-    e = cudaMemcpy(s->d_wide, s->wide_frag.data(), s->wide_frag.size() * sizeof(double), cudaMemcpyHostToDevice);
+  e = cudaMemcpy(base, s->image.data(), s->image.size(), cudaMemcpyHostToDevice);  // status word and result cleared
   if (e != cudaSuccess) return fail_cuda(s, e, "detag_bind: workspace upload");
 
   s->ld = ld;
@@ -781,27 +876,9 @@ int detag_step_host(detag_state* s, int64_t ld_host, float* x, float* y, float* 
   // Graph tables at the head of the staging area, ordered on the caller's stream.  The status word there is
   // cleared when a staging area is first used, not on every call: a time-out stays visible to detag_status.
   int* status_word = reinterpret_cast<int*>(base + l.status);
-  if (s->d_status_host != status_word) e = cudaMemsetAsync(base, 0, detag::kWsAlign, user);
+  const size_t skip = s->d_status_host != status_word ? 0 : l.row_ptr;
   s->d_status_host = status_word;
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(base + l.row_ptr, s->row_ptr.data(), s->row_ptr.size() * sizeof(int32_t),
-                        cudaMemcpyHostToDevice, user);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(base + l.col_idx, s->col_idx.data(), s->col_idx.size() * sizeof(int32_t),
-                        cudaMemcpyHostToDevice, user);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(base + l.vals, s->vals.data(), s->vals.size() * sizeof(double), cudaMemcpyHostToDevice, user);
-  if (e == cudaSuccess && !s->poly.empty())
-    e = cudaMemcpyAsync(base + l.poly, s->poly.data(), s->poly.size() * sizeof(double), cudaMemcpyHostToDevice, user);
-  if (e == cudaSuccess && !s->torus_frag.empty())
-    e = cudaMemcpyAsync(base + l.torus, s->torus_frag.data(), s->torus_frag.size() * sizeof(double),
-                        cudaMemcpyHostToDevice, user);
-  if (e == cudaSuccess && !s->circ_row.empty())
-    e = cudaMemcpyAsync(base + l.circ_row, s->circ_row.data(), s->circ_row.size() * sizeof(double),
-                        cudaMemcpyHostToDevice, user);
-  if (e == cudaSuccess && !s->wide_frag.empty())
-    e = cudaMemcpyAsync(base + l.wide, s->wide_frag.data(), s->wide_frag.size() * sizeof(double), cudaMemcpyHostToDevice,
-                        user);
+  e = cudaMemcpyAsync(base + skip, s->image.data() + skip, s->image.size() - skip, cudaMemcpyHostToDevice, user);
   if (e == cudaSuccess) e = cudaEventRecord(s->host_event[2], user);
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(s->host_stream[k], s->host_event[2], 0);
   if (e != cudaSuccess) return fail_cuda(s, e, "detag_step_host: table upload");
@@ -814,6 +891,7 @@ int detag_step_host(detag_state* s, int64_t ld_host, float* x, float* y, float* 
   p.torus = s->torus_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.torus);
   p.circ_row = s->circ_row.empty() ? nullptr : reinterpret_cast<double*>(base + l.circ_row);
   p.wide = s->wide_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.wide);
+  p.split = s->split.blocks.empty() ? nullptr : base + l.split_blocks;
   p.status = status_word;
   p.y_obs = nullptr;
   p.t_noise = static_cast<uint32_t>(s->t + 1);

@@ -16,6 +16,7 @@ namespace detag {
 constexpr int kMaxWorkers = 1024;       // detag_create limit on n
 constexpr int kMaxDenseWorkers = 64;    // dense-polynomial kernels with P in shared memory: limit on n
 constexpr int kMaxWideWorkers = 128;    // dense-polynomial kernel with P in registers: limit on n
+constexpr int kMaxSplitWorkers = 256;   // integer tensor path: limit on n
 constexpr int kMaxPartials = 2048;      // per-CTA partial sums of the consensus-error reduction
 constexpr size_t kWsAlign = 256;
 
@@ -44,11 +45,12 @@ struct StepParams {
   const double* poly;  // dense P_K(M), row-major n x n (null when n > kMaxDenseWorkers)
   const double* circ_row;  // circulant kernel, dense mode: the first row of P_K(M) (or null)
   const double* wide;  // register-resident dense kernel (64 < n <= 128): the warp strips of P_K(M) in fragment order (or null)
+  const unsigned char* split;  // split kernel: digit blocks, row exponents and P in the workspace (or null)
   const double* torus; // block-circulant kernel: per-frequency 8 x 8 polynomial blocks in fragment order (or null)
   double eta;
   double alpha;
   double sigma;
-  uint32_t seed_lo, seed_hi;
+  uint32_t round_key[20];  // Philox round keys of the noise seed (noise.cuh)
   uint32_t t_noise;  // step index that enters the noise counter
   int grad_at_start;  // nonzero: the gradient is taken at the model the step started from (Algorithm 2 as printed)
   int steps;          // consecutive steps in one launch (multi-step kernel only)
@@ -68,6 +70,17 @@ constexpr int kModeDpsgd = 2;     // D-PSGD: x' = AG_K(x) - alpha g, g' = synthe
 // buffers and kept in the state.
 struct alignas(64) TensorMapSet {
   unsigned char bytes[8 * 128];
+};
+
+// P_K(M) as the split kernel (step_split.cu) takes it: the distinct 32 x 32 blocks of its base-256 digits, their table,
+// the exponent of every row's scale, and P itself (transposed).  Empty when the kernel does not take the matrix.
+struct SplitPoly {
+  std::vector<unsigned char> blocks;
+  std::vector<int32_t> row_exp;
+  std::vector<double> poly_t;  // transposed, rows padded to a multiple of 16, their number to one of 32; or see circulant
+  bool sparse;           // some entry is less than 2^-8 of its row's largest
+  bool circulant;        // blocks depend on their distance only: poly_t holds output workers 0 .. 31
+  unsigned char id[64];  // [output block][input block] -> distinct block, 255: all zero
 };
 
 // host helpers (spectral.cpp)
@@ -107,6 +120,12 @@ void wide_fragments(int n, const std::vector<double>& poly, std::vector<double>&
 bool build_maps_wide(const StepParams& p, TensorMapSet* maps);
 int launch_step_wide(StepParams p, const TensorMapSet& maps, const double* p_frag /* device */, int sm_count,
                      cudaStream_t stream);
+// polynomial on the integer tensor path (step_split.cu): 32 < n <= 256, DeTAG and D-PSGD steps
+void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
+bool build_maps_split(const StepParams& p, TensorMapSet* maps);
+int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const void* blocks /* device */,
+                      const int32_t* row_exp /* device */, const double* poly_t /* device */, bool wide_gradient, int sm_count,
+                      cudaStream_t stream);
 int launch_consensus_error(const StepParams& p, double* partials, double* result, int sm_count, cudaStream_t stream);
 int launch_init_external(const StepParams& p, int sm_count, cudaStream_t stream);  // y = g = g_ext
 int launch_expire_wait(int* status, unsigned polls, cudaStream_t stream);          // a wait nobody ends (self test)
@@ -132,6 +151,8 @@ struct detag_state {
   bool torus = false;
   std::vector<double> torus_frag;
   std::vector<double> wide_frag;  // 64 < n <= 128: P_K(M) as the warp strips of the register-resident kernel
+  detag::SplitPoly split;         // 32 < n <= 256: P_K(M) for the integer tensor path (empty: not taken)
+  std::vector<unsigned char> image;  // the workspace up to the partial sums, as it is uploaded
   int variant_forced = DETAG_VARIANT_AUTO;
   int gradient_point = DETAG_GRADIENT_AT_NEW_MODEL;
   int algorithm = DETAG_ALGORITHM_DETAG;
@@ -157,6 +178,7 @@ struct detag_state {
   double* d_torus = nullptr;
   double* d_circ_row = nullptr;
   double* d_wide = nullptr;
+  unsigned char* d_split = nullptr;  // blocks, row exponents and P of `split`, one after the other (split_at)
   double* d_partials = nullptr;
 
   double sigma = 0.0;

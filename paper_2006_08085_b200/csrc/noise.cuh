@@ -39,6 +39,23 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
   return Philox4{c0, c1, c2, c3};
 }
 
+// The same with the twenty round keys (k0 + round * W0, k1 + round * W1 alternating) laid out by the host in the launch
+// parameters: each is then a constant-bank operand of the exclusive-or that uses it instead of an addition of its own.
+__device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                                 const uint32_t (&round_key)[20]) {
+  constexpr uint32_t kM0 = 0xD2511F53u, kM1 = 0xCD9E8D57u;
+#pragma unroll
+  for (int round = 0; round < 10; ++round) {
+    const unsigned long long p0 = static_cast<unsigned long long>(kM0) * c0;
+    const unsigned long long p1 = static_cast<unsigned long long>(kM1) * c2;
+    c0 = static_cast<uint32_t>(p1 >> 32) ^ c1 ^ round_key[2 * round];
+    c1 = static_cast<uint32_t>(p1);
+    c2 = static_cast<uint32_t>(p0 >> 32) ^ c3 ^ round_key[2 * round + 1];
+    c3 = static_cast<uint32_t>(p0);
+  }
+  return Philox4{c0, c1, c2, c3};
+}
+
 // -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9.
 __device__ __forceinline__ float neg2_ln_unit(uint32_t r) {
   const float v = __uint_as_float(0x3f800000u | (r >> 9));  // 1 + k 2^-23
@@ -73,9 +90,9 @@ __device__ __forceinline__ void box_muller(uint32_t r_even, uint32_t r_odd, floa
 }
 
 // Standard normals of workers 4q..4q+3 at global coordinate j and noise step t.
-__device__ __forceinline__ void normal_quad(uint32_t seed_lo, uint32_t seed_hi, unsigned long long j, uint32_t q,
-                                            uint32_t t, float xi[4]) {
-  const Philox4 r = philox4x32_10(static_cast<uint32_t>(j), static_cast<uint32_t>(j >> 32), q, t, seed_lo, seed_hi);
+__device__ __forceinline__ void normal_quad(const uint32_t (&round_key)[20], unsigned long long j, uint32_t q, uint32_t t,
+                                            float xi[4]) {
+  const Philox4 r = philox4x32_10(static_cast<uint32_t>(j), static_cast<uint32_t>(j >> 32), q, t, round_key);
   box_muller(r.r0, r.r1, xi[0], xi[1]);
   box_muller(r.r2, r.r3, xi[2], xi[3]);
 }

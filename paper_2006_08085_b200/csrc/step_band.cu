@@ -308,7 +308,7 @@ step_band_kernel(const StepParams p, const __grid_constant__ BandMaps maps) {
       for (int e = 0; e < 2; ++e) {
         if (noisy) {
           const uint32_t quad = static_cast<uint32_t>((rb * kR + 8 * pos) / 4 + half);
-          normal_quad(p.seed_lo, p.seed_hi, static_cast<unsigned long long>(p.coord_offset + j + e), quad, p.t_noise,
+          normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + e), quad, p.t_noise,
                       xi[e]);
           transpose4(xi[e], pos);
         } else {

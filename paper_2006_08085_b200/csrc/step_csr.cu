@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepPara
     float xi[4] = {0.f, 0.f, 0.f, 0.f};
     if (sigma != 0.f && !external) {  // every lane takes part (the shuffles want whole warps); idle lanes' draws are unused
       // lane r4 draws coordinate j + r4 for the quad's four workers; the transpose gives it its own row's four
-      normal_quad(p.seed_lo, p.seed_hi, static_cast<unsigned long long>(p.coord_offset + j + r4), static_cast<uint32_t>(q),
+      normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + r4), static_cast<uint32_t>(q),
                   p.t_noise, xi);
       transpose_rows(xi, r4, groups);
     }

@@ -111,7 +111,7 @@ step_mma_many_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           if (noisy) {
-            normal_quad(p.seed_lo, p.seed_hi, static_cast<unsigned long long>(p.coord_offset + j + e),
+            normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + e),
                         static_cast<uint32_t>(r), p.t_noise + static_cast<uint32_t>(step), xi[e]);
           } else {
             xi[e][0] = xi[e][1] = xi[e][2] = xi[e][3] = 0.f;

@@ -325,7 +325,7 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
 #pragma unroll
       for (int hq = 0; hq < 2; ++hq) {
         float v[4];
-        normal_quad(p.seed_lo, p.seed_hi, jn, static_cast<uint32_t>(8 * b + 4 * hq + kq), p.t_noise, v);
+        normal_quad(p.round_key, jn, static_cast<uint32_t>(8 * b + 4 * hq + kq), p.t_noise, v);
         transpose_quad(v, kq);  // v[i]: position kq of quad 8 b + 4 hq + i
 #pragma unroll
         for (int i = 0; i < 4; ++i) xi[4 * hq + i] = v[i];

@@ -1,0 +1,795 @@
+// DeTAG step with the polynomial P = P_K(M) applied on the fifth-generation tensor cores in exact integer arithmetic,
+// for any gossip matrix with 32 < n <= 256 whose distinct 32 x 32 blocks of P fit in shared memory.
+//
+// AG_K(z) = P z.  The float64 tensor path (mma m8n8k4) bounds this product at 64 multiply-adds per clock and SM, which
+// for n = 100 is 3.3 times and for a dense n = 256 eight times the time of the step's HBM traffic.  Here both operands
+// are split into four balanced base-256 digits:
+//     z_j = 2^-s sum_k Z_kj 256^k   (31 bits and sign, one power of two s per coordinate and array, from the largest |z_j|)
+//     P_ij = 2^-r_i sum_l P_lij 256^l   (the same per output worker, split once by the host)
+// and the products of digits are summed by tcgen05.mma kind::i8 into 32-bit integers, exactly.  The ten digit pairs
+// with k + l >= 3 are kept, one accumulator per k + l; the six below weigh less than the rounding of the digits.
+// What is lost is at most 2^-31 of the coordinate's largest operand per term: measured against float64 1e-10 .. 1e-9 of
+// the result in the 2-norm, a twentieth of the rounding of the stored float32 values.  Results that do not contain the
+// largest operand can only be much smaller than it if P is sparse - an entry below 2^-8 of its row's largest.  Then a
+// coordinate of which eight workers in a row all lie more than 2^10 below the largest is not split: its sums are taken in
+// float64 from the operands, which stay staged that long.  So are values outside the scalable range, infinities and NaN,
+// whatever P.  (2^10 leaves such a group 2^-20 of its own largest value.  On the 256-worker ring with 16 rounds, where
+// models vary smoothly from worker to worker and pass through zero, 2^8 met one coordinate in 100 k, 2^10 none in 10^7;
+// each costs its block some 100 us.)
+//
+// A unit of work is a slab of 64 coordinates.  Rows 0..63 of the MMA's M = 128 are the model digits of the slab's
+// coordinates, rows 64..127 its tracker digits, so one instruction serves both arrays: A [128][32 workers] from tensor
+// memory, where the threads that split the operands put it (thread = row = tensor memory lane), B two stacked digit planes
+// [32 output workers][32 workers] of a block of P in shared memory, D [128][2 x 32] the accumulators of two neighbouring
+// weights of an output chunk of 32 workers (two chunks in flight).  An MMA with M = 128 and K = 32 bytes takes 68 cycles
+// for any N up to 128 (measured: N = 16, 32, 64, 96, 128, from tensor or shared memory alike), so two weights share one:
+// six MMAs of N = 64 per block, with a plane of zeros above the highest digit, instead of ten of N = 32.  A thread that reads an accumulator owns one coordinate and consecutive workers:
+// the four workers of a Philox call are its own and shared-memory rows are read 32 coordinates at a time, without
+// conflicts and without swizzle.
+//
+// Roles: 4 or 8 splitting warps; F groups of 4 finishing warps that take half chunks (16 workers) in turn; one thread each for
+// the MMAs, the x, y loads (one slab, handed back block by block while it is split), the g, a, c loads (R stages of 16
+// workers per finishing group, overwritten with g', x', y') and the stores.  Model and tracker sums of a coordinate sit in
+// different warps (lanes 64 apart): each of the two finishes eight of the sixteen workers and hands the sums of the other
+// eight over, through the stage slots of its own eight whose g and a it has already taken into registers.  All sums are
+// taken at the start, so that the accumulators are free again before the noise, the gradient and the fold.
+// Zero blocks of P (rings, tori with few rounds) are skipped; equal blocks (circulant and block-circulant matrices) are
+// kept once.  Every wait is bounded.
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "detag_internal.h"
+#include "noise.cuh"
+#include "pipeline.cuh"
+#include "tensor_memory.cuh"
+#include "tma.cuh"
+
+namespace detag {
+
+namespace {
+
+constexpr int kPS = 64;             // coordinates per slab
+constexpr int kPChunk = 32;         // output workers per accumulator; also workers per block of P
+constexpr int kPUnit = 16;          // workers a finishing group takes at a time
+constexpr int kPWeights = 4;        // accumulators: digit pairs with k + l = 6, 5, 4, 3
+constexpr int kPPlaneBytes = kPChunk * kPChunk;
+constexpr int kPBlockBytes = 5 * kPPlaneBytes;  // one block of P: a plane of zeros and the digit planes 3, 2, 1, 0
+constexpr int kPTileFloats = kPChunk * kPS;          // 32 rows of x or y
+constexpr int kPStageFloats = kPUnit * kPS;          // one array of one unit
+constexpr int kPStageBytes = 3 * kPStageFloats * 4;  // g | a | c  ->  g' | x' | y'
+constexpr int kPScaleSlots = 4;     // slabs whose scales are kept: see the splitting warps
+constexpr int kPMaxGroups = 4, kPMaxStages = 2, kPMaxBlocks = 8;
+// Splitting and finishing warps.  Up to 128 workers two groups of four share the blocks of a slab: its splitting is a
+// serial chain (largest value, then digits) that one group needs 5.6 k cycles for at n = 48, as long as the slab's HBM
+// time.  Beyond, a slab's other stages take longer than its splitting, and the warps finish instead.
+__host__ __device__ constexpr int split_warps(bool big) { return big ? 4 : 8; }
+__host__ __device__ constexpr int finish_groups(bool big) { return big ? 4 : 3; }
+constexpr int kPThreads = 24 * 32;  // both: split_warps + 4 finish_groups + 4
+constexpr int kTmemColumns = 512;
+constexpr int kAccColumn = 256;     // digits below, accumulators from here on
+constexpr int kMaxDigit = 0x7F7F7F7F;  // largest integer with four balanced digits
+constexpr unsigned kRoundUp = 0x18000u;      // mantissas from 1.988 on count as the next power of two (see kMaxDigit)
+constexpr unsigned kSmallest = 0x12800000u;  // 2^-90: smaller maxima leave the range of the float32 scale
+constexpr size_t kPCtrlBytes = 640, kPSmemLimit = 232448;
+
+struct SplitMaps {
+  CUtensorMap x, y;        // boxes {64 coordinates, 32 workers}
+  CUtensorMap g, a, c;     // boxes {64, 16}
+  CUtensorMap xs, ys, gs;  // boxes {64, 16}, ending on a 16-byte boundary: stores
+};
+static_assert(sizeof(SplitMaps) <= sizeof(TensorMapSet), "tensor map storage");
+
+struct SplitTables {
+  const uint4* blocks;     // distinct blocks of P, digit planes in core-matrix order
+  const int* row_exp;      // exponent of each output worker's scale
+  // P itself, for what stays in float64: [input worker, padded to 32][output worker, padded to 16], or, if the blocks of P
+  // depend on their distance only, [input worker][output workers 0 .. 31]
+  const double* poly_t;
+  int circulant;
+  int num_blocks;
+  int nb;                  // 32-worker blocks per side
+  int sparse;              // some entry of P is less than 2^-8 of its row's largest
+  uint64_t id[8];          // [output chunk], a byte per input block: distinct block, 255: all zero
+};
+
+struct SplitPlan {
+  int groups, stages;
+  size_t blocks_at, e_at, scale_at, ctrl_at, bytes;
+};
+
+// Shared memory: x, y of a slab (whole blocks of 32 rows) | blocks of P | g, a, c stages | row exponents, scales, flags |
+// barriers.
+inline SplitPlan plan_for(int nb, int num_blocks, int groups, int stages) {
+  SplitPlan s{};
+  s.groups = groups;
+  s.stages = stages;
+  s.blocks_at = static_cast<size_t>(nb) * 2 * kPTileFloats * 4;
+  s.e_at = s.blocks_at + static_cast<size_t>(num_blocks) * kPBlockBytes;
+  s.scale_at = s.e_at + static_cast<size_t>(groups) * stages * kPStageBytes;
+  s.ctrl_at = s.scale_at + 256 * 4 + kPScaleSlots * 128 * 2 + kPScaleSlots * 4 * 4 + 4 * 128 * 8;
+  s.bytes = s.ctrl_at + kPCtrlBytes;
+  return s;
+}
+
+// Finishing groups and their stages: as many as fit, two stages before a fourth group (bytes = 0: nothing fits).
+inline SplitPlan split_plan(int nb, int num_blocks) {
+  constexpr int tries[4][2] = {{4, 2}, {3, 2}, {4, 1}, {3, 1}};
+  for (const auto& t : tries) {
+    if (t[0] > finish_groups(nb > 4)) continue;
+    const SplitPlan s = plan_for(nb, num_blocks, t[0], t[1]);
+    if (s.bytes <= kPSmemLimit) return s;
+  }
+  return SplitPlan{};
+}
+
+// Integer sums of the four weights -> one float64, exact: a 64-bit integer below 2^51 added to the bits of 1.5 * 2^52.
+// Up to 128 workers the two low weights fit 32 bits together (3 * 128 * 2^14 * 256 < 2^31).
+template <bool kBig>
+__device__ __forceinline__ double join_sums(int s6, int s5, int s4, int s3) {
+  const int hi = s6 * 256 + s5;
+  if (kBig) {
+    const long long lo = static_cast<long long>(s4) * 256 + (s3 + 0x4338000000000000LL);
+    return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - 6755399441055744.0;
+  }
+  const uint32_t lo = static_cast<uint32_t>(s4 * 256 + s3) ^ 0x80000000u;  // offset by 2^31: no sign to extend
+  return __longlong_as_double(static_cast<long long>(hi) * 65536 + (0x4338000000000000LL | lo)) -
+         (6755399441055744.0 + 2147483648.0);
+}
+
+// max(|a|, |b|, |c|), NaN if one of them is
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// kMode: kModeDetag or kModeDpsgd.  kWide: the gradient in float64 (the precision of the rounds kernel, in whose place
+// the call runs) instead of float32 at the rounded model (the other tensor-path kernels').  kBig: n > 128.
+template <int kMode, bool kWide, bool kBig>
+__global__ void __launch_bounds__(kPThreads, 1)
+step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, const __grid_constant__ SplitTables tb,
+                  const __grid_constant__ SplitPlan plan) {
+  constexpr int kSplitWarps = split_warps(kBig), kMmaWarp = kSplitWarps, kLoadXYWarp = kMmaWarp + 1, kLoadEWarp = kMmaWarp + 2, kStoreWarp = kMmaWarp + 3,
+                kFinishWarp = kMmaWarp + 4;
+  constexpr int kDigBuffers = kBig ? 1 : 2;
+  extern __shared__ __align__(128) unsigned char smem[];
+  float* const xy_mem = reinterpret_cast<float*>(smem);                    // [block][x | y][32 rows][64]
+  float* const e_mem = reinterpret_cast<float*>(smem + plan.e_at);
+  int* const row_exp = reinterpret_cast<int*>(smem + plan.scale_at);       // shifted to the exponent field of a double
+  short* const scales = reinterpret_cast<short*>(row_exp + 256);           // [slot][128 rows]
+  unsigned* const flags = reinterpret_cast<unsigned*>(scales + kPScaleSlots * 128);  // [slot][lane quarter]: rows in float64
+  float2* const maxima = reinterpret_cast<float2*>(flags + kPScaleSlots * 4);  // [slab parity][splitting group][128 rows]
+  uint64_t* const xy_full = reinterpret_cast<uint64_t*>(smem + plan.ctrl_at);
+  uint64_t* const xy_empty = xy_full + 1;                                  // [block]
+  uint64_t* const dig_full = xy_empty + kPMaxBlocks;
+  uint64_t* const dig_empty = dig_full + 2;
+  // [group][parity of its unit count]: with three groups both chunks in flight may hold a unit of the same group, and a
+  // parity wait must not find its barrier two phases ahead
+  uint64_t* const acc_full = dig_empty + 2;
+  uint64_t* const acc_empty = acc_full + 2 * kPMaxGroups;                  // [accumulator]
+  uint64_t* const e_full = acc_empty + 2;                                  // [group][stage], like the next two
+  uint64_t* const e_empty = e_full + kPMaxGroups * kPMaxStages;
+  uint64_t* const out_ready = e_empty + kPMaxGroups * kPMaxStages;
+  uint64_t* const pair_bar = out_ready + kPMaxGroups * kPMaxStages;        // [group][warp pair][written, read]
+  uint64_t* const drained = pair_bar + kPMaxGroups * 4;
+  uint64_t* const max_ready = drained + 1;
+  unsigned* const finished = reinterpret_cast<unsigned*>(max_ready + 1);     // [finishing warp]: units done
+  uint32_t* const tmem_slot = finished + 4 * kPMaxGroups;
+  static_assert((1 + kPMaxBlocks + 6 + 2 * kPMaxGroups + 3 * kPMaxGroups * kPMaxStages + 4 * kPMaxGroups + 2) * 8 + (4 * kPMaxGroups + 1) * 4 <= kPCtrlBytes,
+                "barrier area");
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform for the compiler
+  const int n = p.n, nb = tb.nb, groups = plan.groups, stages = plan.stages;
+  const unsigned limit = p.spin_limit;
+  const bool aligned = (s_addr(smem) & 127u) == 0;  // the TMA tiles and core matrices need it
+  {
+    const uint4* src = tb.blocks;
+    uint4* dst = reinterpret_cast<uint4*>(smem + plan.blocks_at);
+    for (int e = tid; e < tb.num_blocks * (kPBlockBytes / 16); e += blockDim.x) dst[e] = src[e];
+    for (int e = tid; e < 256; e += blockDim.x) row_exp[e] = e < n ? tb.row_exp[e] * (1 << 20) : 0;
+  }
+  if (tid == 0) {
+    bar_init(xy_full, 1);
+    for (int b = 0; b < kPMaxBlocks; ++b) bar_init(&xy_empty[b], 4);
+    for (int s = 0; s < 2; ++s) {
+      bar_init(&dig_full[s], kSplitWarps);
+      bar_init(&dig_empty[s], 1);
+      bar_init(&acc_empty[s], 8);
+    }
+    for (int s = 0; s < 2 * kPMaxGroups; ++s) bar_init(&acc_full[s], 1);
+    for (int s = 0; s < kPMaxGroups * kPMaxStages; ++s) {
+      bar_init(&e_full[s], 1);
+      bar_init(&e_empty[s], 1);
+      bar_init(&out_ready[s], 4);
+    }
+    for (int s = 0; s < kPMaxGroups * 4; ++s) bar_init(&pair_bar[s], 2);
+    bar_init(drained, 1);
+    bar_init(max_ready, kSplitWarps);
+    for (int w = 0; w < 4 * kPMaxGroups; ++w) finished[w] = 0;
+    fence_barrier_init();
+    if (!aligned) atomicExch(p.status, 2);
+  }
+  if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemColumns);
+  fence_async_shared();
+  tmem_fence_before();
+  __syncthreads();
+  tmem_fence_after();
+  constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
+
+  // this CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ...; chunk q = slab number * nb + output chunk,
+  // unit v = slab number * units + half chunk
+  const int my_slabs = aligned && *tmem_slot == 0 && blockIdx.x < p.num_slabs
+                           ? static_cast<int>((p.num_slabs - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+  const int units = (n + kPUnit - 1) / kPUnit, total = my_slabs * units;
+  auto slab_col = [&](int k) { return (static_cast<long long>(blockIdx.x) + static_cast<long long>(k) * gridDim.x) * kPS; };
+  auto warp_wait = [&](uint64_t* bar, int phase) {  // every lane polls the same barrier: no broadcast of the verdict
+    return __all_sync(0xffffffffu, bar_wait(bar, phase & 1, limit));
+  };
+
+  if (warp < kSplitWarps) {
+    // ---------------------------------------------------------------- splitting warps: thread = row of A = tensor memory lane
+    const int part = warp >> 2, quarter = warp & 3;
+    const bool tracker = quarter >= 2;
+    const int row = quarter * 32 + lane, coord = (quarter & 1) * 32 + lane;
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(quarter) << 21);
+    const bool idle = kMode == kModeDpsgd && tracker;  // D-PSGD has no tracker: its rows of A are never read back
+    const float* const col = xy_mem + (tracker ? kPTileFloats : 0) + coord;
+    const int first = part == 0 ? 0 : nb / 2, last = kBig || part == 1 ? nb : nb / 2;  // blocks of this group
+    bool ok = true;
+    for (int k = 0; k < my_slabs && ok; ++k) {
+      const int buf = k % kDigBuffers, slot = k % kPScaleSlots;
+      ok = warp_wait(xy_full, k);
+      if (!ok) break;
+      // largest magnitude, and the smallest of the largest magnitudes of eight consecutive workers
+      float top_f = 0.f, low_f = __uint_as_float(0x7f800000u);
+      if (!idle) {
+        for (int b = first; b < last; ++b) {
+          const float* src = col + b * (2 * kPTileFloats);
+#pragma unroll
+          for (int r = 0; r < 32; r += 8)
+            if (r < n - 32 * b) {  // rows beyond n within the eight arrive as zeros
+              const float m = max_abs3(max_abs3(src[r * kPS], src[(r + 1) * kPS], src[(r + 2) * kPS]),
+                                       max_abs3(src[(r + 3) * kPS], src[(r + 4) * kPS], src[(r + 5) * kPS]),
+                                       max_abs3(src[(r + 6) * kPS], src[(r + 7) * kPS], 0.f));
+              top_f = max_abs3(top_f, m, m);
+              if (r + 8 <= n - 32 * b) low_f = fminf(low_f, m);
+            }
+        }
+      }
+      if (!kBig) {  // the other group's blocks
+        float2* const mx = maxima + (k & 1) * 256 + row;  // read again two slabs later, behind the next hand-over
+        mx[part * 128] = make_float2(top_f, low_f);
+        __syncwarp();
+        if (lane == 0) bar_arrive(max_ready);
+        ok = warp_wait(max_ready, k);
+        if (!ok) break;
+        const float2 other = mx[(part ^ 1) * 128];
+        top_f = max_abs3(top_f, other.x, other.x);
+        low_f = fminf(low_f, other.y);
+      }
+      const unsigned top = __float_as_uint(top_f), low = __float_as_uint(low_f);
+      // as float bits: not finite; too small for the scale; eight workers in a row all more than 2^10 below the largest
+      const bool exact = top >= 0x7f800000u || (top != 0 && (top < kSmallest || (tb.sparse != 0 && low + (10u << 23) < top)));
+      const int e = top == 0 || exact ? 30 : static_cast<int>((top + kRoundUp) >> 23) - 127;  // all |z| < 2^(e+1)
+      const float scale = __uint_as_float(static_cast<unsigned>(157 - e) << 23);              // 2^(30 - e)
+      const unsigned exact_lanes = __ballot_sync(0xffffffffu, exact);
+      const bool any_exact = exact_lanes != 0;
+      if (k >= kDigBuffers) ok = warp_wait(&dig_empty[buf], k / kDigBuffers - 1);
+      if (!ok) break;
+      tmem_fence_after();
+      // The slot was last read for slab k - 4: a finishing group reads a unit's scales before it releases the
+      // accumulators, and the MMAs of slab k - 2 (complete: dig_empty) came after that release for all units of k - 4.
+      if (part == 0) {
+        scales[slot * 128 + row] = static_cast<short>(exact ? 0 : e - 6);
+        if (lane == 0) flags[slot * 4 + quarter] = exact_lanes;
+      }
+      for (int b = first; b < last; ++b) {
+        if (!idle) {
+          uint32_t w[32];  // digit plane l of this row's 32 workers in words 8 l .. 8 l + 7
+          const float* src = col + b * (2 * kPTileFloats);
+          const int rows = n - 32 * b;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            w[u] = w[8 + u] = w[16 + u] = w[24 + u] = 0u;
+            if (4 * u < rows) {  // rows beyond n within the four arrive as zeros
+              uint32_t z[4];
+#pragma unroll
+              for (int v = 0; v < 4; ++v)  // balanced digits: q + 0x80808080 has them as bytes offset by 128
+                z[v] = static_cast<uint32_t>(__float2int_rn(src[(4 * u + v) * kPS] * scale)) + 0x80808080u;
+              const uint32_t ab = __byte_perm(z[0], z[1], 0x5140), cd = __byte_perm(z[2], z[3], 0x5140);
+              const uint32_t ef = __byte_perm(z[0], z[1], 0x7362), gh = __byte_perm(z[2], z[3], 0x7362);
+              w[u] = __byte_perm(ab, cd, 0x5410) ^ 0x80808080u;
+              w[8 + u] = __byte_perm(ab, cd, 0x7632) ^ 0x80808080u;
+              w[16 + u] = __byte_perm(ef, gh, 0x5410) ^ 0x80808080u;
+              w[24 + u] = __byte_perm(ef, gh, 0x7632) ^ 0x80808080u;
+            }
+          }
+          tmem_store32(lane_base + buf * 128 + b * 32, w);
+        }
+        __syncwarp();
+        if (lane == 0 && !any_exact) bar_arrive(&xy_empty[b]);  // the loads of the next slab follow block by block
+      }
+      tmem_wait_store();
+      tmem_fence_before();
+      __syncwarp();
+      if (lane == 0) bar_arrive(&dig_full[buf]);
+      if (any_exact) {  // the finishing warps read these rows' operands themselves: keep the slab until they are done with it
+        if (lane == 0) {
+          for (int t = 0; t < groups && ok; ++t) {
+            const unsigned need = static_cast<unsigned>(((k + 1) * units - t + groups - 1) / groups);
+            for (int v = 0; v < 4 && ok; ++v) ok = count_wait(&finished[4 * t + v], need, limit);
+          }
+          for (int b = first; b < last && ok; ++b) bar_arrive(&xy_empty[b]);
+        }
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      }
+    }
+    if (!ok && lane == 0) atomicExch(p.status, 1);
+  } else if (warp >= kFinishWarp) {
+    // ---------------------------------------------------------------- finishing warps
+    const int t = (warp - kFinishWarp) >> 2, quarter = warp & 3;
+    const bool second = quarter >= 2;  // reads the tracker rows; finishes workers 8..15 of every sixteen
+    const int pair = quarter & 1, coord = pair * 32 + lane, mine = second ? 8 : 0;
+    const uint32_t acc_lane = tmem + kAccColumn + (static_cast<uint32_t>(quarter) << 21);
+    float* const e_group = e_mem + static_cast<size_t>(t) * stages * (kPStageBytes / 4) + coord;
+    uint64_t* const written = &pair_bar[4 * t + 2 * pair];
+    uint64_t* const taken = written + 1;
+    const double alpha = p.alpha;
+    const float sigma = static_cast<float>(p.sigma);
+    const bool noisy = p.sigma != 0.0, at_start = p.grad_at_start != 0;
+    const long long d_tma = p.d & ~3LL;  // columns below this are written by the TMA stores
+    int k = 0, h = t, st = 0, st_phase = 0, m = 0;
+    while (h >= units) {
+      h -= units;
+      ++k;
+    }
+    bool ok = true;
+    for (int v = t; v < total && t < groups; v += groups, ++m) {
+      const int q = k * nb + (h >> 1);
+      ok = warp_wait(&acc_full[2 * t + (m & 1)], m >> 1) && warp_wait(&e_full[t * kPMaxStages + st], st_phase);
+      if (!ok) break;
+      tmem_fence_after();
+      const int slot = k % kPScaleSlots;
+      const unsigned exact_lanes = flags[slot * 4 + quarter];
+      const long long j = slab_col(k) + coord;
+      const int w0 = kPUnit * h + mine;  // first of this thread's eight workers
+      float* const sg = e_group + st * (kPStageBytes / 4) + mine * kPS;
+      float* const sa = sg + kPStageFloats;
+      float* const sc = sa + kPStageFloats;
+      float gold[8], av[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        gold[u] = sg[u * kPS];
+        av[u] = sa[u * kPS];
+      }
+      // ---- sums of sixteen workers: eight handed to the other warp of the pair, eight kept
+      double own[8];
+      const int ex = (scales[slot * 128 + coord] + 1023) << 20, ey = (scales[slot * 128 + 64 + coord] + 1023) << 20;
+      int er[8];
+      *reinterpret_cast<int4*>(&er[0]) = *reinterpret_cast<const int4*>(row_exp + w0);
+      *reinterpret_cast<int4*>(&er[4]) = *reinterpret_cast<const int4*>(row_exp + w0 + 4);
+      {
+        const uint32_t acc = acc_lane + (q & 1) * 128 + (h & 1) * kPUnit;
+        int s[kPWeights][8];
+        if (kMode != kModeDpsgd || !second) {
+#pragma unroll
+          for (int w = 0; w < kPWeights; ++w) tmem_load8(acc + w * 32 + (mine ^ 8), s[w]);
+          tmem_wait_load();
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const double give = join_sums<kBig>(s[0][u], s[1][u], s[2][u], s[3][u]);
+            sg[u * kPS] = __int_as_float(__double2hiint(give));
+            sa[u * kPS] = __int_as_float(__double2loint(give));
+          }
+        }
+#pragma unroll
+        for (int w = 0; w < kPWeights; ++w) tmem_load8(acc + w * 32 + mine, s[w]);
+        tmem_wait_load();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) own[u] = join_sums<kBig>(s[0][u], s[1][u], s[2][u], s[3][u]);
+      }
+      if (exact_lanes != 0) {
+        // Rows of this warp that were not split: their sums in float64 from the operands themselves, one row after the
+        // other.  Lanes i and i + 16 sum output worker i of the sixteen over the even and the odd input workers (sixteen
+        // entries of P side by side, eight reads in flight).  The sums replace the integer ones, in units of the scales.
+        const float* const z = xy_mem + (second ? kPTileFloats : 0) + pair * 32;
+        const int c = h >> 1, pitch = tb.circulant ? kPChunk : units * kPUnit;
+        const double* const column = tb.poly_t + (tb.circulant ? kPUnit * (h & 1) : kPUnit * h) + (lane & 15);
+        const int to_units = (2046 << 20) - row_exp[kPUnit * h + (lane & 15)];
+        for (unsigned left = exact_lanes; left != 0; left &= left - 1) {
+          const int src = __ffs(left) - 1;
+          double sum = 0.0;
+          for (int b = 0; b < nb; ++b) {
+            if (static_cast<uint8_t>(tb.id[c] >> (8 * b)) == 0xffu) continue;  // a zero block of P
+            const int pb = !tb.circulant ? b : b >= c ? b - c : b - c + nb;  // block row 0 holds them all
+#pragma unroll 8
+            for (int w = lane >> 4; w < 32; w += 2) {
+              const double pw = column[static_cast<size_t>(32 * pb + w) * pitch];
+              const float zw = z[b * (2 * kPTileFloats) + w * kPS + src];
+              sum = fma(pw, static_cast<double>(pw != 0.0 ? zw : 0.f), sum);  // a zero of P must not make an infinity NaN
+            }
+          }
+          sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+          sum *= __hiloint2double(to_units - __shfl_sync(0xffffffffu, second ? ey : ex, src), 0);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const double keep = __shfl_sync(0xffffffffu, sum, mine + u), give = __shfl_sync(0xffffffffu, sum, (mine ^ 8) + u);
+            if (lane == src) {
+              own[u] = keep;
+              sg[u * kPS] = __int_as_float(__double2hiint(give));
+              sa[u * kPS] = __int_as_float(__double2loint(give));
+            }
+          }
+        }
+      }
+      tmem_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        bar_arrive(written);
+        bar_arrive(&acc_empty[q & 1]);
+        if (h + 1 == units && (h & 1) == 0) bar_arrive(&acc_empty[q & 1]);  // there is no other half of this chunk
+      }
+      // ---- normals of this thread's eight workers, while the other warp arrives
+      float xi[8];
+      if (noisy) {
+        const unsigned long long jn = static_cast<unsigned long long>(p.coord_offset + j);
+#pragma unroll
+        for (int u = 0; u < 8; u += 4) {
+          float quad[4];
+          normal_quad(p.round_key, jn, static_cast<uint32_t>((w0 + u) >> 2), p.t_noise, quad);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) xi[u + i] = sigma * quad[i];
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) xi[u] = 0.f;
+      }
+      ok = warp_wait(written, m);
+      if (!ok) break;
+      // ---- gossiped model and tracker (over `own`), model update, y~ - g
+      const float* const og = sg + (second ? -8 * kPS : 8 * kPS);  // the other warp's slots
+      double xd[8], yg[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const double other = (kMode != kModeDpsgd || second)
+                                 ? __hiloint2double(__float_as_int(og[u * kPS]), __float_as_int(og[kPStageFloats + u * kPS])) : 0.0;
+        const double xt = (second ? other : own[u]) * __hiloint2double(ex + er[u], 0);
+        const double yt = (second ? own[u] : other) * __hiloint2double(ey + er[u], 0);
+        const double gd = static_cast<double>(gold[u]);
+        xd[u] = fma(-alpha, kMode == kModeDpsgd ? gd : yt, xt);
+        yg[u] = yt - gd;
+        own[u] = yt;
+      }
+      if (kMode != kModeDpsgd && p.y_obs != nullptr) {  // optional observer: the gossiped tracker
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (w0 + u < n && j < p.d) p.y_obs[static_cast<long long>(w0 + u) * p.ld + j] = static_cast<float>(own[u]);
+      }
+      __syncwarp();
+      if (lane == 0) bar_arrive(taken);
+      // ---- gradient at the new model, or at the one the step started from - still in global memory, this unit's rows
+      // are stored after this - and fold; the results go over g, a, c
+      float at[8], go[8], xo[8], yo[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) at[u] = xo[u] = static_cast<float>(xd[u]);
+      if (at_start) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          at[u] = w0 + u < n && j < p.d ? p.x[static_cast<long long>(w0 + u) * p.ld + j] : 0.f;
+          if (kWide) xd[u] = static_cast<double>(at[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const float cv = sc[u * kPS];
+        go[u] = kWide ? static_cast<float>(fma(static_cast<double>(av[u]), xd[u] - static_cast<double>(cv), static_cast<double>(xi[u])))
+                      : fmaf(av[u], at[u] - cv, xi[u]);
+        yo[u] = static_cast<float>(yg[u] + static_cast<double>(go[u]));
+      }
+      ok = warp_wait(taken, m);
+      if (!ok) break;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        sg[u * kPS] = go[u];
+        sa[u * kPS] = xo[u];
+        if (kMode != kModeDpsgd) sc[u * kPS] = yo[u];
+      }
+      if (j >= d_tma && j < p.d) {  // TMA clips a store at 16-byte granularity: the last d % 4 columns are written here
+        for (int u = 0; u < 8 && w0 + u < n; ++u) {
+          const long long off = static_cast<long long>(w0 + u) * p.ld + j;
+          p.g[off] = sg[u * kPS];
+          p.x[off] = sa[u * kPS];
+          if (kMode != kModeDpsgd) p.y[off] = sc[u * kPS];
+        }
+      }
+      fence_async_shared();  // results visible to the TMA stores
+      __syncwarp();
+      if (lane == 0) {
+        bar_arrive(&out_ready[t * kPMaxStages + st]);
+        // relaxed: what a reader of the count waits for, this unit's reads of x and y, went into the results above
+        *const_cast<volatile unsigned*>(&finished[warp - kFinishWarp]) = static_cast<unsigned>(m + 1);
+      }
+      if (++st == stages) {
+        st = 0;
+        ++st_phase;
+      }
+      h += groups;
+      while (h >= units) {
+        h -= units;
+        ++k;
+      }
+    }
+    if (!ok && lane == 0) atomicExch(p.status, 1);
+  } else if (warp == kMmaWarp) {
+    // ---------------------------------------------------------------- MMAs
+    // The whole warp walks the loop, one lane issues: operands computed in uniform control flow stay in uniform registers
+    // (issued from inside a one-lane branch each MMA cost 127 cycles, eight times its time on the tensor cores).
+    const uint32_t b_base = s_addr(smem + plan.blocks_at);
+    const bool leader = lane == 0;
+    bool ok = true;
+    int q = 0, t = 0, turn = 0;  // t, turn: group of the next unit and the parity of how many it has had
+    auto hand_over = [&]() {     // the group waits for all MMAs issued so far
+      mma_commit(&acc_full[2 * t + turn], leader);
+      if (++t == groups) {
+        t = 0;
+        turn ^= 1;
+      }
+    };
+    for (int k = 0; k < my_slabs && ok; ++k) {
+      const int buf = k % kDigBuffers;
+      ok = warp_wait(&dig_full[buf], k / kDigBuffers);
+      for (int c = 0; c < nb && ok; ++c, ++q) {
+        if (q >= 2) ok = warp_wait(&acc_empty[q & 1], (q >> 1) - 1);
+        if (!ok) break;
+        tmem_fence_after();
+        const uint32_t acc = tmem + kAccColumn + (q & 1) * 128;
+        unsigned add = 0;  // the first product of an accumulator clears it
+        uint64_t ids = tb.id[c];
+        for (int kb = 0; kb < nb; ++kb, ids >>= 8) {
+          const uint32_t id = static_cast<uint32_t>(ids) & 0xffu;
+          if (id == 0xffu) continue;
+          const uint32_t a = tmem + buf * 128 + kb * 32;
+          const uint64_t b = mma_operand(b_base + id * kPBlockBytes, 256, 128);
+          constexpr int kPlane = kPPlaneBytes / 16;  // planes from b on: zeros, digits 3, 2, 1, 0
+          mma_i8(acc, a + 24, b + 1 * kPlane, kMmaI8Desc128x64, add, leader);      // 3: (3 2) -> weights 6, 5
+          mma_i8(acc + 64, a + 24, b + 3 * kPlane, kMmaI8Desc128x64, add, leader);  //    (1 0) -> 4, 3
+          mma_i8(acc, a + 16, b, kMmaI8Desc128x64, 1u, leader);                     // 2: (- 3) -> 6, 5
+          mma_i8(acc + 64, a + 16, b + 2 * kPlane, kMmaI8Desc128x64, 1u, leader);   //    (2 1) -> 4, 3
+          mma_i8(acc + 64, a + 8, b + 1 * kPlane, kMmaI8Desc128x64, 1u, leader);    // 1: (3 2) -> 4, 3
+          mma_i8(acc + 64, a, b, kMmaI8Desc128x64, 1u, leader);                     // 0: (- 3) -> 4, 3
+          add = 1;
+        }
+        hand_over();
+        if (2 * c + 1 < units) hand_over();
+      }
+      if (ok) mma_commit(&dig_empty[buf], leader);
+    }
+    if (!ok) {  // nothing may be in flight when the tensor memory is given back
+      if (leader) atomicExch(p.status, 1);
+      mma_commit(drained, leader);
+      warp_wait(drained, 0);
+    }
+  } else if (warp == kLoadXYWarp) {
+    if (lane == 0) {
+      const unsigned bytes = (kMode == kModeDpsgd ? 1u : 2u) * nb * kPTileFloats * 4u;
+      int k = 0;
+      bool ok = true;
+      for (; k < my_slabs && ok; ++k) {
+        if (p.stall_after >= 0 && static_cast<long long>(k) * units >= p.stall_after) break;  // self test: the loads stop
+        const int col = static_cast<int>(slab_col(k));
+        for (int b = 0; b < nb; ++b) {
+          if (k > 0) ok = bar_wait(&xy_empty[b], (k - 1) & 1, limit);
+          if (!ok) break;
+          if (b == 0) bar_expect_tx(xy_full, bytes);
+          float* dst = xy_mem + b * (2 * kPTileFloats);
+          tile_load(dst, &maps.x, col, 32 * b, xy_full);
+          if (kMode != kModeDpsgd) tile_load(dst + kPTileFloats, &maps.y, col, 32 * b, xy_full);
+        }
+      }
+      if (!ok) atomicExch(p.status, 1);
+      if (k > 0) bar_wait(xy_full, (k - 1) & 1, limit);  // nothing in flight when the CTA leaves (bounded)
+    }
+    __syncwarp();
+  } else if (warp == kLoadEWarp) {
+    if (lane == 0) {
+      int v = 0, k = 0, h = 0, t = 0, st = 0, phase = 0;  // group and stage of unit v; phase = uses of the stage so far
+      bool ok = true;
+      for (; v < total; ++v) {
+        if (p.stall_after >= 0 && v >= p.stall_after) break;
+        const int s = t * kPMaxStages + st;
+        if (phase > 0) ok = bar_wait(&e_empty[s], (phase - 1) & 1, limit);
+        if (!ok) break;
+        float* dst = e_mem + static_cast<size_t>(t * stages + st) * (kPStageBytes / 4);
+        const int col = static_cast<int>(slab_col(k));
+        bar_expect_tx(&e_full[s], kPStageBytes);
+        tile_load(dst, &maps.g, col, kPUnit * h, &e_full[s]);
+        tile_load(dst + kPStageFloats, &maps.a, col, kPUnit * h, &e_full[s]);
+        tile_load(dst + 2 * kPStageFloats, &maps.c, col, kPUnit * h, &e_full[s]);
+        if (++t == groups) {
+          t = 0;
+          if (++st == stages) {
+            st = 0;
+            ++phase;
+          }
+        }
+        if (++h == units) {
+          h = 0;
+          ++k;
+        }
+      }
+      if (!ok) atomicExch(p.status, 1);
+      for (int back = 1; back <= groups * stages && back <= v; ++back) {
+        const int z = v - back, u = z / groups;
+        bar_wait(&e_full[(z % groups) * kPMaxStages + u % stages], (u / stages) & 1, limit);
+      }
+    }
+    __syncwarp();
+  } else if (warp == kStoreWarp) {
+    if (lane == 0) {
+      int k = 0, h = 0, t = 0, st = 0, phase = 0;
+      for (int v = 0; v < total; ++v) {
+        const int s = t * kPMaxStages + st;
+        if (!bar_wait(&out_ready[s], phase & 1, limit)) {
+          atomicExch(p.status, 1);
+          break;
+        }
+        const float* src = e_mem + static_cast<size_t>(t * stages + st) * (kPStageBytes / 4);  // now g' | x' | y'
+        const long long col = slab_col(k);
+        if (col < (p.d & ~3LL)) {
+          tile_store(&maps.gs, static_cast<int>(col), kPUnit * h, src);
+          tile_store(&maps.xs, static_cast<int>(col), kPUnit * h, src + kPStageFloats);
+          if (kMode != kModeDpsgd) tile_store(&maps.ys, static_cast<int>(col), kPUnit * h, src + 2 * kPStageFloats);
+        }
+        store_commit();
+        store_wait_read();  // the stage may be refilled now
+        bar_arrive(&e_empty[s]);
+        if (++t == groups) {
+          t = 0;
+          if (++st == stages) {
+            st = 0;
+            ++phase;
+          }
+        }
+        if (++h == units) {
+          h = 0;
+          ++k;
+        }
+      }
+      store_wait_all();
+    }
+    __syncwarp();
+  }
+  tmem_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    tmem_fence_after();
+    tmem_free(tmem, kTmemColumns);
+  }
+}
+
+typedef void (*SplitKernel)(const StepParams, const SplitMaps, const SplitTables, const SplitPlan);
+
+template <bool kBig>
+SplitKernel pick_split(const StepParams& p, bool wide) {
+  if (p.mode == kModeDpsgd)
+    return wide ? step_split_kernel<kModeDpsgd, true, kBig> : step_split_kernel<kModeDpsgd, false, kBig>;
+  return wide ? step_split_kernel<kModeDetag, true, kBig> : step_split_kernel<kModeDetag, false, kBig>;
+}
+
+}  // namespace
+
+// Digits of P: distinct 32 x 32 blocks, their table and the rows' exponents.  `poly`: the n x n matrix, or (circulant: the
+// blocks depend on their distance only) its first 32 rows.  Leaves `out` empty when the kernel does not take the matrix:
+// n outside 33 .. 256, an entry or a row that cannot be scaled, too many distinct blocks.
+void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out) {
+  out = SplitPoly{};
+  if (n <= 32 || n > 256 || encode_tiled_fn() == nullptr) return;
+  const int nb = (n + kPChunk - 1) / kPChunk, rows = circulant ? kPChunk : n;
+  std::vector<uint32_t> digits(static_cast<size_t>(circulant ? 1 : nb) * kPChunk * nb * kPChunk, 0);  // balanced digits as bytes
+  std::vector<int32_t> row_exp(n);
+  bool sparse = false;
+  for (int i = 0; i < rows; ++i) {
+    const double* row = &poly[static_cast<size_t>(i) * n];
+    double top = 0.0, low = 1e300;
+    for (int j = 0; j < n; ++j) {
+      const double v = std::fabs(row[j]);
+      if (!(v <= 1e30)) return;  // also NaN
+      top = v > top ? v : top;
+      low = v < low ? v : low;
+    }
+    if (!(top >= 1e-30)) return;
+    sparse = sparse || low < top / 256.0;
+    int e = std::ilogb(top);
+    if (std::nearbyint(std::ldexp(top, 30 - e)) > kMaxDigit) ++e;
+    for (int k = i; k < n; k += rows) row_exp[k] = e - 30;
+    const double scale = std::ldexp(1.0, 30 - e);
+    uint32_t* out_row = &digits[static_cast<size_t>(i) * nb * kPChunk];
+    for (int j = 0; j < n; ++j)
+      out_row[j] = (static_cast<uint32_t>(static_cast<int32_t>(std::lrint(row[j] * scale))) + 0x80808080u) ^ 0x80808080u;
+  }
+  std::vector<unsigned char> blocks;
+  unsigned char id[64];  // [output chunk][input block]
+  std::memset(id, 255, sizeof id);
+  std::vector<unsigned char> block(kPBlockBytes);
+  for (int c = 0; c < (circulant ? 1 : nb); ++c)
+    for (int kb = 0; kb < nb; ++kb) {
+      uint32_t any = 0;
+      for (int r = 0; r < kPChunk; ++r) {
+        const uint32_t* src = &digits[(static_cast<size_t>(c) * kPChunk + r) * nb * kPChunk + kb * kPChunk];
+        // core matrices of 8 rows x 16 bytes, the two of a row group side by side
+        unsigned char* at = &block[(r / 8) * 256 + (r % 8) * 16];
+        for (int w = 0; w < kPChunk; ++w) {
+          any |= src[w];
+          for (int l = 0; l < 4; ++l)
+            at[(4 - l) * kPPlaneBytes + (w / 16) * 128 + w % 16] = static_cast<unsigned char>(src[w] >> (8 * l));
+        }
+      }
+      if (any == 0) continue;
+      const int have = static_cast<int>(blocks.size() / kPBlockBytes);
+      int hit = 0;
+      while (hit < have && std::memcmp(&blocks[static_cast<size_t>(hit) * kPBlockBytes], block.data(), kPBlockBytes) != 0) ++hit;
+      if (hit == have) {
+        if (split_plan(nb, have + 1).bytes == 0) return;
+        blocks.insert(blocks.end(), block.begin(), block.end());
+      }
+      id[c * 8 + kb] = static_cast<unsigned char>(hit);
+    }
+  if (circulant)
+    for (int c = 1; c < nb; ++c)
+      for (int kb = 0; kb < nb; ++kb) id[c * 8 + kb] = id[(kb - c + nb) % nb];
+  const size_t pitch = circulant ? kPChunk : static_cast<size_t>((n + kPUnit - 1) / kPUnit) * kPUnit;
+  out.poly_t.assign(nb * kPChunk * pitch, 0.0);
+  for (int i = 0; i < rows; ++i)
+    for (int j = 0; j < n; ++j) out.poly_t[j * pitch + i] = poly[static_cast<size_t>(i) * n + j];
+  out.blocks.swap(blocks);
+  out.row_exp.swap(row_exp);
+  out.sparse = sparse;
+  out.circulant = circulant;
+  std::memcpy(out.id, id, sizeof id);
+}
+
+bool build_maps_split(const StepParams& p, TensorMapSet* out) {
+  SplitMaps& m = *reinterpret_cast<SplitMaps*>(out->bytes);
+  const float* y = p.mode == kModeDpsgd ? p.x : p.y;  // D-PSGD has no tracker: those maps are never used
+  if (!make_map(&m.x, p.x, p.n, p.d, p.ld, kPChunk, kPS) || !make_map(&m.y, y, p.n, p.d, p.ld, kPChunk, kPS) ||
+      !make_map(&m.g, p.g, p.n, p.d, p.ld, kPUnit, kPS) || !make_map(&m.a, p.a, p.n, p.d, p.ld, kPUnit, kPS) ||
+      !make_map(&m.c, p.c, p.n, p.d, p.ld, kPUnit, kPS))
+    return false;
+  const long long d_tma = p.d & ~3LL;  // the stores' tensor ends on a 16-byte boundary
+  if (d_tma > 0 && (!make_map(&m.xs, p.x, p.n, d_tma, p.ld, kPUnit, kPS) ||
+                    !make_map(&m.ys, y, p.n, d_tma, p.ld, kPUnit, kPS) || !make_map(&m.gs, p.g, p.n, d_tma, p.ld, kPUnit, kPS)))
+    return false;
+  if (d_tma == 0) m.xs = m.ys = m.gs = m.x;  // never used
+  return true;
+}
+
+int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const void* blocks, const int32_t* row_exp,
+                      const double* poly_t, bool wide, int sm_count, cudaStream_t stream) {
+  if (p.mode == kModeExternal || poly.blocks.empty()) return static_cast<int>(cudaErrorInvalidValue);
+  p.S = kPS;
+  p.num_slabs = (p.d + kPS - 1) / kPS;
+  SplitTables tb{};
+  tb.blocks = static_cast<const uint4*>(blocks);
+  tb.row_exp = row_exp;
+  tb.poly_t = poly_t;
+  tb.sparse = poly.sparse ? 1 : 0;
+  tb.circulant = poly.circulant ? 1 : 0;
+  tb.num_blocks = static_cast<int>(poly.blocks.size() / kPBlockBytes);
+  tb.nb = (p.n + kPChunk - 1) / kPChunk;
+  std::memcpy(tb.id, poly.id, sizeof tb.id);
+  const SplitPlan plan = split_plan(tb.nb, tb.num_blocks);
+  const SplitKernel kernel = p.n > 128 ? pick_split<true>(p, wide) : pick_split<false>(p, wide);
+  const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(plan.bytes));
+  if (e != 0) return e;
+  const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;
+  if (grid <= 0) return 0;
+  kernel<<<static_cast<unsigned>(grid), kPThreads, plan.bytes, stream>>>(
+      p, *reinterpret_cast<const SplitMaps*>(maps.bytes), tb, plan);
+  return static_cast<int>(cudaGetLastError());
+}
+
+}  // namespace detag

@@ -263,7 +263,7 @@ step_wide_kernel(const StepParams p, const __grid_constant__ WideMaps maps, cons
     // 8 block + 4 (i & 1) + kq in tile (i >> 1).
     auto draw = [&](int pair, float (&xi)[4]) {
       const unsigned long long jn = static_cast<unsigned long long>(p.coord_offset + j0 + pair * 16 + (kq >> 1) * 8 + crow);
-      normal_quad(p.seed_lo, p.seed_hi, jn, quad, p.t_noise, xi);
+      normal_quad(p.round_key, jn, quad, p.t_noise, xi);
       transpose_quad(xi, kq);
     };
     // Element-wise tail of the pair: model update, gradient, tracker fold; g', x', y' go over g, a, c.

@@ -1,0 +1,170 @@
+"""The polynomial on the integer tensor path (32 < n <= 256): tile edges, block structures, modes, and the coordinates it
+contracts in float64 instead (values too far apart for one scale, infinities, NaN)."""
+import numpy as np
+import pytest
+
+from oracle import detag_oracle as orc
+from paper_2006_08085_b200 import binding as B
+from paper_2006_08085_b200 import build, inputs
+from paper_2006_08085_b200.session import Session
+from parity import HALF_ULP32, one_step_from_rounded_state, oracle_problem, worst_ratio
+
+pytestmark = pytest.mark.gpu
+
+SLABS = 64 * 148  # one slab of 64 coordinates per block
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def _graph(kind, n):
+    if kind == "ring":
+        return inputs.metropolis_weights(inputs.ring_graph(n))
+    if kind == "torus":
+        return inputs.metropolis_weights(inputs.torus_graph(n // 16, 16))
+    if kind == "path":
+        return inputs.metropolis_weights(inputs.path_graph(n))
+    if kind == "directed":
+        return inputs.directed_cycle_blend(n, 0.4, 0.35)
+    return inputs.metropolis_weights(inputs.random_regular4_graph(n, n))
+
+
+def _data(n, d, seed):
+    rng = np.random.default_rng(seed)
+    a = rng.uniform(0.5, 2.0, (n, d)).astype(np.float32)
+    c = (0.1 * (rng.standard_normal((n, d)) + np.arange(n)[:, None] - n / 2)).astype(np.float32)
+    return a, c, rng.standard_normal((n, d)).astype(np.float32)
+
+
+# n: one worker beyond a block, whole blocks, a last unit of one worker, an odd number of half chunks; d: below, at and
+# beyond a slab, tails of 1 .. 3 columns, several slabs per block of the grid
+@pytest.mark.parametrize("n,d,K,kind,at_start", [
+    (33, 1, 2, "regular4", False), (48, 63, 3, "regular4", True), (49, 2 * SLABS + 66, 2, "path", False),
+    (64, 64, 5, "ring", False), (65, 65, 3, "directed", True), (81, 5 * SLABS + 3, 4, "regular4", False),
+    (113, 130, 6, "regular4", False), (128, 3 * SLABS + 31, 9, "regular4", True), (160, 97, 12, "ring", False),
+    (224, 2 * SLABS + 2, 40, "ring", False), (256, 131, 16, "torus", True), (256, 3 * SLABS + 7, 16, "torus", False),
+    (256, 2 * SLABS + 65, 16, "ring", False)])
+def test_one_step_against_the_oracle(n, d, K, kind, at_start):
+    m = _graph(kind, n)
+    eta = 0.3
+    cols = np.unique(np.concatenate([np.arange(min(d, 70)), np.arange(max(0, d - 70), d),
+                                     np.random.default_rng(1).integers(0, d, 60)]))
+    a, c, x0 = _data(n, d, n + d)
+    # the oracle on a sample of the columns (the step never mixes them), the noise index of each being its column
+    ref = {}
+    for lo, hi in _runs(cols):
+        p = oracle_problem(m, K, eta, 0.02, a[:, lo:hi], c[:, lo:hi], 0.1, 11, lo)
+        if at_start:
+            s = orc.PhaseState(x0[:, lo:hi].astype(np.float64), a[:, lo:hi].astype(np.float64),
+                               c[:, lo:hi].astype(np.float64), 0)
+            out = orc.phase_as_printed(p, s)
+            g = orc.stochastic_gradient(p, s.x, 1)
+            ref[lo, hi] = (out.x, None, g, out.y)
+        else:
+            ref[lo, hi] = one_step_from_rounded_state(p, x0[:, lo:hi])
+    with Session(m, d, K, eta, 0.02, a, c, x0, 0.1, 11, observe_gossip=True,
+                 gradient_point=int(at_start)) as s:
+        if at_start:  # any tracker and gradient will do: the objective's arrays
+            s.upload("y", a)
+            s.upload("g", c)
+            B.detag_set_step(s.state, 0)
+        else:
+            s.init()
+        s.step()
+        s.status()
+        got = {k: s.download(k) for k in ("x", "y_gossip", "g", "y")}
+    for (lo, hi), want in ref.items():
+        x, yg, g, yf = want if at_start else want[1]
+        cut = {k: v[:, lo:hi] for k, v in got.items()}
+        assert worst_ratio(cut["x"], x) <= 1.0, (lo, "x")
+        assert worst_ratio(cut["g"], g) <= 1.0, (lo, "g")
+        assert worst_ratio(cut["y"], yf, extra=HALF_ULP32 * np.abs(g)) <= 1.0, (lo, "y")
+        if yg is not None:
+            assert worst_ratio(cut["y_gossip"], yg) <= 1.0, (lo, "y_gossip")
+
+
+def _runs(cols):
+    """Consecutive stretches [lo, hi) of a sorted column list."""
+    cuts = np.flatnonzero(np.diff(cols) > 1) + 1
+    return [(int(r[0]), int(r[-1]) + 1) for r in np.split(cols, cuts)]
+
+
+@pytest.mark.parametrize("n,kind,K", [(40, "ring", 2), (100, "regular4", 2), (100, "regular4", 8), (256, "ring", 9)])
+def test_values_far_apart_keep_their_precision(n, kind, K):
+    """A few workers a million times larger than the rest: results out of their reach must not inherit their scale.  A
+    float64 sum rounded once to float32 is off by half an ulp, 2^-24 of itself, and that is all in those columns if the
+    polynomial has entries below 2^-8 of their row's largest (they are contracted in float64).  Elsewhere the dropped digit
+    pairs add, per term, three products of uniform digits (standard deviation 74) at 2^16 of 2^62 times the two scales,
+    each up to twice the largest operand or entry: 2^-27 of those for 256 terms, bounded by six deviations."""
+    d, eta = 200, 0.2
+    m = _graph(kind, n)
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal((n, d)).astype(np.float32)
+    x[:3, ::7] *= 1e6
+    x[:, 5] = 0.0
+    x[:, 12] = 0.0
+    x[7, 12] = 3e-39  # the only value of its column: below the range of the scale
+    zero = np.zeros((n, d), np.float32)
+    with Session(m, d, K, eta, 0.0, zero, zero, x) as s:
+        s.step()
+        s.status()
+        got = s.download("x").astype(np.float64)
+    x = x.astype(np.float64)
+    top = np.abs(P).max(axis=1, keepdims=True)
+    bound = 2.0 ** -24 * np.abs(P @ x) + 2.0 ** -45 * (np.abs(P) @ np.abs(x)) + 1e-45
+    split = np.ones(d, bool)
+    split[::7] = not (np.abs(P) < top / 256).any()
+    bound += np.where(split, 2.0 ** -24.4 * top * np.abs(x).max(axis=0), 0.0)
+    assert (np.abs(got - P @ x) <= bound).all()
+    assert (got[:, 5] == 0.0).all()
+
+
+@pytest.mark.parametrize("n,bad", [(48, np.inf), (100, np.nan), (256, -np.inf)])
+def test_what_is_not_finite_stays_in_reach(n, bad):
+    d, K, eta = 130, 2, 0.2
+    m = _graph("ring", n)
+    P = _polynomial(m, K, eta)
+    x = np.random.default_rng(n).standard_normal((n, d)).astype(np.float32)
+    x[9, 70] = bad
+    zero = np.zeros((n, d), np.float32)
+    with Session(m, d, K, eta, 0.0, zero, zero, x) as s:
+        s.step()
+        s.status()
+        got = s.download("x")
+    reached = P[:, 9] != 0.0
+    assert not np.isfinite(got[reached, 70]).any()
+    keep = np.ones((n, d), bool)
+    keep[reached, 70] = False
+    x[9, 70] = 0.0
+    assert worst_ratio(got[keep], (P @ x.astype(np.float64))[keep]) <= 1.0
+
+
+def _polynomial(m, K, eta):
+    w = m.to_dense()
+    prev = cur = np.eye(m.n)
+    for _ in range(K):
+        prev, cur = cur, (1.0 + eta) * w @ cur - eta * prev
+    return cur
+
+
+@pytest.mark.parametrize("n,d", [(70, 67), (96, 2 * SLABS + 5), (256, 129)])
+def test_dpsgd(n, d):
+    m = _graph("ring", n)
+    a, c, x0 = _data(n, d, n)
+    K, eta, alpha = 3, 0.2, 0.05
+    with Session(m, d, K, eta, alpha, a, c, x0, 0.1, 3, algorithm=B.DETAG_ALGORITHM_DPSGD) as s:
+        s.upload("g", c)
+        s.upload("y", a)
+        B.detag_set_step(s.state, 0)
+        s.step()
+        s.status()
+        x, g, y = (s.download(k) for k in ("x", "g", "y"))
+    want = _polynomial(m, K, eta) @ x0.astype(np.float64) - alpha * c
+    assert worst_ratio(x, want) <= 1.0
+    for lo, hi in ((0, min(d, 100)), (max(0, d - 100), d)):
+        p = oracle_problem(m, K, eta, alpha, a[:, lo:hi], c[:, lo:hi], 0.1, 3, lo)
+        assert worst_ratio(g[:, lo:hi], orc.stochastic_gradient(p, want[:, lo:hi], 1)) <= 1.0
+    assert np.array_equal(y, a)  # no tracker: untouched
