@@ -430,6 +430,16 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   return variant == DETAG_VARIANT_DENSE || variant == DETAG_VARIANT_RING;
 }
 
+// Up to 16 workers a thread takes a coordinate's whole column.  us per step, tensor-path kernel -> that one: 8 workers,
+// d = 8 M 1005 -> 362; 12, d = 4 M 565 -> 294; 13, d = 4 M 565 -> 461; 16, d = 4 M 568 -> 474, d = 270 k 43 -> 32.
+// Caller-written gradients read four arrays before the first contraction, and have no noise and gradient to save: beyond
+// eight workers they stay (8, d = 8 M 619 -> 307; 13, d = 4 M 381 -> 540; 16, d = 270 k 34.9 -> 36.0).  The
+// failure-detection self test wants bounded waits, of which that kernel has none: it runs the tensor-path kernel.
+bool small_ok(const StepParams& p) {
+  if (p.n > detag::kMaxSmallWorkers || p.stall_after >= 0) return false;
+  return p.mode != detag::kModeExternal || p.n <= 8;
+}
+
 // Picks the kernel variant, plans it for the sizes in `p` and launches it.
 int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   int e = 0;
@@ -469,6 +479,10 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
           const int rc = launch_tail_columns(s, p, d_main, stream, &e);
           if (rc != DETAG_OK) return rc;
         }
+        break;
+      }
+      if (small_ok(p)) {
+        e = detag::launch_step_small(p, s->sm_count, stream);
         break;
       }
       const bool mma = p.n <= 32;
@@ -823,9 +837,14 @@ int detag_step_many(detag_state* s, int count, void* stream) {
       p.t_noise = static_cast<uint32_t>(s->t + 1);
       p.steps = now;
       if (!p.a || !p.c) return fail(s, DETAG_ERR_UNBOUND, "the synthetic gradient needs the objective arrays a and c");
-      const detag::TensorMapSet* maps = maps_for(s, kFamilyMma, p);
-      if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-      const int e = detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream));
+      int e;
+      if (small_ok(p)) {
+        e = detag::launch_step_small(p, s->sm_count, static_cast<cudaStream_t>(stream));
+      } else {
+        const detag::TensorMapSet* maps = maps_for(s, kFamilyMma, p);
+        if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+        e = detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream));
+      }
       if (e != 0) return fail_cuda(s, e, "detag_step_many launch");
       s->t += now;
       done += now;

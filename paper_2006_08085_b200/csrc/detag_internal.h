@@ -16,6 +16,7 @@ namespace detag {
 constexpr int kMaxWorkers = 1024;       // detag_create limit on n
 constexpr int kMaxDenseWorkers = 64;    // dense-polynomial kernels with P in shared memory: limit on n
 constexpr int kMaxWideWorkers = 128;    // dense-polynomial kernel with P in registers: limit on n
+constexpr int kMaxSmallWorkers = 16;    // one thread per coordinate: limit on n
 constexpr int kMaxSplitWorkers = 256;   // integer tensor path: limit on n
 constexpr int kMaxPartials = 2048;      // per-CTA partial sums of the consensus-error reduction
 constexpr size_t kWsAlign = 256;
@@ -120,6 +121,8 @@ void wide_fragments(int n, const std::vector<double>& poly, std::vector<double>&
 bool build_maps_wide(const StepParams& p, TensorMapSet* maps);
 int launch_step_wide(StepParams p, const TensorMapSet& maps, const double* p_frag /* device */, int sm_count,
                      cudaStream_t stream);
+// one thread per coordinate (step_small.cu): n <= 16, all modes; p.steps iterations
+int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
 // polynomial on the integer tensor path (step_split.cu): 32 < n <= 256, DeTAG and D-PSGD steps
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
 bool build_maps_split(const StepParams& p, TensorMapSet* maps);
