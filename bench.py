@@ -38,9 +38,9 @@ BYTES_PER_WC = 32  # read x, y, g, a, c + write x, y, g, float32 each: the fused
 # small case of the same kernel; traffic grows in proportion to n*d).  Keyed by the sha256 prefix of the kernel
 # sources the capture was taken on: a changed kernel reports null until it is captured again.
 KERNEL_SOURCES = {
-    "wide": ("step_wide.cu", "pipeline.cuh", "noise.cuh"),
+    "small": ("step_small.cu", "noise.cuh"),
+    "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh"),
     "mma": ("step_mma.cu", "mma_common.cuh", "pipeline.cuh", "noise.cuh"),
-    "band": ("step_band.cu", "pipeline.cuh", "noise.cuh"),
     "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh"),
     "csr": ("step_csr.cu", "noise.cuh"),
     "torus": ("step_torus.cu", "torus_basis.h", "pipeline.cuh", "noise.cuh"),
@@ -50,14 +50,12 @@ MEASURED_TRAFFIC = {
     ("mma", "dense"): ("22eae46feb506e80", 31.46),     # cfg5 shape at d = 2 M: 1.2949 GB read + 0.7183 GB written / 64 M wc
     ("torus", "torus8"): ("427a2bff49b63d9c", 31.27),  # cfg3 shape at d = 1 M: 1.2803 + 0.7208 GB / 64 M wc
     ("ring", "band"): ("60c16ee651aa8e4f", 31.12),     # cfg4 shape at d = 200 k: 1.0280 + 0.5652 GB / 51.2 M wc
-    ("wide", "dense"): ("77d5b7be943b4c42", 30.83),    # 100-worker random graph at d = 400 k: 0.8011 + 0.4321 GB / 40 M wc
     ("csr", "rounds"): ("bcc2ab2f791da0eb", 31.17),    # the same graph through the rounds kernel: 0.8088 + 0.4381 GB / 40 M wc
 }
 
 # Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes) and that
 # pipe's peak: 64 multiply-adds per clock and SM (measured: 61 with m8n8k4 MMAs from 16 warps) x 148 SMs x max clock.
-FP64_FMA_PER_WC = {("mma", "dense"): 64, ("ring", "band"): 80, ("band", "dense"): 128,
-                   ("torus", "torus8"): 26, ("torus", "torus4"): 28}
+FP64_FMA_PER_WC = {("mma", "dense"): 64, ("ring", "band"): 80, ("torus", "torus8"): 26, ("torus", "torus4"): 28}
 VARIANT_NAMES = {1: "csr", 2: "dense", 3: "ring", 4: "torus"}
 FP64_FMA_PER_CLK_SM = 64
 SM_COUNT = 148
@@ -65,9 +63,9 @@ SM_COUNT = 148
 
 def kernel_key(variant: str, n: int):
     if variant == "dense":
-        return ("mma", "dense") if n <= 32 else ("band", "dense") if n <= 64 else ("wide", "dense")
+        return ("small", "column") if n <= 16 else ("mma", "dense") if n <= 32 else ("split", "digits")
     if variant == "ring":
-        return ("ring", "band")
+        return ("split", "digits") if n <= 256 else ("ring", "band")
     if variant == "csr":
         return ("csr", "rounds")
     if variant == "torus":
@@ -333,7 +331,6 @@ def theorem3_regime(dev, args) -> dict:
         s.status()
         out["runs"].append({"K": K, "variant": VARIANT_NAMES.get(B.detag_get_variant(s.state), "other"),
                             "ms_per_step": ms / steps, "value": cfg.wc / (ms / steps * 1e-3), "unit": UNIT,
-                            "fp64_fma_per_wc": 80 if K == base.K else 2 * cfg.n,
                             "consensus_error_per_wc_by_step": ce})
         s.close()
         del s
@@ -343,8 +340,8 @@ def theorem3_regime(dev, args) -> dict:
 
 def general_graph(dev, args) -> dict:
     """Graphs none of the structured kernels takes - seeded random 4-regular graphs with 100 and with 72 workers,
-    K = 6, d = 2,000,000: step time and roofline fractions of the kernel the library picks (the dense polynomial
-    held in registers, whose bound is the FP64 tensor pipe: 2 * n_padded multiply-adds per worker-coordinate) and,
+    K = 6, d = 2,000,000: step time and roofline fractions of the kernel the library picks (the polynomial on the
+    integer tensor path) and,
     for the 100-worker graph, of the generic rounds kernel that takes every graph."""
     import torch
 
@@ -380,10 +377,6 @@ def general_graph(dev, args) -> dict:
         out = {"workload": f"{n} workers, random 4-regular graph (Metropolis weights), d = {d:,}, K = {K}",
                "variant": variant, "ms_per_step": ms, "value": n * d / (ms * 1e-3), "unit": UNIT, "achieved_gbs": gbs,
                "frac_of_measured_peak": gbs / peak, "frac_of_8TBps_nominal": gbs / 8000.0}
-        if variant == "dense":
-            fma = 2 * ((n + 7) // 8 * 8)
-            out["fp64_fma_per_wc"] = fma
-            out["fp64_pipe_frac"] = fma * out["value"] / (FP64_FMA_PER_CLK_SM * SM_COUNT * 1965e6)
         return out
 
     return {"picked_100": one(100, 0), "rounds_100": one(100, B.DETAG_VARIANT_CSR), "picked_72": one(72, 0)}

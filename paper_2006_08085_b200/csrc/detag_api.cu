@@ -18,7 +18,7 @@ namespace {
 size_t align_up(size_t v) { return (v + detag::kWsAlign - 1) / detag::kWsAlign * detag::kWsAlign; }
 
 struct WsLayout {
-  size_t status, result, row_ptr, col_idx, vals, poly, torus, circ_row, wide, split_blocks, split_exp, split_poly, partials, total;
+  size_t status, result, row_ptr, col_idx, vals, poly, torus, split_blocks, split_exp, split_poly, partials, total;
 };
 
 WsLayout ws_layout(const detag_state* s) {
@@ -37,10 +37,6 @@ WsLayout ws_layout(const detag_state* s) {
   off += align_up(s->poly.size() * sizeof(double));
   l.torus = off;
   off += align_up(s->torus_frag.size() * sizeof(double));
-  l.circ_row = off;
-  off += align_up(s->circ_row.size() * sizeof(double));
-  l.wide = off;
-  off += align_up(s->wide_frag.size() * sizeof(double));
   l.split_blocks = off;
   off += align_up(s->split.blocks.size());
   l.split_exp = off;
@@ -175,7 +171,7 @@ void analyse_circulant(detag_state* s) {
       if (delta > hb) hb = delta;
     }
   s->half_band = hb;
-  if (n <= 256) s->circ_row = cur;  // p(0 .. n-1): the dense mode of the circulant kernel looks its fragments up here
+  if (n <= detag::kMaxSplitWorkers) s->circ_row = cur;
   if (hb <= 16 && n >= 2 * hb + 1)
     for (int delta = -16; delta <= 16; ++delta)
       s->band[delta + 16] = (delta >= -hb && delta <= hb) ? cur[((delta % n) + n) % n] : 0.0;
@@ -260,11 +256,11 @@ void analyse_torus(detag_state* s) {
 
 bool torus_ok(const detag_state* s) { return s->torus && s->d <= 0x7fffffffLL; }
 
-// The circulant kernel: band mode while the polynomial's half-band is at most 16, dense mode (n <= 256) beyond.
+// The circulant kernel takes polynomials whose half-band is at most 16; the integer tensor path any up to 256 workers.
 bool ring_band(const detag_state* s) { return detag::ring_variant_available(s->n, s->half_band); }
 
 bool band_ok(const detag_state* s) {
-  return s->circulant && s->d <= 0x7fffffffLL && (ring_band(s) || detag::ring_dense_available(s->n));
+  return s->circulant && s->d <= 0x7fffffffLL && (ring_band(s) || (detag::ring_variant_available(s->n, 0) && s->n <= detag::kMaxSplitWorkers));
 }
 
 int step_mode(const detag_state* s) {
@@ -291,8 +287,6 @@ StepParams make_params(const detag_state* s) {
   p.vals = s->d_vals;
   p.poly = s->d_poly;
   p.torus = s->d_torus;
-  p.circ_row = s->d_circ_row;
-  p.wide = s->d_wide;
   p.split = s->d_split;
   p.eta = s->eta;
   p.alpha = s->alpha;
@@ -312,17 +306,13 @@ StepParams make_params(const detag_state* s) {
 
 bool dense_ok(const detag_state* s) {
   if (s->d > 0x7fffffffLL) return false;
-  return (!s->poly.empty() && detag::dense_variant_available(s->n)) ||
-         (!s->wide_frag.empty() && detag::wide_variant_available(s->n));
+  return detag::dense_variant_available(s->n);
 }
 
-// Host cost model.  The dense product needs n multiply-adds per element and array against the sparse
-// rounds' K*(nnz per row), but keeps its outputs in registers and needs no barriers; it wins for every
-// n it supports - except that for 32 < n <= 64 a circulant matrix with a narrow band is cheaper through the
-// band kernel (80 instead of 128 MMAs per tile).  Caller-written gradients and D-PSGD run on the dense
-// kernel for n <= 32 and on the generic rounds kernel otherwise.
-// for 32 < n <= 64 a block-circulant matrix (torus) takes the transform kernel: 24 multiply-adds per element
-// and array instead of 64.
+// Host cost model.  The product with the polynomial beats the sparse rounds wherever a kernel takes it: K rounds cost
+// K * (nnz per row) shared-memory gathers of 16 bytes per element and array and two barriers each.  Tori of 8-worker blocks
+// take the transform kernel (24 multiply-adds per element and array).  Caller-written gradients run on the dense kernels
+// for n <= 32 and on the rounds kernel otherwise.
 bool variant_runs_mode(const detag_state* s, int variant) {
   if (step_mode(s) == detag::kModeDetag) return true;
   if (variant == DETAG_VARIANT_RING) return step_mode(s) == detag::kModeDpsgd;
@@ -333,17 +323,17 @@ int resolve_variant(const detag_state* s) {
   if (s->variant_forced != DETAG_VARIANT_AUTO) return s->variant_forced;
   // a ring whose band fits takes the circulant kernel from n = 64 on; with a dense polynomial only beyond the
   // reach of the 64-row dense kernel
-  const bool ring = band_ok(s) && (ring_band(s) || s->n > detag::kMaxDenseWorkers);
+  const bool ring = band_ok(s) && (ring_band(s) || s->n > 64);
   if (step_mode(s) == detag::kModeDpsgd && s->n > 32 && ring) return DETAG_VARIANT_RING;
   if (step_mode(s) != detag::kModeDetag) return (s->n <= 32 && dense_ok(s)) ? DETAG_VARIANT_DENSE : DETAG_VARIANT_CSR;
   if (s->n > 32 && ring) return DETAG_VARIANT_RING;
   if (s->n > 32 && torus_ok(s)) return DETAG_VARIANT_TORUS;
   if (dense_ok(s)) {
-    if (s->n > detag::kMaxDenseWorkers) {
-      // Register-resident polynomial against the sparse rounds, both measured at d = 2 M (ms): the dense kernel is
-      // bound by one warp scheduler's share of the MMAs - blocks / 4 strips (the next multiple of four when one
-      // scheduler is a block short) of n / 4 k-steps - the rounds kernel by a per-worker part and K * nnz
-      // shared-memory gathers.  The rounds win at one or two rounds on graphs of degree four.
+    if (s->n > 64) {
+      // Which of the two names the call goes by, where no structure decides: the rounds' if a float64 product (blocks of
+      // eight workers on four tensor-path schedulers) would take longer than the rounds, measured at d = 2 M (ms) - one
+      // or two rounds on graphs of degree four.  With the integer tensor path both run there (split_ok): 100 workers,
+      // d = 2 M, 1.6 ms for any K against 3.2 ms for one round.
       const int blocks = (s->n + 7) / 8, blocks_eff = blocks % 4 == 3 ? blocks + 1 : blocks;
       const double dense_ms = 0.0412 * blocks_eff * blocks / 2.0;
       const double rounds_ms = 0.024 * s->n + 0.00155 * s->K * static_cast<double>(s->col_idx.size());
@@ -367,7 +357,7 @@ int query_device(detag_state* s) {
 }
 
 // Kernel families that take tensor maps.
-enum { kFamilyMma = 1, kFamilyBand = 2, kFamilyTorus = 3, kFamilyRing = 4, kFamilyWide = 5, kFamilySplit = 6 };
+enum { kFamilyMma = 1, kFamilyTorus = 2, kFamilyRing = 3, kFamilySplit = 4 };
 
 // Tensor maps for the buffers in `p`: built on first use, then found again by buffer addresses and sizes
 // (detag_step always hits; detag_step_host cycles through its two chunk slots and the ragged last chunk).
@@ -391,9 +381,7 @@ const detag::TensorMapSet* maps_for(detag_state* s, int family, const StepParams
   detag_state::MapEntry& en = *slot;
   en.family = 0;  // invalid until built
   const bool ok = family == kFamilyMma    ? detag::build_maps_mma(p, &en.maps)
-                  : family == kFamilyBand ? detag::build_maps_band(p, &en.maps)
                   : family == kFamilyRing ? detag::build_maps_ring(p, &en.maps)
-                  : family == kFamilyWide ? detag::build_maps_wide(p, &en.maps)
                   : family == kFamilySplit ? detag::build_maps_split(p, &en.maps)
                                           : detag::build_maps_torus(p, &en.maps);
   if (!ok) return nullptr;
@@ -462,34 +450,18 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     if (e != 0) return fail_cuda(s, e, "step kernel launch");
     return DETAG_OK;
   }
-  switch (variant) {
+  // what the integer tensor path does not take although its variant promises it (a polynomial whose entries cannot be
+  // scaled, e.g. under an absurd momentum) runs as rounds
+  const bool as_rounds = (variant == DETAG_VARIANT_DENSE && p.n > 32) || (variant == DETAG_VARIANT_RING && !ring_band(s));
+  switch (as_rounds ? DETAG_VARIANT_CSR : variant) {
     case DETAG_VARIANT_DENSE: {
-      if (p.n > detag::kMaxDenseWorkers) {
-        // the register-resident polynomial takes whole 32-coordinate halves; the last d % 32 columns go to the generic kernel
-        const long long d_main = p.d & ~31LL;
-        if (d_main > 0) {
-          StepParams pm = p;
-          pm.d = d_main;
-          const detag::TensorMapSet* maps = maps_for(s, kFamilyWide, pm);
-          if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-          e = detag::launch_step_wide(pm, *maps, p.wide, s->sm_count, stream);
-          if (e != 0) return fail_cuda(s, e, "step kernel launch");
-        }
-        if (d_main < p.d) {
-          const int rc = launch_tail_columns(s, p, d_main, stream, &e);
-          if (rc != DETAG_OK) return rc;
-        }
-        break;
-      }
       if (small_ok(p)) {
         e = detag::launch_step_small(p, s->sm_count, stream);
         break;
       }
-      const bool mma = p.n <= 32;
-      const detag::TensorMapSet* maps = maps_for(s, mma ? kFamilyMma : kFamilyBand, p);
+      const detag::TensorMapSet* maps = maps_for(s, kFamilyMma, p);
       if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-      e = mma ? detag::launch_step_mma(p, *maps, s->sm_count, stream)
-              : detag::launch_step_band(p, *maps, nullptr, s->sm_count, stream);
+      e = detag::launch_step_mma(p, *maps, s->sm_count, stream);
       break;
     }
     case DETAG_VARIANT_RING: {
@@ -500,7 +472,7 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
         pm.d = d_main;
         const detag::TensorMapSet* maps = maps_for(s, kFamilyRing, pm);
         if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-        e = detag::launch_step_ring(pm, *maps, ring_band(s) ? s->band : nullptr, p.circ_row, s->sm_count, stream);
+        e = detag::launch_step_ring(pm, *maps, s->band, s->sm_count, stream);
         if (e != 0) return fail_cuda(s, e, "step kernel launch");
       }
       if (d_main < p.d) {
@@ -571,20 +543,13 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   s->col_idx.assign(col_idx, col_idx + nnz);
   s->vals.assign(vals, vals + nnz);
   std::vector<double> poly;
-  if (n <= detag::kMaxDenseWorkers) {
-    gossip_polynomial(s, s->poly);
-  } else if (n <= detag::kMaxWideWorkers) {  // kept as the warp strips of the register-resident kernel only
-    gossip_polynomial(s, poly);
-    detag::wide_fragments(n, poly, s->wide_frag);
-  }
+  if (n <= 128) gossip_polynomial(s, poly);
+  if (n <= 64) s->poly = poly;  // what the small kernels and the torus analysis use
   analyse_circulant(s);
   analyse_torus(s);
   if (n > 32 && n <= detag::kMaxSplitWorkers) {
     const bool blocks = block_circulant(s);
-    if (blocks)
-      first_block_row(s, poly);
-    else if (!s->poly.empty())
-      poly = s->poly;
+    if (blocks) first_block_row(s, poly);
     if (!poly.empty()) detag::split_polynomial(n, poly, blocks, s->split);  // else: too many distinct blocks
   }
   s->map_cache.reserve(8);
@@ -599,8 +564,6 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   put(l.vals, s->vals.data(), s->vals.size() * sizeof(double));
   put(l.poly, s->poly.data(), s->poly.size() * sizeof(double));
   put(l.torus, s->torus_frag.data(), s->torus_frag.size() * sizeof(double));
-  put(l.circ_row, s->circ_row.data(), s->circ_row.size() * sizeof(double));
-  put(l.wide, s->wide_frag.data(), s->wide_frag.size() * sizeof(double));
   put(l.split_blocks, s->split.blocks.data(), s->split.blocks.size());
   put(l.split_exp, s->split.row_exp.data(), s->split.row_exp.size() * sizeof(int32_t));
   put(l.split_poly, s->split.poly_t.data(), s->split.poly_t.size() * sizeof(double));
@@ -638,8 +601,6 @@ int detag_bind(detag_state* s, int64_t ld, float* x, float* y, float* g, const f
   s->d_vals = reinterpret_cast<double*>(base + l.vals);
   s->d_poly = s->poly.empty() ? nullptr : reinterpret_cast<double*>(base + l.poly);
   s->d_torus = s->torus_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.torus);
-  s->d_circ_row = s->circ_row.empty() ? nullptr : reinterpret_cast<double*>(base + l.circ_row);
-  s->d_wide = s->wide_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.wide);
   s->d_split = s->split.blocks.empty() ? nullptr : base + l.split_blocks;
   s->d_partials = reinterpret_cast<double*>(base + l.partials);
 
@@ -908,8 +869,6 @@ int detag_step_host(detag_state* s, int64_t ld_host, float* x, float* y, float* 
   p.vals = reinterpret_cast<double*>(base + l.vals);
   p.poly = s->poly.empty() ? nullptr : reinterpret_cast<double*>(base + l.poly);
   p.torus = s->torus_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.torus);
-  p.circ_row = s->circ_row.empty() ? nullptr : reinterpret_cast<double*>(base + l.circ_row);
-  p.wide = s->wide_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.wide);
   p.split = s->split.blocks.empty() ? nullptr : base + l.split_blocks;
   p.status = status_word;
   p.y_obs = nullptr;

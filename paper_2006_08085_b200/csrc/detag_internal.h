@@ -14,8 +14,7 @@ typedef struct CUstream_st* cudaStream_t;
 namespace detag {
 
 constexpr int kMaxWorkers = 1024;       // detag_create limit on n
-constexpr int kMaxDenseWorkers = 64;    // dense-polynomial kernels with P in shared memory: limit on n
-constexpr int kMaxWideWorkers = 128;    // dense-polynomial kernel with P in registers: limit on n
+constexpr int kMaxDenseWorkers = 128;   // dense variant: limit on n
 constexpr int kMaxSmallWorkers = 16;    // one thread per coordinate: limit on n
 constexpr int kMaxSplitWorkers = 256;   // integer tensor path: limit on n
 constexpr int kMaxPartials = 2048;      // per-CTA partial sums of the consensus-error reduction
@@ -43,9 +42,7 @@ struct StepParams {
   const int32_t* row_ptr;
   const int32_t* col_idx;
   const double* vals;
-  const double* poly;  // dense P_K(M), row-major n x n (null when n > kMaxDenseWorkers)
-  const double* circ_row;  // circulant kernel, dense mode: the first row of P_K(M) (or null)
-  const double* wide;  // register-resident dense kernel (64 < n <= 128): the warp strips of P_K(M) in fragment order (or null)
+  const double* poly;  // dense P_K(M), row-major n x n (null when n > 64)
   const unsigned char* split;  // split kernel: digit blocks, row exponents and P in the workspace (or null)
   const double* torus; // block-circulant kernel: per-frequency 8 x 8 polynomial blocks in fragment order (or null)
   double eta;
@@ -101,26 +98,14 @@ bool dense_variant_available(int n);  // n <= kMaxDenseWorkers and the driver of
 bool build_maps_mma(const StepParams& p, TensorMapSet* maps);
 int launch_step_mma(StepParams p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);       // n <= 32
 int launch_step_mma_many(StepParams p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);  // p.steps steps
-bool dense_window_available(int n);                // the band kernel's dense mode: 32 < n <= 64
-bool build_maps_band(const StepParams& p, TensorMapSet* maps);
-int launch_step_band(StepParams p, const TensorMapSet& maps, const double* band /* null: dense mode */, int sm_count,
-                     cudaStream_t stream);
-// circulant kernel (step_ring.cu): n % 32 == 0, 64 <= n <= 1024; band mode for half-band <= 16, dense mode for n <= 256
+// circulant kernel (step_ring.cu): n % 32 == 0, 64 <= n <= 1024, half-band <= 16
 bool ring_variant_available(int n, int half_band);
-bool ring_dense_available(int n);
 bool build_maps_ring(const StepParams& p, TensorMapSet* maps);  // p.d a multiple of 64
-int launch_step_ring(StepParams p, const TensorMapSet& maps, const double* band /* null: dense mode */,
-                     const double* p_row /* device: first row of P, dense mode */, int sm_count, cudaStream_t stream);
+int launch_step_ring(StepParams p, const TensorMapSet& maps, const double* band, int sm_count, cudaStream_t stream);
 bool torus_variant_available(int n);               // block-circulant kernel: n = 32 or 64 (4 or 8 blocks of 8)
 bool build_maps_torus(const StepParams& p, TensorMapSet* maps);
 int launch_step_torus(StepParams p, const TensorMapSet& maps, const double* phat_frag /* device */, int sm_count,
                       cudaStream_t stream);
-// dense polynomial held in registers (step_wide.cu): 64 < n <= 128, p.d a multiple of 32, DeTAG step only
-bool wide_variant_available(int n);
-void wide_fragments(int n, const std::vector<double>& poly, std::vector<double>& frag);
-bool build_maps_wide(const StepParams& p, TensorMapSet* maps);
-int launch_step_wide(StepParams p, const TensorMapSet& maps, const double* p_frag /* device */, int sm_count,
-                     cudaStream_t stream);
 // one thread per coordinate (step_small.cu): n <= 16, all modes; p.steps iterations
 int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
 // polynomial on the integer tensor path (step_split.cu): 32 < n <= 256, DeTAG and D-PSGD steps
@@ -144,16 +129,15 @@ struct detag_state {
   double eta = 0.0, alpha = 0.0;
   std::vector<int32_t> row_ptr, col_idx;
   std::vector<double> vals;
-  std::vector<double> poly;  // P_K(M) when n <= kMaxDenseWorkers
+  std::vector<double> poly;  // P_K(M) when n <= 64
   bool circulant = false;    // every row of M is the previous one shifted by one
   int half_band = 0;         // of the circulant P_K(M): P[i][(i+delta) mod n] = 0 for |delta| > half_band
   double band[33] = {0};     // p(delta) at index delta + 16, valid when circulant and half_band <= 16
-  std::vector<double> circ_row;  // first row of the circulant P_K(M) (kept when n <= 256)
+  std::vector<double> circ_row;  // first row of the circulant P_K(M) (kept when n <= kMaxSplitWorkers)
   // block-circulant structure with 8-worker blocks, symmetric in the block distance (tori): the per-frequency
   // 8 x 8 polynomial blocks in MMA fragment order
   bool torus = false;
   std::vector<double> torus_frag;
-  std::vector<double> wide_frag;  // 64 < n <= 128: P_K(M) as the warp strips of the register-resident kernel
   detag::SplitPoly split;         // 32 < n <= 256: P_K(M) for the integer tensor path (empty: not taken)
   std::vector<unsigned char> image;  // the workspace up to the partial sums, as it is uploaded
   int variant_forced = DETAG_VARIANT_AUTO;
@@ -179,8 +163,6 @@ struct detag_state {
   double* d_vals = nullptr;
   double* d_poly = nullptr;
   double* d_torus = nullptr;
-  double* d_circ_row = nullptr;
-  double* d_wide = nullptr;
   unsigned char* d_split = nullptr;  // blocks, row exponents and P of `split`, one after the other (split_at)
   double* d_partials = nullptr;
 

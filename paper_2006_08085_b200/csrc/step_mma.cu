@@ -255,6 +255,8 @@ MmaKernel pick_mode(const StepParams& p) {
 
 }  // namespace
 
+bool dense_variant_available(int n) { return n <= kMaxDenseWorkers && encode_tiled_fn() != nullptr; }
+
 // Tensor maps over the arrays in `p`; false when the driver refuses one.
 bool build_maps_mma(const StepParams& p, TensorMapSet* out) {
   MmaMaps* maps = reinterpret_cast<MmaMaps*>(out->bytes);

@@ -2,12 +2,10 @@
 //
 // For a circulant M (every row is the previous one shifted by one: the ring with uniform weights, the paper's
 // Metropolis ring and its slack matrices) the K-round accelerated gossip AG_K(z) = P z has a circulant
-// P = P_K(M), P[i][j] = p((j - i) mod n).  Two modes:
-//   band   p(delta) = 0 for |delta| > 16 (K times the bandwidth of M at most 16): 32 output rows need a window
-//          of 64 input rows, and of the 16 x 4 blocks of that 64 x 32 slice only 10 per 8-row output block are
-//          non-zero: 80 float64 MMAs (m8n8k4) per 8 coordinates x 32 workers for tracker and model together.
-//   dense  any p (Theorem 3's phase length makes P dense): every output block contracts the whole ring, n / 4
-//          k-steps, with the B fragments looked up in the one stored row of P.  n <= 256.
+// P = P_K(M), P[i][j] = p((j - i) mod n).  While p(delta) = 0 for |delta| > 16 (K times the bandwidth of M at most 16), 32
+// output rows need a window of 64 input rows, and of the 16 x 4 blocks of that 64 x 32 slice only 10 per 8-row output
+// block are non-zero: 80 float64 MMAs (m8n8k4) per 8 coordinates x 32 workers for tracker and model together.  (Up to 256
+// workers the integer tensor path, step_split.cu, comes first.)
 //
 // Layout of the contraction: the eight coordinates of a warp's tile are the M index of the MMA, the input worker
 // the contraction index (k-step s takes window rows 4 s + kq) and the output worker the N index, permuted so that
@@ -23,8 +21,7 @@
 //          order, plus a second copy of chunk 0 in a side buffer, taken before anything of the slab is stored, for
 //          the last tile, whose window wraps around to rows 0..15.  Since no row is fetched again after it was
 //          fetched once (except those two, both handled), the in-place update of x and y needs no further care.
-//          Dense mode: the chunks 0 .. n/16 - 1 of a slab all stay resident until its last tile is done.
-//   g, a, c  of a tile's 32 rows go to one of four (dense: two) stages; the tail overwrites them with g', x', y'
+//   g, a, c  of a tile's 32 rows go to one of four stages; the tail overwrites them with g', x', y'
 //          and three TMA stores send the stage out.
 // Every transfer is one three-dimensional TMA box {32 coordinates, 2 halves, rows} in the 128-byte swizzle: rows
 // arrive as contiguous 256-byte pieces, and with the row ownership above every warp-wide shared-memory access hits
@@ -59,22 +56,17 @@ constexpr int kRConsumerWarps = kRGroups * kRGroupWarps;
 constexpr int kLoadXYWarp = kRConsumerWarps, kLoadEWarp = kRConsumerWarps + 1, kRStoreWarp = kRConsumerWarps + 2,
               kRSignalWarp = kRConsumerWarps + 3;
 constexpr int kRThreads = (kRConsumerWarps + 4) * 32;
-constexpr int kMaxSlots = 16;
 
-template <bool kDense>
-struct RingPlan {
-  static constexpr int kSlots = kDense ? 16 : 12;       // ring of x, y chunks
-  static constexpr int kEStages = kDense ? 2 : 4;       // even: a stage always serves the same consumer group
-  static constexpr int kSideFloats = kDense ? 0 : 2 * kSlotFloats;   // chunk 0 copies, one per slab parity
-  static constexpr int kTableDoubles = kDense ? 256 : 0;             // the stored row of P
-  static constexpr size_t kCtrlOffset = static_cast<size_t>(kSlots) * kSlotFloats * 4 + kSideFloats * 4 +
-                                        static_cast<size_t>(kEStages) * kEStageFloats * 4 + kTableDoubles * 8;
-  // control area: slot barriers, side barriers (2), stage barriers (full, empty, ready), counters
-  static constexpr size_t kCtrlBytes = (kMaxSlots + 2 + 3 * 4) * 8 + (2 + kRConsumerWarps) * 4;
-  static constexpr size_t kSmemBytes = kCtrlOffset + 512 + 1024;     // + slack to align the tiles to 1 KiB
-  static_assert(kCtrlBytes <= 512, "control area");
-  static_assert(kSmemBytes <= 232448, "shared memory plan");
-};
+constexpr int kSlots = 12;    // ring of x, y chunks
+constexpr int kEStages = 4;   // even: a stage always serves the same consumer group
+constexpr int kSideFloats = 2 * kSlotFloats;  // chunk 0 copies, one per slab parity
+constexpr size_t kCtrlOffset =
+    static_cast<size_t>(kSlots) * kSlotFloats * 4 + kSideFloats * 4 + static_cast<size_t>(kEStages) * kEStageFloats * 4;
+// control area: slot barriers, side barriers (2), stage barriers (full, empty, ready), counters
+constexpr size_t kCtrlBytes = (kSlots + 2 + 3 * 4) * 8 + (2 + kRConsumerWarps) * 4;
+constexpr size_t kRingSmemBytes = kCtrlOffset + 512 + 1024;  // + slack to align the tiles to 1 KiB
+static_assert(kCtrlBytes <= 512, "control area");
+static_assert(kRingSmemBytes <= 232448, "shared memory plan");
 
 struct RingMaps {
   CUtensorMap x, y;        // boxes {32, 2, 16 rows}
@@ -84,24 +76,19 @@ struct RingMaps {
 static_assert(sizeof(RingMaps) <= sizeof(TensorMapSet), "tensor map storage");
 
 struct RingCoef {
-  double p[2 * kRHalo + 1];  // band mode: p[delta + 16] = P[i][(i + delta) mod n]
+  double p[2 * kRHalo + 1];  // p[delta + 16] = P[i][(i + delta) mod n]
 };
 
-template <bool kDense>
 __global__ void __launch_bounds__(kRThreads, 1)
-step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, const __grid_constant__ RingCoef coef,
-                 const double* __restrict__ p_row) {
-  using Plan = RingPlan<kDense>;
-  constexpr int kSlots = Plan::kSlots, kEStages = Plan::kEStages;
+step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, const __grid_constant__ RingCoef coef) {
   extern __shared__ unsigned char smem_unaligned[];
   // the swizzle pattern is a function of the shared-memory address: tiles start on 1 KiB boundaries
   unsigned char* smem_raw = smem_unaligned + ((1024u - (s_addr(smem_unaligned) & 1023u)) & 1023u);
   float* ring_mem = reinterpret_cast<float*>(smem_raw);                 // [slot][x chunk | y chunk]
   float* side_mem = ring_mem + kSlots * kSlotFloats;                    // [slab parity][x chunk 0 | y chunk 0]
-  float* e_mem = side_mem + Plan::kSideFloats;                          // [stage][g | a | c]
-  double* table = reinterpret_cast<double*>(e_mem + kEStages * kEStageFloats);   // dense mode: p(0 .. n-1)
-  uint64_t* slot_full = reinterpret_cast<uint64_t*>(smem_raw + Plan::kCtrlOffset);
-  uint64_t* side_full = slot_full + kMaxSlots;
+  float* e_mem = side_mem + kSideFloats;                          // [stage][g | a | c]
+  uint64_t* slot_full = reinterpret_cast<uint64_t*>(smem_raw + kCtrlOffset);
+  uint64_t* side_full = slot_full + kSlots;
   uint64_t* e_full = side_full + 2;
   uint64_t* e_empty = e_full + 4;
   uint64_t* out_ready = e_empty + 4;
@@ -113,9 +100,7 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
   const int n = p.n;
   const int NB = n / kRT;                                    // tiles (row blocks) per slab
   const int NC = n / kChunkRows;                             // chunks per ring
-  const int CPS = kDense ? NC : NC + 1;                      // chunk loads per slab into the slot ring
-  if (kDense)
-    for (int e = tid; e < n; e += kRThreads) table[e] = p_row[e];
+  const int CPS = NC + 1;                      // chunk loads per slab into the slot ring
   if (tid == 0) {
     *landed = 0;
     *side_landed = 0;
@@ -161,29 +146,27 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
       const long long stall_at = p.stall_after >= 0 ? 2 * p.stall_after : -1;
       for (int sl = 0; sl < my_slabs && ok; ++sl) {
         const int half = static_cast<int>((blockIdx.x + static_cast<long long>(sl) * gridDim.x) * 2);
-        if (!kDense) {
-          // second copy of chunk 0 for the slab's last tile; the buffer was last read by the last tile two slabs back
-          if (sl >= 2) ok = wait_released((sl - 1) * NB - 1);
-          if (!ok) break;
-          if (stall_at >= 0 && Q >= stall_at) return;
-          float* sd = side_mem + static_cast<size_t>(sl & 1) * kSlotFloats;
-          bar_expect_tx(&side_full[sl & 1], kSlotFloats * 4);
-          rows_load(sd, &maps.x, half, 0, &side_full[sl & 1]);
-          rows_load(sd + kChunkFloats, &maps.y, half, 0, &side_full[sl & 1]);
-        }
+        // second copy of chunk 0 for the slab's last tile; the buffer was last read by the last tile two slabs back
+        if (sl >= 2) ok = wait_released((sl - 1) * NB - 1);
+        if (!ok) break;
+        if (stall_at >= 0 && Q >= stall_at) return;
+        float* sd = side_mem + static_cast<size_t>(sl & 1) * kSlotFloats;
+        bar_expect_tx(&side_full[sl & 1], kSlotFloats * 4);
+        rows_load(sd, &maps.x, half, 0, &side_full[sl & 1]);
+        rows_load(sd + kChunkFloats, &maps.y, half, 0, &side_full[sl & 1]);
         for (int q = 0; q < CPS && ok; ++q, ++Q) {
           if (stall_at >= 0 && Q >= stall_at) return;
           const int slot = static_cast<int>(Q % kSlots);
           if (Q >= kSlots) {
             // the chunk that held this slot: position q_old of slab sl_old; its last reader is tile q_old / 2 of
-            // that slab (dense mode: the slab's last tile)
+            // that slab
             const int Qo = Q - kSlots, slo = Qo / CPS;
             const int qo = Qo - slo * CPS;
-            const int last_reader = kDense ? NB - 1 : (qo / 2 < NB ? qo / 2 : NB - 1);
+            const int last_reader = qo / 2 < NB ? qo / 2 : NB - 1;
             ok = wait_released(slo * NB + last_reader);
             if (!ok) break;
           }
-          const int chunk = kDense ? q : (q + NC - 1) % NC;  // band mode starts with the chunk before row 0
+          const int chunk = (q + NC - 1) % NC;  // starts with the chunk before row 0
           float* st = ring_mem + static_cast<size_t>(slot) * kSlotFloats;
           bar_expect_tx(&slot_full[slot], kSlotFloats * 4);
           rows_load(st, &maps.x, half, chunk * kChunkRows, &slot_full[slot]);
@@ -204,13 +187,11 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
     if (lane == 0) {
       int Q = 0;
       for (int sl = 0; sl < my_slabs; ++sl) {
-        if (!kDense) {
-          if (!bar_wait(&side_full[sl & 1], (sl >> 1) & 1, limit)) {
-            atomicExch(p.status, 1);
-            return;
-          }
-          count_publish(side_landed, static_cast<unsigned>(sl + 1));
+        if (!bar_wait(&side_full[sl & 1], (sl >> 1) & 1, limit)) {
+          atomicExch(p.status, 1);
+          return;
         }
+        count_publish(side_landed, static_cast<unsigned>(sl + 1));
         for (int q = 0; q < CPS; ++q, ++Q) {
           if (!bar_wait(&slot_full[Q % kSlots], (Q / kSlots) & 1, limit)) {
             atomicExch(p.status, 1);
@@ -262,7 +243,7 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
           break;
         }
         // rows 0..15 are read once more, into the side buffer: nothing of the slab goes out before that copy is in
-        if (!kDense && b == 0 && !count_wait(side_landed, static_cast<unsigned>(sl + 1), limit)) {
+        if (b == 0 && !count_wait(side_landed, static_cast<unsigned>(sl + 1), limit)) {
           atomicExch(p.status, 1);
           break;
         }
@@ -293,16 +274,14 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
   const int half_of_tile = ctile >> 2;
   const int chunk16 = 2 * (ctile & 3) + (crow >> 2);
   const int off = kq * kRS + half_of_tile * kRHalf + (((chunk16 ^ ((2 * kq + half_of_tile) & 7)) << 2) | (crow & 3));
-  // band mode: B fragment of window step u = s - 2t: entry [k = kq][column crow] = p(delta), delta = input row -
+  // B fragment of window step u = s - 2t: entry [k = kq][column crow] = p(delta), delta = input row -
   // output row = (4 u + kq) - 16 - (crow / 2 + 4 (crow & 1)); the same for every tile
-  double bfrag[kDense ? 1 : kBandSteps];
+  double bfrag[kBandSteps];
   const int out_pos = (crow >> 1) + 4 * (crow & 1);  // tile row (within its 8-row block) that MMA column `crow` stands for
-  if (!kDense) {
 #pragma unroll
-    for (int u = 0; u < kBandSteps; ++u) {
-      const int delta = 4 * u + kq - kRHalo - out_pos;
-      bfrag[u] = (delta >= -kRHalo && delta <= kRHalo) ? coef.p[delta + kRHalo] : 0.0;
-    }
+  for (int u = 0; u < kBandSteps; ++u) {
+    const int delta = 4 * u + kq - kRHalo - out_pos;
+    bfrag[u] = (delta >= -kRHalo && delta <= kRHalo) ? coef.p[delta + kRHalo] : 0.0;
   }
 
   unsigned done = 0;  // tiles this group has finished
@@ -334,11 +313,11 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
 #pragma unroll
       for (int m = 0; m < 8; ++m) xi[m] = 0.f;
     }
-    // ---- the window: band mode chunks at loading positions 2b .. 2b+3 (the last one of the slab's last tile is
-    // the side copy of chunk 0); dense mode all NC chunks of the slab
-    const int q_first = kDense ? 0 : 2 * b;
-    const int q_last = kDense ? NC - 1 : (2 * b + 3 < CPS ? 2 * b + 3 : CPS - 1);
-    const bool wraps = !kDense && 2 * b + 3 >= CPS;
+    // ---- the window: chunks at loading positions 2b .. 2b+3 (the last one of the slab's last tile is the side copy of
+    // chunk 0)
+    const int q_first = 2 * b;
+    const int q_last = 2 * b + 3 < CPS ? 2 * b + 3 : CPS - 1;
+    const bool wraps = 2 * b + 3 >= CPS;
     bool ok = true;
     if (lane == 0) {
       ok = count_wait_relaxed(landed, static_cast<unsigned>(Qbase + q_last + 1), limit);
@@ -365,43 +344,23 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
     double cx[4][2], cy[4][2];
 #pragma unroll
     for (int t = 0; t < 4; ++t) cx[t][0] = cx[t][1] = cy[t][0] = cy[t][1] = 0.0;
-    if (!kDense) {
-      // cx accumulates P x, cy accumulates P y; the model update x' = x~ - alpha y~ happens in the tail
+    // cx accumulates P x, cy accumulates P y; the model update x' = x~ - alpha y~ happens in the tail
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {  // window chunk w: rows 32 b - 16 + 16 w ..; the slab's last tile ends in the side copy
-        const int q = 2 * b + w;
-        const float* ch = (q < CPS) ? ring_mem + static_cast<size_t>((Qbase + q) % kSlots) * kSlotFloats
-                                    : side_mem + static_cast<size_t>(sl & 1) * kSlotFloats;
+    for (int w = 0; w < 4; ++w) {  // window chunk w: rows 32 b - 16 + 16 w ..; the slab's last tile ends in the side copy
+      const int q = 2 * b + w;
+      const float* ch = (q < CPS) ? ring_mem + static_cast<size_t>((Qbase + q) % kSlots) * kSlotFloats
+                                  : side_mem + static_cast<size_t>(sl & 1) * kSlotFloats;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {  // k-step s = 4 w + i: window rows 4 s + kq
-          const int s = 4 * w + i;
-          const double zx = static_cast<double>(ch[off + i * 256]);
-          const double zy = static_cast<double>(ch[kChunkFloats + off + i * 256]);
+      for (int i = 0; i < 4; ++i) {  // k-step s = 4 w + i: window rows 4 s + kq
+        const int s = 4 * w + i;
+        const double zx = static_cast<double>(ch[off + i * 256]);
+        const double zy = static_cast<double>(ch[kChunkFloats + off + i * 256]);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int u = s - 2 * t;  // compile-time after unrolling: only the band's blocks are issued
-            if (u >= 0 && u < kBandSteps) {
-              if (!dpsgd) dmma(cy[t], zy, bfrag[u]);
-              dmma(cx[t], zx, bfrag[u]);
-            }
-          }
-        }
-      }
-    } else {
-      for (int c = 0; c < NC; ++c) {  // every chunk of the ring
-        const float* ch = ring_mem + static_cast<size_t>((Qbase + c) % kSlots) * kSlotFloats;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int in_row = c * kChunkRows + 4 * i + kq;
-          const float xv = ch[off + i * 256], yv = ch[kChunkFloats + off + i * 256];
-          const double by = static_cast<double>(yv), bx = static_cast<double>(xv);
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            int delta = in_row - (b * kRT + 8 * t + out_pos);  // P[out][in] = p((in - out) mod n)
-            delta += delta < 0 ? n : 0;
-            const double bv = table[delta];
-            if (!dpsgd) dmma(cy[t], by, bv);
-            dmma(cx[t], bx, bv);
+        for (int t = 0; t < 4; ++t) {
+          const int u = s - 2 * t;  // compile-time after unrolling: only the band's blocks are issued
+          if (u >= 0 && u < kBandSteps) {
+            if (!dpsgd) dmma(cy[t], zy, bfrag[u]);
+            dmma(cx[t], zx, bfrag[u]);
           }
         }
       }
@@ -409,7 +368,7 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
     // gradient point of Algorithm 2 as printed: this lane's own rows of the old model, still in their chunks
     float x_old[8];
     if (p.grad_at_start) {
-      const int q_own = kDense ? 2 * b : 2 * b + 1;
+      const int q_own = 2 * b + 1;
 #pragma unroll
       for (int m = 0; m < 8; ++m)
         x_old[m] = ring_mem[static_cast<size_t>((Qbase + q_own + (m >> 2)) % kSlots) * kSlotFloats + off + (m & 3) * 256];
@@ -468,8 +427,6 @@ bool ring_variant_available(int n, int half_band) {
   return n % kRT == 0 && n >= 64 && n <= kMaxWorkers && half_band <= kRHalo && encode_tiled_fn() != nullptr;
 }
 
-bool ring_dense_available(int n) { return n % kRT == 0 && n >= 64 && n <= 256 && encode_tiled_fn() != nullptr; }
-
 // p.d must be a multiple of 64 (the caller hands the remaining columns to the generic kernel).
 bool build_maps_ring(const StepParams& p, TensorMapSet* out) {
   RingMaps& m = *reinterpret_cast<RingMaps*>(out->bytes);
@@ -480,25 +437,18 @@ bool build_maps_ring(const StepParams& p, TensorMapSet* out) {
          make_half_map(&m.ys, y, p.n, p.d, p.ld, kRT);
 }
 
-// band != nullptr: band mode, the 33 entries p(delta) at index delta + 16.  band == nullptr: dense mode, p_row is a
-// device pointer to the n entries p(0 .. n-1) of the first row of the circulant P.
-int launch_step_ring(StepParams p, const TensorMapSet& maps, const double* band, const double* p_row, int sm_count,
-                     cudaStream_t stream) {
+// band: the 33 entries p(delta) at index delta + 16.
+int launch_step_ring(StepParams p, const TensorMapSet& maps, const double* band, int sm_count, cudaStream_t stream) {
   if (p.mode == kModeExternal || p.d % kRS != 0) return static_cast<int>(cudaErrorInvalidValue);
   RingCoef coef{};
-  const bool dense = band == nullptr;
-  if (!dense)
-    for (int k = 0; k < 2 * kRHalo + 1; ++k) coef.p[k] = band[k];
+  for (int k = 0; k < 2 * kRHalo + 1; ++k) coef.p[k] = band[k];
   p.S = kRS;
   p.num_slabs = p.d / kRS;
-  auto kernel = dense ? step_ring_kernel<true> : step_ring_kernel<false>;
-  const size_t smem = dense ? RingPlan<true>::kSmemBytes : RingPlan<false>::kSmemBytes;
-  const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(smem));
+  const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(step_ring_kernel), static_cast<int>(kRingSmemBytes));
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;
   if (grid <= 0) return 0;
-  kernel<<<static_cast<unsigned>(grid), kRThreads, smem, stream>>>(p, *reinterpret_cast<const RingMaps*>(maps.bytes), coef,
-                                                                   p_row);
+  step_ring_kernel<<<static_cast<unsigned>(grid), kRThreads, kRingSmemBytes, stream>>>(p, *reinterpret_cast<const RingMaps*>(maps.bytes), coef);
   return static_cast<int>(cudaGetLastError());
 }
 
