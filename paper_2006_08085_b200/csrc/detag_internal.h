@@ -78,7 +78,8 @@ struct SplitPoly {
   std::vector<double> poly_t;  // transposed, rows padded to a multiple of 16, their number to one of 32; or see circulant
   bool sparse;           // some entry is less than 2^-8 of its row's largest
   bool circulant;        // blocks depend on their distance only: poly_t holds output workers 0 .. 31
-  unsigned char id[64];  // [output block][input block] -> distinct block, 255: all zero
+  unsigned char id[64];  // [output block][input block] -> distinct block, 255: no digit of it is set
+  unsigned char reach[8];  // [output block], a bit per input block: some entry of P is not zero
 };
 
 // host helpers (spectral.cpp)

@@ -33,7 +33,7 @@
 // different warps (lanes 64 apart): each of the two finishes eight of the sixteen workers and hands the sums of the other
 // eight over, through the stage slots of its own eight whose g and a it has already taken into registers.  All sums are
 // taken at the start, so that the accumulators are free again before the noise, the gradient and the fold.
-// Zero blocks of P (rings, tori with few rounds) are skipped; equal blocks (circulant and block-circulant matrices) are
+// Blocks of P without a digit (rings, tori with few rounds) are skipped; equal blocks (circulant and block-circulant matrices) are
 // kept once.  Every wait is bounded.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -93,7 +93,8 @@ struct SplitTables {
   int num_blocks;
   int nb;                  // 32-worker blocks per side
   int sparse;              // some entry of P is less than 2^-8 of its row's largest
-  uint64_t id[8];          // [output chunk], a byte per input block: distinct block, 255: all zero
+  uint64_t id[8];          // [output chunk], a byte per input block: distinct block, 255: no digit of it is set
+  uint8_t reach[8];        // [output chunk], a bit per input block: some entry of P itself is not zero
 };
 
 struct SplitPlan {
@@ -404,7 +405,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
           const int src = __ffs(left) - 1;
           double sum = 0.0;
           for (int b = 0; b < nb; ++b) {
-            if (static_cast<uint8_t>(tb.id[c] >> (8 * b)) == 0xffu) continue;  // a zero block of P
+            if ((tb.reach[c] >> b & 1) == 0) continue;  // a zero block of P (the digits may vanish before P does)
             const int pb = !tb.circulant ? b : b >= c ? b - c : b - c + nb;  // block row 0 holds them all
 #pragma unroll 8
             for (int w = lane >> 4; w < 32; w += 2) {
@@ -714,10 +715,14 @@ void split_polynomial(int n, const std::vector<double>& poly, bool circulant, Sp
   std::vector<unsigned char> blocks;
   unsigned char id[64];  // [output chunk][input block]
   std::memset(id, 255, sizeof id);
+  unsigned char reach[8] = {0};
   std::vector<unsigned char> block(kPBlockBytes);
   for (int c = 0; c < (circulant ? 1 : nb); ++c)
     for (int kb = 0; kb < nb; ++kb) {
       uint32_t any = 0;
+      for (int i = c * kPChunk; i < std::min((c + 1) * kPChunk, rows); ++i)
+        for (int j = kb * kPChunk; j < std::min((kb + 1) * kPChunk, n); ++j)
+          if (poly[static_cast<size_t>(i) * n + j] != 0.0) reach[c] |= static_cast<unsigned char>(1u << kb);
       for (int r = 0; r < kPChunk; ++r) {
         const uint32_t* src = &digits[(static_cast<size_t>(c) * kPChunk + r) * nb * kPChunk + kb * kPChunk];
         // core matrices of 8 rows x 16 bytes, the two of a row group side by side
@@ -740,7 +745,10 @@ void split_polynomial(int n, const std::vector<double>& poly, bool circulant, Sp
     }
   if (circulant)
     for (int c = 1; c < nb; ++c)
-      for (int kb = 0; kb < nb; ++kb) id[c * 8 + kb] = id[(kb - c + nb) % nb];
+      for (int kb = 0; kb < nb; ++kb) {
+        id[c * 8 + kb] = id[(kb - c + nb) % nb];
+        reach[c] |= static_cast<unsigned char>((reach[0] >> ((kb - c + nb) % nb) & 1) << kb);
+      }
   const size_t pitch = circulant ? kPChunk : static_cast<size_t>((n + kPUnit - 1) / kPUnit) * kPUnit;
   out.poly_t.assign(nb * kPChunk * pitch, 0.0);
   for (int i = 0; i < rows; ++i)
@@ -750,6 +758,7 @@ void split_polynomial(int n, const std::vector<double>& poly, bool circulant, Sp
   out.sparse = sparse;
   out.circulant = circulant;
   std::memcpy(out.id, id, sizeof id);
+  std::memcpy(out.reach, reach, sizeof reach);
 }
 
 bool build_maps_split(const StepParams& p, TensorMapSet* out) {
@@ -781,6 +790,7 @@ int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& p
   tb.num_blocks = static_cast<int>(poly.blocks.size() / kPBlockBytes);
   tb.nb = (p.n + kPChunk - 1) / kPChunk;
   std::memcpy(tb.id, poly.id, sizeof tb.id);
+  std::memcpy(tb.reach, poly.reach, sizeof tb.reach);
   const SplitPlan plan = split_plan(tb.nb, tb.num_blocks);
   const SplitKernel kernel = p.n > 128 ? pick_split<true>(p, wide) : pick_split<false>(p, wide);
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(plan.bytes));

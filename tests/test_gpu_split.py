@@ -142,6 +142,30 @@ def test_what_is_not_finite_stays_in_reach(n, bad):
     assert worst_ratio(got[keep], (P @ x.astype(np.float64))[keep]) <= 1.0
 
 
+@pytest.mark.parametrize("n,K,worker", [(256, 34, 31), (256, 33, 224), (128, 35, 31)])
+def test_faint_entries_reach_as_far_as_the_polynomial(n, K, worker):
+    """Entries of P far below the largest of their row (1e-10 .. 1e-16 of it, whole blocks of them): an infinity travels
+    through them, and so does an operand large enough to make up for them."""
+    d, eta = 65, 0.2
+    m = _graph("ring", n)
+    P = _polynomial(m, K, eta)
+    x = np.random.default_rng(n + K).standard_normal((n, d)).astype(np.float32)
+    x[worker, 3] = np.inf
+    x[worker, 40] = 1e20
+    zero = np.zeros((n, d), np.float32)
+    with Session(m, d, K, eta, 0.0, zero, zero, x) as s:
+        s.step()
+        s.status()
+        got = s.download("x")
+    reached = P[:, worker] != 0.0
+    faint = np.abs(P[:, worker]) < 2.0 ** -32 * np.abs(P).max()
+    assert (reached & faint).any()
+    assert not np.isfinite(got[reached, 3]).any() and np.isfinite(got[~reached, 3]).all()
+    x = x.astype(np.float64)
+    bound = 2.0 ** -24 * np.abs(P @ x[:, 40]) + 2.0 ** -45 * (np.abs(P) @ np.abs(x[:, 40]))
+    assert (np.abs(got[:, 40] - P @ x[:, 40]) <= bound).all()
+
+
 def _polynomial(m, K, eta):
     w = m.to_dense()
     prev = cur = np.eye(m.n)
