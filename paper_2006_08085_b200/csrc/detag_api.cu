@@ -946,7 +946,7 @@ int detag_status(detag_state* s, void* stream) {
     e = cudaMemcpyAsync(&word[1], s->d_status_host, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail_cuda(s, e, "detag_status");
-  if (word[0] == 2 || word[1] == 2) return fail(s, DETAG_ERR_CUDA, "a kernel found its shared memory misaligned");
+  if (word[0] == 2 || word[1] == 2) return fail(s, DETAG_ERR_CUDA, "a kernel found its shared or tensor memory misplaced");
   if (word[0] != 0 || word[1] != 0) return fail(s, DETAG_ERR_TIMEOUT, "a device-side wait gave up");
   s->d_status_host = nullptr;  // read and clean: the staging area is not referred to again until the next host step
   return DETAG_OK;

@@ -34,7 +34,8 @@
 // eight over, through the stage slots of its own eight whose g and a it has already taken into registers.  All sums are
 // taken at the start, so that the accumulators are free again before the noise, the gradient and the fold.
 // Blocks of P without a digit (rings, tori with few rounds) are skipped; equal blocks (circulant and block-circulant matrices) are
-// kept once.  Every wait is bounded.
+// kept once.  Every wait is bounded but the allocation of tensor memory, which waits for kernels that do not depend on this
+// one.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -220,6 +221,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   __syncthreads();
   tmem_fence_after();
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
+  if (tid == 0 && *tmem_slot != 0) atomicExch(p.status, 2);
 
   // this CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ...; chunk q = slab number * nb + output chunk,
   // unit v = slab number * units + half chunk
