@@ -18,7 +18,7 @@ namespace {
 size_t align_up(size_t v) { return (v + detag::kWsAlign - 1) / detag::kWsAlign * detag::kWsAlign; }
 
 struct WsLayout {
-  size_t status, result, row_ptr, col_idx, vals, poly, torus, split_blocks, split_exp, split_poly, partials, total;
+  size_t status, result, row_ptr, col_idx, vals, poly, torus, split_blocks, split_exp, split_guard, split_poly, partials, total;
 };
 
 WsLayout ws_layout(const detag_state* s) {
@@ -41,6 +41,8 @@ WsLayout ws_layout(const detag_state* s) {
   off += align_up(s->split.blocks.size());
   l.split_exp = off;
   off += align_up(s->split.row_exp.size() * sizeof(int32_t));
+  l.split_guard = off;
+  off += align_up(s->split.guard.size() * sizeof(int32_t));
   l.split_poly = off;
   off += align_up(s->split.poly_t.size() * sizeof(double));
   l.partials = off;
@@ -443,10 +445,10 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     const detag::TensorMapSet* maps = maps_for(s, kFamilySplit, p);
     if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
     const WsLayout l = ws_layout(s);
-    e = detag::launch_step_split(p, *maps, s->split, p.split,
-                                 reinterpret_cast<const int32_t*>(p.split + (l.split_exp - l.split_blocks)),
-                                 reinterpret_cast<const double*>(p.split + (l.split_poly - l.split_blocks)),
-                                 variant == DETAG_VARIANT_CSR, s->sm_count, stream);
+    const detag::SplitDevice tables{p.split, reinterpret_cast<const int32_t*>(p.split + (l.split_exp - l.split_blocks)),
+                                    reinterpret_cast<const int32_t*>(p.split + (l.split_guard - l.split_blocks)),
+                                    reinterpret_cast<const double*>(p.split + (l.split_poly - l.split_blocks))};
+    e = detag::launch_step_split(p, *maps, s->split, tables, variant == DETAG_VARIANT_CSR, s->sm_count, stream);
     if (e != 0) return fail_cuda(s, e, "step kernel launch");
     return DETAG_OK;
   }
@@ -566,6 +568,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   put(l.torus, s->torus_frag.data(), s->torus_frag.size() * sizeof(double));
   put(l.split_blocks, s->split.blocks.data(), s->split.blocks.size());
   put(l.split_exp, s->split.row_exp.data(), s->split.row_exp.size() * sizeof(int32_t));
+  put(l.split_guard, s->split.guard.data(), s->split.guard.size() * sizeof(int32_t));
   put(l.split_poly, s->split.poly_t.data(), s->split.poly_t.size() * sizeof(double));
   *out = s;
   return DETAG_OK;

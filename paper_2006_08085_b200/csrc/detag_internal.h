@@ -43,7 +43,7 @@ struct StepParams {
   const int32_t* col_idx;
   const double* vals;
   const double* poly;  // dense P_K(M), row-major n x n (null when n > 64)
-  const unsigned char* split;  // split kernel: digit blocks, row exponents and P in the workspace (or null)
+  const unsigned char* split;  // split kernel: digit blocks, row exponents, guard and P in the workspace (or null)
   const double* torus; // block-circulant kernel: per-frequency 8 x 8 polynomial blocks in fragment order (or null)
   double eta;
   double alpha;
@@ -71,12 +71,15 @@ struct alignas(64) TensorMapSet {
 };
 
 // P_K(M) as the split kernel (step_split.cu) takes it: the distinct 32 x 32 blocks of its base-256 digits, their table,
-// the exponent of every row's scale, and P itself (transposed).  Empty when the kernel does not take the matrix.
+// the exponent of every row's scale, the groups of inputs that tell when a coordinate's operands may share one scale, and P
+// itself (transposed).  Empty when the kernel does not take the matrix.
 struct SplitPoly {
   std::vector<unsigned char> blocks;
   std::vector<int32_t> row_exp;
   std::vector<double> poly_t;  // transposed, rows padded to a multiple of 16, their number to one of 32; or see circulant
-  bool sparse;           // some entry is less than 2^-8 of its row's largest
+  std::vector<int32_t> guard;  // groups of guard_size inputs, as offsets into a staged column
+  int guard_size;
+  float guard_tau;       // each group's largest operand must be at least this share of the coordinate's largest
   bool circulant;        // blocks depend on their distance only: poly_t holds output workers 0 .. 31
   unsigned char id[64];  // [output block][input block] -> distinct block, 255: no digit of it is set
   unsigned char reach[8];  // [output block], a bit per input block: some entry of P is not zero
@@ -112,9 +115,14 @@ int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
 // polynomial on the integer tensor path (step_split.cu): 32 < n <= 256, DeTAG and D-PSGD steps
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
 bool build_maps_split(const StepParams& p, TensorMapSet* maps);
-int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const void* blocks /* device */,
-                      const int32_t* row_exp /* device */, const double* poly_t /* device */, bool wide_gradient, int sm_count,
-                      cudaStream_t stream);
+struct SplitDevice {  // the tables of a SplitPoly in the workspace
+  const void* blocks;
+  const int32_t* row_exp;
+  const int32_t* guard;
+  const double* poly_t;
+};
+int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& tables,
+                      bool wide_gradient, int sm_count, cudaStream_t stream);
 int launch_consensus_error(const StepParams& p, double* partials, double* result, int sm_count, cudaStream_t stream);
 int launch_init_external(const StepParams& p, int sm_count, cudaStream_t stream);  // y = g = g_ext
 int launch_expire_wait(int* status, unsigned polls, cudaStream_t stream);          // a wait nobody ends (self test)
@@ -164,7 +172,7 @@ struct detag_state {
   double* d_vals = nullptr;
   double* d_poly = nullptr;
   double* d_torus = nullptr;
-  unsigned char* d_split = nullptr;  // blocks, row exponents and P of `split`, one after the other (split_at)
+  unsigned char* d_split = nullptr;  // blocks, row exponents, guard and P of `split`, one after the other (ws_layout)
   double* d_partials = nullptr;
 
   double sigma = 0.0;

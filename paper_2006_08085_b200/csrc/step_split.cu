@@ -3,31 +3,33 @@
 //
 // AG_K(z) = P z.  The float64 tensor path (mma m8n8k4) bounds this product at 64 multiply-adds per clock and SM, which
 // for n = 100 is 3.3 times and for a dense n = 256 eight times the time of the step's HBM traffic.  Here both operands
-// are split into four balanced base-256 digits:
-//     z_j = 2^-s sum_k Z_kj 256^k   (31 bits and sign, one power of two s per coordinate and array, from the largest |z_j|)
+// are split into five balanced base-256 digits:
+//     z_j = 2^-s sum_k Z_kj 256^k   (39 bits and sign, one power of two s per coordinate and array, from the largest |z_j|)
 //     P_ij = 2^-r_i sum_l P_lij 256^l   (the same per output worker, split once by the host)
-// and the products of digits are summed by tcgen05.mma kind::i8 into 32-bit integers, exactly.  The ten digit pairs
-// with k + l >= 3 are kept, one accumulator per k + l; the six below weigh less than the rounding of the digits.
-// What is lost is at most 2^-31 of the coordinate's largest operand per term: measured against float64 1e-10 .. 1e-9 of
-// the result in the 2-norm, a twentieth of the rounding of the stored float32 values.  Results that do not contain the
-// largest operand can only be much smaller than it if P is sparse - an entry below 2^-8 of its row's largest.  Then a
-// coordinate of which eight workers in a row all lie more than 2^10 below the largest is not split: its sums are taken in
-// float64 from the operands, which stay staged that long.  So are values outside the scalable range, infinities and NaN,
-// whatever P.  (2^10 leaves such a group 2^-20 of its own largest value.  On the 256-worker ring with 16 rounds, where
-// models vary smoothly from worker to worker and pass through zero, 2^8 met one coordinate in 100 k, 2^10 none in 10^7;
-// each costs its block some 100 us.)
+// and the products of digits are summed by tcgen05.mma kind::i8 into 32-bit integers, exactly.  The fifteen digit pairs
+// with k + l >= 4 are kept, one accumulator per k + l.  What is dropped is, for an output of m terms, some 2^-38 sqrt(m) of
+// its largest weight times the coordinate's largest operand: 1e-11 .. 1e-12 of the result in the 2-norm.
+//
+// That scale is the coordinate's; an output that reads no operand near the largest must not inherit its error.  The host
+// therefore chooses groups of inputs such that every output gives every input of one of the groups at least `theta` of its
+// largest weight (split_guard below).  If the largest operand of each group is at least tau of the coordinate's largest,
+// every sum of magnitudes sum_j |P_ij z_j| is at least theta tau of largest weight times largest operand, and
+// tau = 2^-12 sqrt(m) / theta keeps the error below 2^-24 of that sum by more than five standard deviations (largest found on
+// rings, tori and random graphs of 36 .. 256 workers, magnitudes spread in various ways: a fifth of it).  A coordinate that fails the test - or holds infinities, NaN or values outside
+// the scalable range - is summed in float64: the warp that owns it takes its 32 coordinates through the float64 tensor path,
+// from the operands, which stay staged that long.  Operands drawn alike fail less than once in a thousand coordinates.
 //
 // A unit of work is a slab of 64 coordinates.  Rows 0..63 of the MMA's M = 128 are the model digits of the slab's
 // coordinates, rows 64..127 its tracker digits, so one instruction serves both arrays: A [128][32 workers] from tensor
-// memory, where the threads that split the operands put it (thread = row = tensor memory lane), B two stacked digit planes
-// [32 output workers][32 workers] of a block of P in shared memory, D [128][2 x 32] the accumulators of two neighbouring
-// weights of an output chunk of 32 workers (two chunks in flight).  An MMA with M = 128 and K = 32 bytes takes 68 cycles
-// for any N up to 128 (measured: N = 16, 32, 64, 96, 128, from tensor or shared memory alike), so two weights share one:
-// six MMAs of N = 64 per block, with a plane of zeros above the highest digit, instead of ten of N = 32.  A thread that reads an accumulator owns one coordinate and consecutive workers:
-// the four workers of a Philox call are its own and shared-memory rows are read 32 coordinates at a time, without
-// conflicts and without swizzle.
+// memory, where the threads that split the operands put it (thread = row = tensor memory lane), B the stacked digit planes
+// of a block of P in shared memory, D the accumulators of an output chunk side by side.  An MMA with M = 128 and K = 32
+// bytes takes 68 cycles for any N up to 128 (measured: N = 16, 32, 64, 96, 128, from tensor or shared memory alike), so a
+// digit of z meets all planes it is kept with in one: five MMAs (N = 160 .. 32) per block of 32 x 32 weights, digit k with
+// the planes 4 .. 4 - k, whose accumulators are neighbours.  Two chunks of 32 output workers are in flight, one beyond 128
+// workers.  A thread that reads an accumulator owns one coordinate and consecutive workers: the four workers of a Philox
+// call are its own and shared-memory rows are read 32 coordinates at a time, without conflicts and without swizzle.
 //
-// Roles: 4 or 8 splitting warps; F groups of 4 finishing warps that take half chunks (16 workers) in turn; one thread each for
+// Roles: 4 or 8 splitting warps; F groups of 4 finishing warps that take 16 workers (a unit) in turn; one thread each for
 // the MMAs, the x, y loads (one slab, handed back block by block while it is split), the g, a, c loads (R stages of 16
 // workers per finishing group, overwritten with g', x', y') and the stores.  Model and tracker sums of a coordinate sit in
 // different warps (lanes 64 apart): each of the two finishes eight of the sixteen workers and hands the sums of the other
@@ -42,6 +44,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <utility>
 
 #include "detag_internal.h"
 #include "noise.cuh"
@@ -54,11 +57,10 @@ namespace detag {
 namespace {
 
 constexpr int kPS = 64;             // coordinates per slab
-constexpr int kPChunk = 32;         // output workers per accumulator; also workers per block of P
+constexpr int kPChunk = 32;         // workers per block of P and of the staged slab
 constexpr int kPUnit = 16;          // workers a finishing group takes at a time
-constexpr int kPWeights = 4;        // accumulators: digit pairs with k + l = 6, 5, 4, 3
-constexpr int kPPlaneBytes = kPChunk * kPChunk;
-constexpr int kPBlockBytes = 5 * kPPlaneBytes;  // one block of P: a plane of zeros and the digit planes 3, 2, 1, 0
+constexpr int kPDigits = 5;         // of z and of P; also accumulators: digit pairs with k + l = 8, 7, 6, 5, 4
+constexpr int kPBlockBytes = kPDigits * kPChunk * kPChunk;  // one block of P: the digit planes 4, 3, 2, 1, 0
 constexpr int kPTileFloats = kPChunk * kPS;          // 32 rows of x or y
 constexpr int kPStageFloats = kPUnit * kPS;          // one array of one unit
 constexpr int kPStageBytes = 3 * kPStageFloats * 4;  // g | a | c  ->  g' | x' | y'
@@ -70,10 +72,17 @@ constexpr int kPMaxGroups = 4, kPMaxStages = 2, kPMaxBlocks = 8;
 __host__ __device__ constexpr int split_warps(bool big) { return big ? 4 : 8; }
 __host__ __device__ constexpr int finish_groups(bool big) { return big ? 4 : 3; }
 constexpr int kPThreads = 24 * 32;  // both: split_warps + 4 finish_groups + 4
-constexpr int kTmemColumns = 512;
-constexpr int kAccColumn = 256;     // digits below, accumulators from here on
-constexpr int kMaxDigit = 0x7F7F7F7F;  // largest integer with four balanced digits
-constexpr unsigned kRoundUp = 0x18000u;      // mantissas from 1.988 on count as the next power of two (see kMaxDigit)
+constexpr int kTmemColumns = 512, kPAccColumns = kPDigits * kPChunk;
+// Tensor memory: digits of a slab (forty columns per block of 32 workers) and accumulators.  Two accumulators, i.e. four
+// units in flight, hide the finishing warps' way from one unit to the next and come before a second slab's digits.
+__host__ __device__ constexpr int digit_buffers(int nb) { return nb <= 2 ? 2 : 1; }
+__host__ __device__ constexpr int accumulators(bool big) { return big ? 1 : 2; }
+static_assert(digit_buffers(2) * 40 * 2 + accumulators(false) * kPAccColumns <= kTmemColumns &&
+                  digit_buffers(4) * 40 * 4 + accumulators(false) * kPAccColumns <= kTmemColumns &&
+                  digit_buffers(8) * 40 * 8 + accumulators(true) * kPAccColumns <= kTmemColumns,
+              "tensor memory plan");
+constexpr long long kMaxDigits = 0x7F7F7F7F7FLL;  // largest integer with five balanced digits
+constexpr unsigned kRoundUp = 0x18000u;      // mantissas from 1.988 on count as the next power of two (see kMaxDigits)
 constexpr unsigned kSmallest = 0x12800000u;  // 2^-90: smaller maxima leave the range of the float32 scale
 constexpr size_t kPCtrlBytes = 640, kPSmemLimit = 232448;
 
@@ -93,53 +102,77 @@ struct SplitTables {
   int circulant;
   int num_blocks;
   int nb;                  // 32-worker blocks per side
-  int sparse;              // some entry of P is less than 2^-8 of its row's largest
+  const int* guard;        // guard_groups x guard_size inputs, as offsets into a coordinate's staged column
+  int guard_groups, guard_size;  // size 2 or a multiple of 4
+  float guard_tau;
   uint64_t id[8];          // [output chunk], a byte per input block: distinct block, 255: no digit of it is set
   uint8_t reach[8];        // [output chunk], a bit per input block: some entry of P itself is not zero
 };
 
 struct SplitPlan {
   int groups, stages;
-  size_t blocks_at, e_at, scale_at, ctrl_at, bytes;
+  size_t blocks_at, e_at, guard_at, scale_at, ctrl_at, bytes;
 };
 
-// Shared memory: x, y of a slab (whole blocks of 32 rows) | blocks of P | g, a, c stages | row exponents, scales, flags |
-// barriers.
-inline SplitPlan plan_for(int nb, int num_blocks, int groups, int stages) {
+// Shared memory: x, y of a slab (whole blocks of 32 rows) | blocks of P | g, a, c stages | groups of the guard | row
+// exponents, scales, flags, maxima | barriers.
+inline SplitPlan plan_for(int nb, int num_blocks, int guard_entries, int groups, int stages) {
   SplitPlan s{};
   s.groups = groups;
   s.stages = stages;
   s.blocks_at = static_cast<size_t>(nb) * 2 * kPTileFloats * 4;
   s.e_at = s.blocks_at + static_cast<size_t>(num_blocks) * kPBlockBytes;
-  s.scale_at = s.e_at + static_cast<size_t>(groups) * stages * kPStageBytes;
+  s.guard_at = s.e_at + static_cast<size_t>(groups) * stages * kPStageBytes;
+  s.scale_at = s.guard_at + static_cast<size_t>(guard_entries + 3) / 4 * 16;
   s.ctrl_at = s.scale_at + 256 * 4 + kPScaleSlots * 128 * 2 + kPScaleSlots * 4 * 4 + 4 * 128 * 8;
   s.bytes = s.ctrl_at + kPCtrlBytes;
   return s;
 }
 
 // Finishing groups and their stages: as many as fit, two stages before a fourth group (bytes = 0: nothing fits).
-inline SplitPlan split_plan(int nb, int num_blocks) {
+inline SplitPlan split_plan(int nb, int num_blocks, int guard_entries) {
   constexpr int tries[4][2] = {{4, 2}, {3, 2}, {4, 1}, {3, 1}};
   for (const auto& t : tries) {
     if (t[0] > finish_groups(nb > 4)) continue;
-    const SplitPlan s = plan_for(nb, num_blocks, t[0], t[1]);
+    const SplitPlan s = plan_for(nb, num_blocks, guard_entries, t[0], t[1]);
     if (s.bytes <= kPSmemLimit) return s;
   }
   return SplitPlan{};
 }
 
-// Integer sums of the four weights -> one float64, exact: a 64-bit integer below 2^51 added to the bits of 1.5 * 2^52.
-// Up to 128 workers the two low weights fit 32 bits together (3 * 128 * 2^14 * 256 < 2^31).
+// Integer sums of the five weights -> one float64 in units of 256^5, exact but for the rounding of the lowest: a 64-bit
+// integer below 2^51 added to the bits of 1.5 * 2^52.  `hi` = s8 * 256 + s7.  Up to 128 workers the rest fits 32 bits
+// (3 * 128 * 2^14 * 256 < 2^31).
 template <bool kBig>
-__device__ __forceinline__ double join_sums(int s6, int s5, int s4, int s3) {
-  const int hi = s6 * 256 + s5;
+__device__ __forceinline__ double join_sums(int hi, int s6, int s5, int s4) {
+  const int low = s5 + ((s4 + 128) >> 8);
   if (kBig) {
-    const long long lo = static_cast<long long>(s4) * 256 + (s3 + 0x4338000000000000LL);
+    const long long lo = static_cast<long long>(s6) * 256 + (low + 0x4338000000000000LL);
     return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - 6755399441055744.0;
   }
-  const uint32_t lo = static_cast<uint32_t>(s4 * 256 + s3) ^ 0x80000000u;  // offset by 2^31: no sign to extend
+  const uint32_t lo = static_cast<uint32_t>(s6 * 256 + low) ^ 0x80000000u;  // offset by 2^31: no sign to extend
   return __longlong_as_double(static_cast<long long>(hi) * 65536 + (0x4338000000000000LL | lo)) -
          (6755399441055744.0 + 2147483648.0);
+}
+
+// Eight joined sums of this thread's coordinate from the accumulators at `acc` (whole warp).
+template <bool kBig>
+__device__ __forceinline__ void take_sums(uint32_t acc, double (&out)[8]) {
+  int hi[8], s6[8], s5[8], s4[8];
+  {
+    int s7[8];
+    tmem_load8(acc, hi);
+    tmem_load8(acc + kPChunk, s7);
+    tmem_wait_load();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) hi[u] = hi[u] * 256 + s7[u];
+  }
+  tmem_load8(acc + 2 * kPChunk, s6);
+  tmem_load8(acc + 3 * kPChunk, s5);
+  tmem_load8(acc + 4 * kPChunk, s4);
+  tmem_wait_load();
+#pragma unroll
+  for (int u = 0; u < 8; ++u) out[u] = join_sums<kBig>(hi[u], s6[u], s5[u], s4[u]);
 }
 
 // max(|a|, |b|, |c|), NaN if one of them is
@@ -147,6 +180,68 @@ __device__ __forceinline__ float max_abs3(float a, float b, float c) {
   float r;
   asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
+}
+
+// Largest magnitude of a block's 32 staged rows (those beyond n are zeros), with what came before.
+__device__ __forceinline__ float block_max(const float* src, float top) {
+#pragma unroll
+  for (int r = 0; r < 32; r += 8) {
+    const float m = max_abs3(max_abs3(src[r * kPS], src[(r + 1) * kPS], src[(r + 2) * kPS]),
+                             max_abs3(src[(r + 3) * kPS], src[(r + 4) * kPS], src[(r + 5) * kPS]),
+                             max_abs3(src[(r + 6) * kPS], src[(r + 7) * kPS], 0.f));
+    top = max_abs3(top, m, m);
+  }
+  return top;
+}
+
+// Smallest of the largest magnitudes of groups first, first + step, ... of `size` inputs (2, or a multiple of 4).
+__device__ __forceinline__ float group_low(const float* col, const int* guard, int groups, int size, int first, int step) {
+  float low = __uint_as_float(0x7f800000u);
+  if (size == 2) {
+#pragma unroll 4
+    for (int q = first; q < groups; q += step) {
+      const int2 at = *reinterpret_cast<const int2*>(guard + 2 * q);
+      low = fminf(low, max_abs3(col[at.x], col[at.y], 0.f));
+    }
+    return low;
+  }
+  for (int q = first; q < groups; q += step) {
+    float m = 0.f;
+#pragma unroll 2
+    for (int i = 0; i < size; i += 4) {
+      const int4 at = *reinterpret_cast<const int4*>(guard + q * size + i);
+      m = max_abs3(max_abs3(m, col[at.x], col[at.y]), col[at.z], col[at.w]);
+    }
+    low = fminf(low, m);
+  }
+  return low;
+}
+
+// Digits of a block's 32 workers (zeros beyond n): digit 0 in w0, digit k in words 8 (k - 1) .. 8 k - 1 of w.  The value
+// z scale, at most 31 bits before the point, in two steps that float32 does exactly: its multiple of 2^14 next to it, and
+// what is left in 1/256, each as the low bits of 1.5 * 2^23 plus it.  With the 40-bit integer q of both, q + 0x8080808080
+// has the balanced digits as bytes offset by 128.  No conversions: they run on a pipe a quarter as wide.  No test per row:
+// the splitting is a serial chain, and so its loads and chains overlap.
+__device__ __forceinline__ void block_digits(const float* src, float scale, uint32_t (&w)[32], uint32_t (&w0)[8]) {
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    uint32_t z[4], f[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const float x = src[(4 * u + v) * kPS];
+      const float high = fmaf(x, scale, 206158430208.f);                                   // 1.5 * 2^37
+      const float rest = fmaf(x, scale, -__fadd_rn(high, -206158430208.f));
+      f[v] = __float_as_uint(fmaf(rest, 256.f, 12583040.f));                               // 1.5 * 2^23 + 128
+      z[v] = (__float_as_uint(high) << 14) + ((f[v] >> 8) + (0x80808080u - 0x4B4000u));
+    }
+    const uint32_t ab = __byte_perm(z[0], z[1], 0x5140), cd = __byte_perm(z[2], z[3], 0x5140);
+    const uint32_t ef = __byte_perm(z[0], z[1], 0x7362), gh = __byte_perm(z[2], z[3], 0x7362);
+    w0[u] = __byte_perm(__byte_perm(f[0], f[1], 0x0040), __byte_perm(f[2], f[3], 0x0040), 0x5410) ^ 0x80808080u;
+    w[u] = __byte_perm(ab, cd, 0x5410) ^ 0x80808080u;
+    w[8 + u] = __byte_perm(ab, cd, 0x7632) ^ 0x80808080u;
+    w[16 + u] = __byte_perm(ef, gh, 0x5410) ^ 0x80808080u;
+    w[24 + u] = __byte_perm(ef, gh, 0x7632) ^ 0x80808080u;
+  }
 }
 
 // kMode: kModeDetag or kModeDpsgd.  kWide: the gradient in float64 (the precision of the rounds kernel, in whose place
@@ -157,10 +252,11 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
                   const __grid_constant__ SplitPlan plan) {
   constexpr int kSplitWarps = split_warps(kBig), kMmaWarp = kSplitWarps, kLoadXYWarp = kMmaWarp + 1, kLoadEWarp = kMmaWarp + 2, kStoreWarp = kMmaWarp + 3,
                 kFinishWarp = kMmaWarp + 4;
-  constexpr int kDigBuffers = kBig ? 1 : 2;
+  constexpr int kAccs = accumulators(kBig);
   extern __shared__ __align__(128) unsigned char smem[];
   float* const xy_mem = reinterpret_cast<float*>(smem);                    // [block][x | y][32 rows][64]
   float* const e_mem = reinterpret_cast<float*>(smem + plan.e_at);
+  int* const guard = reinterpret_cast<int*>(smem + plan.guard_at);          // [group][guard_size]
   int* const row_exp = reinterpret_cast<int*>(smem + plan.scale_at);       // shifted to the exponent field of a double
   short* const scales = reinterpret_cast<short*>(row_exp + 256);           // [slot][128 rows]
   unsigned* const flags = reinterpret_cast<unsigned*>(scales + kPScaleSlots * 128);  // [slot][lane quarter]: rows in float64
@@ -173,7 +269,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   // parity wait must not find its barrier two phases ahead
   uint64_t* const acc_full = dig_empty + 2;
   uint64_t* const acc_empty = acc_full + 2 * kPMaxGroups;                  // [accumulator]
-  uint64_t* const e_full = acc_empty + 2;                                  // [group][stage], like the next two
+  uint64_t* const e_full = acc_empty + 2;                           // [group][stage], like the next two
   uint64_t* const e_empty = e_full + kPMaxGroups * kPMaxStages;
   uint64_t* const out_ready = e_empty + kPMaxGroups * kPMaxStages;
   uint64_t* const pair_bar = out_ready + kPMaxGroups * kPMaxStages;        // [group][warp pair][written, read]
@@ -193,6 +289,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     uint4* dst = reinterpret_cast<uint4*>(smem + plan.blocks_at);
     for (int e = tid; e < tb.num_blocks * (kPBlockBytes / 16); e += blockDim.x) dst[e] = src[e];
     for (int e = tid; e < 256; e += blockDim.x) row_exp[e] = e < n ? tb.row_exp[e] * (1 << 20) : 0;
+    for (int e = tid; e < tb.guard_groups * tb.guard_size; e += blockDim.x) guard[e] = tb.guard[e];
   }
   if (tid == 0) {
     bar_init(xy_full, 1);
@@ -223,6 +320,11 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
   if (tid == 0 && *tmem_slot != 0) atomicExch(p.status, 2);
 
+  // Tensor memory: digits 4 .. 1 of a slab in 32 columns per block (digit k in the eight from 8 (k - 1) on), digit 0 in
+  // eight per block, the accumulators behind all buffers of both: weight 8, 7, 6, 5, 4 in 32 columns each.
+  const int dig_buffers = kBig ? 1 : digit_buffers(nb);
+  const uint32_t low_column = tmem + dig_buffers * 32 * nb, acc_column = tmem + dig_buffers * 40 * nb;
+
   // this CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ...; chunk q = slab number * nb + output chunk,
   // unit v = slab number * units + half chunk
   const int my_slabs = aligned && *tmem_slot == 0 && blockIdx.x < p.num_slabs
@@ -238,30 +340,22 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     const int part = warp >> 2, quarter = warp & 3;
     const bool tracker = quarter >= 2;
     const int row = quarter * 32 + lane, coord = (quarter & 1) * 32 + lane;
-    const uint32_t lane_base = tmem + (static_cast<uint32_t>(quarter) << 21);
+    const uint32_t lane_base = static_cast<uint32_t>(quarter) << 21;
     const bool idle = kMode == kModeDpsgd && tracker;  // D-PSGD has no tracker: its rows of A are never read back
     const float* const col = xy_mem + (tracker ? kPTileFloats : 0) + coord;
     const int first = part == 0 ? 0 : nb / 2, last = kBig || part == 1 ? nb : nb / 2;  // blocks of this group
     bool ok = true;
     for (int k = 0; k < my_slabs && ok; ++k) {
-      const int buf = k % kDigBuffers, slot = k % kPScaleSlots;
+      const int buf = dig_buffers == 2 ? k & 1 : 0, use = dig_buffers == 2 ? k >> 1 : k, slot = k % kPScaleSlots;
       ok = warp_wait(xy_full, k);
       if (!ok) break;
-      // largest magnitude, and the smallest of the largest magnitudes of eight consecutive workers
+      // largest magnitude, and the smallest of the largest magnitudes of the guard's groups
       float top_f = 0.f, low_f = __uint_as_float(0x7f800000u);
       if (!idle) {
         for (int b = first; b < last; ++b) {
-          const float* src = col + b * (2 * kPTileFloats);
-#pragma unroll
-          for (int r = 0; r < 32; r += 8)
-            if (r < n - 32 * b) {  // rows beyond n within the eight arrive as zeros
-              const float m = max_abs3(max_abs3(src[r * kPS], src[(r + 1) * kPS], src[(r + 2) * kPS]),
-                                       max_abs3(src[(r + 3) * kPS], src[(r + 4) * kPS], src[(r + 5) * kPS]),
-                                       max_abs3(src[(r + 6) * kPS], src[(r + 7) * kPS], 0.f));
-              top_f = max_abs3(top_f, m, m);
-              if (r + 8 <= n - 32 * b) low_f = fminf(low_f, m);
-            }
+          top_f = block_max(col + b * (2 * kPTileFloats), top_f);
         }
+        low_f = group_low(col, guard, tb.guard_groups, tb.guard_size, kBig ? 0 : part, kBig ? 1 : 2);
       }
       if (!kBig) {  // the other group's blocks
         float2* const mx = maxima + (k & 1) * 256 + row;  // read again two slabs later, behind the next hand-over
@@ -274,44 +368,29 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
         top_f = max_abs3(top_f, other.x, other.x);
         low_f = fminf(low_f, other.y);
       }
-      const unsigned top = __float_as_uint(top_f), low = __float_as_uint(low_f);
-      // as float bits: not finite; too small for the scale; eight workers in a row all more than 2^10 below the largest
-      const bool exact = top >= 0x7f800000u || (top != 0 && (top < kSmallest || (tb.sparse != 0 && low + (10u << 23) < top)));
+      const unsigned top = __float_as_uint(top_f);
+      // as float bits: not finite, too small for the scale; an output may read nothing near the largest operand
+      const bool exact = top >= 0x7f800000u || (top != 0 && (top < kSmallest || low_f < tb.guard_tau * top_f));
       const int e = top == 0 || exact ? 30 : static_cast<int>((top + kRoundUp) >> 23) - 127;  // all |z| < 2^(e+1)
       const float scale = __uint_as_float(static_cast<unsigned>(157 - e) << 23);              // 2^(30 - e)
       const unsigned exact_lanes = __ballot_sync(0xffffffffu, exact);
       const bool any_exact = exact_lanes != 0;
-      if (k >= kDigBuffers) ok = warp_wait(&dig_empty[buf], k / kDigBuffers - 1);
+      if (use > 0) ok = warp_wait(&dig_empty[buf], use - 1);
       if (!ok) break;
       tmem_fence_after();
       // The slot was last read for slab k - 4: a finishing group reads a unit's scales before it releases the
-      // accumulators, and the MMAs of slab k - 2 (complete: dig_empty) came after that release for all units of k - 4.
+      // accumulators, and the MMAs of slab k - 2 (complete: dig_empty) came after that release for all units of k - 4 (two
+      // slabs have at least as many chunks as there are accumulators).
       if (part == 0) {
         scales[slot * 128 + row] = static_cast<short>(exact ? 0 : e - 6);
         if (lane == 0) flags[slot * 4 + quarter] = exact_lanes;
       }
       for (int b = first; b < last; ++b) {
         if (!idle) {
-          uint32_t w[32];  // digit plane l of this row's 32 workers in words 8 l .. 8 l + 7
-          const float* src = col + b * (2 * kPTileFloats);
-          const int rows = n - 32 * b;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            w[u] = w[8 + u] = w[16 + u] = w[24 + u] = 0u;
-            if (4 * u < rows) {  // rows beyond n within the four arrive as zeros
-              uint32_t z[4];
-#pragma unroll
-              for (int v = 0; v < 4; ++v)  // balanced digits: q + 0x80808080 has them as bytes offset by 128
-                z[v] = static_cast<uint32_t>(__float2int_rn(src[(4 * u + v) * kPS] * scale)) + 0x80808080u;
-              const uint32_t ab = __byte_perm(z[0], z[1], 0x5140), cd = __byte_perm(z[2], z[3], 0x5140);
-              const uint32_t ef = __byte_perm(z[0], z[1], 0x7362), gh = __byte_perm(z[2], z[3], 0x7362);
-              w[u] = __byte_perm(ab, cd, 0x5410) ^ 0x80808080u;
-              w[8 + u] = __byte_perm(ab, cd, 0x7632) ^ 0x80808080u;
-              w[16 + u] = __byte_perm(ef, gh, 0x5410) ^ 0x80808080u;
-              w[24 + u] = __byte_perm(ef, gh, 0x7632) ^ 0x80808080u;
-            }
-          }
-          tmem_store32(lane_base + buf * 128 + b * 32, w);
+          uint32_t w[32], w0[8];
+          block_digits(col + b * (2 * kPTileFloats), scale, w, w0);
+          tmem_store32(lane_base + tmem + (buf * nb + b) * 32, w);
+          tmem_store8(lane_base + low_column + (buf * nb + b) * 8, w0);
         }
         __syncwarp();
         if (lane == 0 && !any_exact) bar_arrive(&xy_empty[b]);  // the loads of the next slab follow block by block
@@ -321,14 +400,13 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
       __syncwarp();
       if (lane == 0) bar_arrive(&dig_full[buf]);
       if (any_exact) {  // the finishing warps read these rows' operands themselves: keep the slab until they are done with it
-        if (lane == 0) {
-          for (int t = 0; t < groups && ok; ++t) {
-            const unsigned need = static_cast<unsigned>(((k + 1) * units - t + groups - 1) / groups);
-            for (int v = 0; v < 4 && ok; ++v) ok = count_wait(&finished[4 * t + v], need, limit);
-          }
+        if (lane < 4 * groups)  // a lane per finishing warp
+          ok = count_wait_relaxed(&finished[lane], static_cast<unsigned>(((k + 1) * units - (lane >> 2) + groups - 1) / groups), limit);
+        ok = __all_sync(0xffffffffu, ok);
+        asm volatile("fence.acq_rel.cta;" ::: "memory");
+        if (lane == 0)
           for (int b = first; b < last && ok; ++b) bar_arrive(&xy_empty[b]);
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        __syncwarp();
       }
     }
     if (!ok && lane == 0) atomicExch(p.status, 1);
@@ -337,7 +415,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     const int t = (warp - kFinishWarp) >> 2, quarter = warp & 3;
     const bool second = quarter >= 2;  // reads the tracker rows; finishes workers 8..15 of every sixteen
     const int pair = quarter & 1, coord = pair * 32 + lane, mine = second ? 8 : 0;
-    const uint32_t acc_lane = tmem + kAccColumn + (static_cast<uint32_t>(quarter) << 21);
+    const uint32_t acc_lane = acc_column + (static_cast<uint32_t>(quarter) << 21);
     float* const e_group = e_mem + static_cast<size_t>(t) * stages * (kPStageBytes / 4) + coord;
     uint64_t* const written = &pair_bar[4 * t + 2 * pair];
     uint64_t* const taken = written + 1;
@@ -352,7 +430,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     }
     bool ok = true;
     for (int v = t; v < total && t < groups; v += groups, ++m) {
-      const int q = k * nb + (h >> 1);
+      const int a = (k * nb + (h >> 1)) & (kAccs - 1);
       ok = warp_wait(&acc_full[2 * t + (m & 1)], m >> 1) && warp_wait(&e_full[t * kPMaxStages + st], st_phase);
       if (!ok) break;
       tmem_fence_after();
@@ -372,59 +450,96 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
       // ---- sums of sixteen workers: eight handed to the other warp of the pair, eight kept
       double own[8];
       const int ex = (scales[slot * 128 + coord] + 1023) << 20, ey = (scales[slot * 128 + 64 + coord] + 1023) << 20;
-      int er[8];
-      *reinterpret_cast<int4*>(&er[0]) = *reinterpret_cast<const int4*>(row_exp + w0);
-      *reinterpret_cast<int4*>(&er[4]) = *reinterpret_cast<const int4*>(row_exp + w0 + 4);
-      {
-        const uint32_t acc = acc_lane + (q & 1) * 128 + (h & 1) * kPUnit;
-        int s[kPWeights][8];
+      if (exact_lanes == 0) {
+        const uint32_t acc = acc_lane + a * kPAccColumns + (h & 1) * kPUnit;
         if (kMode != kModeDpsgd || !second) {
-#pragma unroll
-          for (int w = 0; w < kPWeights; ++w) tmem_load8(acc + w * 32 + (mine ^ 8), s[w]);
-          tmem_wait_load();
+          double give[8];
+          take_sums<kBig>(acc + (mine ^ 8), give);
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            const double give = join_sums<kBig>(s[0][u], s[1][u], s[2][u], s[3][u]);
-            sg[u * kPS] = __int_as_float(__double2hiint(give));
-            sa[u * kPS] = __int_as_float(__double2loint(give));
+            sg[u * kPS] = __int_as_float(__double2hiint(give[u]));
+            sa[u * kPS] = __int_as_float(__double2loint(give[u]));
           }
         }
-#pragma unroll
-        for (int w = 0; w < kPWeights; ++w) tmem_load8(acc + w * 32 + mine, s[w]);
-        tmem_wait_load();
-#pragma unroll
-        for (int u = 0; u < 8; ++u) own[u] = join_sums<kBig>(s[0][u], s[1][u], s[2][u], s[3][u]);
-      }
-      if (exact_lanes != 0) {
-        // Rows of this warp that were not split: their sums in float64 from the operands themselves, one row after the
-        // other.  Lanes i and i + 16 sum output worker i of the sixteen over the even and the odd input workers (sixteen
-        // entries of P side by side, eight reads in flight).  The sums replace the integer ones, in units of the scales.
+        take_sums<kBig>(acc + mine, own);
+      } else {
+        // Some row of this warp was not split: all 32 in float64, from the operands themselves, in units of the scales.
         const float* const z = xy_mem + (second ? kPTileFloats : 0) + pair * 32;
+        const int to_units = (2046 << 20) - (second ? ey : ex);
+        float* const hi_word = sg - lane;  // this warp's part of the mailbox, [worker][coordinate]
+        float* const lo_word = sa - lane;
         const int c = h >> 1, pitch = tb.circulant ? kPChunk : units * kPUnit;
-        const double* const column = tb.poly_t + (tb.circulant ? kPUnit * (h & 1) : kPUnit * h) + (lane & 15);
-        const int to_units = (2046 << 20) - row_exp[kPUnit * h + (lane & 15)];
-        for (unsigned left = exact_lanes; left != 0; left &= left - 1) {
-          const int src = __ffs(left) - 1;
-          double sum = 0.0;
+        const double* const columns = tb.poly_t + (tb.circulant ? kPUnit * (h & 1) : kPUnit * h);
+        bool finite = true;
+        __syncwarp();  // every lane has taken its g and a out of the mailbox
+        // Products on the float64 tensor path: four tiles of eight coordinates (M) by eight output workers (N)
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const int to = half == 0 ? mine : mine ^ 8;
+          double sum[4][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
           for (int b = 0; b < nb; ++b) {
-            if ((tb.reach[c] >> b & 1) == 0) continue;  // a zero block of P (the digits may vanish before P does)
+            if ((tb.reach[c] >> b & 1) == 0) continue;  // a zero block of P
             const int pb = !tb.circulant ? b : b >= c ? b - c : b - c + nb;  // block row 0 holds them all
-#pragma unroll 8
-            for (int w = lane >> 4; w < 32; w += 2) {
-              const double pw = column[static_cast<size_t>(32 * pb + w) * pitch];
-              const float zw = z[b * (2 * kPTileFloats) + w * kPS + src];
-              sum = fma(pw, static_cast<double>(pw != 0.0 ? zw : 0.f), sum);  // a zero of P must not make an infinity NaN
-            }
+            const double* const pw = columns + static_cast<size_t>(32 * pb + (lane & 3)) * pitch + to + (lane >> 2);
+            const float* const zb = z + b * (2 * kPTileFloats) + (lane & 3) * kPS + (lane >> 2);
+            double w[8];  // P comes from L2: all of a block's at once
+#pragma unroll
+            for (int s = 0; s < 8; ++s) w[s] = __ldg(pw + static_cast<size_t>(4 * s) * pitch);
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) dmma(sum[i], static_cast<double>(zb[4 * s * kPS + 8 * i]), w[s]);
           }
-          sum += __shfl_xor_sync(0xffffffffu, sum, 16);
-          sum *= __hiloint2double(to_units - __shfl_sync(0xffffffffu, second ? ey : ex, src), 0);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const int at = (2 * (lane & 3) + e) * kPS + 8 * i + (lane >> 2);
+              hi_word[at] = __int_as_float(__double2hiint(sum[i][e]));
+              lo_word[at] = __int_as_float(__double2loint(sum[i][e]));
+            }
+          __syncwarp();
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            const double keep = __shfl_sync(0xffffffffu, sum, mine + u), give = __shfl_sync(0xffffffffu, sum, (mine ^ 8) + u);
-            if (lane == src) {
-              own[u] = keep;
-              sg[u * kPS] = __int_as_float(__double2hiint(give));
-              sa[u * kPS] = __int_as_float(__double2loint(give));
+            const double v = __hiloint2double(__float_as_int(sg[u * kPS]), __float_as_int(sa[u * kPS]));
+            finite = finite && (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+            const double scaled = v * __hiloint2double(to_units - row_exp[kPUnit * h + to + u], 0);
+            if (half == 0) {
+              own[u] = scaled;
+            } else {  // this lane's own column
+              sg[u * kPS] = __int_as_float(__double2hiint(scaled));
+              sa[u * kPS] = __int_as_float(__double2loint(scaled));
+            }
+          }
+          __syncwarp();
+        }
+        if (__any_sync(0xffffffffu, !finite)) {
+          // Infinities or NaN among the operands: a lane sums its own coordinate, without the zeros of P, which the products
+          // above turn into NaN.
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const int to = half == 0 ? mine : mine ^ 8;
+            double sum[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+            for (int b = 0; b < nb; ++b) {
+              if ((tb.reach[c] >> b & 1) == 0) continue;
+              const int pb = !tb.circulant ? b : b >= c ? b - c : b - c + nb;
+              for (int w = 0; w < 32; ++w) {
+                const double zw = static_cast<double>(z[b * (2 * kPTileFloats) + w * kPS + lane]);
+                const double* const pw = columns + static_cast<size_t>(32 * pb + w) * pitch + to;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                  if (pw[u] != 0.0) sum[u] = fma(pw[u], zw, sum[u]);
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const double scaled = sum[u] * __hiloint2double(to_units - row_exp[kPUnit * h + to + u], 0);
+              if (half == 0) {
+                own[u] = scaled;
+              } else {
+                sg[u * kPS] = __int_as_float(__double2hiint(scaled));
+                sa[u * kPS] = __int_as_float(__double2loint(scaled));
+              }
             }
           }
         }
@@ -433,8 +548,8 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
       __syncwarp();
       if (lane == 0) {
         bar_arrive(written);
-        bar_arrive(&acc_empty[q & 1]);
-        if (h + 1 == units && (h & 1) == 0) bar_arrive(&acc_empty[q & 1]);  // there is no other half of this chunk
+        bar_arrive(&acc_empty[a]);
+        if (h + 1 == units && (h & 1) == 0) bar_arrive(&acc_empty[a]);  // there is no other half of this chunk
       }
       // ---- normals of this thread's eight workers, while the other warp arrives
       float xi[8];
@@ -455,6 +570,9 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
       if (!ok) break;
       // ---- gossiped model and tracker (over `own`), model update, y~ - g
       const float* const og = sg + (second ? -8 * kPS : 8 * kPS);  // the other warp's slots
+      int er[8];
+      *reinterpret_cast<int4*>(&er[0]) = *reinterpret_cast<const int4*>(row_exp + w0);
+      *reinterpret_cast<int4*>(&er[4]) = *reinterpret_cast<const int4*>(row_exp + w0 + 4);
       double xd[8], yg[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -531,7 +649,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     // ---------------------------------------------------------------- MMAs
     // The whole warp walks the loop, one lane issues: operands computed in uniform control flow stay in uniform registers
     // (issued from inside a one-lane branch each MMA cost 127 cycles, eight times its time on the tensor cores).
-    const uint32_t b_base = s_addr(smem + plan.blocks_at);
+    const uint64_t b_base = mma_operand(s_addr(smem + plan.blocks_at), 256, 128);
     const bool leader = lane == 0;
     bool ok = true;
     int q = 0, t = 0, turn = 0;  // t, turn: group of the next unit and the parity of how many it has had
@@ -543,27 +661,26 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
       }
     };
     for (int k = 0; k < my_slabs && ok; ++k) {
-      const int buf = k % kDigBuffers;
-      ok = warp_wait(&dig_full[buf], k / kDigBuffers);
+      const int buf = dig_buffers == 2 ? k & 1 : 0, use = dig_buffers == 2 ? k >> 1 : k;
+      ok = warp_wait(&dig_full[buf], use);
       for (int c = 0; c < nb && ok; ++c, ++q) {
-        if (q >= 2) ok = warp_wait(&acc_empty[q & 1], (q >> 1) - 1);
+        if (q >= kAccs) ok = warp_wait(&acc_empty[q & (kAccs - 1)], q / kAccs - 1);
         if (!ok) break;
         tmem_fence_after();
-        const uint32_t acc = tmem + kAccColumn + (q & 1) * 128;
+        const uint32_t acc = acc_column + (q & (kAccs - 1)) * kPAccColumns;
         unsigned add = 0;  // the first product of an accumulator clears it
         uint64_t ids = tb.id[c];
-        for (int kb = 0; kb < nb; ++kb, ids >>= 8) {
+        uint32_t z = tmem + buf * nb * 32, z0 = low_column + buf * nb * 8;
+        for (int kb = 0; kb < nb; ++kb, ids >>= 8, z += 32, z0 += 8) {
           const uint32_t id = static_cast<uint32_t>(ids) & 0xffu;
           if (id == 0xffu) continue;
-          const uint32_t a = tmem + buf * 128 + kb * 32;
-          const uint64_t b = mma_operand(b_base + id * kPBlockBytes, 256, 128);
-          constexpr int kPlane = kPPlaneBytes / 16;  // planes from b on: zeros, digits 3, 2, 1, 0
-          mma_i8(acc, a + 24, b + 1 * kPlane, kMmaI8Desc128x64, add, leader);      // 3: (3 2) -> weights 6, 5
-          mma_i8(acc + 64, a + 24, b + 3 * kPlane, kMmaI8Desc128x64, add, leader);  //    (1 0) -> 4, 3
-          mma_i8(acc, a + 16, b, kMmaI8Desc128x64, 1u, leader);                     // 2: (- 3) -> 6, 5
-          mma_i8(acc + 64, a + 16, b + 2 * kPlane, kMmaI8Desc128x64, 1u, leader);   //    (2 1) -> 4, 3
-          mma_i8(acc + 64, a + 8, b + 1 * kPlane, kMmaI8Desc128x64, 1u, leader);    // 1: (3 2) -> 4, 3
-          mma_i8(acc + 64, a, b, kMmaI8Desc128x64, 1u, leader);                     // 0: (- 3) -> 4, 3
+          const uint64_t b = b_base + id * (kPBlockBytes / 16);
+          // digit k of z with the planes 4 .. 4 - k of P -> weights 4 + k .. 4
+          mma_i8(acc, z + 24, b, mma_i8_desc(5 * kPChunk), add, leader);
+          mma_i8(acc + kPChunk, z + 16, b, mma_i8_desc(4 * kPChunk), 1u, leader);
+          mma_i8(acc + 2 * kPChunk, z + 8, b, mma_i8_desc(3 * kPChunk), 1u, leader);
+          mma_i8(acc + 3 * kPChunk, z, b, mma_i8_desc(2 * kPChunk), 1u, leader);
+          mma_i8(acc + 4 * kPChunk, z0, b, mma_i8_desc(kPChunk), 1u, leader);
           add = 1;
         }
         hand_over();
@@ -685,54 +802,145 @@ SplitKernel pick_split(const StepParams& p, bool wide) {
 
 }  // namespace
 
+// Groups of inputs for the test described at the top, for the n x n matrix whose first `rows` rows are given (the others
+// follow from the block structure).  For each theta and group size a greedy cover: take an output that no group serves yet
+// and add those of its inputs, one after the other, that keep the most other such outputs served.  Kept is the one with the
+// least expected work: reads of its groups against coordinates in float64, if operands were drawn alike (an operand is below
+// tau of the largest with a probability of about 2 tau, a group with its size's power of that) and, weighing less, if their
+// magnitudes were spread evenly over four decades.
+void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& out) {
+  constexpr int kWords = 4, kLevels = 7;
+  // level[i][j] = k: output i gives input j between 2^-k and 2^(1 - k) of its largest weight (0: all of it)
+  std::vector<uint8_t> level(static_cast<size_t>(n) * n, 255);
+  int terms = 1;
+  for (int i = 0; i < n; ++i) {
+    const double* row = &poly[static_cast<size_t>(i % rows) * n];
+    const int shift = i / rows * rows;  // rows beyond the given ones: the block structure moves them
+    double top = 0.0;
+    int count = 0;
+    for (int j = 0; j < n; ++j) {
+      top = std::fmax(top, std::fabs(row[j]));
+      count += row[j] != 0.0 ? 1 : 0;
+    }
+    terms = std::max(terms, count);
+    for (int j = 0; j < n; ++j) {
+      const double r = std::fabs(row[j]) / (0.999999 * top);
+      const int k = r >= 1.0 ? 0 : r >= 1.0 / (1 << (kLevels - 1)) ? -std::ilogb(r) : 255;
+      level[static_cast<size_t>(i) * n + (j + shift < n ? j + shift : j + shift - n)] = static_cast<uint8_t>(k);
+    }
+  }
+  const int stride = n % 2 == 0 ? n / 2 - (n % 4 == 0 ? 1 : 2) : n / 2;  // coprime to n: ties go to inputs far apart
+  double best = 1e300;
+  std::vector<uint64_t> readers(static_cast<size_t>(n) * kWords, 0);  // [input]: outputs that give it at least theta
+  std::vector<int> inputs;
+  std::vector<int32_t> groups;
+  for (int k = 0; k < kLevels; ++k) {
+    const double tau = std::sqrt(static_cast<double>(terms)) / 4096.0 * (1 << k);
+    if (tau > 0.5) break;
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j)
+        if (level[static_cast<size_t>(i) * n + j] == k) readers[static_cast<size_t>(j) * kWords + i / 64] |= 1ull << (i % 64);
+    const double small = std::fmax(0.0, 1.0 - std::log2(1.0 / tau) / 13.3);
+    int largest = 32;  // of a group, as far as its outputs have such inputs
+    for (int size = 2; size <= 32 && size / 2 < largest; size *= 2) {
+      uint64_t open[kWords] = {0, 0, 0, 0};
+      for (int i = 0; i < n; ++i) open[i / 64] |= 1ull << (i % 64);
+      groups.clear();
+      largest = 0;
+      double fail = 0.0, fail_spread = 0.0;
+      for (int i = 0; i < n && groups.size() <= 2 * static_cast<size_t>(n) && groups.size() < best; ++i) {
+        if ((open[i / 64] >> (i % 64) & 1) == 0) continue;
+        inputs.clear();
+        for (int v = 0, j = i; v < n; ++v, j = j + stride < n ? j + stride : j + stride - n)
+          if (level[static_cast<size_t>(i) * n + j] <= k) inputs.push_back(j);
+        uint64_t served[kWords];
+        std::copy(open, open + kWords, served);
+        int have = 0, last = 0;
+        double p = 1.0, p_spread = 1.0;
+        for (; have < size && have < static_cast<int>(inputs.size()); ++have, p *= 2.0 * tau, p_spread *= small) {
+          int pick = have, most = -1;
+          for (int v = have; v < static_cast<int>(inputs.size()); ++v) {
+            const uint64_t* r = &readers[static_cast<size_t>(inputs[v]) * kWords];
+            int count = 0;
+            for (int w = 0; w < kWords; ++w) count += __builtin_popcountll(served[w] & r[w]);
+            if (count > most) {
+              most = count;
+              pick = v;
+            }
+          }
+          std::swap(inputs[have], inputs[pick]);
+          const int j = inputs[have];
+          for (int w = 0; w < kWords; ++w) served[w] &= readers[static_cast<size_t>(j) * kWords + w];
+          last = j / kPChunk * (2 * kPTileFloats) + j % kPChunk * kPS;
+          groups.push_back(last);
+        }
+        largest = std::max(largest, have);
+        for (; have < size; ++have) groups.push_back(last);
+        for (int w = 0; w < kWords; ++w) open[w] &= ~served[w];
+        fail += p;
+        fail_spread += p_spread;
+      }
+      const double work = groups.size() + n * (640.0 * std::fmin(fail, 1.0) + 4.0 * std::fmin(fail_spread, 1.0));
+      if (groups.size() <= 2 * static_cast<size_t>(n) && work < best) {
+        best = work;
+        out.guard = groups;
+        out.guard_size = size;
+        out.guard_tau = static_cast<float>(tau);
+      }
+    }
+  }
+  if (out.guard.empty()) {  // nothing to tell the coordinates by: all in float64 (one input is as good as another)
+    out.guard.assign(2, 0);
+    out.guard_size = 2;
+    out.guard_tau = 2.f;
+  }
+}
+
 // Digits of P: distinct 32 x 32 blocks, their table and the rows' exponents.  `poly`: the n x n matrix, or (circulant: the
 // blocks depend on their distance only) its first 32 rows.  Leaves `out` empty when the kernel does not take the matrix:
 // n outside 33 .. 256, an entry or a row that cannot be scaled, too many distinct blocks.
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out) {
   out = SplitPoly{};
   if (n <= 32 || n > 256 || encode_tiled_fn() == nullptr) return;
-  const int nb = (n + kPChunk - 1) / kPChunk, rows = circulant ? kPChunk : n;
-  std::vector<uint32_t> digits(static_cast<size_t>(circulant ? 1 : nb) * kPChunk * nb * kPChunk, 0);  // balanced digits as bytes
+  const int nb = (n + kPChunk - 1) / kPChunk, rows = circulant ? kPChunk : n, wide = nb * kPChunk;
+  std::vector<int64_t> digits(static_cast<size_t>(circulant ? 1 : nb) * kPChunk * wide, 0);  // balanced digits as bytes
   std::vector<int32_t> row_exp(n);
-  bool sparse = false;
   for (int i = 0; i < rows; ++i) {
     const double* row = &poly[static_cast<size_t>(i) * n];
-    double top = 0.0, low = 1e300;
+    double top = 0.0;
     for (int j = 0; j < n; ++j) {
       const double v = std::fabs(row[j]);
       if (!(v <= 1e30)) return;  // also NaN
       top = v > top ? v : top;
-      low = v < low ? v : low;
     }
     if (!(top >= 1e-30)) return;
-    sparse = sparse || low < top / 256.0;
     int e = std::ilogb(top);
-    if (std::nearbyint(std::ldexp(top, 30 - e)) > kMaxDigit) ++e;
+    if (std::nearbyint(std::ldexp(top, 38 - e)) > static_cast<double>(kMaxDigits)) ++e;
     for (int k = i; k < n; k += rows) row_exp[k] = e - 30;
-    const double scale = std::ldexp(1.0, 30 - e);
-    uint32_t* out_row = &digits[static_cast<size_t>(i) * nb * kPChunk];
+    const double scale = std::ldexp(1.0, 38 - e);
     for (int j = 0; j < n; ++j)
-      out_row[j] = (static_cast<uint32_t>(static_cast<int32_t>(std::lrint(row[j] * scale))) + 0x80808080u) ^ 0x80808080u;
+      digits[static_cast<size_t>(i) * wide + j] = (std::llrint(row[j] * scale) + 0x8080808080LL) ^ 0x8080808080LL;
   }
+  SplitPoly made{};
+  split_guard(n, poly, rows, made);
   std::vector<unsigned char> blocks;
-  unsigned char id[64];  // [output chunk][input block]
-  std::memset(id, 255, sizeof id);
-  unsigned char reach[8] = {0};
+  std::memset(made.id, 255, sizeof made.id);
   std::vector<unsigned char> block(kPBlockBytes);
+  constexpr int plane = kPChunk * kPChunk;  // bytes
   for (int c = 0; c < (circulant ? 1 : nb); ++c)
     for (int kb = 0; kb < nb; ++kb) {
-      uint32_t any = 0;
+      int64_t any = 0;
       for (int i = c * kPChunk; i < std::min((c + 1) * kPChunk, rows); ++i)
         for (int j = kb * kPChunk; j < std::min((kb + 1) * kPChunk, n); ++j)
-          if (poly[static_cast<size_t>(i) * n + j] != 0.0) reach[c] |= static_cast<unsigned char>(1u << kb);
+          if (poly[static_cast<size_t>(i) * n + j] != 0.0) made.reach[c] |= static_cast<unsigned char>(1u << kb);
       for (int r = 0; r < kPChunk; ++r) {
-        const uint32_t* src = &digits[(static_cast<size_t>(c) * kPChunk + r) * nb * kPChunk + kb * kPChunk];
-        // core matrices of 8 rows x 16 bytes, the two of a row group side by side
+        const int64_t* src = &digits[(static_cast<size_t>(c) * kPChunk + r) * wide + kb * kPChunk];
+        // planes 4 .. 0 of core matrices of 8 rows x 16 bytes, the two of a row group side by side
         unsigned char* at = &block[(r / 8) * 256 + (r % 8) * 16];
         for (int w = 0; w < kPChunk; ++w) {
           any |= src[w];
-          for (int l = 0; l < 4; ++l)
-            at[(4 - l) * kPPlaneBytes + (w / 16) * 128 + w % 16] = static_cast<unsigned char>(src[w] >> (8 * l));
+          for (int l = 0; l < kPDigits; ++l)
+            at[(kPDigits - 1 - l) * plane + (w / 16) * 128 + w % 16] = static_cast<unsigned char>(src[w] >> (8 * l));
         }
       }
       if (any == 0) continue;
@@ -740,27 +948,25 @@ void split_polynomial(int n, const std::vector<double>& poly, bool circulant, Sp
       int hit = 0;
       while (hit < have && std::memcmp(&blocks[static_cast<size_t>(hit) * kPBlockBytes], block.data(), kPBlockBytes) != 0) ++hit;
       if (hit == have) {
-        if (split_plan(nb, have + 1).bytes == 0) return;
+        if (split_plan(nb, have + 1, static_cast<int>(made.guard.size())).bytes == 0) return;
         blocks.insert(blocks.end(), block.begin(), block.end());
       }
-      id[c * 8 + kb] = static_cast<unsigned char>(hit);
+      made.id[c * 8 + kb] = static_cast<unsigned char>(hit);
     }
   if (circulant)
     for (int c = 1; c < nb; ++c)
       for (int kb = 0; kb < nb; ++kb) {
-        id[c * 8 + kb] = id[(kb - c + nb) % nb];
-        reach[c] |= static_cast<unsigned char>((reach[0] >> ((kb - c + nb) % nb) & 1) << kb);
+        made.id[c * 8 + kb] = made.id[(kb - c + nb) % nb];
+        made.reach[c] |= static_cast<unsigned char>((made.reach[0] >> ((kb - c + nb) % nb) & 1) << kb);
       }
   const size_t pitch = circulant ? kPChunk : static_cast<size_t>((n + kPUnit - 1) / kPUnit) * kPUnit;
-  out.poly_t.assign(nb * kPChunk * pitch, 0.0);
+  made.poly_t.assign(wide * pitch, 0.0);
   for (int i = 0; i < rows; ++i)
-    for (int j = 0; j < n; ++j) out.poly_t[j * pitch + i] = poly[static_cast<size_t>(i) * n + j];
-  out.blocks.swap(blocks);
-  out.row_exp.swap(row_exp);
-  out.sparse = sparse;
-  out.circulant = circulant;
-  std::memcpy(out.id, id, sizeof id);
-  std::memcpy(out.reach, reach, sizeof reach);
+    for (int j = 0; j < n; ++j) made.poly_t[j * pitch + i] = poly[static_cast<size_t>(i) * n + j];
+  made.blocks.swap(blocks);
+  made.row_exp.swap(row_exp);
+  made.circulant = circulant;
+  out = std::move(made);
 }
 
 bool build_maps_split(const StepParams& p, TensorMapSet* out) {
@@ -778,22 +984,25 @@ bool build_maps_split(const StepParams& p, TensorMapSet* out) {
   return true;
 }
 
-int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const void* blocks, const int32_t* row_exp,
-                      const double* poly_t, bool wide, int sm_count, cudaStream_t stream) {
+int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& dev, bool wide,
+                      int sm_count, cudaStream_t stream) {
   if (p.mode == kModeExternal || poly.blocks.empty()) return static_cast<int>(cudaErrorInvalidValue);
   p.S = kPS;
   p.num_slabs = (p.d + kPS - 1) / kPS;
   SplitTables tb{};
-  tb.blocks = static_cast<const uint4*>(blocks);
-  tb.row_exp = row_exp;
-  tb.poly_t = poly_t;
-  tb.sparse = poly.sparse ? 1 : 0;
+  tb.blocks = static_cast<const uint4*>(dev.blocks);
+  tb.row_exp = dev.row_exp;
+  tb.poly_t = dev.poly_t;
+  tb.guard = dev.guard;
+  tb.guard_size = poly.guard_size;
+  tb.guard_groups = static_cast<int>(poly.guard.size()) / poly.guard_size;
+  tb.guard_tau = poly.guard_tau;
   tb.circulant = poly.circulant ? 1 : 0;
   tb.num_blocks = static_cast<int>(poly.blocks.size() / kPBlockBytes);
   tb.nb = (p.n + kPChunk - 1) / kPChunk;
   std::memcpy(tb.id, poly.id, sizeof tb.id);
   std::memcpy(tb.reach, poly.reach, sizeof tb.reach);
-  const SplitPlan plan = split_plan(tb.nb, tb.num_blocks);
+  const SplitPlan plan = split_plan(tb.nb, tb.num_blocks, static_cast<int>(poly.guard.size()));
   const SplitKernel kernel = p.n > 128 ? pick_split<true>(p, wide) : pick_split<false>(p, wide);
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(plan.bytes));
   if (e != 0) return e;

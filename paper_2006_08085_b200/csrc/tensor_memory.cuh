@@ -40,6 +40,12 @@ __device__ __forceinline__ void tmem_store32(uint32_t addr, const uint32_t (&w)[
       : "memory");
 }
 
+__device__ __forceinline__ void tmem_store8(uint32_t addr, const uint32_t (&w)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+
 // Eight columns; the values may be used after tmem_wait_load().
 __device__ __forceinline__ void tmem_load8(uint32_t addr, int (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -49,8 +55,10 @@ __device__ __forceinline__ void tmem_load8(uint32_t addr, int (&v)[8]) {
 }
 
 // Instruction descriptor of kind::i8: 32-bit integer sums (2 at bit 4), signed bytes for A and B (1 at bits 7 and 10),
-// both K-major, N = 64 (N / 8 at bit 17), M = 128 (M / 16 at bit 24).
-constexpr uint32_t kMmaI8Desc128x64 = (2u << 4) | (1u << 7) | (1u << 10) | ((64u / 8) << 17) | ((128u / 16) << 24);
+// both K-major, N a multiple of 16 up to 256 (N / 8 at bit 17), M = 128 (M / 16 at bit 24).
+__host__ __device__ constexpr uint32_t mma_i8_desc(int n) {
+  return (2u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n / 8) << 17) | ((128u / 16) << 24);
+}
 
 // Descriptor of an operand in shared memory: K-major core matrices of 8 rows x 16 bytes without swizzle, row groups
 // `row_stride` bytes apart, the two halves of K `k_stride` bytes apart.  Addresses advance by 16 bytes per unit.

@@ -1,5 +1,5 @@
 """The polynomial on the integer tensor path (32 < n <= 256): tile edges, block structures, modes, and the coordinates it
-contracts in float64 instead (values too far apart for one scale, infinities, NaN)."""
+contracts in float64 instead (an output may read nothing near the largest operand, infinities, NaN)."""
 import numpy as np
 import pytest
 
@@ -93,11 +93,10 @@ def _runs(cols):
 
 @pytest.mark.parametrize("n,kind,K", [(40, "ring", 2), (100, "regular4", 2), (100, "regular4", 8), (256, "ring", 9)])
 def test_values_far_apart_keep_their_precision(n, kind, K):
-    """A few workers a million times larger than the rest: results out of their reach must not inherit their scale.  A
-    float64 sum rounded once to float32 is off by half an ulp, 2^-24 of itself, and that is all in those columns if the
-    polynomial has entries below 2^-8 of their row's largest (they are contracted in float64).  Elsewhere the dropped digit
-    pairs add, per term, three products of uniform digits (standard deviation 74) at 2^16 of 2^62 times the two scales,
-    each up to twice the largest operand or entry: 2^-27 of those for 256 terms, bounded by six deviations."""
+    """A few neighbouring workers a million times larger than the rest: results out of their reach must not inherit their
+    scale.  A float64 sum rounded once to float32 is off by half an ulp, 2^-24 of itself, and that is all in those columns
+    if the polynomial has entries below 2^-8 of their row's largest.  Elsewhere the bound allows 2^-24.4 of the largest
+    operand times the row's largest entry, far more than the kernel's digits leave out (2^-37)."""
     d, eta = 200, 0.2
     m = _graph(kind, n)
     P = _polynomial(m, K, eta)
@@ -120,6 +119,53 @@ def test_values_far_apart_keep_their_precision(n, kind, K):
     bound += np.where(split, 2.0 ** -24.4 * top * np.abs(x).max(axis=0), 0.0)
     assert (np.abs(got - P @ x) <= bound).all()
     assert (got[:, 5] == 0.0).all()
+
+
+def _unequal(pattern, n, d, rng):
+    z = rng.standard_normal((n, d))
+    if pattern == "one larger":
+        z[n // 3] *= 2.0 ** 9
+    elif pattern == "every eighth":
+        z[::8] *= 10.0 ** rng.integers(3, 9, d)
+    elif pattern == "all but the last":
+        z[:n - n % 8 - (n % 8 == 0) * 4] *= 1e6
+    elif pattern == "sorted":
+        z *= (10.0 ** np.linspace(-2, 2, n))[:, None]
+    elif pattern == "log-uniform":
+        z *= 10.0 ** rng.uniform(-2, 2, (n, d))
+    elif pattern == "one alone":
+        z[np.arange(n) != n // 2] = 0.0
+    elif pattern == "consensus":
+        z = z[:1] + 1e-6 * z
+    return z.astype(np.float32)
+
+
+@pytest.mark.parametrize("kind,n", [("ring", 36), ("regular4", 48), ("ring", 100), ("regular4", 100), ("directed", 128),
+                                    ("ring", 224), ("torus", 256)])
+@pytest.mark.parametrize("K", [1, 2, 6, 16])
+def test_every_result_is_as_precise_as_what_it_reads(kind, n, K):
+    """P z per element, model and tracker, against float64: half an ulp of the stored value, 2^-24 |P z|, and as much again
+    for the sum, 2^-24 |P| |z| - the magnitudes that this very output reads, whatever the other workers hold."""
+    d, eta = 150, 0.2
+    m = _graph(kind, n)
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(n * 31 + K)
+    zero = np.zeros((n, d), np.float32)
+    patterns = ["alike", "one larger", "every eighth", "all but the last", "sorted", "log-uniform", "one alone", "consensus"]
+    with Session(m, d, K, eta, 0.0, zero, zero, zero) as s:
+        for k, pattern in enumerate(patterns):
+            state = {"x": _unequal(pattern, n, d, rng), "y": _unequal(patterns[k - 1], n, d, rng)}
+            s.upload("g", zero)
+            for name, v in state.items():
+                s.upload(name, v)
+            B.detag_set_step(s.state, 0)
+            s.step()
+            s.status()
+            for name, v in state.items():
+                got, z = s.download(name).astype(np.float64), v.astype(np.float64)
+                bound = 2.0 ** -24 * (np.abs(P @ z) + np.abs(P) @ np.abs(z)) + 1e-45
+                worst = (np.abs(got - P @ z) / bound).max()
+                assert worst <= 1.0, (pattern if name == "x" else patterns[k - 1], name, worst)
 
 
 @pytest.mark.parametrize("n,bad", [(48, np.inf), (100, np.nan), (256, -np.inf)])
