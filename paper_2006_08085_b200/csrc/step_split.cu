@@ -834,7 +834,7 @@ void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& ou
   std::vector<uint64_t> readers(static_cast<size_t>(n) * kWords, 0);  // [input]: outputs that give it at least theta
   std::vector<int> inputs;
   std::vector<int32_t> groups;
-  for (int k = 0; k < kLevels; ++k) {
+  for (int k = 0; k < kLevels && best > 0.25 * n; ++k) {
     const double tau = std::sqrt(static_cast<double>(terms)) / 4096.0 * (1 << k);
     if (tau > 0.5) break;
     for (int i = 0; i < n; ++i)
@@ -842,7 +842,7 @@ void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& ou
         if (level[static_cast<size_t>(i) * n + j] == k) readers[static_cast<size_t>(j) * kWords + i / 64] |= 1ull << (i % 64);
     const double small = std::fmax(0.0, 1.0 - std::log2(1.0 / tau) / 13.3);
     int largest = 32;  // of a group, as far as its outputs have such inputs
-    for (int size = 2; size <= 32 && size / 2 < largest; size *= 2) {
+    for (int size = 2; size <= 32 && size / 2 <= largest && best > 0.25 * n; size *= 2) {
       uint64_t open[kWords] = {0, 0, 0, 0};
       for (int i = 0; i < n; ++i) open[i / 64] |= 1ull << (i % 64);
       groups.clear();
@@ -880,7 +880,7 @@ void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& ou
         fail += p;
         fail_spread += p_spread;
       }
-      const double work = groups.size() + n * (640.0 * std::fmin(fail, 1.0) + 4.0 * std::fmin(fail_spread, 1.0));
+      const double work = groups.size() + n * (6000.0 * std::fmin(fail, 1.0) + 40.0 * std::fmin(fail_spread, 1.0));
       if (groups.size() <= 2 * static_cast<size_t>(n) && work < best) {
         best = work;
         out.guard = groups;
