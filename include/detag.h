@@ -56,8 +56,10 @@ enum {
 
 /* Kernel variants of the gossip part of the step; all compute the same result.  The polynomial variants of 32 < n <= 256
    workers run on the integer tensor path where its shared-memory plan holds P_K(M) (any matrix up to n = 128, beyond that
-   matrices whose 32 x 32 blocks depend on their distance only), a few coordinates excepted in float64; otherwise they run
-   as rounds. */
+   matrices whose 32 x 32 blocks depend on their distance only); coordinates in which an output may read operands far below
+   the largest are summed in float64 instead, which takes up to five times as long when it concerns all of them (one or two
+   rounds on sparse graphs, workers of very different magnitude).  Circulant bands run in float64 throughout.  What neither
+   takes runs as rounds. */
 enum {
   DETAG_VARIANT_AUTO = 0,  /* host cost model picks */
   DETAG_VARIANT_CSR = 1,   /* K rounds of neighbour-indexed sums over the CSR rows, slab staged on chip: any graph, n <= 1024.
@@ -65,8 +67,8 @@ enum {
                               polynomial if the integer tensor path takes it; forced, the rounds run as such */
   DETAG_VARIANT_DENSE = 2, /* one product with the host-precomputed polynomial P_K(M), n <= 128 (any M) */
   DETAG_VARIANT_RING = 3,  /* circulant M (rings), n % 32 == 0, 64 <= n <= 1024: the circulant polynomial P_K(M), a band
-                              while K * bandwidth <= 16, or any (n <= 256), e.g. at Theorem 3's phase length; for n > 256 the
-                              last d % 64 coordinates run through the CSR kernel in the same call */
+                              while K * bandwidth <= 16, or any (n <= 256), e.g. at Theorem 3's phase length; a band's last
+                              d % 64 coordinates run through another kernel in the same call */
   DETAG_VARIANT_TORUS = 4  /* block-circulant M with 8-worker blocks, symmetric in the block distance (R x 8 tori, n = 32 or 64):
                               Fourier transform along the block axis, one 8 x 8 polynomial block per frequency, transform back */
 };

@@ -258,7 +258,7 @@ void analyse_torus(detag_state* s) {
 
 bool torus_ok(const detag_state* s) { return s->torus && s->d <= 0x7fffffffLL; }
 
-// The circulant kernel takes polynomials whose half-band is at most 16; the integer tensor path any up to 256 workers.
+// The circulant kernel takes polynomials whose half-band is at most 16; the integer tensor path the others up to 256 workers.
 bool ring_band(const detag_state* s) { return detag::ring_variant_available(s->n, s->half_band); }
 
 bool band_ok(const detag_state* s) {
@@ -323,8 +323,8 @@ bool variant_runs_mode(const detag_state* s, int variant) {
 
 int resolve_variant(const detag_state* s) {
   if (s->variant_forced != DETAG_VARIANT_AUTO) return s->variant_forced;
-  // a ring whose band fits takes the circulant kernel from n = 64 on; with a dense polynomial only beyond the
-  // reach of the 64-row dense kernel
+  // a ring whose band fits takes the circulant kernel from n = 64 on; rings with a dense polynomial go by that name too,
+  // beyond 64 workers
   const bool ring = band_ok(s) && (ring_band(s) || s->n > 64);
   if (step_mode(s) == detag::kModeDpsgd && s->n > 32 && ring) return DETAG_VARIANT_RING;
   if (step_mode(s) != detag::kModeDetag) return (s->n <= 32 && dense_ok(s)) ? DETAG_VARIANT_DENSE : DETAG_VARIANT_CSR;
@@ -332,10 +332,11 @@ int resolve_variant(const detag_state* s) {
   if (s->n > 32 && torus_ok(s)) return DETAG_VARIANT_TORUS;
   if (dense_ok(s)) {
     if (s->n > 64) {
-      // Which of the two names the call goes by, where no structure decides: the rounds' if a float64 product (blocks of
-      // eight workers on four tensor-path schedulers) would take longer than the rounds, measured at d = 2 M (ms) - one
-      // or two rounds on graphs of degree four.  With the integer tensor path both run there (split_ok): 100 workers,
-      // d = 2 M, 1.6 ms for any K against 3.2 ms for one round.
+      // Where no structure decides, the rounds if a float64 product on the tensor path (blocks of eight workers on four
+      // schedulers) would take longer, in ms at d = 2 M: one or two rounds on graphs of degree four.  Both run on the
+      // integer tensor path now where that takes the matrix (split_ok; 100 workers, d = 2 M: 2.0 ms for two rounds, 3.9 as
+      // rounds); what the choice still decides is the name the call goes by and with it the precision of the gradient, which
+      // the rounds evaluate in float64 and the products in float32 at the stored model.
       const int blocks = (s->n + 7) / 8, blocks_eff = blocks % 4 == 3 ? blocks + 1 : blocks;
       const double dense_ms = 0.0412 * blocks_eff * blocks / 2.0;
       const double rounds_ms = 0.024 * s->n + 0.00155 * s->K * static_cast<double>(s->col_idx.size());
@@ -394,9 +395,20 @@ const detag::TensorMapSet* maps_for(detag_state* s, int family, const StepParams
   return &en.maps;
 }
 
-// The columns from `first` on through the generic rounds kernel (the tensor-path kernels that take whole 32- or
-// 64-coordinate pieces hand their remainder here, in the same call).
-int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cudaStream_t stream, int* cuda_error) {
+int launch_split(detag_state* s, const StepParams& p, bool wide, cudaStream_t stream) {
+  const detag::TensorMapSet* maps = maps_for(s, kFamilySplit, p);
+  if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+  const WsLayout l = ws_layout(s);
+  const detag::SplitDevice tables{p.split, reinterpret_cast<const int32_t*>(p.split + (l.split_exp - l.split_blocks)),
+                                  reinterpret_cast<const int32_t*>(p.split + (l.split_guard - l.split_blocks)),
+                                  reinterpret_cast<const double*>(p.split + (l.split_poly - l.split_blocks))};
+  const int e = detag::launch_step_split(p, *maps, s->split, tables, wide, s->sm_count, stream);
+  return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
+}
+
+// The columns from `first` on, which the circulant kernel leaves (it takes whole 64-coordinate slabs), in the same call:
+// through the integer tensor path where that takes the matrix (one slab), else through the generic rounds kernel.
+int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cudaStream_t stream) {
   StepParams pt = p;
   pt.d = p.d - first;
   pt.coord_offset = p.coord_offset + first;
@@ -406,22 +418,26 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   pt.a = p.a + first;
   pt.c = p.c + first;
   if (p.y_obs) pt.y_obs = p.y_obs + first;
+  if (!s->split.blocks.empty()) return launch_split(s, pt, false, stream);
   const int rc = detag::plan_step_csr(pt, s->smem_optin);
   if (rc != DETAG_OK) return fail(s, rc, "graph too large for the shared-memory plan");
-  *cuda_error = detag::launch_step_csr(pt, s->sm_count, stream);
-  return DETAG_OK;
+  const int e = detag::launch_step_csr(pt, s->sm_count, stream);
+  return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
 }
 
 // The integer tensor path takes the dense and circulant products with 32 < n <= 256, and, where the choice is the
-// library's, the rounds of such matrices too.
+// library's, the rounds of such matrices too.  Circulant bands stay on their float64 kernel, which needs no test of the
+// operands; us per step, integer path -> that one: 64 workers, d = 2 M, K = 1 1099 -> 1035, K = 16 1020 -> 1035; 128, d = 1 M,
+// K = 1 1260 -> 1031, K = 16 1103 -> 1031; 224, d = 500 k, K = 16 1198 -> 927; 256, d = 1 M, K = 1 3157 -> 2032, K = 16
+// 2620 -> 2032; 256, d = 4096 82 -> 30.
 bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   if (s->split.blocks.empty() || p.mode == detag::kModeExternal || p.d > 0x7fffffffLL) return false;
   if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
-  return variant == DETAG_VARIANT_DENSE || variant == DETAG_VARIANT_RING;
+  return variant == DETAG_VARIANT_DENSE || (variant == DETAG_VARIANT_RING && !ring_band(s));
 }
 
 // Up to 16 workers a thread takes a coordinate's whole column.  us per step, tensor-path kernel -> that one: 8 workers,
-// d = 8 M 1005 -> 362; 12, d = 4 M 565 -> 294; 13, d = 4 M 565 -> 461; 16, d = 4 M 568 -> 474, d = 270 k 43 -> 32.
+// d = 8 M 1005 -> 362; 12, d = 4 M 565 -> 294; 13, d = 4 M 565 -> 461; 16, d = 4 M 568 -> 474, d = 270 k 47 -> 42.
 // Caller-written gradients read four arrays before the first contraction, and have no noise and gradient to save: beyond
 // eight workers they stay (8, d = 8 M 619 -> 307; 13, d = 4 M 381 -> 540; 16, d = 270 k 34.9 -> 36.0).  The
 // failure-detection self test wants bounded waits, of which that kernel has none: it runs the tensor-path kernel.
@@ -441,17 +457,7 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     return fail(s, DETAG_ERR_UNBOUND, "the synthetic gradient needs the objective arrays a and c");
   if (p.mode == detag::kModeExternal && !p.g_ext)
     return fail(s, DETAG_ERR_UNBOUND, "caller-written gradients selected but no gradient array given");
-  if (split_ok(s, p, variant)) {
-    const detag::TensorMapSet* maps = maps_for(s, kFamilySplit, p);
-    if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-    const WsLayout l = ws_layout(s);
-    const detag::SplitDevice tables{p.split, reinterpret_cast<const int32_t*>(p.split + (l.split_exp - l.split_blocks)),
-                                    reinterpret_cast<const int32_t*>(p.split + (l.split_guard - l.split_blocks)),
-                                    reinterpret_cast<const double*>(p.split + (l.split_poly - l.split_blocks))};
-    e = detag::launch_step_split(p, *maps, s->split, tables, variant == DETAG_VARIANT_CSR, s->sm_count, stream);
-    if (e != 0) return fail_cuda(s, e, "step kernel launch");
-    return DETAG_OK;
-  }
+  if (split_ok(s, p, variant)) return launch_split(s, p, variant == DETAG_VARIANT_CSR, stream);
   // what the integer tensor path does not take although its variant promises it (a polynomial whose entries cannot be
   // scaled, e.g. under an absurd momentum) runs as rounds
   const bool as_rounds = (variant == DETAG_VARIANT_DENSE && p.n > 32) || (variant == DETAG_VARIANT_RING && !ring_band(s));
@@ -467,7 +473,6 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
       break;
     }
     case DETAG_VARIANT_RING: {
-      // the circulant kernel takes whole 64-coordinate slabs; the last d % 64 columns go to the generic kernel
       const long long d_main = p.d & ~63LL;
       if (d_main > 0) {
         StepParams pm = p;
@@ -478,7 +483,7 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
         if (e != 0) return fail_cuda(s, e, "step kernel launch");
       }
       if (d_main < p.d) {
-        const int rc = launch_tail_columns(s, p, d_main, stream, &e);
+        const int rc = launch_tail_columns(s, p, d_main, stream);
         if (rc != DETAG_OK) return rc;
       }
       break;

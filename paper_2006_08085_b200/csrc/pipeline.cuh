@@ -166,6 +166,13 @@ __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
                : "d"(a), "d"(b));
 }
 
+// max(|a|, |b|, |c|), NaN if one of them is
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // 4 x 4 transpose over four neighbouring lanes (lane bits 0 and 1): lane kq gives row kq = v[0..3] and receives
 // column kq.
 __device__ __forceinline__ void transpose_quad(float (&v)[4], int kq) {

@@ -4,8 +4,7 @@
 // Metropolis ring and its slack matrices) the K-round accelerated gossip AG_K(z) = P z has a circulant
 // P = P_K(M), P[i][j] = p((j - i) mod n).  While p(delta) = 0 for |delta| > 16 (K times the bandwidth of M at most 16), 32
 // output rows need a window of 64 input rows, and of the 16 x 4 blocks of that 64 x 32 slice only 10 per 8-row output
-// block are non-zero: 80 float64 MMAs (m8n8k4) per 8 coordinates x 32 workers for tracker and model together.  (Up to 256
-// workers the integer tensor path, step_split.cu, comes first.)
+// block are non-zero: 80 float64 MMAs (m8n8k4) per 8 coordinates x 32 workers for tracker and model together.
 //
 // Layout of the contraction: the eight coordinates of a warp's tile are the M index of the MMA, the input worker
 // the contraction index (k-step s takes window rows 4 s + kq) and the output worker the N index, permuted so that
@@ -25,7 +24,7 @@
 //          and three TMA stores send the stage out.
 // Every transfer is one three-dimensional TMA box {32 coordinates, 2 halves, rows} in the 128-byte swizzle: rows
 // arrive as contiguous 256-byte pieces, and with the row ownership above every warp-wide shared-memory access hits
-// 32 different banks.  The kernel takes whole slabs only: the host hands the last d % 64 columns to the generic
+// 32 different banks.  The kernel takes whole slabs only: the host hands the last d % 64 columns to another
 // kernel.
 // Roles: 16 consumer warps in two groups taking alternate tiles; one thread loading x, y chunks, one loading
 // g, a, c stages, one storing, one publishing how many chunks have landed (so that no consumer ever starts a
@@ -363,6 +362,32 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
             dmma(cx[t], zx, bfrag[u]);
           }
         }
+      }
+    }
+    // Infinities or NaN in the window: the band's zeros have carried them to every row of the tile.  Each lane then sums its
+    // own rows anew, without those.  (As float bits the upper half of a double that is not finite is a NaN.)
+    float seen = 0.f;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      seen = max_abs3(seen, __int_as_float(__double2hiint(cx[t][0])), __int_as_float(__double2hiint(cx[t][1])));
+      seen = max_abs3(seen, __int_as_float(__double2hiint(cy[t][0])), __int_as_float(__double2hiint(cy[t][1])));
+    }
+    if (__any_sync(0xffffffffu, seen != seen)) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        double sx = 0.0, sy = 0.0;
+        for (int d = 0; d <= 2 * kRHalo; ++d) {
+          const double w = coef.p[d];
+          if (w == 0.0) continue;
+          const int row = kq + 4 * m + d, q = 2 * b + (row >> 4), r = row & (kChunkRows - 1);  // in the window, its chunk, in that
+          const float* ch = (q < CPS) ? ring_mem + static_cast<size_t>((Qbase + q) % kSlots) * kSlotFloats
+                                      : side_mem + static_cast<size_t>(sl & 1) * kSlotFloats;
+          const int o = r * kRS + half_of_tile * kRHalf + (((chunk16 ^ ((2 * r + half_of_tile) & 7)) << 2) | (crow & 3));
+          sx = fma(w, static_cast<double>(ch[o]), sx);
+          if (!dpsgd) sy = fma(w, static_cast<double>(ch[kChunkFloats + o]), sy);
+        }
+        cx[m >> 1][m & 1] = sx;
+        cy[m >> 1][m & 1] = sy;
       }
     }
     // gradient point of Algorithm 2 as printed: this lane's own rows of the old model, still in their chunks

@@ -175,13 +175,6 @@ __device__ __forceinline__ void take_sums(uint32_t acc, double (&out)[8]) {
   for (int u = 0; u < 8; ++u) out[u] = join_sums<kBig>(hi[u], s6[u], s5[u], s4[u]);
 }
 
-// max(|a|, |b|, |c|), NaN if one of them is
-__device__ __forceinline__ float max_abs3(float a, float b, float c) {
-  float r;
-  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
 // Largest magnitude of a block's 32 staged rows (those beyond n are zeros), with what came before.
 __device__ __forceinline__ float block_max(const float* src, float top) {
 #pragma unroll

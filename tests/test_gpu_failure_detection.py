@@ -56,12 +56,15 @@ def test_a_wait_that_nothing_ends_gives_up_and_is_reported():
 @pytest.mark.parametrize("n,d,K,variant,after", [
     (16, 64 * 148 * 4 + 17, 3, B.DETAG_VARIANT_DENSE, 1),   # dense kernel, n <= 32: several slabs per CTA
     (16, 64 * 148 * 4 + 17, 3, B.DETAG_VARIANT_DENSE, 0),   # nothing is ever loaded
-    (64, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_RING, 3),     # band kernel, ring
-    (48, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # band kernel, dense window mode
+    (64, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_RING, 3),     # circulant band kernel
+    (288, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_RING, 5),
+    (48, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # integer tensor path, two slabs' digits
     (64, 64 * 148 * 3 + 5, 2, B.DETAG_VARIANT_TORUS, 2),    # block-circulant transform kernel
     (32, 64 * 148 * 3 + 5, 2, B.DETAG_VARIANT_TORUS, 0),
-    (72, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # dense kernel with the polynomial in registers, two stages of g, a, c
-    (128, 64 * 148 * 2 + 37, 2, B.DETAG_VARIANT_DENSE, 0),  # ... one stage
+    (72, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # ... one slab's digits
+    (128, 64 * 148 * 2 + 37, 2, B.DETAG_VARIANT_DENSE, 0),
+    (160, 64 * 148 + 5, 17, B.DETAG_VARIANT_RING, 1),       # ... more than 128 workers, beyond the band kernel's reach
+    (256, 64 * 148 + 5, 17, B.DETAG_VARIANT_RING, 18),
 ])
 def test_a_stalled_loader_times_out_every_waiter_and_the_state_recovers(n, d, K, variant, after):
     m, a, c, x0 = _case(n, d, n, torus=variant == B.DETAG_VARIANT_TORUS)

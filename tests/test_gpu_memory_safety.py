@@ -50,7 +50,8 @@ def _guarded_state(torch, m, d, ld, K, eta, observe, variant, where):
 @pytest.mark.parametrize("n,d,ld,K,variant", [
     (5, 30, 48, 2, B.DETAG_VARIANT_DENSE), (32, 131, 132, 3, B.DETAG_VARIANT_DENSE), (3, 2, 4, 1, B.DETAG_VARIANT_DENSE),
     (33, 67, 68, 2, B.DETAG_VARIANT_DENSE), (50, 130, 136, 3, B.DETAG_VARIANT_DENSE), (64, 65, 68, 2, B.DETAG_VARIANT_DENSE),
-    (64, 67, 72, 4, B.DETAG_VARIANT_RING), (96, 130, 132, 2, B.DETAG_VARIANT_RING),
+    (64, 67, 72, 4, B.DETAG_VARIANT_RING), (96, 130, 132, 2, B.DETAG_VARIANT_RING), (288, 130, 132, 2, B.DETAG_VARIANT_RING),
+    (160, 67, 72, 17, B.DETAG_VARIANT_RING), (256, 130, 132, 17, B.DETAG_VARIANT_RING),
     (64, 67, 72, 4, B.DETAG_VARIANT_TORUS), (32, 130, 132, 2, B.DETAG_VARIANT_TORUS), (64, 3, 4, 2, B.DETAG_VARIANT_TORUS),
     (72, 67, 68, 2, B.DETAG_VARIANT_DENSE), (100, 130, 132, 3, B.DETAG_VARIANT_DENSE), (128, 31, 32, 2, B.DETAG_VARIANT_DENSE),
     (9, 77, 80, 3, B.DETAG_VARIANT_CSR), (70, 33, 36, 2, B.DETAG_VARIANT_CSR)])

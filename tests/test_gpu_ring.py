@@ -1,0 +1,97 @@
+"""The circulant band kernel (K * bandwidth <= 16) over several slabs per block: reuse of the ring of chunks, of the side copy
+and of the stages from slab to slab, both gradient points, D-PSGD, and the columns beyond the last whole slab."""
+import numpy as np
+import pytest
+
+from oracle import detag_oracle as orc
+from paper_2006_08085_b200 import binding as B
+from paper_2006_08085_b200 import build, inputs
+from paper_2006_08085_b200.session import Session
+from parity import HALF_ULP32, oracle_problem, worst_ratio
+
+pytestmark = pytest.mark.gpu
+
+SLABS = 64 * 148  # one slab of 64 coordinates per block
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def _matrix(kind, n):
+    if kind == "ring":
+        return inputs.metropolis_weights(inputs.ring_graph(n))
+    return inputs.directed_cycle_blend(n, 0.4, 0.35)
+
+
+@pytest.mark.parametrize("n,d,K,kind", [
+    (64, 3 * SLABS + 5, 16, "ring"), (96, 2 * SLABS + 65, 1, "directed"), (256, 3 * SLABS + 7, 4, "ring"),
+    (288, 3 * SLABS + 5, 5, "directed"), (512, 2 * SLABS + 130, 16, "ring"), (1024, SLABS + 64, 3, "ring")])
+@pytest.mark.parametrize("mode", ["new", "start", "dpsgd"])
+def test_one_step_against_the_oracle(n, d, K, kind, mode):
+    m = _matrix(kind, n)
+    eta, alpha = 0.3, 0.02
+    rng = np.random.default_rng(n + d)
+    a = rng.random((n, d), dtype=np.float32) + np.float32(0.5)
+    c, x0, y0, g0 = (rng.standard_normal((n, d), dtype=np.float32) for _ in range(4))
+    with Session(m, d, K, eta, alpha, a, c, x0, 0.1, 11, observe_gossip=mode != "dpsgd", variant=B.DETAG_VARIANT_RING,
+                 gradient_point=int(mode == "start"), algorithm=int(mode == "dpsgd")) as s:
+        s.upload("y", y0)
+        s.upload("g", g0)
+        B.detag_set_step(s.state, 0)
+        s.step()
+        s.status()
+        got = {k: s.download(k) for k in ("x", "y", "g") + (() if mode == "dpsgd" else ("y_gossip",))}
+    w = m.to_dense()
+    prev = P = np.eye(n)
+    for _ in range(K):
+        prev, P = P, (1.0 + eta) * w @ P - eta * prev
+    # a few stretches of columns: both ends, and one in every slab of the first and of the last block
+    starts = {0, 30, d - 70, *(64 * (148 * k) + 20 for k in range(d // SLABS + 1)),
+              *(64 * (148 * k + 147) + 10 for k in range(d // SLABS + 1))}
+    for lo in sorted(v for v in starts if v < d):
+        cut = slice(lo, min(d, lo + 70))
+        x, y, g = (v[:, cut].astype(np.float64) for v in (x0, y0, g0))
+        p = oracle_problem(m, K, eta, alpha, a[:, cut], c[:, cut], 0.1, 11, lo)
+        y_gossip = P @ y
+        x_new = P @ x - alpha * (g if mode == "dpsgd" else y_gossip)
+        g_new = orc.stochastic_gradient(p, x if mode == "start" else x_new, 1)
+        assert worst_ratio(got["x"][:, cut], x_new) <= 1.0, (lo, "x")
+        assert worst_ratio(got["g"][:, cut], g_new) <= 1.0, (lo, "g")
+        if mode == "dpsgd":
+            assert np.array_equal(got["y"][:, cut], y0[:, cut])
+            continue
+        assert worst_ratio(got["y_gossip"][:, cut], y_gossip) <= 1.0, (lo, "y_gossip")
+        assert worst_ratio(got["y"][:, cut], y_gossip + g_new - g, extra=HALF_ULP32 * np.abs(g_new)) <= 1.0, (lo, "y")
+
+
+@pytest.mark.parametrize("n,worker,K,bad", [(64, 63, 16, np.inf), (96, 0, 3, np.nan), (256, 31, 1, -np.inf), (288, 270, 5, np.inf)])
+def test_what_is_not_finite_stays_in_reach(n, worker, K, bad):
+    """One operand of the model and one of the tracker; the band's zeros must not carry them further, also around the end."""
+    d, eta = 130, 0.2
+    m = _matrix("ring", n)
+    x, y = np.random.default_rng(n).standard_normal((2, n, d)).astype(np.float32)
+    x[worker, 9] = bad
+    y[worker, 64] = bad
+    zero = np.zeros((n, d), np.float32)
+    with Session(m, d, K, eta, 0.0, zero, zero, x, observe_gossip=True, variant=B.DETAG_VARIANT_RING) as s:
+        s.upload("y", y)
+        B.detag_set_step(s.state, 0)
+        s.step()
+        s.status()
+        got = {"x": s.download("x"), "y_gossip": s.download("y_gossip")}
+    P = np.eye(n)
+    prev, w = P, m.to_dense()
+    for _ in range(K):
+        prev, P = P, (1.0 + eta) * w @ P - eta * prev
+    reached = P[:, worker] != 0.0
+    assert reached.sum() == 2 * K + 1
+    for (name, z), col in zip((("x", x), ("y_gossip", y)), (9, 64)):
+        assert not np.isfinite(got[name][reached, col]).any(), name
+        keep = np.ones((n, d), bool)
+        keep[reached, col] = False
+        if name == "x":
+            keep[reached, 64] = False  # x' = P x - 0 * P y
+        z[worker, col] = 0.0
+        assert worst_ratio(got[name][keep], (P @ z.astype(np.float64))[keep]) <= 1.0, name
