@@ -44,8 +44,9 @@ namespace {
 
 // kMode: what the step computes (kModeDetag / kModeExternal / kModeDpsgd).
 // kAtStart: the gradient is taken at the model the step started from (Algorithm 2 as printed) instead of the new one.
-// kKs: number of 4-worker input blocks that can be non-zero, ceil(n / 4) rounded up to 2, 4 or 8; the MMAs of the
-// all-zero blocks of the padded P are not issued.
+// kKs: 4-worker input blocks that are multiplied, 8 (n <= 32) or, for caller-written gradients of at most 16 workers, 4; the
+// other steps of so few workers run on the kernel with a thread per coordinate (step_small.cu), and here only for the
+// failure-detection self test, on the padded matrix.
 template <int kMode, bool kAtStart, int kKs>
 __global__ void __launch_bounds__(kMmaThreads, 1)
 step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
@@ -246,11 +247,10 @@ step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
 
 typedef void (*MmaKernel)(const StepParams, const MmaMaps);
 
-template <int kKs>
 MmaKernel pick_mode(const StepParams& p) {
-  if (p.mode == kModeExternal) return step_mma_kernel<kModeExternal, false, kKs>;
-  if (p.mode == kModeDpsgd) return step_mma_kernel<kModeDpsgd, false, kKs>;
-  return p.grad_at_start ? step_mma_kernel<kModeDetag, true, kKs> : step_mma_kernel<kModeDetag, false, kKs>;
+  if (p.mode == kModeExternal) return p.n <= 16 ? step_mma_kernel<kModeExternal, false, 4> : step_mma_kernel<kModeExternal, false, 8>;
+  if (p.mode == kModeDpsgd) return step_mma_kernel<kModeDpsgd, false, 8>;
+  return p.grad_at_start ? step_mma_kernel<kModeDetag, true, 8> : step_mma_kernel<kModeDetag, false, 8>;
 }
 
 }  // namespace
@@ -278,7 +278,7 @@ bool build_maps_mma(const StepParams& p, TensorMapSet* out) {
 int launch_step_mma(StepParams p, const TensorMapSet& maps, int sm_count, cudaStream_t stream) {
   p.S = kS;
   p.num_slabs = (p.d + kS - 1) / kS;
-  const MmaKernel kernel = p.n <= 8 ? pick_mode<2>(p) : p.n <= 16 ? pick_mode<4>(p) : pick_mode<8>(p);
+  const MmaKernel kernel = pick_mode(p);
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(kMmaSmemBytes));
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;

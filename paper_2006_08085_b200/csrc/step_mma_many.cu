@@ -18,9 +18,7 @@ namespace detag {
 
 namespace {
 
-// kKs: number of 4-worker input blocks that can be non-zero, ceil(n / 4) rounded up to 2, 4 or 8; the MMAs of the
-// all-zero blocks of the padded P are not issued.
-template <bool kAtStart, int kKs>
+template <bool kAtStart>
 __global__ void __launch_bounds__(kMmaThreads, 1)
 step_mma_many_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
   // No static shared memory in this kernel: the dynamic array starts at the CTA's shared window, whose
@@ -87,7 +85,7 @@ step_mma_many_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
           cx[t][0] = cx[t][1] = 0.0;
         }
 #pragma unroll
-        for (int ks = 0; ks < kKs; ++ks) {
+        for (int ks = 0; ks < kN / 4; ++ks) {
           const int src = (4 * ks + kq) * kPitchXY + cl + r;
           const double by = static_cast<double>(sy[src]);
           const double bx = fma(-alpha, by, static_cast<double>(sx[src]));
@@ -181,13 +179,7 @@ int launch_step_mma_many(StepParams p, const TensorMapSet& maps, int sm_count, c
   if (p.steps < 1 || p.mode != kModeDetag) return static_cast<int>(cudaErrorInvalidValue);
   p.S = kS;
   p.num_slabs = (p.d + kS - 1) / kS;
-  void (*kernel)(const StepParams, const MmaMaps);
-  if (p.n <= 8)
-    kernel = p.grad_at_start ? step_mma_many_kernel<true, 2> : step_mma_many_kernel<false, 2>;
-  else if (p.n <= 16)
-    kernel = p.grad_at_start ? step_mma_many_kernel<true, 4> : step_mma_many_kernel<false, 4>;
-  else
-    kernel = p.grad_at_start ? step_mma_many_kernel<true, 8> : step_mma_many_kernel<false, 8>;
+  void (*const kernel)(const StepParams, const MmaMaps) = p.grad_at_start ? step_mma_many_kernel<true> : step_mma_many_kernel<false>;
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(kMmaSmemBytes));
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;

@@ -309,9 +309,8 @@ def test_circulant_kernel_with_a_dense_polynomial(n, d, K, kind):
                                         (88, 31, 4, "regular4"), (96, 1057, 5, "directed"), (104, 64, 8, "regular4"),
                                         (127, 97, 3, "path"), (128, 160, 12, "regular4")])
 def test_dense_polynomial_held_in_registers(n, d, K, kind):
-    """64 < n <= 128, any matrix: the polynomial as register-resident warp strips.  Unstructured, non-symmetric and
-    irregular matrices, worker counts on and off the 8-row blocks, d below, on and off the 32-column halves the
-    kernel takes (the remainder runs on the generic kernel in the same call)."""
+    """64 < n <= 128, any matrix: the dense polynomial on the integer tensor path.  Unstructured, non-symmetric and irregular
+    matrices, worker counts on and off the 32-worker blocks, d below, on and off the 64-column slabs."""
     rng = np.random.default_rng(n * 31 + d)
     if kind == "regular4":
         m = inputs.metropolis_weights(inputs.random_regular4_graph(n, n + K))
