@@ -429,11 +429,17 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
 // library's, the rounds of such matrices too.  Circulant bands stay on their float64 kernel, which needs no test of the
 // operands; us per step, integer path -> that one: 64 workers, d = 2 M, K = 1 1099 -> 1035, K = 16 1020 -> 1035; 128, d = 1 M,
 // K = 1 1260 -> 1031, K = 16 1103 -> 1031; 224, d = 500 k, K = 16 1198 -> 927; 256, d = 1 M, K = 1 3157 -> 2032, K = 16
-// 2620 -> 2032; 256, d = 4096 82 -> 30.
+// 2620 -> 2032; 256, d = 4096 82 -> 30.  Unless d is ragged and short:
+// the columns beyond the last whole slab are a second launch, a slab's latency long, where the integer path takes everything
+// in one.  Two launches -> one: 64 workers, K = 4, d = 9001 26 -> 16; 128, K = 4, d = 9001 39 -> 24, but K = 1, d = 20001
+// 61 -> 60; 256, K = 4, d = 4097 71 -> 43, but K = 1, d = 9001 70 -> 82.
 bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   if (s->split.blocks.empty() || p.mode == detag::kModeExternal || p.d > 0x7fffffffLL) return false;
   if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
-  return variant == DETAG_VARIANT_DENSE || (variant == DETAG_VARIANT_RING && !ring_band(s));
+  if (variant == DETAG_VARIANT_DENSE) return true;
+  if (variant != DETAG_VARIANT_RING) return false;
+  // by the length of the state, not of a staged chunk: host-resident stepping gives the same bits
+  return !ring_band(s) || (s->d % 64 != 0 && s->d <= (s->n <= 128 ? 2LL : 1LL) * 64 * s->sm_count);
 }
 
 // Up to 16 workers a thread takes a coordinate's whole column.  us per step, tensor-path kernel -> that one: 8 workers,

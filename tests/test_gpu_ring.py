@@ -69,7 +69,7 @@ def test_one_step_against_the_oracle(n, d, K, kind, mode):
 @pytest.mark.parametrize("n,worker,K,bad", [(64, 63, 16, np.inf), (96, 0, 3, np.nan), (256, 31, 1, -np.inf), (288, 270, 5, np.inf)])
 def test_what_is_not_finite_stays_in_reach(n, worker, K, bad):
     """One operand of the model and one of the tracker; the band's zeros must not carry them further, also around the end."""
-    d, eta = 130, 0.2
+    d, eta = 128, 0.2
     m = _matrix("ring", n)
     x, y = np.random.default_rng(n).standard_normal((2, n, d)).astype(np.float32)
     x[worker, 9] = bad
