@@ -47,10 +47,12 @@ KERNEL_SOURCES = {
 }
 MEASURED_TRAFFIC = {
     # (kernel, mode): (source digest, bytes per wc)
-    ("mma", "dense"): ("22eae46feb506e80", 31.46),     # cfg5 shape at d = 2 M: 1.2949 GB read + 0.7183 GB written / 64 M wc
-    ("torus", "torus8"): ("427a2bff49b63d9c", 31.27),  # cfg3 shape at d = 1 M: 1.2803 + 0.7208 GB / 64 M wc
-    ("ring", "band"): ("60c16ee651aa8e4f", 31.12),     # cfg4 shape at d = 200 k: 1.0280 + 0.5652 GB / 51.2 M wc
-    ("csr", "rounds"): ("bcc2ab2f791da0eb", 31.17),    # the same graph through the rounds kernel: 0.8088 + 0.4381 GB / 40 M wc
+    ("small", "column"): ("2d293cc7edde3135", 29.00),   # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1440 GB written / 16 M wc
+    ("mma", "dense"): ("98fc5c149709161c", 31.37),     # cfg5 shape at d = 2 M: 1.2899 + 0.7176 GB / 64 M wc
+    ("torus", "torus8"): ("22f3bc13d621a2ed", 31.26),  # cfg3 shape at d = 1 M: 1.2801 + 0.7204 GB / 64 M wc
+    ("ring", "band"): ("1a16972a0d29d375", 31.09),     # cfg4 shape at d = 200 k: 1.0279 + 0.5637 GB / 51.2 M wc
+    ("split", "digits"): ("b1eb219985913d27", 30.81),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4321 GB / 40 M wc
+    ("csr", "rounds"): ("bd6f6c1d0ef487a7", 31.16),     # the same graph through the rounds kernel: 0.8089 + 0.4374 GB / 40 M wc
 }
 
 # Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes) and that
@@ -65,7 +67,7 @@ def kernel_key(variant: str, n: int):
     if variant == "dense":
         return ("small", "column") if n <= 16 else ("mma", "dense") if n <= 32 else ("split", "digits")
     if variant == "ring":
-        return ("split", "digits") if n <= 256 else ("ring", "band")
+        return ("ring", "band")  # K times the bandwidth at most 16, as in the configurations
     if variant == "csr":
         return ("csr", "rounds")
     if variant == "torus":

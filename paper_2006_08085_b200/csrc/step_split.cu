@@ -36,7 +36,15 @@
 // eight over, through the stage slots of its own eight whose g and a it has already taken into registers.  All sums are
 // taken at the start, so that the accumulators are free again before the noise, the gradient and the fold.
 // Blocks of P without a digit (rings, tori with few rounds) are skipped; equal blocks (circulant and block-circulant matrices) are
-// kept once.  Every wait is bounded but the allocation of tensor memory, which waits for kernels that do not depend on this
+// kept once.
+//
+// Bound by the finishing warps' chain (207 instructions per worker-coordinate in all, 60 % of the issue slots at n = 100), at a
+// dense n = 256 by MMAs and splitting, which take turns.  us per step, the float64 kernels this one replaced -> now: 48
+// workers, printed timing, d = 1.0 M 861 -> 470; 100 workers, d = 2 M 3518 -> 2060; 256-ring at K = 196, d = 200 k
+// 1940 -> 640; 16 x 16 torus, d = 500 k 8992 -> 1640.  (Four digits and four accumulators took 417, 1680, 566 and 1420, but
+// left 2^-31 of the coordinate's largest operand in every result.)  With every coordinate in float64: 48 workers, K = 1,
+// d = 1 M 477 -> 1410; 100 workers, K = 2 1040 -> 4730; the torus 1570 -> 8710 - P comes from L2 and the slab is held.
+// Every wait is bounded but the allocation of tensor memory, which waits for kernels that do not depend on this
 // one.
 #include <cuda.h>
 #include <cuda_runtime.h>
