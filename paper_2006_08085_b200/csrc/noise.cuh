@@ -56,34 +56,43 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
   return Philox4{c0, c1, c2, c3};
 }
 
-// -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9.
+// 1 + (r >> 9) 2^-23: the exponent bits of 1.0 come in from above as the word is shifted, one instruction for both.
+__device__ __forceinline__ float one_to_two(uint32_t r) { return __uint_as_float(__funnelshift_r(r, 0x7fu, 9)); }
+
+// -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9.  The factor -2 is in the argument F = -2 f and in the coefficients, scaled by
+// powers of two: the bits are those of -2 times the logarithm.
 __device__ __forceinline__ float neg2_ln_unit(uint32_t r) {
-  const float v = __uint_as_float(0x3f800000u | (r >> 9));  // 1 + k 2^-23
-  const float u = v - 0x1.fffffep-1f;                        // (2k+1) 2^-24, exact
+  const float u = one_to_two(r) - 0x1.fffffep-1f;            // (2k+1) 2^-24, exact
   const int bits = __float_as_int(u);
-  const int e = (bits - 0x3f2aaaab) >> 23;                   // u = m 2^e with m in [2/3, 4/3)
-  const float m = __int_as_float(bits - (e << 23));
-  const float f = m - 1.0f;
-  // ln(1+f) = f + f^2 r(f) on |f| <= 1/3 (Chebyshev fit of (ln(1+f) - f)/f^2, degree 7)
-  float r7 = 0.13756538927555084f;
-  r7 = fmaf(r7, f, -0.1504942923784256f);
-  r7 = fmaf(r7, f, 0.1405421793460846f);
-  r7 = fmaf(r7, f, -0.16481579840183258f);
-  r7 = fmaf(r7, f, 0.2000732272863388f);
-  r7 = fmaf(r7, f, -0.25004205107688904f);
-  r7 = fmaf(r7, f, 0.33333271741867065f);
-  r7 = fmaf(r7, f, -0.49999985098838806f);
-  float ln = fmaf(f * f, r7, f);
-  const float ef = __int_as_float(0x4b400000 + e) - 12582912.0f;  // e as a float, no conversion instruction
-  ln = fmaf(ef, 1.42860677e-06f, ln);
-  ln = fmaf(ef, 0.693145751953125f, ln);
-  return -2.0f * ln;
+  const int eb = (bits - 0x3f2aaaab) & 0xff800000;           // u = m 2^e with m in [2/3, 4/3); eb = e 2^23
+  const float m = __int_as_float(bits - eb);
+  const float F = fmaf(m, -2.0f, 2.0f);                      // -2 f, f = m - 1, exact
+  // ln(1+f) = f + f^2 r(f) on |f| <= 1/3 (Chebyshev fit of (ln(1+f) - f)/f^2, degree 7); here -r(-F/2) / 2
+  float r7 = 0.13756538927555084f * 0x1p-8f;
+  r7 = fmaf(r7, F, 0.1504942923784256f * 0x1p-7f);
+  r7 = fmaf(r7, F, 0.1405421793460846f * 0x1p-6f);
+  r7 = fmaf(r7, F, 0.16481579840183258f * 0x1p-5f);
+  r7 = fmaf(r7, F, 0.2000732272863388f * 0x1p-4f);
+  r7 = fmaf(r7, F, 0.25004205107688904f * 0x1p-3f);
+  r7 = fmaf(r7, F, 0.33333271741867065f * 0x1p-2f);
+  r7 = fmaf(r7, F, 0.49999985098838806f * 0x1p-1f);
+  float ln = fmaf(F * F, r7, F);
+  const float ef = __int2float_rn(eb);                       // e 2^23, exact
+  ln = fmaf(ef, -1.42860677e-06f * 0x1p-22f, ln);
+  return fmaf(ef, -0.693145751953125f * 0x1p-22f, ln);
+}
+
+// Approximate reciprocal square root of a normal number (rsqrtf() tests for subnormal arguments first).
+__device__ __forceinline__ float rsqrt_normal(float v) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
 }
 
 __device__ __forceinline__ void box_muller(uint32_t r_even, uint32_t r_odd, float& first, float& second) {
-  const float t = neg2_ln_unit(r_even);                                   // > 0
-  const float rad = t * rsqrtf(t);
-  const float w = __uint_as_float(0x3f800000u | (r_odd >> 9)) - 1.5f;     // u_ang - 1/2 in [-1/2, 1/2), exact
+  const float t = neg2_ln_unit(r_even);                                   // 1.2e-7 .. 33.3
+  const float rad = t * rsqrt_normal(t);
+  const float w = one_to_two(r_odd) - 1.5f;                               // u_ang - 1/2 in [-1/2, 1/2), exact
   const float theta = w * 6.283185307179586f;                             // 2 pi u_ang - pi
   first = -rad * __cosf(theta);                                           // cos(2 pi u) = -cos(2 pi u - pi)
   second = -rad * __sinf(theta);
