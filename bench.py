@@ -38,7 +38,7 @@ BYTES_PER_WC = 32  # read x, y, g, a, c + write x, y, g, float32 each: the fused
 # small case of the same kernel; traffic grows in proportion to n*d).  Keyed by the sha256 prefix of the kernel
 # sources the capture was taken on: a changed kernel reports null until it is captured again.
 KERNEL_SOURCES = {
-    "small": ("step_small.cu", "noise.cuh"),
+    "small": ("step_small.cu", "noise.cuh", "pipeline.cuh"),
     "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh"),
     "mma": ("step_mma.cu", "mma_common.cuh", "pipeline.cuh", "noise.cuh"),
     "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh"),

@@ -442,14 +442,12 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   return !ring_band(s) || (s->d % 64 != 0 && s->d <= (s->n <= 128 ? 2LL : 1LL) * 64 * s->sm_count);
 }
 
-// Up to 16 workers a thread takes a coordinate's whole column.  us per step, tensor-path kernel -> that one: 8 workers,
-// d = 8 M 1005 -> 362; 12, d = 4 M 565 -> 294; 13, d = 4 M 565 -> 461; 16, d = 4 M 568 -> 474, d = 270 k 47 -> 42.
-// Caller-written gradients read four arrays before the first contraction, and have no noise and gradient to save: beyond
-// eight workers they stay (8, d = 8 M 619 -> 307; 13, d = 4 M 381 -> 540; 16, d = 270 k 34.9 -> 36.0).  The
-// failure-detection self test wants bounded waits, of which that kernel has none: it runs the tensor-path kernel.
+// Up to 16 workers the step runs in registers, without staging.  us per step, tensor-path kernel with its stages and barriers
+// -> that one: 8 workers, d = 8 M 1005 -> 327; 12, d = 4 M 565 -> 273; 13, d = 4 M 565 -> 350; 16, d = 4 M 568 -> 378, d = 270 k
+// 47 -> 29; caller-written gradients, 16, d = 4 M 415 -> 321, d = 270 k 34.9 -> 24.9.  The failure-detection self test wants
+// bounded waits, of which that kernel has none: it runs the tensor-path kernel.
 bool small_ok(const StepParams& p) {
-  if (p.n > detag::kMaxSmallWorkers || p.stall_after >= 0) return false;
-  return p.mode != detag::kModeExternal || p.n <= 8;
+  return p.n <= detag::kMaxSmallWorkers && p.stall_after < 0;
 }
 
 // Picks the kernel variant, plans it for the sizes in `p` and launches it.

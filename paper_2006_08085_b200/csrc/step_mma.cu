@@ -44,10 +44,8 @@ namespace {
 
 // kMode: what the step computes (kModeDetag / kModeExternal / kModeDpsgd).
 // kAtStart: the gradient is taken at the model the step started from (Algorithm 2 as printed) instead of the new one.
-// kKs: 4-worker input blocks that are multiplied, 8 (n <= 32) or, for caller-written gradients of at most 16 workers, 4; the
-// other steps of so few workers run on the kernel with a thread per coordinate (step_small.cu), and here only for the
-// failure-detection self test, on the padded matrix.
-template <int kMode, bool kAtStart, int kKs>
+// At most 16 workers run on step_small.cu, and here, on the padded matrix, only for the failure-detection self test.
+template <int kMode, bool kAtStart>
 __global__ void __launch_bounds__(kMmaThreads, 1)
 step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
   // No static shared memory in this kernel: the dynamic array starts at the CTA's shared window, whose
@@ -120,7 +118,7 @@ step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
         }
       }
 #pragma unroll
-      for (int ks = 0; ks < kKs; ++ks) {
+      for (int ks = 0; ks < kN / 4; ++ks) {
         const int src = (4 * ks + kq) * kPitchXY + cl + r;
         double by = 0.0, bx;
         if (kMode == kModeDpsgd) {
@@ -248,9 +246,9 @@ step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
 typedef void (*MmaKernel)(const StepParams, const MmaMaps);
 
 MmaKernel pick_mode(const StepParams& p) {
-  if (p.mode == kModeExternal) return p.n <= 16 ? step_mma_kernel<kModeExternal, false, 4> : step_mma_kernel<kModeExternal, false, 8>;
-  if (p.mode == kModeDpsgd) return step_mma_kernel<kModeDpsgd, false, 8>;
-  return p.grad_at_start ? step_mma_kernel<kModeDetag, true, 8> : step_mma_kernel<kModeDetag, false, 8>;
+  if (p.mode == kModeExternal) return step_mma_kernel<kModeExternal, false>;
+  if (p.mode == kModeDpsgd) return step_mma_kernel<kModeDpsgd, false>;
+  return p.grad_at_start ? step_mma_kernel<kModeDetag, true> : step_mma_kernel<kModeDetag, false>;
 }
 
 }  // namespace

@@ -1,21 +1,30 @@
-// DeTAG step for at most 16 workers: a thread takes the whole column of workers of a coordinate.
+// DeTAG step for at most 16 workers, held in registers from the loads to the stores.
 //
-// AG_K(z) = P z with P = P_K(M) from the host.  A column of n <= 16 workers is 2 n^2 float64 multiply-adds for the two
-// contractions, at most 32 per worker-coordinate: half a clock per worker-coordinate and SM on the scalar float64 pipe
-// against 1.3 clocks of HBM traffic, so the tensor path has nothing to win here - it works on 32 padded rows, which for
-// eight workers is three quarters of its noise, gradient and shared-memory work for nothing.  P sits in shared memory, four
-// output workers of one input worker side by side (two 16-byte broadcasts for eight multiply-adds).  Rows are read and written as neighbouring
-// lanes' neighbouring words; nothing is staged, no thread waits for another, and the remainder of d needs no path of its
-// own.  Several steps per launch keep the column in registers from one to the next.
+// AG_K(z) = P z with P = P_K(M) from the host, on the float64 tensor path (mma m8n8k4) with the operands' roles chosen so that
+// nothing has to move between lanes: eight coordinates are the M index, the input workers the contraction index and the
+// output workers the N index, permuted so that column 2 q + e of the output block b stands for worker q + 4 (2 b + e).  A
+// lane (c = lane / 4, q = lane % 4) then supplies workers q, q + 4, ... of coordinate c and receives the same workers of the
+// same coordinate: it loads its elements from global memory, takes them through all of the step and writes them back.  No
+// shared memory, no barriers; the next step of several in one launch finds its operands in place.
 //
-// Bound: HBM up to 12 workers (8 workers, d = 8 M: 362 us, 0.86 of the copy rate; the tensor-path kernel took 1005 us), at
-// 16 the issue slots, 133 instructions per worker-coordinate (d = 4 M: 474 us, before 568; address arithmetic with one
-// byte offset per row for all arrays instead of one per access took it from 178 instructions and 537 us; two coordinates
-// per thread cost 962 us for want of warps).  Twenty steps in one launch, 8 workers, d = 62 k: 45 us, before 127.
+// A warp takes 8 V coordinates; lane c owns the V neighbouring ones from V c on, so that a row is read as V-word vectors, and
+// its tile t consists of the t-th of every lane.  The four workers of a Philox call are the four lanes of a coordinate at the
+// same place: each lane draws whole calls, as many as there are for four lanes, and a 4 x 4 transpose hands them out.
+//
+// Bound: HBM for single steps (n = 8, d = 8 M 327 us, 0.96 of the copy rate; n = 16, d = 4 M 378 us, 0.83), at d = 270 k the launch
+// and the loads' latency (n = 16 29 us for 21 of HBM time); for many steps the special-function pipe, five conversions per
+// worker-coordinate and step beside the normals (n = 8, d = 62 k, twenty steps: 28 us).  One thread per coordinate, its column in
+// shared memory and the sums on the scalar float64 pipe, took 133 instructions per worker-coordinate at n = 16 and 399, 499, 41
+// and 45 us; caller-written gradients of 16 workers, d = 270 k, went from 35 us on the staged kernel to 25.
+//
+// Measured on the way: loads behind a branch (rows beyond n) 599 us at n = 13, d = 4 M, clamped and selected 350; V = 2 for
+// single steps 514 us at n = 8, d = 8 M (64-byte row pieces), within 2 % at n = 16, d = 270 k; 128 registers instead of 168 at
+// n = 16 421 us for d = 4 M; blocks of 64 threads the same.
 #include <cuda_runtime.h>
 
 #include "detag_internal.h"
 #include "noise.cuh"
+#include "pipeline.cuh"
 
 namespace detag {
 
@@ -23,225 +32,196 @@ namespace {
 
 constexpr int kSmallThreads = 128;
 
-// Blocks per SM the registers are planned for.
-constexpr int small_blocks(int N, bool many) { return many ? (N <= 8 ? 3 : 2) : 6; }
+template <int V>
+struct Vec;
+template <>
+struct Vec<2> {
+  typedef float2 Type;
+};
+template <>
+struct Vec<4> {
+  typedef float4 Type;
+};
 
-// N: n rounded up to a multiple of four, kFull: n == N.  kMany: p.steps iterations (DeTAG with the synthetic gradient only).
-template <int N, bool kFull, int kMode, bool kAtStart, bool kMany>
-__global__ void __launch_bounds__(kSmallThreads, small_blocks(N, kMany)) step_small_kernel(const StepParams p) {
-  __shared__ __align__(16) double poly[N / 4][N][4];  // [output quad][input worker][output], zero beyond n
-  // The column's operands of the contractions, u = x - alpha y (D-PSGD: x) and the tracker, widened once; every thread its
-  // own entries.  In registers they would leave room for half the warps.
-  __shared__ double operands[(kMode == kModeDpsgd ? 1 : 2) * N * kSmallThreads];
-  double* const op_u = operands + threadIdx.x;
-  double* const op_y = op_u + N * kSmallThreads;
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int i = e / N, k = e % N;
-    poly[i >> 2][k][i & 3] = i < p.n && k < p.n ? p.poly[i * p.n + k] : 0.0;
-  }
-  __syncthreads();
-  const long long j = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  if (j >= p.d) return;
-  const int n = kFull ? N : p.n;
+// Blocks per SM the registers are planned for: what the five arrays' vectors and the sums need without spills.  More blocks
+// at fewer registers lose (n = 16: above), fewer do not gain; many steps at n = 16 in 6 blocks 76 us for 68.
+constexpr int small_blocks(int R, int V, bool many) { return many ? 4 : R * V <= 8 ? 5 : R * V <= 12 ? 4 : 3; }
+
+// R: workers per lane, n rounded up to 4 R; kFull: n == 4 R.  V: coordinates per lane.  kMany: p.steps iterations (DeTAG with
+// the synthetic gradient only).
+template <int R, bool kFull, int V, int kMode, bool kAtStart, bool kMany>
+__global__ void __launch_bounds__(kSmallThreads, small_blocks(R, V, kMany)) step_small_kernel(const StepParams p) {
+  typedef typename Vec<V>::Type VecT;
+  constexpr int kBlocks = (R + 1) / 2;        // output blocks of eight workers
+  constexpr int kDraws = (R * V + 3) / 4;     // Philox calls of a lane
+  const int lane = threadIdx.x & 31, q = lane & 3, c = lane >> 2;
+  const long long warp = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) >> 5;
+  const long long first = warp * (8 * V);     // the warp's first coordinate
+  if (first >= p.d) return;                   // whole warps
+  const long long j = first + V * c;          // this lane's first coordinate; rows are padded to a multiple of four
+  const bool inside = j < p.d;
+  const int n = kFull ? 4 * R : p.n;
   const double alpha = p.alpha;
   const float sigma = static_cast<float>(p.sigma);
-  const bool noisy = p.sigma != 0.0;
-  const unsigned long long jn = static_cast<unsigned long long>(p.coord_offset + j);
-  // One byte offset per row serves all arrays.
-  const long long pitch = p.ld * 4, start = j * 4;
-  auto at = [](const float* base, long long off) { return reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + off); };
-  // Rows beyond n read row n - 1 and count as zero: no branch around a read.
-  auto rows4 = [&](const float* base, int q, const long long (&off)[4], float (&v)[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float t = *at(base, off[i]);
-      v[i] = kFull || q + i < n ? t : 0.f;
-    }
-  };
-  auto offsets = [&](int q, long long (&off)[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) off[i] = start + (kFull || q + i < n ? q + i : n - 1) * pitch;
-  };
+  const bool noisy = kMode != kModeExternal && p.sigma != 0.0;
   const float* const pa = kMode == kModeExternal ? p.g_ext : p.a;
 
-  float xs[kMany ? N / 4 : 1][4], ys[kMany ? N / 4 : 1][4], gs[kMany ? N / 4 : 1][4], as[kMany ? N / 4 : 1][4],
-      cs[kMany ? N / 4 : 1][4];
-  // all rows are asked for before the first is used
-  constexpr int kQuads = N / 4;
+  // ---- everything is asked for before anything is used.  Workers beyond n and coordinates beyond d count as zero; they read
+  // a row and a column that are there, so that no branch keeps the loads apart.
+  const long long at = inside ? j : first;
+  auto load = [&](const float* base, float (&v)[R][V]) {
 #pragma unroll
-  for (int f = 0; f < N / 4; f += kQuads) {
-    float xv[kQuads][4], yv[kQuads][4], gv[kQuads][4], gn[kQuads][4];
+    for (int i = 0; i < R; ++i) {
+      const int row = q + 4 * i;
+      const VecT w = *reinterpret_cast<const VecT*>(base + (kFull || row < n ? row : n - 1) * p.ld + at);
+      const float* const e = reinterpret_cast<const float*>(&w);
 #pragma unroll
-    for (int q = 0; q < kQuads; ++q) {
-      long long off[4];
-      offsets(4 * (f + q), off);
-      rows4(p.x, 4 * (f + q), off, xv[q]);
-      if (kMode != kModeDpsgd) rows4(p.y, 4 * (f + q), off, yv[q]);
-      if (kMode == kModeExternal) {
-        rows4(pa, 4 * (f + q), off, gn[q]);
-        rows4(p.g, 4 * (f + q), off, gv[q]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < kQuads; ++q)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = 4 * (f + q) + i;
-        double y = kMode == kModeDpsgd ? 0.0 : static_cast<double>(yv[q][i]);
-        // Algorithm 2's tracker update with the caller's newest gradient
-        if (kMode == kModeExternal) y += static_cast<double>(gn[q][i]) - static_cast<double>(gv[q][i]);
-        op_u[k * kSmallThreads] = kMode == kModeDpsgd ? static_cast<double>(xv[q][i]) : fma(-alpha, y, static_cast<double>(xv[q][i]));
-        if (kMode != kModeDpsgd) op_y[k * kSmallThreads] = y;
-        if (kMany) xs[f + q][i] = xv[q][i];
-      }
-  }
-
-  // Four output workers: contractions, noise, gradient, fold.  x_at: the model the step started from (kAtStart).
-  auto quad = [&](int q, uint32_t t, const float (&gv)[4], const float (&av)[4], const float (&cv)[4], const float (&x_at)[4],
-                  float (&xo)[4], float (&yo)[4], float (&go)[4], double (&cy)[4]) {
-    double cx[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      cx[i] = kMode == kModeDpsgd ? -alpha * static_cast<double>(gv[i]) : 0.0;
-      cy[i] = kMode == kModeDetag ? static_cast<double>(-gv[i]) : 0.0;  // ends as y~ - g
-    }
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      // a few shared-memory reads in flight at a time: all of a quad's, moved to its front, would not fit in registers
-      if (k % 4 == 0) asm volatile("" ::: "memory");
-      const double2 p01 = *reinterpret_cast<const double2*>(&poly[q >> 2][k][0]);
-      const double2 p23 = *reinterpret_cast<const double2*>(&poly[q >> 2][k][2]);
-      const double pk[4] = {p01.x, p01.y, p23.x, p23.y};
-      const double u = op_u[k * kSmallThreads], y = kMode == kModeDpsgd ? 0.0 : op_y[k * kSmallThreads];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        cx[i] = fma(pk[i], u, cx[i]);
-        if (kMode != kModeDpsgd) cy[i] = fma(pk[i], y, cy[i]);
-      }
-    }
-    float xi[4] = {0.f, 0.f, 0.f, 0.f};
-    if (kMode != kModeExternal && noisy) normal_quad(p.round_key, jn, static_cast<uint32_t>(q >> 2), t, xi);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      xo[i] = static_cast<float>(cx[i]);  // x' (float64 sum, rounded once)
-      if (kMode == kModeExternal) {
-        go[i] = av[i];                      // the gradient just folded becomes g_old
-        yo[i] = static_cast<float>(cy[i]);  // the gossiped tracker
-      } else {
-        go[i] = fmaf(av[i], (kAtStart ? x_at[i] : xo[i]) - cv[i], sigma * xi[i]);  // stochastic gradient
-        yo[i] = static_cast<float>(cy[i] + static_cast<double>(go[i]));            // fold: (y~ - g) + g', g' as stored
-      }
+      for (int t = 0; t < V; ++t) v[i][t] = kFull || row < n ? e[t] : 0.f;
     }
   };
-  auto store4 = [&](float* base, int q, const long long (&off)[4], const float (&v)[4]) {
+  float x[R][V], y[R][V], g[R][V], a[R][V], cc[R][V];
+  load(p.x, x);
+  if (kMode != kModeDpsgd) load(p.y, y);
+  load(p.g, g);
+  load(pa, a);
+  if (kMode != kModeExternal) load(p.c, cc);
+  double frag[R][kBlocks];  // [input step][output block]: P[worker of column c][worker q of the step]
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (kFull || q + i < n) *const_cast<float*>(at(base, off[i])) = v[i];
-  };
-
-  if (kMany) {
+  for (int k = 0; k < R; ++k)
 #pragma unroll
-    for (int q = 0; q < N / 4; ++q) {
-      long long off[4];
-      offsets(4 * q, off);
-      rows4(p.g, 4 * q, off, gs[q]);
-      rows4(pa, 4 * q, off, as[q]);
-      rows4(p.c, 4 * q, off, cs[q]);
+    for (int b = 0; b < kBlocks; ++b) {
+      const int out = (c >> 1) + 4 * (2 * b + (c & 1)), in = 4 * k + q;
+      frag[k][b] = out < n && in < n ? p.poly[out * n + in] : 0.0;
     }
-#pragma unroll 1
-    for (int step = 0; step < p.steps; ++step) {
+
+  double gd[R][V];  // the old gradient widened; the next of several steps starts from what this one folded
 #pragma unroll
-      for (int q = 0; q < N / 4; ++q) {
-        double cy[4];
-        float g4[4], x4[4];
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          g4[i] = gs[q][i];
-          x4[i] = xs[q][i];
+    for (int t = 0; t < V; ++t) gd[i][t] = static_cast<double>(g[i][t]);
+
+  auto step = [&](uint32_t t_noise) {
+    float xi[R][V];
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int t = 0; t < V; ++t) xi[i][t] = 0.f;
+    if (noisy) {
+#pragma unroll
+      for (int h = 0; h < kDraws; ++h) {
+        // call 4 h + lane's place: coordinate (its number) % V, quad (its number) / V
+        const int mine_t = V == 4 ? q : q % V, mine_i = V == 4 ? h : (4 / V) * h + q / V;
+        float v[4];
+        normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + mine_t), static_cast<uint32_t>(mine_i), t_noise, v);
+        transpose_quad(v, q);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const int number = 4 * h + s;
+          if (number / V < R) xi[number / V][number % V] = v[s];
         }
-        quad(4 * q, p.t_noise + static_cast<uint32_t>(step), g4, as[q], cs[q], x4, xs[q], ys[q], gs[q], cy);
-      }
-      if (step + 1 < p.steps) {
-#pragma unroll
-        for (int q = 0; q < N / 4; ++q)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const double y = static_cast<double>(ys[q][i]);
-            op_u[(4 * q + i) * kSmallThreads] = fma(-alpha, y, static_cast<double>(xs[q][i]));
-            op_y[(4 * q + i) * kSmallThreads] = y;
-          }
       }
     }
 #pragma unroll
-    for (int q = 0; q < N / 4; ++q) {
-      long long off[4];
-      offsets(4 * q, off);
-      store4(p.x, 4 * q, off, xs[q]);
-      store4(p.y, 4 * q, off, ys[q]);
-      store4(p.g, 4 * q, off, gs[q]);
+    for (int t = 0; t < V; ++t) {
+      // cx ends as x' = P (x - alpha y), by linearity; cy starts at -g and ends as y~ - g, so that the fold is cy + g'.
+      // Caller-written gradients: the operand is the tracker folded with them, cy starts at zero.  D-PSGD: cx starts at
+      // -alpha g and sums P x.
+      double cx[kBlocks][2], cy[kBlocks][2];
+#pragma unroll
+      for (int i = 0; i < 2 * kBlocks; ++i) {
+        const double old = i < R && kMode != kModeExternal ? -gd[i < R ? i : 0][t] : 0.0;
+        cx[i >> 1][i & 1] = kMode == kModeDpsgd ? alpha * old : 0.0;
+        cy[i >> 1][i & 1] = kMode == kModeDetag ? old : 0.0;
+      }
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        double u = static_cast<double>(x[k][t]), yd = 0.0;
+        if (kMode != kModeDpsgd) {
+          yd = static_cast<double>(y[k][t]);
+          if (kMode == kModeExternal) yd += static_cast<double>(a[k][t]) - gd[k][t];  // Algorithm 2's tracker update
+          u = fma(-alpha, yd, u);
+        }
+#pragma unroll
+        for (int b = 0; b < kBlocks; ++b) {
+          if (kMode != kModeDpsgd) dmma(cy[b], yd, frag[k][b]);
+          dmma(cx[b], u, frag[k][b]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const double sy = cy[i >> 1][i & 1];
+        const float xn = static_cast<float>(cx[i >> 1][i & 1]);  // x' (float64 sum, rounded once)
+        if (!kMany && kMode != kModeDpsgd && p.y_obs != nullptr && (kFull || q + 4 * i < n) && j + t < p.d)  // optional observer: the gossiped tracker
+          p.y_obs[(q + 4 * i) * p.ld + j + t] = static_cast<float>(kMode == kModeDetag ? sy + gd[i][t] : sy);
+        if (kMode == kModeExternal) {
+          g[i][t] = a[i][t];                    // the gradient just folded becomes g_old
+          y[i][t] = static_cast<float>(sy);     // the gossiped tracker
+        } else {
+          const float gn = fmaf(a[i][t], (kAtStart ? x[i][t] : xn) - cc[i][t], sigma * xi[i][t]);  // stochastic gradient
+          gd[i][t] = static_cast<double>(gn);
+          if (kMode == kModeDetag) y[i][t] = static_cast<float>(sy + gd[i][t]);  // fold: (y~ - g) + g', g' as stored
+          g[i][t] = gn;
+        }
+        x[i][t] = xn;
+      }
     }
-    return;
-  }
-  float gn[4], an[4], cn[4], xn[4];  // the next quad's rows are on their way while one is worked on
-  long long next[4];
-  auto fetch = [&](int q) {
-    if (kMode != kModeExternal) {
-      rows4(p.g, q, next, gn);
-      rows4(p.c, q, next, cn);
-    }
-    rows4(pa, q, next, an);
-    if (kAtStart) rows4(p.x, q, next, xn);  // still the old model: this thread overwrites it below
   };
-  offsets(0, next);
-  fetch(0);
+  if (kMany) {
 #pragma unroll 1
-  for (int q = 0; q < N; q += 4) {
-    float gv[4], av[4], cv[4], xv[4], xo[4], yo[4], go[4];
-    double cy[4];
-    long long off[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      gv[i] = gn[i];
-      av[i] = an[i];
-      cv[i] = cn[i];
-      xv[i] = xn[i];
-      off[i] = next[i];
-      if (kFull) next[i] += 4 * pitch;
-    }
-    if (!kFull) offsets(q + 4, next);
-    if (q + 4 < N) fetch(q + 4);
-    quad(q, p.t_noise, gv, av, cv, xv, xo, yo, go, cy);
-    store4(p.x, q, off, xo);
-    if (kMode != kModeDpsgd) store4(p.y, q, off, yo);
-    store4(p.g, q, off, go);
-    if (kMode != kModeDpsgd && p.y_obs != nullptr) {  // optional observer: the gossiped tracker
-      float yg[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        yg[i] = kMode == kModeDetag ? static_cast<float>(cy[i] + static_cast<double>(gv[i])) : yo[i];
-      store4(p.y_obs, q, off, yg);
-    }
+    for (int s = 0; s < p.steps; ++s) step(p.t_noise + static_cast<uint32_t>(s));
+  } else {
+    step(p.t_noise);
   }
+
+  if (!inside) return;
+  auto store = [&](float* base, const float (&v)[R][V]) {
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      if (!kFull && q + 4 * i >= n) continue;
+      float* const to = base + (q + 4 * i) * p.ld + j;
+      if (j + V <= p.d) {
+        VecT w;
+        float* const e = reinterpret_cast<float*>(&w);
+#pragma unroll
+        for (int t = 0; t < V; ++t) e[t] = v[i][t];
+        *reinterpret_cast<VecT*>(to) = w;
+      } else {  // nothing beyond column d is written
+#pragma unroll
+        for (int t = 0; t < V; ++t)
+          if (j + t < p.d) to[t] = v[i][t];
+      }
+    }
+  };
+  store(p.x, x);
+  if (kMode != kModeDpsgd) store(p.y, y);
+  store(p.g, g);
 }
 
 typedef void (*SmallKernel)(const StepParams);
 
-template <int N, bool kFull>
+template <int R, bool kFull>
 SmallKernel pick_small(const StepParams& p) {
-  if (p.steps > 1)
-    return p.grad_at_start ? step_small_kernel<N, kFull, kModeDetag, true, true> : step_small_kernel<N, kFull, kModeDetag, false, true>;
-  if (p.mode == kModeExternal) return step_small_kernel<(N <= 8 ? N : 8), kFull, kModeExternal, false, false>;  // n <= 8
-  if (p.mode == kModeDpsgd) return step_small_kernel<N, kFull, kModeDpsgd, false, false>;
-  return p.grad_at_start ? step_small_kernel<N, kFull, kModeDetag, true, false> : step_small_kernel<N, kFull, kModeDetag, false, false>;
+  if (p.mode == kModeExternal) return step_small_kernel<R, kFull, 4, kModeExternal, false, false>;
+  if (p.mode == kModeDpsgd) return step_small_kernel<R, kFull, 4, kModeDpsgd, false, false>;
+  return p.grad_at_start ? step_small_kernel<R, kFull, 4, kModeDetag, true, false> : step_small_kernel<R, kFull, 4, kModeDetag, false, false>;
 }
 
-template <int N>
+template <int R, bool kFull>
+SmallKernel pick_many(const StepParams& p) {
+  return p.grad_at_start ? step_small_kernel<R, kFull, 2, kModeDetag, true, true> : step_small_kernel<R, kFull, 2, kModeDetag, false, true>;
+}
+
+template <int R>
 int launch_small(const StepParams& p, int sm_count, cudaStream_t stream) {
-  const SmallKernel kernel = p.n == N ? pick_small<N, true>(p) : pick_small<N, false>(p);
-  // short vectors: smaller blocks, so that every SM gets a share
-  const int threads = p.d >= kSmallThreads * static_cast<long long>(sm_count) ? kSmallThreads : p.d >= 64LL * sm_count ? 64 : 32;
-  const long long grid = (p.d + threads - 1) / threads;
-  kernel<<<static_cast<unsigned>(grid), threads, 0, stream>>>(p);
+  const bool many = p.steps > 1, full = p.n == 4 * R;
+  const SmallKernel kernel = many ? (full ? pick_many<R, true>(p) : pick_many<R, false>(p))
+                                  : (full ? pick_small<R, true>(p) : pick_small<R, false>(p));
+  // Many steps: half as many coordinates to a warp, twice the warps to hide the chain of a step behind.  Short vectors: smaller
+  // blocks, so that every SM gets a share.
+  const int width = 8 * (many ? 2 : 4);
+  const long long warps = (p.d + width - 1) / width;
+  const int per_block = warps >= 4LL * sm_count ? 4 : warps >= 2LL * sm_count ? 2 : 1;
+  kernel<<<static_cast<unsigned>((warps + per_block - 1) / per_block), 32 * per_block, 0, stream>>>(p);
   return static_cast<int>(cudaGetLastError());
 }
 
@@ -249,11 +229,11 @@ int launch_small(const StepParams& p, int sm_count, cudaStream_t stream) {
 
 // p.steps > 1: that many iterations.
 int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream) {
-  if (p.n > kMaxSmallWorkers || p.d <= 0 || (p.mode == kModeExternal && p.n > 8) || (p.steps > 1 && p.mode != kModeDetag)) return static_cast<int>(cudaErrorInvalidValue);
-  if (p.n <= 4) return launch_small<4>(p, sm_count, stream);
-  if (p.n <= 8) return launch_small<8>(p, sm_count, stream);
-  if (p.n <= 12) return launch_small<12>(p, sm_count, stream);
-  return launch_small<16>(p, sm_count, stream);
+  if (p.n > kMaxSmallWorkers || p.d <= 0 || (p.steps > 1 && p.mode != kModeDetag)) return static_cast<int>(cudaErrorInvalidValue);
+  if (p.n <= 4) return launch_small<1>(p, sm_count, stream);
+  if (p.n <= 8) return launch_small<2>(p, sm_count, stream);
+  if (p.n <= 12) return launch_small<3>(p, sm_count, stream);
+  return launch_small<4>(p, sm_count, stream);
 }
 
 }  // namespace detag

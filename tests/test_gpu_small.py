@@ -1,4 +1,4 @@
-"""At most 16 workers, a thread per coordinate: worker counts on and off the quads, vectors below, at and beyond a block of
+"""At most 16 workers, the step in registers: worker counts on and off the quads, vectors below, at and beyond a block of
 every size the launch picks (32, 64, 128 threads), all modes, one step against the oracle per element."""
 import numpy as np
 import pytest
@@ -54,3 +54,32 @@ def test_one_step_against_the_oracle(n, d, mode):
     g_ref = orc.stochastic_gradient(p, x if mode == "start" else x_new, 1)
     assert worst_ratio(got["g"], g_ref) <= 1.0
     assert worst_ratio(got["y"], y_gossip + g_ref - g, extra=HALF_ULP32 * np.abs(g_ref)) <= 1.0
+
+
+@pytest.mark.parametrize("n", [2, 6, 16])
+@pytest.mark.parametrize("d", [2, 31, 32, 2 * 32 * 148 + 1, 4 * 32 * 148 + 3])
+@pytest.mark.parametrize("steps", [1, 3])
+def test_columns_keep_to_themselves(n, d, steps):
+    """A warp's 16 or 32 coordinates, the vectors of a row and the blocks of the launch end anywhere: nothing beyond column d
+    changes, and an infinity stays in its coordinate."""
+    m = inputs.csr_from_dense(np.full((2, 2), 0.5)) if n == 2 else inputs.metropolis_weights(inputs.ring_graph(n))
+    rng = np.random.default_rng(n * 17 + d)
+    arrays = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c")}
+    hit = d // 2
+    got = []
+    for bad in (False, True):
+        with Session(m, d, 2, 0.2, 0.05, sigma=0.1, seed=3, ld=(d + 3) // 4 * 4 + 4) as s:
+            for k, v in arrays.items():
+                s.upload(k, v)
+                getattr(s, k)[:, d:] = 7.0
+            if bad:
+                s.x[0, hit] = float("inf")
+            B.detag_set_step(s.state, 0)
+            s.step_many(steps)
+            s.status()
+            got.append({k: getattr(s, k).cpu().numpy() for k in ("x", "y", "g")})
+    keep = np.arange(d) != hit
+    for k in ("x", "y", "g"):
+        assert np.all(got[0][k][:, d:] == 7.0) and np.all(got[1][k][:, d:] == 7.0)
+        assert np.all(np.isfinite(got[0][k])) and np.array_equal(got[0][k][:, :d][:, keep], got[1][k][:, :d][:, keep])
+    assert not np.isfinite(got[1]["x"][0, hit])
