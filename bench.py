@@ -38,12 +38,12 @@ BYTES_PER_WC = 32  # read x, y, g, a, c + write x, y, g, float32 each: the fused
 # small case of the same kernel; traffic grows in proportion to n*d).  Keyed by the sha256 prefix of the kernel
 # sources the capture was taken on: a changed kernel reports null until it is captured again.
 KERNEL_SOURCES = {
-    "small": ("step_small.cu", "noise.cuh", "pipeline.cuh"),
-    "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh"),
-    "mma": ("step_mma.cu", "mma_common.cuh", "pipeline.cuh", "noise.cuh"),
-    "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh"),
-    "csr": ("step_csr.cu", "noise.cuh"),
-    "torus": ("step_torus.cu", "torus_basis.h", "pipeline.cuh", "noise.cuh"),
+    "small": ("step_small.cu", "noise.cuh", "packed.cuh", "pipeline.cuh"),
+    "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh"),
+    "mma": ("step_mma.cu", "mma_common.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh"),
+    "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh", "packed.cuh"),
+    "csr": ("step_csr.cu", "noise.cuh", "packed.cuh"),
+    "torus": ("step_torus.cu", "torus_basis.h", "pipeline.cuh", "noise.cuh", "packed.cuh"),
 }
 MEASURED_TRAFFIC = {
     # (kernel, mode): (source digest, bytes per wc)

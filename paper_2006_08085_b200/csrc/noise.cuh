@@ -16,6 +16,8 @@
 
 #include <cstdint>
 
+#include "packed.cuh"
+
 namespace detag {
 
 struct Philox4 {
@@ -59,27 +61,27 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
 // 1 + (r >> 9) 2^-23: the exponent bits of 1.0 come in from above as the word is shifted, one instruction for both.
 __device__ __forceinline__ float one_to_two(uint32_t r) { return __uint_as_float(__funnelshift_r(r, 0x7fu, 9)); }
 
-// -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9.  The factor -2 is in the argument F = -2 f and in the coefficients, scaled by
-// powers of two: the bits are those of -2 times the logarithm.
-__device__ __forceinline__ float neg2_ln_unit(uint32_t r) {
-  const float u = one_to_two(r) - 0x1.fffffep-1f;            // (2k+1) 2^-24, exact
-  const int bits = __float_as_int(u);
-  const int eb = (bits - 0x3f2aaaab) & 0xff800000;           // u = m 2^e with m in [2/3, 4/3); eb = e 2^23
-  const float m = __int_as_float(bits - eb);
-  const float F = fmaf(m, -2.0f, 2.0f);                      // -2 f, f = m - 1, exact
+// -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9, of two words.  The factor -2 is in the argument F = -2 f and in the coefficients,
+// scaled by powers of two: the bits are those of -2 times the logarithm.
+__device__ __forceinline__ F2 neg2_ln_unit(uint32_t r0, uint32_t r1) {
+  float u0, u1;
+  unpack2(add2(pack2(one_to_two(r0), one_to_two(r1)), both(-0x1.fffffep-1f)), u0, u1);  // (2k+1) 2^-24, exact
+  const int b0 = __float_as_int(u0), b1 = __float_as_int(u1);
+  const int e0 = (b0 - 0x3f2aaaab) & 0xff800000, e1 = (b1 - 0x3f2aaaab) & 0xff800000;   // u = m 2^e with m in [2/3, 4/3); here e 2^23
+  const F2 F = fma2(pack2(__int_as_float(b0 - e0), __int_as_float(b1 - e1)), both(-2.0f), both(2.0f));  // -2 f, f = m - 1, exact
   // ln(1+f) = f + f^2 r(f) on |f| <= 1/3 (Chebyshev fit of (ln(1+f) - f)/f^2, degree 7); here -r(-F/2) / 2
-  float r7 = 0.13756538927555084f * 0x1p-8f;
-  r7 = fmaf(r7, F, 0.1504942923784256f * 0x1p-7f);
-  r7 = fmaf(r7, F, 0.1405421793460846f * 0x1p-6f);
-  r7 = fmaf(r7, F, 0.16481579840183258f * 0x1p-5f);
-  r7 = fmaf(r7, F, 0.2000732272863388f * 0x1p-4f);
-  r7 = fmaf(r7, F, 0.25004205107688904f * 0x1p-3f);
-  r7 = fmaf(r7, F, 0.33333271741867065f * 0x1p-2f);
-  r7 = fmaf(r7, F, 0.49999985098838806f * 0x1p-1f);
-  float ln = fmaf(F * F, r7, F);
-  const float ef = __int2float_rn(eb);                       // e 2^23, exact
-  ln = fmaf(ef, -1.42860677e-06f * 0x1p-22f, ln);
-  return fmaf(ef, -0.693145751953125f * 0x1p-22f, ln);
+  F2 r7 = both(0.13756538927555084f * 0x1p-8f);
+  r7 = fma2(r7, F, both(0.1504942923784256f * 0x1p-7f));
+  r7 = fma2(r7, F, both(0.1405421793460846f * 0x1p-6f));
+  r7 = fma2(r7, F, both(0.16481579840183258f * 0x1p-5f));
+  r7 = fma2(r7, F, both(0.2000732272863388f * 0x1p-4f));
+  r7 = fma2(r7, F, both(0.25004205107688904f * 0x1p-3f));
+  r7 = fma2(r7, F, both(0.33333271741867065f * 0x1p-2f));
+  r7 = fma2(r7, F, both(0.49999985098838806f * 0x1p-1f));
+  F2 ln = fma2(mul2(F, F), r7, F);
+  const F2 ef = pack2(__int2float_rn(e0), __int2float_rn(e1));                          // exact
+  ln = fma2(ef, both(-1.42860677e-06f * 0x1p-22f), ln);
+  return fma2(ef, both(-0.693145751953125f * 0x1p-22f), ln);
 }
 
 // Approximate reciprocal square root of a normal number (rsqrtf() tests for subnormal arguments first).
@@ -89,21 +91,33 @@ __device__ __forceinline__ float rsqrt_normal(float v) {
   return r;
 }
 
-__device__ __forceinline__ void box_muller(uint32_t r_even, uint32_t r_odd, float& first, float& second) {
-  const float t = neg2_ln_unit(r_even);                                   // 1.2e-7 .. 33.3
-  const float rad = t * rsqrt_normal(t);
-  const float w = one_to_two(r_odd) - 1.5f;                               // u_ang - 1/2 in [-1/2, 1/2), exact
-  const float theta = w * 6.283185307179586f;                             // 2 pi u_ang - pi
-  first = -rad * __cosf(theta);                                           // cos(2 pi u) = -cos(2 pi u - pi)
-  second = -rad * __sinf(theta);
+// Both Box-Muller transforms of a Philox call: (first, third) and (second, fourth) normal.
+__device__ __forceinline__ void box_muller(const Philox4& r, F2& even, F2& odd) {
+  const F2 t = neg2_ln_unit(r.r0, r.r2);  // 1.2e-7 .. 33.3
+  float t0, t1, a0, a1;
+  unpack2(t, t0, t1);
+  const F2 rad = mul2(t, pack2(-rsqrt_normal(t0), -rsqrt_normal(t1)));                                              // negated
+  const F2 theta = mul2(add2(pack2(one_to_two(r.r1), one_to_two(r.r3)), both(-1.5f)), both(6.283185307179586f));    // 2 pi u_ang - pi
+  unpack2(theta, a0, a1);
+  even = mul2(rad, pack2(__cosf(a0), __cosf(a1)));  // cos(2 pi u) = -cos(2 pi u - pi)
+  odd = mul2(rad, pack2(__sinf(a0), __sinf(a1)));
 }
 
 // Standard normals of workers 4q..4q+3 at global coordinate j and noise step t.
-__device__ __forceinline__ void normal_quad(const uint32_t (&round_key)[20], unsigned long long j, uint32_t q, uint32_t t,
-                                            float xi[4]) {
-  const Philox4 r = philox4x32_10(static_cast<uint32_t>(j), static_cast<uint32_t>(j >> 32), q, t, round_key);
-  box_muller(r.r0, r.r1, xi[0], xi[1]);
-  box_muller(r.r2, r.r3, xi[2], xi[3]);
+__device__ __forceinline__ void normal_quad(const uint32_t (&round_key)[20], unsigned long long j, uint32_t q, uint32_t t, float (&xi)[4]) {
+  F2 even, odd;
+  box_muller(philox4x32_10(static_cast<uint32_t>(j), static_cast<uint32_t>(j >> 32), q, t, round_key), even, odd);
+  unpack2(even, xi[0], xi[2]);
+  unpack2(odd, xi[1], xi[3]);
+}
+
+// `scale` times those.
+__device__ __forceinline__ void normal_quad(const uint32_t (&round_key)[20], unsigned long long j, uint32_t q, uint32_t t, float scale,
+                                            float (&xi)[4]) {
+  F2 even, odd;
+  box_muller(philox4x32_10(static_cast<uint32_t>(j), static_cast<uint32_t>(j >> 32), q, t, round_key), even, odd);
+  unpack2(mul2(even, both(scale)), xi[0], xi[2]);
+  unpack2(mul2(odd, both(scale)), xi[1], xi[3]);
 }
 
 }  // namespace detag

@@ -165,7 +165,7 @@ step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
       for (int e = 0; e < 2; ++e) {
         if (kMode != kModeExternal && noisy) {
           normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + e),
-                      static_cast<uint32_t>(r), p.t_noise, xi[e]);
+                      static_cast<uint32_t>(r), p.t_noise, sigma, xi[e]);
         } else {
           xi[e][0] = xi[e][1] = xi[e][2] = xi[e][3] = 0.f;
         }
@@ -190,8 +190,8 @@ step_mma_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
             x_at.x = j < p.d ? p.x[off] : 0.f;
             x_at.y = j + 1 < p.d ? p.x[off + 1] : 0.f;
           }
-          go.x = fmaf(av.x, x_at.x - cv.x, sigma * xi[0][t]);            // stochastic gradient
-          go.y = fmaf(av.y, x_at.y - cv.y, sigma * xi[1][t]);
+          go.x = fmaf(av.x, x_at.x - cv.x, xi[0][t]);            // stochastic gradient
+          go.y = fmaf(av.y, x_at.y - cv.y, xi[1][t]);
           yo.x = static_cast<float>(cy[t][0] + static_cast<double>(go.x));  // fold: (y~ - g) + g', g' as stored
           yo.y = static_cast<float>(cy[t][1] + static_cast<double>(go.y));
         }

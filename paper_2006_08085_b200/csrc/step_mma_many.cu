@@ -110,7 +110,7 @@ step_mma_many_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
         for (int e = 0; e < 2; ++e) {
           if (noisy) {
             normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + e),
-                        static_cast<uint32_t>(r), p.t_noise + static_cast<uint32_t>(step), xi[e]);
+                        static_cast<uint32_t>(r), p.t_noise + static_cast<uint32_t>(step), sigma, xi[e]);
           } else {
             xi[e][0] = xi[e][1] = xi[e][2] = xi[e][3] = 0.f;
           }
@@ -128,8 +128,8 @@ step_mma_many_kernel(const StepParams p, const __grid_constant__ MmaMaps maps) {
           xo.y = static_cast<float>(cx[t][1]);
           // gradient point: the new model, or (Algorithm 2 as printed) the staged model this step started from
           const float2 x_at = kAtStart ? *reinterpret_cast<const float2*>(sx + xoff) : xo;
-          go.x = fmaf(av.x, x_at.x - cv.x, sigma * xi[0][t]);            // stochastic gradient
-          go.y = fmaf(av.y, x_at.y - cv.y, sigma * xi[1][t]);
+          go.x = fmaf(av.x, x_at.x - cv.x, xi[0][t]);            // stochastic gradient
+          go.y = fmaf(av.y, x_at.y - cv.y, xi[1][t]);
           yo.x = static_cast<float>(cy[t][0] + static_cast<double>(go.x));  // fold: (y~ - g) + g', g' as stored
           yo.y = static_cast<float>(cy[t][1] + static_cast<double>(go.y));
           if (!final_step) {

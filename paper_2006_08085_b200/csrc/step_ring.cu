@@ -303,7 +303,7 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
 #pragma unroll
       for (int hq = 0; hq < 2; ++hq) {
         float v[4];
-        normal_quad(p.round_key, jn, static_cast<uint32_t>(8 * b + 4 * hq + kq), p.t_noise, v);
+        normal_quad(p.round_key, jn, static_cast<uint32_t>(8 * b + 4 * hq + kq), p.t_noise, sigma, v);
         transpose_quad(v, kq);  // v[i]: position kq of quad 8 b + 4 hq + i
 #pragma unroll
         for (int i = 0; i < 4; ++i) xi[4 * hq + i] = v[i];
@@ -428,7 +428,7 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
       // model update: x' = x~ - alpha y~ (D-PSGD: x~ - alpha g)
       xo[m] = static_cast<float>(fma(-alpha, dpsgd ? static_cast<double>(gv[m]) : cy[t][e], cx[t][e]));
       const float x_at = p.grad_at_start ? x_old[m] : xo[m];  // gradient point: new model, or the one the step started from
-      go[m] = fmaf(av[m], x_at - cv[m], sigma * xi[m]);
+      go[m] = fmaf(av[m], x_at - cv[m], xi[m]);
       yo[m] = static_cast<float>((cy[t][e] - static_cast<double>(gv[m])) + static_cast<double>(go[m]));  // fold
     }
 #pragma unroll

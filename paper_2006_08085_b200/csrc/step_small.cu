@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kSmallThreads, small_blocks(R, V, kMany)) step
         // call 4 h + lane's place: coordinate (its number) % V, quad (its number) / V
         const int mine_t = V == 4 ? q : q % V, mine_i = V == 4 ? h : (4 / V) * h + q / V;
         float v[4];
-        normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + mine_t), static_cast<uint32_t>(mine_i), t_noise, v);
+        normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + mine_t), static_cast<uint32_t>(mine_i), t_noise, sigma, v);
         transpose_quad(v, q);
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kSmallThreads, small_blocks(R, V, kMany)) step
           g[i][t] = a[i][t];                    // the gradient just folded becomes g_old
           y[i][t] = static_cast<float>(sy);     // the gossiped tracker
         } else {
-          const float gn = fmaf(a[i][t], (kAtStart ? x[i][t] : xn) - cc[i][t], sigma * xi[i][t]);  // stochastic gradient
+          const float gn = fmaf(a[i][t], (kAtStart ? x[i][t] : xn) - cc[i][t], xi[i][t]);  // stochastic gradient
           gd[i][t] = static_cast<double>(gn);
           if (kMode == kModeDetag) y[i][t] = static_cast<float>(sy + gd[i][t]);  // fold: (y~ - g) + g', g' as stored
           g[i][t] = gn;

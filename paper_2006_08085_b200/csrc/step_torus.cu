@@ -179,13 +179,13 @@ __device__ __forceinline__ void torus_gradient(const StepParams& p, const float*
   for (int t = 0; t < R / 2; ++t) {  // quads 4 t .. 4 t + 3: blocks r = 2 t, 2 t + 1
     float xi[4] = {0.f, 0.f, 0.f, 0.f};
     if (noisy) {
-      normal_quad(p.round_key, jn, static_cast<uint32_t>(4 * t + kq), p.t_noise, xi);
+      normal_quad(p.round_key, jn, static_cast<uint32_t>(4 * t + kq), p.t_noise, sigma, xi);
       transpose_quad(xi, kq);  // xi[i]: this lane's position of quad 4 t + i, i.e. r = 2 t + (i >> 1), e = i & 1
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = 2 * t + (i >> 1), e = i & 1, o = off + r * 512 + e * 256;
-      sc[o] = fmaf(sa[o], x_at[e][r] - sc[o], sigma * xi[i]);
+      sc[o] = fmaf(sa[o], x_at[e][r] - sc[o], xi[i]);
     }
   }
 }
