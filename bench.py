@@ -40,7 +40,7 @@ BYTES_PER_WC = 32  # read x, y, g, a, c + write x, y, g, float32 each: the fused
 KERNEL_SOURCES = {
     "small": ("step_small.cu", "noise.cuh", "packed.cuh", "pipeline.cuh"),
     "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh"),
-    "mma": ("step_mma.cu", "mma_common.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh"),
+    "dense": ("step_dense.cu", "pipeline.cuh", "noise.cuh", "packed.cuh"),
     "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh", "packed.cuh"),
     "csr": ("step_csr.cu", "noise.cuh", "packed.cuh"),
     "torus": ("step_torus.cu", "torus_basis.h", "pipeline.cuh", "noise.cuh", "packed.cuh"),
@@ -48,7 +48,7 @@ KERNEL_SOURCES = {
 MEASURED_TRAFFIC = {
     # (kernel, mode): (source digest, bytes per wc)
     ("small", "column"): ("2d293cc7edde3135", 29.00),   # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1440 GB written / 16 M wc
-    ("mma", "dense"): ("98fc5c149709161c", 31.37),     # cfg5 shape at d = 2 M: 1.2899 + 0.7176 GB / 64 M wc
+    ("dense", "product"): ("98fc5c149709161c", 31.37),     # cfg5 shape at d = 2 M: 1.2899 + 0.7176 GB / 64 M wc
     ("torus", "torus8"): ("22f3bc13d621a2ed", 31.26),  # cfg3 shape at d = 1 M: 1.2801 + 0.7204 GB / 64 M wc
     ("ring", "band"): ("1a16972a0d29d375", 31.09),     # cfg4 shape at d = 200 k: 1.0279 + 0.5637 GB / 51.2 M wc
     ("split", "digits"): ("b1eb219985913d27", 30.81),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4321 GB / 40 M wc
@@ -57,7 +57,7 @@ MEASURED_TRAFFIC = {
 
 # Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes) and that
 # pipe's peak: 64 multiply-adds per clock and SM (measured: 61 with m8n8k4 MMAs from 16 warps) x 148 SMs x max clock.
-FP64_FMA_PER_WC = {("mma", "dense"): 64, ("ring", "band"): 80, ("torus", "torus8"): 26, ("torus", "torus4"): 28}
+FP64_FMA_PER_WC = {("dense", "product"): 64, ("ring", "band"): 80, ("torus", "torus8"): 26, ("torus", "torus4"): 28}
 VARIANT_NAMES = {1: "csr", 2: "dense", 3: "ring", 4: "torus"}
 FP64_FMA_PER_CLK_SM = 64
 SM_COUNT = 148
@@ -65,7 +65,7 @@ SM_COUNT = 148
 
 def kernel_key(variant: str, n: int):
     if variant == "dense":
-        return ("small", "column") if n <= 16 else ("mma", "dense") if n <= 32 else ("split", "digits")
+        return ("small", "column") if n <= 16 else ("dense", "product") if n <= 48 else ("split", "digits")
     if variant == "ring":
         return ("ring", "band")  # K times the bandwidth at most 16, as in the configurations
     if variant == "csr":

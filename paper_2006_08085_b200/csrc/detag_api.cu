@@ -360,7 +360,7 @@ int query_device(detag_state* s) {
 }
 
 // Kernel families that take tensor maps.
-enum { kFamilyMma = 1, kFamilyTorus = 2, kFamilyRing = 3, kFamilySplit = 4 };
+enum { kFamilyMma = 1, kFamilyTorus = 2, kFamilyRing = 3, kFamilySplit = 4, kFamilyDense = 5 };
 
 // Tensor maps for the buffers in `p`: built on first use, then found again by buffer addresses and sizes
 // (detag_step always hits; detag_step_host cycles through its two chunk slots and the ragged last chunk).
@@ -386,6 +386,7 @@ const detag::TensorMapSet* maps_for(detag_state* s, int family, const StepParams
   const bool ok = family == kFamilyMma    ? detag::build_maps_mma(p, &en.maps)
                   : family == kFamilyRing ? detag::build_maps_ring(p, &en.maps)
                   : family == kFamilySplit ? detag::build_maps_split(p, &en.maps)
+                  : family == kFamilyDense ? detag::build_maps_dense(p, &en.maps)
                                           : detag::build_maps_torus(p, &en.maps);
   if (!ok) return nullptr;
   en.family = family;
@@ -450,6 +451,20 @@ bool small_ok(const StepParams& p) {
   return p.n <= detag::kMaxSmallWorkers && p.stall_after < 0;
 }
 
+// Groups of warps with a slab each take the dense product of 17 to 48 workers, in all modes, and where the choice is the
+// library's what the rounds would run there (caller-written gradients and D-PSGD beyond 32).  us per step, the kernel with
+// padded tiles (up to 32) or the integer tensor path -> that one: 17 workers, d = 3 M 582 -> 340; 24 569 -> 414; 28 572 -> 531; 32
+// 600 -> 580, d = 25.6 M 5030 -> 4805, printed timing, d = 3 M 790 -> 578; 33, d = 1 M 411 -> 272; 40 427 -> 292; 48 430 -> 393; D-PSGD
+// of 32, d = 3 M 415 -> 405, of 48, d = 1 M 444 -> 265; caller-written gradients of 24, d = 3 M 448 -> 410, of 48, d = 1 M 664 (rounds)
+// -> 391.  But caller-written gradients of 28 470 -> 496, of 32 498 -> 535; and from 41 workers on a slab takes long enough that with
+// one per SM the integer path is ahead: 48, d = 9400 12.3 -> 13.9, d = 18000 16.4 -> 14.4 (40, d = 9400: 12.3 both).  The length is the
+// state's, not a staged chunk's: host-resident stepping gives the same bits.
+bool dense_step_ok(const detag_state* s, const StepParams& p, int variant) {
+  if (p.n <= detag::kMaxSmallWorkers || p.n > detag::kMaxDenseStepWorkers || p.stall_after >= 0 || p.poly == nullptr || p.d > 0x7fffffffLL) return false;
+  if (p.mode == detag::kModeExternal ? p.n > 24 && p.n <= 32 : p.n > 40 && s->d <= 64LL * s->sm_count) return false;
+  return variant == DETAG_VARIANT_DENSE || (variant == DETAG_VARIANT_CSR && s->variant_forced == DETAG_VARIANT_AUTO);
+}
+
 // Picks the kernel variant, plans it for the sizes in `p` and launches it.
 int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   int e = 0;
@@ -461,6 +476,12 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     return fail(s, DETAG_ERR_UNBOUND, "the synthetic gradient needs the objective arrays a and c");
   if (p.mode == detag::kModeExternal && !p.g_ext)
     return fail(s, DETAG_ERR_UNBOUND, "caller-written gradients selected but no gradient array given");
+  if (dense_step_ok(s, p, variant)) {
+    const detag::TensorMapSet* maps = maps_for(s, kFamilyDense, p);
+    if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+    e = detag::launch_step_dense(p, *maps, variant == DETAG_VARIANT_CSR && p.mode == detag::kModeDpsgd, s->sm_count, stream);
+    return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
+  }
   if (split_ok(s, p, variant)) return launch_split(s, p, variant == DETAG_VARIANT_CSR, stream);
   // what the integer tensor path does not take although its variant promises it (a polynomial whose entries cannot be
   // scaled, e.g. under an absurd momentum) runs as rounds
@@ -798,9 +819,10 @@ int detag_step_many(detag_state* s, int count, void* stream) {
   if (!s->bound) return fail(s, DETAG_ERR_UNBOUND, "detag_step_many before detag_bind");
   if (count >= 2 && step_mode(s) == detag::kModeExternal)
     return fail(s, DETAG_ERR_ARG, "detag_step_many: caller-written gradients need one call per step");
-  // the fused kernel exists for the dense polynomial with n <= 32; the observer wants every step's tracker
+  // the fused kernels exist for the dense polynomial with n <= 32; the observer wants every step's tracker, the
+  // failure-detection self test the kernel with a loading thread
   if (count >= 2 && resolve_variant(s) == DETAG_VARIANT_DENSE && s->n <= 32 && s->y_obs == nullptr &&
-      step_mode(s) == detag::kModeDetag) {
+      step_mode(s) == detag::kModeDetag && s->stall_after < 0) {
     // A launch is cut off at kMaxFusedSteps so that no thread of the kernel waits on a peer for longer than its
     // bounded waits allow (a tile of 1024 steps takes some tens of milliseconds; the waits give up after seconds).
     constexpr int kMaxFusedSteps = 1024;
@@ -814,9 +836,15 @@ int detag_step_many(detag_state* s, int count, void* stream) {
       if (small_ok(p)) {
         e = detag::launch_step_small(p, s->sm_count, static_cast<cudaStream_t>(stream));
       } else {
-        const detag::TensorMapSet* maps = maps_for(s, kFamilyMma, p);
+        // Groups of four warps take a slab's steps in turn; the kernel with padded tiles puts eight warps on one, which is ahead
+        // while there are at most two slabs per SM.  us for ten steps, padded -> groups: 17 workers, d = 9000 26.6 -> 22.5,
+        // d = 72 k 127 -> 71; 24, d = 9000 26.6 -> 23.9; 28, d = 18 k 39.0 -> 41.0, d = 36 k 68 -> 59; 32, d = 9000 26.6 -> 32.8, d = 18 k
+        // 39 -> 43, d = 36 k 70 -> 66, d = 72 k 130 -> 128.
+        const bool padded = p.n > 24 && p.d <= 128LL * s->sm_count;
+        const detag::TensorMapSet* maps = maps_for(s, padded ? kFamilyMma : kFamilyDense, p);
         if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-        e = detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream));
+        e = padded ? detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream))
+                   : detag::launch_step_dense_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream));
       }
       if (e != 0) return fail_cuda(s, e, "detag_step_many launch");
       s->t += now;
