@@ -246,7 +246,9 @@ def detag_init(state, stream=None) -> None:
 
 
 def detag_step(state, stream=None) -> None:
-    _check(lib().detag_step(state, _stream_handle(stream)), "detag_step", state)
+    code = (_lib or lib()).detag_step(state, _stream_handle(stream))
+    if code != DETAG_OK:
+        _check(code, "detag_step", state)
 
 
 def detag_step_many(state, count: int, stream=None) -> None:

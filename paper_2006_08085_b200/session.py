@@ -9,6 +9,9 @@ import numpy as np
 from . import binding as B
 
 
+_raw_current_stream = None  # torch's accessor for the current stream's handle, once a session exists
+
+
 def _round_up(v: int, m: int) -> int:
     return (v + m - 1) // m * m
 
@@ -31,6 +34,8 @@ class Session:
 
         if not torch.cuda.is_available():
             raise RuntimeError("the DeTAG step runs on a CUDA device only; none is available")
+        global _raw_current_stream
+        _raw_current_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
         self.torch = torch
         self.device = torch.device(device)
         torch.cuda.set_device(self.device)
@@ -79,16 +84,23 @@ class Session:
     def stream(self):
         return self.torch.cuda.current_stream(self.device)
 
+    def _raw_stream(self) -> int:
+        """Handle of ``stream()``.  On short vectors a step is its launch: the handle itself takes 0.1 us to get, the stream
+        object around it 2.2, and with it a call with 8 workers and d = 4096 took 11.2 us instead of 8.7."""
+        if _raw_current_stream is None or self.device.index is None:
+            return int(self.stream().cuda_stream)
+        return _raw_current_stream(self.device.index)
+
     def init(self) -> None:
         B.detag_init(self.state, self.stream())
 
     def step(self, count: int = 1) -> None:
-        st = self.stream()
+        st = self._raw_stream()
         for _ in range(count):
             B.detag_step(self.state, st)
 
     def step_many(self, count: int) -> None:
-        B.detag_step_many(self.state, count, self.stream())
+        B.detag_step_many(self.state, count, self._raw_stream())
 
     def consensus_error(self) -> float:
         return B.detag_consensus_error(self.state, self.stream())
