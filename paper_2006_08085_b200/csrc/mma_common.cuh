@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
 #include "pipeline.cuh"
@@ -91,6 +92,8 @@ __device__ __forceinline__ bool mma_setup(const StepParams& p, unsigned char* sm
   }
   fence_async_shared();
   __syncthreads();
+  chain_wait();
+  chain_next();
   return true;
 }
 

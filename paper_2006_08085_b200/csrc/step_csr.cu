@@ -28,6 +28,7 @@
 // mode only the model is gossiped and x' = x~ - alpha g.
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
 
@@ -105,6 +106,8 @@ __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepPara
     cols = s_col;
     __syncthreads();  // the tables are read right below
   }
+  chain_wait();
+  chain_next();
   // item = ((row quad * 4 + row within quad) * groups + coordinate group): a row's threads side by side, the four
   // rows of a Philox call `groups` lanes apart in one warp (groups is a power of two, at most 8)
   const int groups = W >> 2, half = W >> 1, quads = (n + 3) / 4;
@@ -313,8 +316,7 @@ int launch_step_csr(const StepParams& p, int sm_count, cudaStream_t stream) {
   const long long ctas = static_cast<long long>(sm_count) * (kCsrThreads / p.csr_threads);
   const long long grid = p.num_slabs < ctas ? p.num_slabs : ctas;
   if (grid <= 0) return 0;
-  kernel<<<static_cast<unsigned>(grid), p.csr_threads, smem, stream>>>(p);
-  return static_cast<int>(cudaGetLastError());
+  return launch_chained(kernel, static_cast<unsigned>(grid), p.csr_threads, smem, stream, p);
 }
 
 }  // namespace detag

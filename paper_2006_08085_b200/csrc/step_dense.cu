@@ -28,6 +28,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
 #include "packed.cuh"
@@ -124,6 +125,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
     *in_done = *tail_done = 0;
     fence_barrier_init();
     fence_async_shared();
+    chain_wait();
     if (slab < whole) {
       load_operands(slab);
       load_tail(slab);
@@ -136,6 +138,8 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
     frag[e] = out < n && in < n ? p.poly[out * n + in] : 0.0;
   }
   __syncthreads();
+  chain_wait();
+  chain_next();
   bool owes = false;  // this thread sent the last results out and has not yet asked for the next inputs
   bool ok = true;
   int use = 0;
@@ -378,8 +382,7 @@ int launch_kernel(DenseKernel kernel, const StepParams& p, const TensorMapSet& m
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), dense_smem_bytes(R));
   if (e != 0) return e;
   const long long slabs = (p.d + kDS - 1) / kDS, grid = slabs < sm_count ? slabs : sm_count;
-  kernel<<<static_cast<unsigned>(grid), dense_groups(R) * 128, dense_smem_bytes(R), stream>>>(p, *reinterpret_cast<const DenseMaps*>(maps.bytes));
-  return static_cast<int>(cudaGetLastError());
+  return launch_chained(kernel, static_cast<unsigned>(grid), dense_groups(R) * 128, dense_smem_bytes(R), stream, p, *reinterpret_cast<const DenseMaps*>(maps.bytes));
 }
 
 template <int R>

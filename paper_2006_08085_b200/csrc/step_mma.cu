@@ -281,8 +281,7 @@ int launch_step_mma(StepParams p, const TensorMapSet& maps, int sm_count, cudaSt
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;
   if (grid <= 0) return 0;
-  kernel<<<static_cast<unsigned>(grid), kMmaThreads, kMmaSmemBytes, stream>>>(p, *reinterpret_cast<const MmaMaps*>(maps.bytes));
-  return static_cast<int>(cudaGetLastError());
+  return launch_chained(kernel, static_cast<unsigned>(grid), kMmaThreads, kMmaSmemBytes, stream, p, *reinterpret_cast<const MmaMaps*>(maps.bytes));
 }
 
 }  // namespace detag

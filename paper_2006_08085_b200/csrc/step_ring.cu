@@ -32,6 +32,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
 #include "pipeline.cuh"
@@ -115,6 +116,8 @@ step_ring_kernel(const StepParams p, const __grid_constant__ RingMaps maps, cons
   }
   fence_async_shared();
   __syncthreads();
+  chain_wait();
+  chain_next();
 
   // this CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ...
   // 32-bit bookkeeping throughout: the launcher admits d < 2^31, so slab, tile and chunk counts of a CTA fit easily,
@@ -473,8 +476,7 @@ int launch_step_ring(StepParams p, const TensorMapSet& maps, const double* band,
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;
   if (grid <= 0) return 0;
-  step_ring_kernel<<<static_cast<unsigned>(grid), kRThreads, kRingSmemBytes, stream>>>(p, *reinterpret_cast<const RingMaps*>(maps.bytes), coef);
-  return static_cast<int>(cudaGetLastError());
+  return launch_chained(step_ring_kernel, static_cast<unsigned>(grid), kRThreads, kRingSmemBytes, stream, p, *reinterpret_cast<const RingMaps*>(maps.bytes), coef);
 }
 
 }  // namespace detag

@@ -54,6 +54,7 @@
 #include <cstring>
 #include <utility>
 
+#include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
 #include "pipeline.cuh"
@@ -318,6 +319,8 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   tmem_fence_before();
   __syncthreads();
   tmem_fence_after();
+  chain_wait();
+  chain_next();
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
   if (tid == 0 && *tmem_slot != 0) atomicExch(p.status, 2);
 
@@ -1009,9 +1012,7 @@ int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& p
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;
   if (grid <= 0) return 0;
-  kernel<<<static_cast<unsigned>(grid), kPThreads, plan.bytes, stream>>>(
-      p, *reinterpret_cast<const SplitMaps*>(maps.bytes), tb, plan);
-  return static_cast<int>(cudaGetLastError());
+  return launch_chained(kernel, static_cast<unsigned>(grid), kPThreads, plan.bytes, stream, p, *reinterpret_cast<const SplitMaps*>(maps.bytes), tb, plan);
 }
 
 }  // namespace detag

@@ -40,6 +40,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
 #include "pipeline.cuh"
@@ -224,6 +225,8 @@ step_torus_kernel(const StepParams p, const __grid_constant__ TorusMaps maps, co
   }
   fence_async_shared();
   __syncthreads();
+  chain_wait();
+  chain_next();
 
   // this CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ...; k counts them
   const long long my_slabs = blockIdx.x < p.num_slabs ? (p.num_slabs - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
@@ -504,9 +507,7 @@ int launch_step_torus(StepParams p, const TensorMapSet& maps, const double* phat
   if (e != 0) return e;
   const long long grid = p.num_slabs < sm_count ? p.num_slabs : sm_count;
   if (grid <= 0) return 0;
-  kernel<<<static_cast<unsigned>(grid), kTThreads, smem, stream>>>(p, *reinterpret_cast<const TorusMaps*>(maps.bytes),
-                                                                   phat_frag);
-  return static_cast<int>(cudaGetLastError());
+  return launch_chained(kernel, static_cast<unsigned>(grid), kTThreads, smem, stream, p, *reinterpret_cast<const TorusMaps*>(maps.bytes), phat_frag);
 }
 
 }  // namespace detag

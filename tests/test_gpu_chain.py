@@ -1,0 +1,71 @@
+"""Steps that follow one another on a stream, each launch beginning while the one before it finishes: the same bits as with the
+device idle between them, on every kernel, from a captured graph too, and between other work on the stream."""
+import numpy as np
+import pytest
+
+from paper_2006_08085_b200 import binding as B
+from paper_2006_08085_b200 import build, inputs
+from paper_2006_08085_b200.session import Session
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # n, d, K, graph, variant, mode
+    (8, 4096, 2, "ring", B.DETAG_VARIANT_AUTO, "detag"), (16, 33_001, 2, "ring", B.DETAG_VARIANT_AUTO, "external"),
+    (24, 20_003, 3, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (30, 20_003, 3, "regular4", B.DETAG_VARIANT_AUTO, "external"),
+    (48, 30_001, 3, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (64, 20_010, 4, "torus", B.DETAG_VARIANT_AUTO, "detag"),
+    (100, 30_002, 4, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (256, 3_003, 9, "torus", B.DETAG_VARIANT_AUTO, "detag"),
+    (96, 40_005, 4, "ring", B.DETAG_VARIANT_AUTO, "detag"),  # band kernel, its last columns in a launch of their own
+    (60, 5_003, 3, "regular4", B.DETAG_VARIANT_CSR, "detag")]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def _session(n, d, K, graph, variant, mode):
+    m = inputs.metropolis_weights(inputs.ring_graph(n) if graph == "ring" else inputs.torus_graph(n // 8, 8)
+                                  if graph == "torus" else inputs.random_regular4_graph(n, n))
+    rng = np.random.default_rng(n + d)
+    s = Session(m, d, K, 0.2, 0.02, sigma=0.1, seed=5, variant=variant, external_gradient=mode == "external")
+    for k in ("x", "y", "g", "a", "c") + (("g_new",) if mode == "external" else ()):
+        s.upload(k, rng.standard_normal((n, d)).astype(np.float32))
+    B.detag_set_step(s.state, 0)
+    return s
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[0]}-{c[3]}-{c[5]}")
+def test_back_to_back_as_with_the_device_idle_between(case):
+    import torch
+
+    got = []
+    for how in ("idle", "chained", "captured"):
+        with _session(*case) as s:
+            stream = torch.cuda.Stream()
+            stream.wait_stream(torch.cuda.current_stream())
+
+            def steps(count):
+                for _ in range(count):
+                    if s.g_new is not None:  # another kernel between the steps, which the next one reads from
+                        s.g_new.mul_(0.5)
+                    s.step()
+                    if how == "idle":
+                        torch.cuda.synchronize()
+
+            with torch.cuda.stream(stream):
+                steps(2)
+                if how == "captured":
+                    stream.synchronize()
+                    graph, t = torch.cuda.CUDAGraph(), B.detag_get_step(s.state)
+                    with torch.cuda.graph(graph, stream=stream):
+                        steps(6)
+                    assert B.detag_get_step(s.state) == t + 6
+                    graph.replay()
+                else:
+                    steps(6)
+            stream.synchronize()
+            s.status()
+            got.append({k: s.download(k) for k in ("x", "y", "g")})
+    for other in got[1:]:
+        for k in ("x", "y", "g"):
+            assert np.array_equal(got[0][k], other[k]), k
