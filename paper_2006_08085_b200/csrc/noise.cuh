@@ -120,5 +120,36 @@ __device__ __forceinline__ void normal_quad(const uint32_t (&round_key)[20], uns
   unpack2(mul2(odd, both(scale)), xi[1], xi[3]);
 }
 
+// `scale` times the normals of workers 4q..4q+7 at one coordinate.  The two calls differ in the third counter word alone: of
+// the first round's products one is common and the other grows by the multiplier, of the second round's one is common.
+__device__ __forceinline__ void normal_eight(const uint32_t (&round_key)[20], unsigned long long j, uint32_t q, uint32_t t, float scale,
+                                             float (&xi)[8]) {
+  constexpr uint32_t kM0 = 0xD2511F53u, kM1 = 0xCD9E8D57u;
+  const unsigned long long pj = static_cast<unsigned long long>(kM0) * static_cast<uint32_t>(j);
+  const uint32_t c2 = static_cast<uint32_t>(pj >> 32) ^ t ^ round_key[1], c3 = static_cast<uint32_t>(pj);
+  const unsigned long long p1 = static_cast<unsigned long long>(kM1) * c2;
+  unsigned long long pq = static_cast<unsigned long long>(kM1) * q;
+#pragma unroll
+  for (int h = 0; h < 2; ++h, pq += kM1) {
+    const uint32_t c0 = static_cast<uint32_t>(pq >> 32) ^ static_cast<uint32_t>(j >> 32) ^ round_key[0];
+    const unsigned long long p0 = static_cast<unsigned long long>(kM0) * c0;
+    Philox4 r{static_cast<uint32_t>(p1 >> 32) ^ static_cast<uint32_t>(pq) ^ round_key[2], static_cast<uint32_t>(p1),
+              static_cast<uint32_t>(p0 >> 32) ^ c3 ^ round_key[3], static_cast<uint32_t>(p0)};
+#pragma unroll
+    for (int round = 2; round < 10; ++round) {
+      const unsigned long long a = static_cast<unsigned long long>(kM0) * r.r0;
+      const unsigned long long b = static_cast<unsigned long long>(kM1) * r.r2;
+      r.r0 = static_cast<uint32_t>(b >> 32) ^ r.r1 ^ round_key[2 * round];
+      r.r1 = static_cast<uint32_t>(b);
+      r.r2 = static_cast<uint32_t>(a >> 32) ^ r.r3 ^ round_key[2 * round + 1];
+      r.r3 = static_cast<uint32_t>(a);
+    }
+    F2 even, odd;
+    box_muller(r, even, odd);
+    unpack2(mul2(even, both(scale)), xi[4 * h], xi[4 * h + 2]);
+    unpack2(mul2(odd, both(scale)), xi[4 * h + 1], xi[4 * h + 3]);
+  }
+}
+
 }  // namespace detag
 #endif  // DETAG_NOISE_CUH

@@ -38,12 +38,20 @@
 // Blocks of P without a digit (rings, tori with few rounds) are skipped; equal blocks (circulant and block-circulant matrices) are
 // kept once.
 //
-// Bound by the finishing warps' chain (207 instructions per worker-coordinate in all, 60 % of the issue slots at n = 100), at a
-// dense n = 256 by MMAs and splitting, which take turns.  us per step, the float64 kernels this one replaced -> now: 48
-// workers, printed timing, d = 1.0 M 861 -> 470; 100 workers, d = 2 M 3518 -> 2060; 256-ring at K = 196, d = 200 k
-// 1940 -> 640; 16 x 16 torus, d = 500 k 8992 -> 1640.  (Four digits and four accumulators took 417, 1680, 566 and 1420, but
-// left 2^-31 of the coordinate's largest operand in every result.)  With every coordinate in float64: 48 workers, K = 1,
-// d = 1 M 477 -> 1410; 100 workers, K = 2 1040 -> 4730; the torus 1570 -> 8710 - P comes from L2 and the slab is held.
+// Bound by the issue slots and the latency of what the six warps of a scheduler do, at a dense n = 256 by the MMAs, which take
+// turns with splitting and with reading the one accumulator there is room for.  us per step, the float64 kernels this one
+// replaced -> now: 100 workers, d = 2 M 3518 -> 1880; 256-ring at K = 196, d = 200 k 1940 -> 607; 16 x 16 torus, d = 500 k
+// 8992 -> 1470.  (Four digits and four accumulators took 1680, 566 and 1420 when this took 2060, 640 and 1640, but left 2^-31 of the
+// coordinate's largest operand in every result.)  From those figures it came by fewer instructions in the finishing and more
+// registers for it: the scale of a coordinate sits in the number that joins the sums, a row's scale is one factor of x~ - alpha y~
+// and one of the fold, doubles are handed over whole, digits, normals and gradients are made in packed float32, and the issuing
+// warps give 48 registers each to the finishing ones, without which the former changes do not pay (100 workers 2100 us).
+// With every coordinate in float64: 100 workers, K = 2, d = 1 M 1040 -> 4730; the torus 1570 -> 8710 - P comes from L2 and the slab is
+// held.
+//
+// Measured without gain (us for the 1880 of 100 workers; the torus; the ring): digits and their places handed over block by
+// block 1915, 1550, 680 (the splitting takes issue slots from the MMAs it then runs beside); an MMA warp per accumulator 1955; the
+// normals between model update and gradient instead of before the other warp's sums 1915.
 // Every wait is bounded but the allocation of tensor memory, which waits for kernels that do not depend on this
 // one.
 #include <cuda.h>
@@ -57,6 +65,7 @@
 #include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
+#include "packed.cuh"
 #include "pipeline.cuh"
 #include "tensor_memory.cuh"
 #include "tma.cuh"
@@ -124,7 +133,7 @@ struct SplitPlan {
 };
 
 // Shared memory: x, y of a slab (whole blocks of 32 rows) | blocks of P | g, a, c stages | groups of the guard | row
-// exponents, scales, flags, maxima | barriers.
+// scales, scales, flags, maxima | barriers.
 inline SplitPlan plan_for(int nb, int num_blocks, int guard_entries, int groups, int stages) {
   SplitPlan s{};
   s.groups = groups;
@@ -133,7 +142,7 @@ inline SplitPlan plan_for(int nb, int num_blocks, int guard_entries, int groups,
   s.e_at = s.blocks_at + static_cast<size_t>(num_blocks) * kPBlockBytes;
   s.guard_at = s.e_at + static_cast<size_t>(groups) * stages * kPStageBytes;
   s.scale_at = s.guard_at + static_cast<size_t>(guard_entries + 3) / 4 * 16;
-  s.ctrl_at = s.scale_at + 256 * 4 + kPScaleSlots * 128 * 2 + kPScaleSlots * 4 * 4 + 4 * 128 * 8;
+  s.ctrl_at = s.scale_at + 256 * 8 + kPScaleSlots * 128 * 2 + kPScaleSlots * 4 * 4 + 4 * 128 * 8;
   s.bytes = s.ctrl_at + kPCtrlBytes;
   return s;
 }
@@ -149,24 +158,25 @@ inline SplitPlan split_plan(int nb, int num_blocks, int guard_entries) {
   return SplitPlan{};
 }
 
-// Integer sums of the five weights -> one float64 in units of 256^5, exact but for the rounding of the lowest: a 64-bit
-// integer below 2^51 added to the bits of 1.5 * 2^52.  `hi` = s8 * 256 + s7.  Up to 128 workers the rest fits 32 bits
+// Integer sums of the five weights -> one float64, exact but for the rounding of the lowest: a 64-bit integer below 2^51, in units
+// of 256^5, added to the bits of 1.5 * 2^52 with the coordinate's scale in its exponent field (`magic_hi`: the upper word; `magic`:
+// that number), which is then subtracted.  `hi` = s8 * 256 + s7.  Up to 128 workers the rest fits 32 bits
 // (3 * 128 * 2^14 * 256 < 2^31).
 template <bool kBig>
-__device__ __forceinline__ double join_sums(int hi, int s6, int s5, int s4) {
+__device__ __forceinline__ double join_sums(int hi, int s6, int s5, int s4, int magic_hi, double magic) {
   const int low = s5 + ((s4 + 128) >> 8);
   if (kBig) {
-    const long long lo = static_cast<long long>(s6) * 256 + (low + 0x4338000000000000LL);
-    return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - 6755399441055744.0;
+    const long long lo = static_cast<long long>(s6) * 256 + (low + (static_cast<long long>(magic_hi) << 32));
+    return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - magic;
   }
-  const uint32_t lo = static_cast<uint32_t>(s6 * 256 + low) ^ 0x80000000u;  // offset by 2^31: no sign to extend
-  return __longlong_as_double(static_cast<long long>(hi) * 65536 + (0x4338000000000000LL | lo)) -
-         (6755399441055744.0 + 2147483648.0);
+  const int lo = s6 * 256 + low;
+  const unsigned long long upper = static_cast<uint32_t>(magic_hi + (lo >> 31));
+  return __longlong_as_double(static_cast<long long>(hi) * 65536 + static_cast<long long>(upper << 32 | static_cast<uint32_t>(lo))) - magic;
 }
 
 // Eight joined sums of this thread's coordinate from the accumulators at `acc` (whole warp).
 template <bool kBig>
-__device__ __forceinline__ void take_sums(uint32_t acc, double (&out)[8]) {
+__device__ __forceinline__ void take_sums(uint32_t acc, int magic_hi, double magic, double (&out)[8]) {
   int hi[8], s6[8], s5[8], s4[8];
   {
     int s7[8];
@@ -181,7 +191,7 @@ __device__ __forceinline__ void take_sums(uint32_t acc, double (&out)[8]) {
   tmem_load8(acc + 4 * kPChunk, s4);
   tmem_wait_load();
 #pragma unroll
-  for (int u = 0; u < 8; ++u) out[u] = join_sums<kBig>(hi[u], s6[u], s5[u], s4[u]);
+  for (int u = 0; u < 8; ++u) out[u] = join_sums<kBig>(hi[u], s6[u], s5[u], s4[u], magic_hi, magic);
 }
 
 // Largest magnitude of a block's 32 staged rows (those beyond n are zeros), with what came before.
@@ -221,20 +231,26 @@ __device__ __forceinline__ float group_low(const float* col, const int* guard, i
 
 // Digits of a block's 32 workers (zeros beyond n): digit 0 in w0, digit k in words 8 (k - 1) .. 8 k - 1 of w.  The value
 // z scale, at most 31 bits before the point, in two steps that float32 does exactly: its multiple of 2^14 next to it, and
-// what is left in 1/256, each as the low bits of 1.5 * 2^23 plus it.  With the 40-bit integer q of both, q + 0x8080808080
-// has the balanced digits as bytes offset by 128.  No conversions: they run on a pipe a quarter as wide.  No test per row:
+// what is left in 1/256, each as the low bits of 1.5 * 2^23 plus it.  With the 40-bit integer q of both, q + 0x0080808080
+// has the balanced digits as bytes, all but the top one offset by 128.  No conversions: they run on a pipe a quarter as wide.  No test per row:
 // the splitting is a serial chain, and so its loads and chains overlap.
 __device__ __forceinline__ void block_digits(const float* src, float scale, uint32_t (&w)[32], uint32_t (&w0)[8]) {
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     uint32_t z[4], f[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const float x = src[(4 * u + v) * kPS];
-      const float high = fmaf(x, scale, 206158430208.f);                                   // 1.5 * 2^37
-      const float rest = fmaf(x, scale, -__fadd_rn(high, -206158430208.f));
-      f[v] = __float_as_uint(fmaf(rest, 256.f, 12583040.f));                               // 1.5 * 2^23 + 128
-      z[v] = (__float_as_uint(high) << 14) + ((f[v] >> 8) + (0x80808080u - 0x4B4000u));
+    for (int v = 0; v < 4; v += 2) {
+      const F2 x = pack2(src[(4 * u + v) * kPS], src[(4 * u + v + 1) * kPS]);
+      const F2 high = fma2(x, both(scale), both(206158430208.f));                          // 1.5 * 2^37
+      const F2 rest = fma2(x, both(scale), sub2(both(206158430208.f), high));
+      const F2 low = fma2(rest, both(256.f), both(12583040.f));                            // 1.5 * 2^23 + 128
+      float h0, h1, f0, f1;
+      unpack2(high, h0, h1);
+      unpack2(low, f0, f1);
+      f[v] = __float_as_uint(f0);
+      f[v + 1] = __float_as_uint(f1);
+      z[v] = (__float_as_uint(h0) << 14) + ((f[v] >> 8) + (0x00808080u - 0x4B4000u));
+      z[v + 1] = (__float_as_uint(h1) << 14) + ((f[v + 1] >> 8) + (0x00808080u - 0x4B4000u));
     }
     const uint32_t ab = __byte_perm(z[0], z[1], 0x5140), cd = __byte_perm(z[2], z[3], 0x5140);
     const uint32_t ef = __byte_perm(z[0], z[1], 0x7362), gh = __byte_perm(z[2], z[3], 0x7362);
@@ -242,7 +258,7 @@ __device__ __forceinline__ void block_digits(const float* src, float scale, uint
     w[u] = __byte_perm(ab, cd, 0x5410) ^ 0x80808080u;
     w[8 + u] = __byte_perm(ab, cd, 0x7632) ^ 0x80808080u;
     w[16 + u] = __byte_perm(ef, gh, 0x5410) ^ 0x80808080u;
-    w[24 + u] = __byte_perm(ef, gh, 0x7632) ^ 0x80808080u;
+    w[24 + u] = __byte_perm(ef, gh, 0x7632);
   }
 }
 
@@ -259,8 +275,8 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   float* const xy_mem = reinterpret_cast<float*>(smem);                    // [block][x | y][32 rows][64]
   float* const e_mem = reinterpret_cast<float*>(smem + plan.e_at);
   int* const guard = reinterpret_cast<int*>(smem + plan.guard_at);          // [group][guard_size]
-  int* const row_exp = reinterpret_cast<int*>(smem + plan.scale_at);       // shifted to the exponent field of a double
-  short* const scales = reinterpret_cast<short*>(row_exp + 256);           // [slot][128 rows]
+  double* const row_scale = reinterpret_cast<double*>(smem + plan.scale_at);  // a power of two per output worker
+  short* const scales = reinterpret_cast<short*>(row_scale + 256);         // [slot][128 rows]
   unsigned* const flags = reinterpret_cast<unsigned*>(scales + kPScaleSlots * 128);  // [slot][lane quarter]: rows in float64
   float2* const maxima = reinterpret_cast<float2*>(flags + kPScaleSlots * 4);  // [slab parity][splitting group][128 rows]
   uint64_t* const xy_full = reinterpret_cast<uint64_t*>(smem + plan.ctrl_at);
@@ -290,7 +306,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     const uint4* src = tb.blocks;
     uint4* dst = reinterpret_cast<uint4*>(smem + plan.blocks_at);
     for (int e = tid; e < tb.num_blocks * (kPBlockBytes / 16); e += blockDim.x) dst[e] = src[e];
-    for (int e = tid; e < 256; e += blockDim.x) row_exp[e] = e < n ? tb.row_exp[e] * (1 << 20) : 0;
+    for (int e = tid; e < 256; e += blockDim.x) row_scale[e] = __hiloint2double((1023 + (e < n ? tb.row_exp[e] : 0)) << 20, 0);
     for (int e = tid; e < tb.guard_groups * tb.guard_size; e += blockDim.x) guard[e] = tb.guard[e];
   }
   if (tid == 0) {
@@ -339,6 +355,15 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     return __all_sync(0xffffffffu, bar_wait(bar, phase & 1, limit));
   };
 
+  // Registers from the warps that only issue to those that finish: of the 768 x 80 the block is launched with, 80 per splitting
+  // thread, 32 per issuing thread and 96 (88 beyond 128 workers) per finishing thread.
+  constexpr int kFinishRegisters = kBig ? 88 : 96;
+  static_assert(kSplitWarps * 80 + 4 * 32 + (24 - kSplitWarps - 4) * kFinishRegisters <= 24 * 80, "register split");
+  if (warp >= kFinishWarp) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFinishRegisters));
+  } else if (warp >= kSplitWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+  }
   if (warp < kSplitWarps) {
     // ---------------------------------------------------------------- splitting warps: thread = row of A = tensor memory lane
     const int part = warp >> 2, quarter = warp & 3;
@@ -451,31 +476,34 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
         gold[u] = sg[u * kPS];
         av[u] = sa[u * kPS];
       }
-      // ---- sums of sixteen workers: eight handed to the other warp of the pair, eight kept
+      // ---- sums of sixteen workers, but for the factor of their rows: eight handed to the other warp of the pair, eight kept.
+      // A handed double lies across this warp's part of two rows, so that half a warp's are 128 bytes in a row.
       double own[8];
-      const int ex = (scales[slot * 128 + coord] + 1023) << 20, ey = (scales[slot * 128 + 64 + coord] + 1023) << 20;
+      const double magic = __hiloint2double(0x43380000 + scales[slot * 128 + (second ? 64 : 0) + coord] * (1 << 20), 0);
+      const int magic_hi = __double2hiint(magic);
+      double* const box = reinterpret_cast<double*>(e_mem + (static_cast<size_t>(t) * stages + st) * (kPStageBytes / 4) + pair * 32 + (lane >> 4) * kPS) + (lane & 15);
+      double* const my_box = box + mine * (kPS / 2);
+      auto box_at = [](int u) { return (u >> 2) * (kPStageFloats / 2) + (u & 3) * kPS; };
+      __syncwarp();  // every lane has taken its g and a out
       if (exact_lanes == 0) {
         const uint32_t acc = acc_lane + a * kPAccColumns + (h & 1) * kPUnit;
         if (kMode != kModeDpsgd || !second) {
           double give[8];
-          take_sums<kBig>(acc + (mine ^ 8), give);
+          take_sums<kBig>(acc + (mine ^ 8), magic_hi, magic, give);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            sg[u * kPS] = __int_as_float(__double2hiint(give[u]));
-            sa[u * kPS] = __int_as_float(__double2loint(give[u]));
-          }
+          for (int u = 0; u < 8; ++u) my_box[box_at(u)] = give[u];
         }
-        take_sums<kBig>(acc + mine, own);
+        take_sums<kBig>(acc + mine, magic_hi, magic, own);
       } else {
-        // Some row of this warp was not split: all 32 in float64, from the operands themselves, in units of the scales.
+        // Some row of this warp was not split: all 32 in float64, from the operands themselves.
         const float* const z = xy_mem + (second ? kPTileFloats : 0) + pair * 32;
-        const int to_units = (2046 << 20) - (second ? ey : ex);
         float* const hi_word = sg - lane;  // this warp's part of the mailbox, [worker][coordinate]
         float* const lo_word = sa - lane;
         const int c = h >> 1, pitch = tb.circulant ? kPChunk : units * kPUnit;
         const double* const columns = tb.poly_t + (tb.circulant ? kPUnit * (h & 1) : kPUnit * h);
         bool finite = true;
-        __syncwarp();  // every lane has taken its g and a out of the mailbox
+        // 1 / the row's scale
+        auto unscale = [&](int row) { return __hiloint2double((2046 << 20) - __double2hiint(row_scale[row]), 0); };
         // Products on the float64 tensor path: four tiles of eight coordinates (M) by eight output workers (N)
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -503,19 +531,22 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
               lo_word[at] = __int_as_float(__double2loint(sum[i][e]));
             }
           __syncwarp();
+          double take[8];
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
             const double v = __hiloint2double(__float_as_int(sg[u * kPS]), __float_as_int(sa[u * kPS]));
             finite = finite && (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
-            const double scaled = v * __hiloint2double(to_units - row_exp[kPUnit * h + to + u], 0);
-            if (half == 0) {
-              own[u] = scaled;
-            } else {  // this lane's own column
-              sg[u * kPS] = __int_as_float(__double2hiint(scaled));
-              sa[u * kPS] = __int_as_float(__double2loint(scaled));
-            }
+            take[u] = v * unscale(kPUnit * h + to + u);
           }
           __syncwarp();
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (half == 0) {
+              own[u] = take[u];
+            } else {
+              my_box[box_at(u)] = take[u];
+            }
+          }
         }
         if (__any_sync(0xffffffffu, !finite)) {
           // Infinities or NaN among the operands: a lane sums its own coordinate, without the zeros of P, which the products
@@ -537,12 +568,11 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const double scaled = sum[u] * __hiloint2double(to_units - row_exp[kPUnit * h + to + u], 0);
+              const double scaled = sum[u] * unscale(kPUnit * h + to + u);
               if (half == 0) {
                 own[u] = scaled;
               } else {
-                sg[u * kPS] = __int_as_float(__double2hiint(scaled));
-                sa[u * kPS] = __int_as_float(__double2loint(scaled));
+                my_box[box_at(u)] = scaled;
               }
             }
           }
@@ -559,62 +589,56 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
       float xi[8];
       if (noisy) {
         const unsigned long long jn = static_cast<unsigned long long>(p.coord_offset + j);
-#pragma unroll
-        for (int u = 0; u < 8; u += 4) {
-          float quad[4];
-          normal_quad(p.round_key, jn, static_cast<uint32_t>((w0 + u) >> 2), p.t_noise, quad);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) xi[u + i] = sigma * quad[i];
-        }
+        normal_eight(p.round_key, jn, static_cast<uint32_t>(w0 >> 2), p.t_noise, sigma, xi);
       } else {
 #pragma unroll
         for (int u = 0; u < 8; ++u) xi[u] = 0.f;
       }
+      // gradient point of Algorithm 2 as printed: the model the step started from, still in global memory - this unit's rows are
+      // stored after this
+      float start[8];
+      if (at_start) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) start[u] = w0 + u < n && j < p.d ? p.x[static_cast<long long>(w0 + u) * p.ld + j] : 0.f;
+      }
       ok = warp_wait(written, m);
       if (!ok) break;
-      // ---- gossiped model and tracker (over `own`), model update, y~ - g
-      const float* const og = sg + (second ? -8 * kPS : 8 * kPS);  // the other warp's slots
-      int er[8];
-      *reinterpret_cast<int4*>(&er[0]) = *reinterpret_cast<const int4*>(row_exp + w0);
-      *reinterpret_cast<int4*>(&er[4]) = *reinterpret_cast<const int4*>(row_exp + w0 + 4);
-      double xd[8], yg[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const double other = (kMode != kModeDpsgd || second)
-                                 ? __hiloint2double(__float_as_int(og[u * kPS]), __float_as_int(og[kPStageFloats + u * kPS])) : 0.0;
-        const double xt = (second ? other : own[u]) * __hiloint2double(ex + er[u], 0);
-        const double yt = (second ? own[u] : other) * __hiloint2double(ey + er[u], 0);
-        const double gd = static_cast<double>(gold[u]);
-        xd[u] = fma(-alpha, kMode == kModeDpsgd ? gd : yt, xt);
-        yg[u] = yt - gd;
-        own[u] = yt;
-      }
+      const double* const other_box = box + (mine ^ 8) * (kPS / 2);
       if (kMode != kModeDpsgd && p.y_obs != nullptr) {  // optional observer: the gossiped tracker
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (w0 + u < n && j < p.d) p.y_obs[static_cast<long long>(w0 + u) * p.ld + j] = static_cast<float>(own[u]);
+          if (w0 + u < n && j < p.d)
+            p.y_obs[static_cast<long long>(w0 + u) * p.ld + j] = static_cast<float>((second ? own[u] : other_box[box_at(u)]) * row_scale[w0 + u]);
+      }
+      // ---- gossiped model and tracker, model update, y~ - g
+      double yg[8];
+      float at[8], go[8], xo[8], yo[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const double other = (kMode != kModeDpsgd || second) ? other_box[box_at(u)] : 0.0;
+        const double factor = row_scale[w0 + u];  // a power of two: its products are exact
+        const double xt = second ? other : own[u], yt = second ? own[u] : other, gd = static_cast<double>(gold[u]);
+        const double xd = kMode == kModeDpsgd ? fma(-alpha, gd, xt * factor) : fma(-alpha, yt, xt) * factor;
+        yg[u] = fma(yt, factor, -gd);
+        xo[u] = static_cast<float>(xd);
+        at[u] = at_start ? start[u] : xo[u];
+        if (kWide) own[u] = at_start ? static_cast<double>(at[u]) : xd;
+      }
+      // ---- gradient and fold
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        const float c0 = sc[u * kPS], c1 = sc[(u + 1) * kPS];
+        if (kWide) {
+          go[u] = static_cast<float>(fma(static_cast<double>(av[u]), own[u] - static_cast<double>(c0), static_cast<double>(xi[u])));
+          go[u + 1] = static_cast<float>(fma(static_cast<double>(av[u + 1]), own[u + 1] - static_cast<double>(c1), static_cast<double>(xi[u + 1])));
+        } else {
+          unpack2(fma2(pack2(av[u], av[u + 1]), sub2(pack2(at[u], at[u + 1]), pack2(c0, c1)), pack2(xi[u], xi[u + 1])), go[u], go[u + 1]);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) yo[u + e] = static_cast<float>(yg[u + e] + static_cast<double>(go[u + e]));
       }
       __syncwarp();
       if (lane == 0) bar_arrive(taken);
-      // ---- gradient at the new model, or at the one the step started from - still in global memory, this unit's rows
-      // are stored after this - and fold; the results go over g, a, c
-      float at[8], go[8], xo[8], yo[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) at[u] = xo[u] = static_cast<float>(xd[u]);
-      if (at_start) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          at[u] = w0 + u < n && j < p.d ? p.x[static_cast<long long>(w0 + u) * p.ld + j] : 0.f;
-          if (kWide) xd[u] = static_cast<double>(at[u]);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float cv = sc[u * kPS];
-        go[u] = kWide ? static_cast<float>(fma(static_cast<double>(av[u]), xd[u] - static_cast<double>(cv), static_cast<double>(xi[u])))
-                      : fmaf(av[u], at[u] - cv, xi[u]);
-        yo[u] = static_cast<float>(yg[u] + static_cast<double>(go[u]));
-      }
       ok = warp_wait(taken, m);
       if (!ok) break;
 #pragma unroll
