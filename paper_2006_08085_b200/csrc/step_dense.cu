@@ -6,7 +6,8 @@
 // the same ones: operands, sums and the element-wise tail of a coordinate never leave the lane.
 //
 // Four warps (a group) take a slab of 64 coordinates, sixteen each, a lane two neighbours (both share a fragment of P, which
-// comes from shared memory).  Slabs of 64 because rows have to travel in pieces of 256 bytes: warps on their own with 64-byte
+// comes from shared memory); beyond 32 workers eight warps with a coordinate per lane, for the sums of two would leave room for
+// half the warps.  Slabs of 64 because rows have to travel in pieces of 256 bytes: warps on their own with 64-byte
 // pieces reached 0.38 of the copy rate, by TMA and by cp.async alike.  A group has one buffer for the operands of the products
 // (x, y; up to 32 workers g) and one for the rest, over which the results are written.  There is no loading and no storing
 // thread: the warp that is the last of its group to be done with the operands asks for the next slab's, which travel while the
@@ -17,14 +18,16 @@
 // every access of a half warp falls into different banks.  The last d % 64 coordinates are read and written by their lanes.
 //
 // Bound: HBM and the power cap up to 32 workers (d = 25.6 M, six rounds 4.8 ms in short runs, 0.83 of the copy rate; the kernel
-// with padded tiles, a loading and a storing thread 5.17; D-PSGD, d = 3 M 421 us, 0.84), beyond them the FP64 pipe: 12 MMAs of
+// with padded tiles, a loading and a storing thread 5.17; D-PSGD, d = 3 M 417 us, 0.84), beyond them the FP64 pipe: 12 MMAs of
 // 16.3 cycles and three scalar operations per 32 worker-coordinates and scheduler at 48 workers, 200 cycles for 176 of HBM, of which
-// three warps per scheduler keep 0.7 busy (d = 1 M 390 us; the integer tensor path 428).  Up to 24 workers padding was what it
+// six warps per scheduler keep 0.7 busy (d = 1 M 372 us; the integer tensor path 428).  Up to 24 workers padding was what it
 // saves: 24, d = 3 M 569 -> 400 us, 17 582 -> 340.
 //
 // Measured on the way (us): the normals drawn in the tail instead of before the wait for its inputs, 32 workers d = 25.6 M 4900
-// for 4805, at 48 workers 390 for 395; products in a loop unrolled twice 5190 at 32 workers, at 48 390 where the straight line of
-// 288 MMAs takes 410; loads of a ragged slab one after the other 17 instead of 12 at d = 9000.
+// for 4805; products in a loop unrolled twice 5190 at 32 workers, at 48 390 where the straight line of MMAs takes 410; loads of a
+// ragged slab one after the other 17 instead of 12 at d = 9000.  Two coordinates per lane and three groups of four warps beyond 32
+// workers: 48 382 for 372, printed timing 411 for 395, 33 276 for 258, 33 with d = 100 k 37.2 for 33.9, but caller-written gradients of
+// 48 391 for 397; two groups of eight 380.  One coordinate per lane up to 32: 24 456 for 408, 32 with d = 30 k 14.5 for 12.4.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -40,7 +43,11 @@ namespace detag {
 namespace {
 
 constexpr int kDS = 64;  // coordinates per slab
+// Coordinates per lane, warps per group, threads per CTA.
+__host__ __device__ constexpr int dense_coords(int R) { return R <= 8 ? 2 : 1; }
+__host__ __device__ constexpr int dense_warps(int R) { return 8 / dense_coords(R); }
 __host__ __device__ constexpr int dense_groups(int R) { return R <= 8 ? 4 : 3; }
+__host__ __device__ constexpr int dense_threads(int R) { return dense_groups(R) * dense_warps(R) * 32; }
 __host__ __device__ constexpr int dense_blocks(int R) { return (R + 1) / 2; }
 __host__ __device__ constexpr int dense_frag_bytes(int R) { return R * dense_blocks(R) * 32 * 8; }
 __host__ __device__ constexpr int dense_group_bytes(int R) { return (R <= 8 ? 6 : 5) * R * 1024; }
@@ -61,17 +68,19 @@ __device__ __forceinline__ bool last_of(unsigned* counter, unsigned of) {
   return before % of == of - 1;
 }
 
-// The first `bytes` (0, 4 or 8) of eight bytes, then zeros; asynchronous.
-__device__ __forceinline__ void copy8(float* to, const float* from, int bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(s_addr(to)), "l"(from), "r"(bytes) : "memory");
+// The first `bytes` of kBytes (4 or 8) bytes, then zeros; asynchronous.
+template <int kBytes>
+__device__ __forceinline__ void copy_bytes(float* to, const float* from, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(s_addr(to)), "l"(from), "n"(kBytes), "r"(bytes) : "memory");
 }
 
 // R: workers per lane, n rounded up to 4 R.  kWide: the gradient in float64 instead of float32 at the rounded model.
 // kMany: p.steps iterations (DeTAG with the synthetic gradient, up to 32 workers): every lane's results take the places of its
 // own operands.
 template <int R, int kMode, bool kAtStart, bool kWide, bool kMany = false>
-__global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(const StepParams p, const __grid_constant__ DenseMaps maps) {
+__global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const StepParams p, const __grid_constant__ DenseMaps maps) {
   constexpr int kBlocks = dense_blocks(R), kGroups = dense_groups(R), kTile = R * 256;  // floats of an array's tile
+  constexpr int V = dense_coords(R), kWarps = dense_warps(R);
   // Where g is: with the operands (up to 32 workers, so that y~ - g is what the products sum up to, as in the kernel of
   // several steps), or with the tail's inputs.
   constexpr bool kEarly = R <= 8;
@@ -79,7 +88,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* const smem = smem_unaligned + ((1024u - (s_addr(smem_unaligned) & 1023u)) & 1023u);
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), q = lane & 3, c = lane >> 2;
-  const int group = warp >> 2, quarter = warp & 3;
+  const int group = warp / kWarps, part = warp % kWarps;
   float* const tiles = reinterpret_cast<float*>(smem + group * dense_group_bytes(R));
   double* const frag = reinterpret_cast<double*>(smem + kGroups * dense_group_bytes(R));  // [input step][output block][lane]
   uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + kGroups * dense_group_bytes(R) + dense_frag_bytes(R));
@@ -94,11 +103,26 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
   float* const t_gout = kEarly ? tg + kTile : tg;
   float* const ta = t_gout + kTile;
   float* const tc = ta + kTile;
-  // this lane's two coordinates of row q; rows q + 4 i are 256 floats apart and have the same place in the swizzle
-  const int half = quarter >> 1, chunk = (quarter & 1) * 4 + (c >> 1);
-  const int off = q * kDS + half * 32 + ((chunk ^ ((2 * q + half) & 7)) << 2) + (c & 1) * 2;
-  auto get = [&](const float* tile, int i) { return *reinterpret_cast<const float2*>(tile + off + i * 256); };
-  auto put = [&](float* tile, int i, float2 v) { *reinterpret_cast<float2*>(tile + off + i * 256) = v; };
+  // this lane's coordinates of row q; rows q + 4 i are 256 floats apart and have the same place in the swizzle
+  const int within = 8 * V * part + V * c, half = within >> 5, chunk = (within & 31) >> 2;
+  auto place = [&](int row) { return row * kDS + half * 32 + ((chunk ^ ((2 * row + half) & 7)) << 2) + (within & 3); };
+  const int off = place(q);
+  // Two elements at a time: of row i its two coordinates, or of rows i and i + 1 the one.
+  auto row_of = [](int i, int m) { return V == 2 ? i : i + m; };
+  auto coord_of = [](int m) { return V == 2 ? m : 0; };
+  auto get = [&](const float* tile, int i) {
+    if (V == 2) return *reinterpret_cast<const float2*>(tile + off + i * 256);
+    return make_float2(tile[off + i * 256], i + 1 < R ? tile[off + (i + 1) * 256] : 0.f);
+  };
+  auto put = [&](float* tile, int i, float2 v) {
+    if (V == 2) {
+      *reinterpret_cast<float2*>(tile + off + i * 256) = v;
+    } else {
+      tile[off + i * 256] = v.x;
+      if (i + 1 < R) tile[off + (i + 1) * 256] = v.y;
+    }
+  };
+  auto one = [&](const float* tile, int i, int t) { return tile[off + i * 256 + t]; };
 
   const double alpha = p.alpha;
   const float sigma = static_cast<float>(p.sigma);
@@ -119,7 +143,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
     rows_load(ta, &maps.a, 2 * s, 0, tail_full);
     if (kMode != kModeExternal) rows_load(tc, &maps.c, 2 * s, 0, tail_full);
   };
-  if (quarter == 0 && lane == 0) {
+  if (part == 0 && lane == 0) {
     bar_init(in_full, 1);
     bar_init(tail_full, 1);
     *in_done = *tail_done = 0;
@@ -132,7 +156,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
     }
   }
 #pragma unroll
-  for (int e = threadIdx.x; e < R * kBlocks * 32; e += kGroups * 128) {  // while the first loads are on their way
+  for (int e = threadIdx.x; e < R * kBlocks * 32; e += dense_threads(R)) {  // while the first loads are on their way
     const int l = e & 31, b = (e >> 5) % kBlocks, k = (e >> 5) / kBlocks;
     const int out = (l >> 3) + 4 * (2 * b + ((l >> 2) & 1)), in = 4 * k + (l & 3);
     frag[e] = out < n && in < n ? p.poly[out * n + in] : 0.0;
@@ -145,8 +169,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
   int use = 0;
   for (; slab < slabs; slab += stride, ++use) {
     const bool ragged = slab >= whole;
-    const long long j = static_cast<long long>(slab) * kDS + 16 * quarter + 2 * c;  // this lane's first coordinate
-    const bool inside = j < p.d, both_inside = j + 1 < p.d;
+    const long long j = static_cast<long long>(slab) * kDS + within;  // this lane's first coordinate
     if (!ragged) ok = bar_wait(in_full, use & 1, limit);
     if (owes) {
       store_wait_read();
@@ -165,12 +188,12 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
     ok = __all_sync(0xffffffffu, ok) != 0;
     if (!ok) break;
     if (ragged) {
-      const int bytes = both_inside ? 8 : inside ? 4 : 0;  // the others become zeros
+      const int bytes = j + V <= p.d ? 4 * V : j < p.d ? 4 : 0;  // the others become zeros
       auto take = [&](float* tile, const float* base) {
 #pragma unroll 1
         for (int i = 0; i < R; ++i) {
-          const bool there = inside && q + 4 * i < n;
-          copy8(tile + off + i * 256, there ? base + (q + 4 * i) * p.ld + j : base, there ? bytes : 0);
+          const bool there = bytes != 0 && q + 4 * i < n;
+          copy_bytes<4 * V>(tile + off + i * 256, there ? base + (q + 4 * i) * p.ld + j : base, there ? bytes : 0);
         }
       };
       take(tx, p.x);
@@ -186,40 +209,37 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
       const uint32_t t_noise = p.t_noise + (kMany ? static_cast<uint32_t>(step) : 0u);
       // cx ends as x' = P (x - alpha y), by linearity; cy starts at -g and ends as y~ - g, or ends as y~.  Caller-written gradients:
       // the operand is the tracker folded with them.  D-PSGD: cx starts at -alpha g, or ends without it, and sums P x.
-      double cx[kBlocks][2][2], cy[kBlocks][2][2];  // [block][coordinate][worker of the lane's two]
+      double cx[kBlocks][V][2], cy[kBlocks][V][2];  // [block][coordinate][worker of the lane's two]
 #pragma unroll
-      for (int i = 0; i < 2 * kBlocks; ++i) {
-        float2 g = make_float2(0.f, 0.f);
-        if (kEarly && kMode != kModeExternal && i < R) g = get(tg, i);
-        cx[i >> 1][0][i & 1] = kMode == kModeDpsgd && kEarly ? -alpha * static_cast<double>(g.x) : 0.0;
-        cx[i >> 1][1][i & 1] = kMode == kModeDpsgd && kEarly ? -alpha * static_cast<double>(g.y) : 0.0;
-        cy[i >> 1][0][i & 1] = kMode == kModeDetag && kEarly ? static_cast<double>(-g.x) : 0.0;
-        cy[i >> 1][1][i & 1] = kMode == kModeDetag && kEarly ? static_cast<double>(-g.y) : 0.0;
-      }
-      float2 x_old[kAtStart ? R : 1];
+      for (int i = 0; i < 2 * kBlocks; ++i)
+#pragma unroll
+        for (int t = 0; t < V; ++t) {
+          const float g = kEarly && kMode != kModeExternal && i < R ? one(tg, i, t) : 0.f;
+          cx[i >> 1][t][i & 1] = kMode == kModeDpsgd && kEarly ? -alpha * static_cast<double>(g) : 0.0;
+          cy[i >> 1][t][i & 1] = kMode == kModeDetag && kEarly ? static_cast<double>(-g) : 0.0;
+        }
+      float x_old[kAtStart ? R : 1][V];
       constexpr int kUnroll = kAtStart || R <= 10 ? R : 2;  // the printed timing keeps the old model in registers
 #pragma unroll kUnroll
       for (int k = 0; k < R; ++k) {
-        const float2 x = get(tx, k);
-        if (kAtStart) x_old[kAtStart ? k : 0] = x;
-        double u[2] = {static_cast<double>(x.x), static_cast<double>(x.y)}, y[2] = {0.0, 0.0};
-        if (kMode != kModeDpsgd) {
-          const float2 yf = get(ty, k);
-          y[0] = static_cast<double>(yf.x);
-          y[1] = static_cast<double>(yf.y);
-          if (kMode == kModeExternal) {  // Algorithm 2's tracker update
-            const float2 gn = get(ta, k), go = get(tg, k);
-            y[0] += static_cast<double>(gn.x) - static_cast<double>(go.x);
-            y[1] += static_cast<double>(gn.y) - static_cast<double>(go.y);
+        double u[V], y[V];
+#pragma unroll
+        for (int t = 0; t < V; ++t) {
+          const float x = one(tx, k, t);
+          if (kAtStart) x_old[kAtStart ? k : 0][t] = x;
+          u[t] = static_cast<double>(x);
+          y[t] = 0.0;
+          if (kMode != kModeDpsgd) {
+            y[t] = static_cast<double>(one(ty, k, t));
+            if (kMode == kModeExternal) y[t] += static_cast<double>(one(ta, k, t)) - static_cast<double>(one(tg, k, t));  // Algorithm 2's tracker update
+            u[t] = fma(-alpha, y[t], u[t]);
           }
-          u[0] = fma(-alpha, y[0], u[0]);
-          u[1] = fma(-alpha, y[1], u[1]);
         }
 #pragma unroll
         for (int b = 0; b < kBlocks; ++b) {
           const double f = frag[(k * kBlocks + b) * 32 + lane];
 #pragma unroll
-          for (int t = 0; t < 2; ++t) {
+          for (int t = 0; t < V; ++t) {
             if (kMode != kModeDpsgd) dmma(cy[b][t], y[t], f);
             dmma(cx[b][t], u[t], f);
           }
@@ -232,7 +252,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
 #pragma unroll
         for (int b = 0; b < kBlocks; ++b)
 #pragma unroll
-          for (int t = 0; t < 2; ++t) {
+          for (int t = 0; t < V; ++t) {
             seen = max_abs3(seen, __int_as_float(__double2hiint(cx[b][t][0])), __int_as_float(__double2hiint(cx[b][t][1])));
             if (kMode != kModeDpsgd) seen = max_abs3(seen, __int_as_float(__double2hiint(cy[b][t][0])), __int_as_float(__double2hiint(cy[b][t][1])));
           }
@@ -240,7 +260,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
 #pragma unroll
           for (int b = 0; b < kBlocks; ++b)
 #pragma unroll
-            for (int t = 0; t < 2; ++t)
+            for (int t = 0; t < V; ++t)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 double sx = 0.0, sy = 0.0;
@@ -248,7 +268,7 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
                 for (int in = 0; in < n; ++in) {
                   const double w = frag[((in >> 2) * kBlocks + b) * 32 + q * 8 + e * 4 + (in & 3)];
                   if (w == 0.0) continue;
-                  const int at = (in >> 2) * 256 + (in & 3) * kDS + half * 32 + ((chunk ^ ((2 * (in & 3) + half) & 7)) << 2) + (c & 1) * 2 + t;
+                  const int at = (in >> 2) * 256 + place(in & 3) + t;
                   double u = static_cast<double>(tx[at]), y = 0.0;
                   if (kMode != kModeDpsgd) {
                     y = static_cast<double>(ty[at]);
@@ -265,87 +285,99 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
       }
       if (!kMany) {  // several steps write their results over the operands
         __syncwarp();
-        if (lane == 0 && last_of(in_done, 4) && slab + stride < whole) load_operands(slab + stride);
+        if (lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride);
       }
-      // Normals of workers q + 8 h, q + 8 h + 4 of both coordinates: lane q draws coordinate q % 2, quad q / 2 of the two, and
-      // entry s of what it gets in return is coordinate s % 2, quad s / 2.  All before the wait, where their registers allow it.
-      float v[kBlocks][4];
+      // Normals, all before the wait where their registers allow it.  Two coordinates: lane q draws coordinate q % 2, quad
+      // 2 h + q / 2, and entry s of what it gets in return is coordinate s % 2, quad 2 h + s / 2.  One: lane q draws quad 4 h + q.
+      constexpr int kDraws = V == 2 ? kBlocks : (R + 3) / 4;
+      float v[kDraws][4];
       auto draw = [&](int h) {
         v[h][0] = v[h][1] = v[h][2] = v[h][3] = 0.f;
         if (noisy) {
-          normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + (q & 1)), static_cast<uint32_t>(2 * h + (q >> 1)), t_noise, sigma, v[h]);
+          normal_quad(p.round_key, static_cast<unsigned long long>(p.coord_offset + j + (V == 2 ? q & 1 : 0)),
+                      static_cast<uint32_t>(V == 2 ? 2 * h + (q >> 1) : 4 * h + q), t_noise, sigma, v[h]);
           transpose_quad(v[h], q);
         }
       };
-      constexpr bool kDrawFirst = R <= 10;
+      auto normal = [&](int i, int t) { return V == 2 ? v[i >> 1][2 * (i & 1) + t] : v[i >> 2][i & 3]; };
+      constexpr bool kDrawFirst = R <= 10 || V == 1;
       if (kDrawFirst) {
 #pragma unroll
-        for (int h = 0; h < kBlocks; ++h) draw(h);
+        for (int h = 0; h < kDraws; ++h) draw(h);
       }
       if (kMode != kModeExternal && !ragged && step == 0) ok = bar_wait(tail_full, use & 1, limit);
       ok = __all_sync(0xffffffffu, ok) != 0;
       if (!ok) break;
-      // ---- element-wise tail, four elements at a time
+      // ---- element-wise tail, two elements at a time
 #pragma unroll
-      for (int h = 0; h < kBlocks; ++h) {
-        if (!kDrawFirst) draw(h);
+      for (int i = 0; i < R; i += 3 - V) {
+        if (!kDrawFirst && (i & 1) == 0) draw(i >> 1);
+        double sx[2], sy[2];
+        float nv[2] = {0.f, 0.f}, old[2] = {0.f, 0.f};
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int i = 2 * h + e;
-          if (i >= R) continue;
-          double sx[2] = {cx[h][0][e], cx[h][1][e]}, sy[2] = {cy[h][0][e], cy[h][1][e]};
-          float2 go, g = make_float2(0.f, 0.f);
-          if (!kEarly && kMode != kModeExternal) {
-            g = get(tg, i);
-            if (kMode == kModeDpsgd) {
-              sx[0] = fma(-alpha, static_cast<double>(g.x), sx[0]);
-              sx[1] = fma(-alpha, static_cast<double>(g.y), sx[1]);
-            } else {
-              sy[0] -= static_cast<double>(g.x);
-              sy[1] -= static_cast<double>(g.y);
-            }
-          }
-          const float2 xo = make_float2(static_cast<float>(sx[0]), static_cast<float>(sx[1]));  // x' (float64 sum, rounded once)
-          float2 yo = xo;
-          if (kMode == kModeExternal) {
-            go = get(ta, i);  // the gradient just folded becomes g_old
-            yo = make_float2(static_cast<float>(sy[0]), static_cast<float>(sy[1]));  // the gossiped tracker
+        for (int m = 0; m < 2; ++m) {
+          const int r = row_of(i, m), t = coord_of(m);
+          sx[m] = r < R ? cx[r >> 1][t][r & 1] : 0.0;
+          sy[m] = r < R ? cy[r >> 1][t][r & 1] : 0.0;
+          if (r < R) nv[m] = normal(r, t);
+          if (kAtStart && r < R) old[m] = x_old[kAtStart ? r : 0][t];
+        }
+        float2 go, g = make_float2(0.f, 0.f);
+        if (!kEarly && kMode != kModeExternal) {
+          g = get(tg, i);
+          if (kMode == kModeDpsgd) {
+            sx[0] = fma(-alpha, static_cast<double>(g.x), sx[0]);
+            sx[1] = fma(-alpha, static_cast<double>(g.y), sx[1]);
           } else {
-            const float2 a = get(ta, i), cc = get(tc, i);
-            if (kWide) {
-              go.x = static_cast<float>(fma(static_cast<double>(a.x), sx[0] - static_cast<double>(cc.x), static_cast<double>(v[h][2 * e])));
-              go.y = static_cast<float>(fma(static_cast<double>(a.y), sx[1] - static_cast<double>(cc.y), static_cast<double>(v[h][2 * e + 1])));
-            } else {
-              const float2 at = kAtStart ? x_old[kAtStart ? i : 0] : xo;  // stochastic gradient
-              unpack2(fma2(pack2(a.x, a.y), sub2(pack2(at.x, at.y), pack2(cc.x, cc.y)), pack2(v[h][2 * e], v[h][2 * e + 1])), go.x, go.y);
-            }
-            if (kMode == kModeDetag)  // fold: (y~ - g) + g', g' as stored
-              yo = make_float2(static_cast<float>(sy[0] + static_cast<double>(go.x)), static_cast<float>(sy[1] + static_cast<double>(go.y)));
+            sy[0] -= static_cast<double>(g.x);
+            sy[1] -= static_cast<double>(g.y);
           }
-          if (!kMany && kMode != kModeDpsgd && p.y_obs != nullptr && q + 4 * i < n && inside) {  // optional observer: the gossiped tracker
-            const long long at = (q + 4 * i) * p.ld + j;
-            if (kMode == kModeDetag && kEarly) g = make_float2(p.g[at], both_inside ? p.g[at + 1] : 0.f);  // not yet stored over
-            p.y_obs[at] = static_cast<float>(sy[0] + static_cast<double>(g.x));
-            if (both_inside) p.y_obs[at + 1] = static_cast<float>(sy[1] + static_cast<double>(g.y));
+        }
+        const float2 xo = make_float2(static_cast<float>(sx[0]), static_cast<float>(sx[1]));  // x' (float64 sum, rounded once)
+        float2 yo = xo;
+        if (kMode == kModeExternal) {
+          go = get(ta, i);  // the gradient just folded becomes g_old
+          yo = make_float2(static_cast<float>(sy[0]), static_cast<float>(sy[1]));  // the gossiped tracker
+        } else {
+          const float2 a = get(ta, i), cc = get(tc, i);
+          if (kWide) {
+            go.x = static_cast<float>(fma(static_cast<double>(a.x), sx[0] - static_cast<double>(cc.x), static_cast<double>(nv[0])));
+            go.y = static_cast<float>(fma(static_cast<double>(a.y), sx[1] - static_cast<double>(cc.y), static_cast<double>(nv[1])));
+          } else {
+            const F2 at = kAtStart ? pack2(old[0], old[1]) : pack2(xo.x, xo.y);  // stochastic gradient
+            unpack2(fma2(pack2(a.x, a.y), sub2(at, pack2(cc.x, cc.y)), pack2(nv[0], nv[1])), go.x, go.y);
           }
-          if (!final_step) {
-            put(tg, i, go);
-            put(tx, i, xo);
-            put(ty, i, yo);
-          } else if (!ragged) {
-            put(t_gout, i, go);
-            put(ta, i, xo);
-            if (kMode != kModeDpsgd) put(tc, i, yo);
-          } else if (q + 4 * i < n && inside) {
-            const long long at = (q + 4 * i) * p.ld + j;
-            p.g[at] = go.x;
-            p.x[at] = xo.x;
-            if (kMode != kModeDpsgd) p.y[at] = yo.x;
-            if (both_inside) {
-              p.g[at + 1] = go.y;
-              p.x[at + 1] = xo.y;
-              if (kMode != kModeDpsgd) p.y[at + 1] = yo.y;
-            }
+          if (kMode == kModeDetag)  // fold: (y~ - g) + g', g' as stored
+            yo = make_float2(static_cast<float>(sy[0] + static_cast<double>(go.x)), static_cast<float>(sy[1] + static_cast<double>(go.y)));
+        }
+        if (!kMany && kMode != kModeDpsgd && p.y_obs != nullptr) {  // optional observer: the gossiped tracker
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const int row = q + 4 * row_of(i, m);
+            const long long at = row * p.ld + j + coord_of(m);
+            if (row_of(i, m) >= R || row >= n || j + coord_of(m) >= p.d) continue;
+            // g: where the products have taken it in already it is still in global memory, not yet stored over
+            const float old_g = kMode == kModeDetag && kEarly ? p.g[at] : m == 0 ? g.x : g.y;
+            p.y_obs[at] = static_cast<float>(sy[m] + static_cast<double>(old_g));
+          }
+        }
+        if (!final_step) {
+          put(tg, i, go);
+          put(tx, i, xo);
+          put(ty, i, yo);
+        } else if (!ragged) {
+          put(t_gout, i, go);
+          put(ta, i, xo);
+          if (kMode != kModeDpsgd) put(tc, i, yo);
+        } else {
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const int row = q + 4 * row_of(i, m);
+            const long long at = row * p.ld + j + coord_of(m);
+            if (row_of(i, m) >= R || row >= n || j + coord_of(m) >= p.d) continue;
+            p.g[at] = m == 0 ? go.x : go.y;
+            p.x[at] = m == 0 ? xo.x : xo.y;
+            if (kMode != kModeDpsgd) p.y[at] = m == 0 ? yo.x : yo.y;
           }
         }
       }
@@ -353,12 +385,12 @@ __global__ void __launch_bounds__(dense_groups(R) * 128, 1) step_dense_kernel(co
     if (!ok) break;
     if (kMany) {
       __syncwarp();
-      if (lane == 0 && last_of(in_done, 4) && slab + stride < whole) load_operands(slab + stride);
+      if (lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride);
     }
     if (!ragged) {
       fence_async_shared();  // results visible to the TMA stores
       __syncwarp();
-      if (lane == 0 && last_of(tail_done, 4)) {
+      if (lane == 0 && last_of(tail_done, kWarps)) {
         rows_store(&maps.g, 2 * slab, 0, t_gout);
         rows_store(&maps.x, 2 * slab, 0, ta);
         if (kMode != kModeDpsgd) rows_store(&maps.y, 2 * slab, 0, tc);
@@ -382,7 +414,7 @@ int launch_kernel(DenseKernel kernel, const StepParams& p, const TensorMapSet& m
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), dense_smem_bytes(R));
   if (e != 0) return e;
   const long long slabs = (p.d + kDS - 1) / kDS, grid = slabs < sm_count ? slabs : sm_count;
-  return launch_chained(kernel, static_cast<unsigned>(grid), dense_groups(R) * 128, dense_smem_bytes(R), stream, p, *reinterpret_cast<const DenseMaps*>(maps.bytes));
+  return launch_chained(kernel, static_cast<unsigned>(grid), dense_threads(R), dense_smem_bytes(R), stream, p, *reinterpret_cast<const DenseMaps*>(maps.bytes));
 }
 
 template <int R>
