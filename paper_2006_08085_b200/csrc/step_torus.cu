@@ -167,28 +167,34 @@ __device__ __forceinline__ void torus_finish(const double (&acc)[R][2], int e, d
 }
 
 
-// Gradient phase of a lane: g' = a (x_at - c) + sigma xi for its 2R elements (element (r, e) at off + r * 512 + e * 256),
-// written over c in the stage (c is not needed again; the tracker phase picks g' up from there).  x_at: the model
-// at which the gradient is taken.  Noise: the lane's workers 8 r + 4 e + kq are position kq of the Philox quads
+// sigma times the normals of a lane's 2R elements.  The lane's workers 8 r + 4 e + kq are position kq of the Philox quads
 // 2 r + e, which the four lanes of a coordinate share: each draws every fourth quad (all four normals of it) and a
 // 4 x 4 transpose over the lanes hands everybody its own position.
 template <int R>
-__device__ __forceinline__ void torus_gradient(const StepParams& p, const float* sa, float* sc, int off,
-                                               const float (&x_at)[2][R], int kq, long long j, float sigma, bool noisy) {
-  unsigned long long jn = static_cast<unsigned long long>(p.coord_offset + j);
+__device__ __forceinline__ void torus_normals(const StepParams& p, int kq, long long j, float sigma, bool noisy, float (&xi)[R / 2][4]) {
+  const unsigned long long jn = static_cast<unsigned long long>(p.coord_offset + j);
 #pragma unroll
   for (int t = 0; t < R / 2; ++t) {  // quads 4 t .. 4 t + 3: blocks r = 2 t, 2 t + 1
-    float xi[4] = {0.f, 0.f, 0.f, 0.f};
+    xi[t][0] = xi[t][1] = xi[t][2] = xi[t][3] = 0.f;
     if (noisy) {
-      normal_quad(p.round_key, jn, static_cast<uint32_t>(4 * t + kq), p.t_noise, sigma, xi);
-      transpose_quad(xi, kq);  // xi[i]: this lane's position of quad 4 t + i, i.e. r = 2 t + (i >> 1), e = i & 1
+      normal_quad(p.round_key, jn, static_cast<uint32_t>(4 * t + kq), p.t_noise, sigma, xi[t]);
+      transpose_quad(xi[t], kq);  // xi[t][i]: this lane's position of quad 4 t + i, i.e. r = 2 t + (i >> 1), e = i & 1
     }
+  }
+}
+
+// Gradient phase of a lane: g' = a (x_at - c) + sigma xi for its 2R elements (element (r, e) at off + r * 512 + e * 256),
+// written over c in the stage (c is not needed again; the tracker phase picks g' up from there).  x_at: the model
+// at which the gradient is taken.
+template <int R>
+__device__ __forceinline__ void torus_gradient(const float* sa, float* sc, int off, const float (&x_at)[2][R], const float (&xi)[R / 2][4]) {
+#pragma unroll
+  for (int t = 0; t < R / 2; ++t)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = 2 * t + (i >> 1), e = i & 1, o = off + r * 512 + e * 256;
-      sc[o] = fmaf(sa[o], x_at[e][r] - sc[o], xi[i]);
+      sc[o] = fmaf(sa[o], x_at[e][r] - sc[o], xi[t][i]);
     }
-  }
 }
 
 template <int R, bool kAtStart>
@@ -383,6 +389,10 @@ step_torus_kernel(const StepParams p, const __grid_constant__ TorusMaps maps, co
         for (int r = 0; r < R; ++r) xv[e][r] = static_cast<float>(out[r]);  // rounded once
       }
     }
+    // The normals need no data: drawn while g, a, c may still be on their way (8 x 8, d = 100 k 50.0 -> 44.6 us, d = 11.2 M 4243 ->
+    // 4226) - but with the printed timing, whose tail holds the old model too, only after (d = 2 M 776 us, before the wait 782).
+    float xi[R / 2][4];
+    if (!kAtStart) torus_normals<R>(p, kq, j, sigma, noisy, xi);
     // g, a, c are needed from here on; their loads had the model contraction to arrive in
     if (lane == 0) {
       // The stage last held slab k - 3, which belongs to the other group (odd stage count): a parity wait must not
@@ -408,15 +418,16 @@ step_torus_kernel(const StepParams p, const __grid_constant__ TorusMaps maps, co
         }
     }
     if (active) {
+      if (kAtStart) torus_normals<R>(p, kq, j, sigma, noisy, xi);
       if (kAtStart) {  // Algorithm 2 as printed: the gradient at the model the step started from (still staged)
         float xold[2][R];
 #pragma unroll
         for (int e = 0; e < 2; ++e)
 #pragma unroll
           for (int r = 0; r < R; ++r) xold[e][r] = sxp[off + r * 512 + e * 256];
-        torus_gradient<R>(p, sa, sc, off, xold, kq, j, sigma, noisy);
+        torus_gradient<R>(sa, sc, off, xold, xi);
       } else {
-        torus_gradient<R>(p, sa, sc, off, xv, kq, j, sigma, noisy);
+        torus_gradient<R>(sa, sc, off, xv, xi);
       }
 #pragma unroll
       for (int e = 0; e < 2; ++e)
