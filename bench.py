@@ -38,21 +38,21 @@ BYTES_PER_WC = 32  # read x, y, g, a, c + write x, y, g, float32 each: the fused
 # small case of the same kernel; traffic grows in proportion to n*d).  Keyed by the sha256 prefix of the kernel
 # sources the capture was taken on: a changed kernel reports null until it is captured again.
 KERNEL_SOURCES = {
-    "small": ("step_small.cu", "noise.cuh", "packed.cuh", "pipeline.cuh"),
-    "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh"),
-    "dense": ("step_dense.cu", "pipeline.cuh", "noise.cuh", "packed.cuh"),
-    "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh", "packed.cuh"),
-    "csr": ("step_csr.cu", "noise.cuh", "packed.cuh"),
-    "torus": ("step_torus.cu", "torus_basis.h", "pipeline.cuh", "noise.cuh", "packed.cuh"),
+    "small": ("step_small.cu", "noise.cuh", "packed.cuh", "pipeline.cuh", "chain.cuh"),
+    "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
+    "dense": ("step_dense.cu", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
+    "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
+    "csr": ("step_csr.cu", "noise.cuh", "packed.cuh", "chain.cuh"),
+    "torus": ("step_torus.cu", "torus_basis.h", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
 }
 MEASURED_TRAFFIC = {
     # (kernel, mode): (source digest, bytes per wc)
-    ("small", "column"): ("2d293cc7edde3135", 29.00),   # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1440 GB written / 16 M wc
-    ("dense", "product"): ("98fc5c149709161c", 31.37),     # cfg5 shape at d = 2 M: 1.2899 + 0.7176 GB / 64 M wc
-    ("torus", "torus8"): ("22f3bc13d621a2ed", 31.26),  # cfg3 shape at d = 1 M: 1.2801 + 0.7204 GB / 64 M wc
-    ("ring", "band"): ("1a16972a0d29d375", 31.09),     # cfg4 shape at d = 200 k: 1.0279 + 0.5637 GB / 51.2 M wc
-    ("split", "digits"): ("b1eb219985913d27", 30.81),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4321 GB / 40 M wc
-    ("csr", "rounds"): ("bd6f6c1d0ef487a7", 31.16),     # the same graph through the rounds kernel: 0.8089 + 0.4374 GB / 40 M wc
+    ("small", "column"): ("26f1b4f3eccbed2b", 28.81),  # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1410 GB written / 16 M wc
+    ("dense", "product"): ("070f126e2d58dbf8", 31.22),  # cfg5 shape at d = 2 M: 1.2802 + 0.7177 GB / 64 M wc
+    ("torus", "torus8"): ("4ccde3daf94c6d39", 31.24),  # cfg3 shape at d = 1 M: 1.2801 + 0.7193 GB / 64 M wc
+    ("ring", "band"): ("a9f574115be24d04", 31.08),  # cfg4 shape at d = 200 k: 1.0275 + 0.5641 GB / 51.2 M wc
+    ("split", "digits"): ("70667638fd698bcb", 30.80),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4315 GB / 40 M wc
+    ("csr", "rounds"): ("b8924f0a1b9a670d", 30.67),  # 300-worker random graph at d = 100 k: 0.6017 + 0.3183 GB / 30 M wc
 }
 
 # Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes) and that

@@ -314,7 +314,7 @@ bool dense_ok(const detag_state* s) {
 // Host cost model.  The product with the polynomial beats the sparse rounds wherever a kernel takes it: K rounds cost
 // K * (nnz per row) shared-memory gathers of 16 bytes per element and array and two barriers each.  Tori of 8-worker blocks
 // take the transform kernel (24 multiply-adds per element and array).  Caller-written gradients run on the dense kernels
-// for n <= 32 and on the rounds kernel otherwise.
+// for n <= 48 (under the rounds' name beyond 32) and on the rounds kernel otherwise.
 bool variant_runs_mode(const detag_state* s, int variant) {
   if (step_mode(s) == detag::kModeDetag) return true;
   if (variant == DETAG_VARIANT_RING) return step_mode(s) == detag::kModeDpsgd;
