@@ -133,7 +133,7 @@ struct SplitPlan {
 };
 
 // Shared memory: x, y of a slab (whole blocks of 32 rows) | blocks of P | g, a, c stages | groups of the guard | row
-// scales, scales, flags, maxima | barriers.
+// scales, scales, flags, maxima (two splitting groups only) | barriers.
 inline SplitPlan plan_for(int nb, int num_blocks, int guard_entries, int groups, int stages) {
   SplitPlan s{};
   s.groups = groups;
@@ -142,7 +142,7 @@ inline SplitPlan plan_for(int nb, int num_blocks, int guard_entries, int groups,
   s.e_at = s.blocks_at + static_cast<size_t>(num_blocks) * kPBlockBytes;
   s.guard_at = s.e_at + static_cast<size_t>(groups) * stages * kPStageBytes;
   s.scale_at = s.guard_at + static_cast<size_t>(guard_entries + 3) / 4 * 16;
-  s.ctrl_at = s.scale_at + 256 * 8 + kPScaleSlots * 128 * 2 + kPScaleSlots * 4 * 4 + 4 * 128 * 8;
+  s.ctrl_at = s.scale_at + 256 * 8 + kPScaleSlots * 128 * 2 + kPScaleSlots * 4 * 4 + (nb <= 4 ? 4 * 128 * 8 : 0);
   s.bytes = s.ctrl_at + kPCtrlBytes;
   return s;
 }
