@@ -159,7 +159,9 @@ int detag_get_variant(const detag_state* s, int* variant);
  * the phase started from, and folds g_(k) - g_(k-1) into the tracker at the end of the phase; its
  * gradients are therefore one phase older than with the default, which evaluates at the new model:
  *     g'  = a o (x - c) + sigma * xi     (x = the model before this step's update)
- * Everything else in the step listing at the top is unchanged, and so is detag_init.  Errors: ARG.
+ * Everything else in the step listing at the top is unchanged, and so is detag_init.  It holds for D-PSGD
+ * steps too (a step then moves along the gradient at the model before the one it starts from), with every
+ * kernel and any number of coordinates; caller-written gradients do not use it.  Errors: ARG.
  */
 int detag_set_gradient_point(detag_state* s, int where);
 int detag_get_gradient_point(const detag_state* s, int* where);
@@ -169,7 +171,8 @@ int detag_get_gradient_point(const detag_state* s, int* where);
  * every worker averages its neighbours' models with the gossip matrix and takes a step along its own
  * stochastic gradient).  With DETAG_ALGORITHM_DPSGD a step is
  *     x'  = AG_K(x) - alpha * g          (plain D-PSGD is K = 1, eta = 0: x' = M x - alpha g)
- *     g'  = a o (x' - c) + sigma * xi    (the gradient the NEXT step uses, evaluated at the new model)
+ *     g'  = a o (x' - c) + sigma * xi    (the gradient the NEXT step uses, evaluated at the new model, or where
+ *                                         detag_set_gradient_point says)
  * on the same kernels, with one contraction and no tracker: the y buffer is neither read nor written, and
  * 24 bytes per worker-coordinate cross HBM instead of 32.  detag_init then sets g = gradient at the bound x only.
  * Synthetic gradient only.  Errors: ARG, UNSUPPORTED (combined with caller-written gradients).

@@ -479,7 +479,7 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   if (dense_step_ok(s, p, variant)) {
     const detag::TensorMapSet* maps = maps_for(s, kFamilyDense, p);
     if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
-    e = detag::launch_step_dense(p, *maps, variant == DETAG_VARIANT_CSR && p.mode == detag::kModeDpsgd, s->sm_count, stream);
+    e = detag::launch_step_dense(p, *maps, s->sm_count, stream);
     return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
   }
   if (split_ok(s, p, variant)) return launch_split(s, p, variant == DETAG_VARIANT_CSR, stream);

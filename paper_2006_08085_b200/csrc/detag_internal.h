@@ -15,8 +15,8 @@ namespace detag {
 
 constexpr int kMaxWorkers = 1024;       // detag_create limit on n
 constexpr int kMaxDenseWorkers = 128;   // dense variant: limit on n
-constexpr int kMaxSmallWorkers = 16;    // one thread per coordinate: limit on n
-constexpr int kMaxDenseStepWorkers = 48;  // dense product, a warp on its own: limit on n
+constexpr int kMaxSmallWorkers = 16;    // step in registers: limit on n
+constexpr int kMaxDenseStepWorkers = 48;  // dense product, groups of warps: limit on n
 constexpr int kMaxSplitWorkers = 256;   // integer tensor path: limit on n
 constexpr int kMaxPartials = 2048;      // per-CTA partial sums of the consensus-error reduction
 constexpr size_t kWsAlign = 256;
@@ -111,11 +111,11 @@ bool torus_variant_available(int n);               // block-circulant kernel: n 
 bool build_maps_torus(const StepParams& p, TensorMapSet* maps);
 int launch_step_torus(StepParams p, const TensorMapSet& maps, const double* phat_frag /* device */, int sm_count,
                       cudaStream_t stream);
-// one thread per coordinate (step_small.cu): n <= 16, all modes; p.steps iterations
+// the step in registers (step_small.cu): n <= 16, all modes; p.steps iterations
 int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
-// dense product, every warp on its own (step_dense.cu): 16 < n <= 48, all modes; wide: D-PSGD's gradient in float64
+// dense product, groups of warps with a slab each (step_dense.cu): 16 < n <= 48, all modes
 bool build_maps_dense(const StepParams& p, TensorMapSet* maps);
-int launch_step_dense(const StepParams& p, const TensorMapSet& maps, bool wide, int sm_count, cudaStream_t stream);
+int launch_step_dense(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);
 int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);  // n <= 32, p.steps steps
 // polynomial on the integer tensor path (step_split.cu): 32 < n <= 256, DeTAG and D-PSGD steps
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);

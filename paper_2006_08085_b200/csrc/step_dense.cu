@@ -341,8 +341,8 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
         } else {
           const float2 a = get(ta, i), cc = get(tc, i);
           if (kWide) {
-            go.x = static_cast<float>(fma(static_cast<double>(a.x), sx[0] - static_cast<double>(cc.x), static_cast<double>(nv[0])));
-            go.y = static_cast<float>(fma(static_cast<double>(a.y), sx[1] - static_cast<double>(cc.y), static_cast<double>(nv[1])));
+            go.x = static_cast<float>(fma(static_cast<double>(a.x), (kAtStart ? static_cast<double>(old[0]) : sx[0]) - static_cast<double>(cc.x), static_cast<double>(nv[0])));
+            go.y = static_cast<float>(fma(static_cast<double>(a.y), (kAtStart ? static_cast<double>(old[1]) : sx[1]) - static_cast<double>(cc.y), static_cast<double>(nv[1])));
           } else {
             const F2 at = kAtStart ? pack2(old[0], old[1]) : pack2(xo.x, xo.y);  // stochastic gradient
             unpack2(fma2(pack2(a.x, a.y), sub2(at, pack2(cc.x, cc.y)), pack2(nv[0], nv[1])), go.x, go.y);
@@ -418,11 +418,13 @@ int launch_kernel(DenseKernel kernel, const StepParams& p, const TensorMapSet& m
 }
 
 template <int R>
-int launch_dense(const StepParams& p, const TensorMapSet& maps, bool wide, int sm_count, cudaStream_t stream) {
-  const DenseKernel kernel = p.mode == kModeExternal ? step_dense_kernel<R, kModeExternal, false, false>
-                             : p.mode == kModeDpsgd  ? (wide ? step_dense_kernel<R, kModeDpsgd, false, (R > 8)> : step_dense_kernel<R, kModeDpsgd, false, false>)
-                             : p.grad_at_start       ? step_dense_kernel<R, kModeDetag, true, false>
-                                                     : step_dense_kernel<R, kModeDetag, false, false>;
+int launch_dense(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream) {
+  DenseKernel kernel = step_dense_kernel<R, kModeExternal, false, false>;
+  if (p.mode == kModeDpsgd) {  // beyond 32 workers it goes by the rounds' name and has their gradient in float64
+    kernel = p.grad_at_start ? step_dense_kernel<R, kModeDpsgd, true, (R > 8)> : step_dense_kernel<R, kModeDpsgd, false, (R > 8)>;
+  } else if (p.mode == kModeDetag) {
+    kernel = p.grad_at_start ? step_dense_kernel<R, kModeDetag, true, false> : step_dense_kernel<R, kModeDetag, false, false>;
+  }
   return launch_kernel<R>(kernel, p, maps, sm_count, stream);
 }
 
@@ -455,18 +457,17 @@ int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm
   }
 }
 
-int launch_step_dense(const StepParams& p, const TensorMapSet& maps, bool wide, int sm_count, cudaStream_t stream) {
-  if (p.n <= kMaxSmallWorkers || p.n > kMaxDenseStepWorkers || p.d <= 0 || p.d > 0x7fffffffLL || (wide && (p.mode != kModeDpsgd || p.n <= 32)))
-    return static_cast<int>(cudaErrorInvalidValue);
+int launch_step_dense(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream) {
+  if (p.n <= kMaxSmallWorkers || p.n > kMaxDenseStepWorkers || p.d <= 0 || p.d > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidValue);
   switch ((p.n + 3) / 4) {
-    case 5: return launch_dense<5>(p, maps, wide, sm_count, stream);
-    case 6: return launch_dense<6>(p, maps, wide, sm_count, stream);
-    case 7: return launch_dense<7>(p, maps, wide, sm_count, stream);
-    case 8: return launch_dense<8>(p, maps, wide, sm_count, stream);
-    case 9: return launch_dense<9>(p, maps, wide, sm_count, stream);
-    case 10: return launch_dense<10>(p, maps, wide, sm_count, stream);
-    case 11: return launch_dense<11>(p, maps, wide, sm_count, stream);
-    default: return launch_dense<12>(p, maps, wide, sm_count, stream);
+    case 5: return launch_dense<5>(p, maps, sm_count, stream);
+    case 6: return launch_dense<6>(p, maps, sm_count, stream);
+    case 7: return launch_dense<7>(p, maps, sm_count, stream);
+    case 8: return launch_dense<8>(p, maps, sm_count, stream);
+    case 9: return launch_dense<9>(p, maps, sm_count, stream);
+    case 10: return launch_dense<10>(p, maps, sm_count, stream);
+    case 11: return launch_dense<11>(p, maps, sm_count, stream);
+    default: return launch_dense<12>(p, maps, sm_count, stream);
   }
 }
 

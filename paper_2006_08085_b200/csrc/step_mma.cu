@@ -248,7 +248,7 @@ typedef void (*MmaKernel)(const StepParams, const MmaMaps);
 
 MmaKernel pick_mode(const StepParams& p) {
   if (p.mode == kModeExternal) return step_mma_kernel<kModeExternal, false>;
-  if (p.mode == kModeDpsgd) return step_mma_kernel<kModeDpsgd, false>;
+  if (p.mode == kModeDpsgd) return p.grad_at_start ? step_mma_kernel<kModeDpsgd, true> : step_mma_kernel<kModeDpsgd, false>;
   return p.grad_at_start ? step_mma_kernel<kModeDetag, true> : step_mma_kernel<kModeDetag, false>;
 }
 

@@ -205,7 +205,7 @@ typedef void (*SmallKernel)(const StepParams);
 template <int R, bool kFull>
 SmallKernel pick_small(const StepParams& p) {
   if (p.mode == kModeExternal) return step_small_kernel<R, kFull, 4, kModeExternal, false, false>;
-  if (p.mode == kModeDpsgd) return step_small_kernel<R, kFull, 4, kModeDpsgd, false, false>;
+  if (p.mode == kModeDpsgd) return p.grad_at_start ? step_small_kernel<R, kFull, 4, kModeDpsgd, true, false> : step_small_kernel<R, kFull, 4, kModeDpsgd, false, false>;
   return p.grad_at_start ? step_small_kernel<R, kFull, 4, kModeDetag, true, false> : step_small_kernel<R, kFull, 4, kModeDetag, false, false>;
 }
 

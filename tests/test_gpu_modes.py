@@ -204,3 +204,35 @@ def test_dpsgd_fused_call_and_host_resident_stepping_agree_with_single_steps():
             out.append((s.download("x"), s.download("g")))
     for k in (1, 2):
         assert np.array_equal(out[0][0], out[k][0]) and np.array_equal(out[0][1], out[k][1])
+
+
+# a worker count, length and variant for every kernel; (16, .., stalled far away): the kernel with padded tiles
+@pytest.mark.parametrize("n,d,K,kind,variant", [
+    (3, 37, 2, "path", B.DETAG_VARIANT_AUTO), (13, 5003, 2, "ring", B.DETAG_VARIANT_AUTO),
+    (16, 1025, 2, "ring", "padded"), (17, 700, 3, "regular4", B.DETAG_VARIANT_AUTO),
+    (32, 9602, 3, "regular4", B.DETAG_VARIANT_AUTO), (33, 130, 3, "regular4", B.DETAG_VARIANT_AUTO),
+    (40, 20_001, 2, "regular4", B.DETAG_VARIANT_AUTO), (48, 9400, 3, "regular4", B.DETAG_VARIANT_AUTO),
+    (48, 9600, 3, "regular4", B.DETAG_VARIANT_AUTO), (40, 301, 2, "regular4", B.DETAG_VARIANT_CSR),
+    (100, 1030, 4, "regular4", B.DETAG_VARIANT_AUTO), (96, 130, 4, "ring", B.DETAG_VARIANT_RING),
+    (96, 9602, 30, "ring", B.DETAG_VARIANT_RING), (96, 70, 4, "ring", B.DETAG_VARIANT_CSR)])
+@pytest.mark.parametrize("where", [B.DETAG_GRADIENT_AT_NEW_MODEL, B.DETAG_GRADIENT_AT_PHASE_START])
+def test_dpsgd_gradient_point(n, d, K, kind, variant, where):
+    """The gradient point holds for D-PSGD too, on every kernel and at every length."""
+    rng = np.random.default_rng(n * 19 + d)
+    m = _graph(kind, n)
+    a, c = _objective(rng, n, d)
+    x, g = (rng.standard_normal((n, d)).astype(np.float32) for _ in range(2))
+    p = oracle_problem(m, K, 0.2, 0.05, a, c, 0.1, 13, 77)
+    with Session(m, d, K, 0.2, 0.05, a, c, x, 0.1, 13, coord_offset=77, gradient_point=where,
+                 variant=B.DETAG_VARIANT_DENSE if variant == "padded" else variant,
+                 algorithm=B.DETAG_ALGORITHM_DPSGD) as s:
+        s.upload("g", g)
+        if variant == "padded":
+            B.detag_debug_inject_stall(s.state, 1 << 40, 1 << 20)  # never reached
+        B.detag_set_step(s.state, 0)
+        s.step()
+        s.status()
+        want = orc.dpsgd_step(p, orc.DpsgdState(x.astype(np.float64), g.astype(np.float64), 0))
+        assert worst_ratio(s.download("x"), want.x) <= 1.0
+        at = x.astype(np.float64) if where == B.DETAG_GRADIENT_AT_PHASE_START else want.x
+        assert worst_ratio(s.download("g"), orc.stochastic_gradient(p, at, 1)) <= 1.0
