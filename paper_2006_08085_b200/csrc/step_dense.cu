@@ -383,13 +383,12 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
       }
     }
     if (!ok) break;
-    if (kMany) {
-      __syncwarp();
-      if (lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride);
-    }
+    // What was written here comes before what the TMA does next: the results before their stores and, of several steps, the
+    // intermediate ones before the next operands that are loaded over them.
+    fence_async_shared();
+    __syncwarp();
+    if (kMany && lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride);
     if (!ragged) {
-      fence_async_shared();  // results visible to the TMA stores
-      __syncwarp();
       if (lane == 0 && last_of(tail_done, kWarps)) {
         rows_store(&maps.g, 2 * slab, 0, t_gout);
         rows_store(&maps.x, 2 * slab, 0, ta);

@@ -49,6 +49,15 @@ def test_fused_steps_equal_single_steps_bit_for_bit(n, d, K, count, where):
         assert np.array_equal(got[0][k], got[1][k]), k
 
 
+@pytest.mark.parametrize("n,d,count", [
+    (25, 9001, 3), (28, 18_944, 2), (32, 257, 4),              # padded tiles where single steps run by groups of warps
+    (17, 9001, 3), (23, 20_003, 3), (28, 20_003, 3),           # groups of warps, 5, 6 and 7 workers per lane
+    (20, 64 * 148 * 9 + 35, 3), (32, 64 * 148 * 9 + 35, 2)])   # several slabs per group, loaded over the last one's steps
+@pytest.mark.parametrize("where", [B.DETAG_GRADIENT_AT_NEW_MODEL, B.DETAG_GRADIENT_AT_PHASE_START])
+def test_fused_steps_of_17_to_32_workers(n, d, count, where):
+    test_fused_steps_equal_single_steps_bit_for_bit(n, d, 3, count, where)
+
+
 def test_fused_trajectory_against_the_oracle():
     n, d, K, steps = 16, 3_001, 4, 12
     m, eta, a, c, x0 = _case(n, d, 5)
