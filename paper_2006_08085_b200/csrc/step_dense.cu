@@ -201,7 +201,8 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
       take(tg, p.g);
       take(ta, kMode == kModeExternal ? p.g_ext : p.a);
       if (kMode != kModeExternal) take(tc, p.c);
-      asm volatile("cp.async.wait_all;" ::: "memory");  // every lane reads its own
+      asm volatile("cp.async.wait_all;" ::: "memory");  // every lane reads its own,
+      if (R > 8) __syncwarp();                          // and the other lanes' where a sum is not finite
     }
 #pragma unroll 1
     for (int step = 0; step < (kMany ? p.steps : 1); ++step) {

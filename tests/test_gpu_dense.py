@@ -90,6 +90,32 @@ def test_what_is_not_finite_reaches_those_that_hear_of_it(n, bad, mode):
     assert finite[:, np.setdiff1d(np.arange(d), cols)].all()
 
 
+@pytest.mark.parametrize("n,d", [(33, 61), (44, 64 * 444 + 61), (48, 3)])
+@pytest.mark.parametrize("mode", ["new", "external", "dpsgd"])
+def test_what_is_not_finite_in_a_ragged_slab(n, d, mode):
+    """The first slab of its group and a later one; one worker's model is infinite in every column, and the workers that do not
+    hear of it get what they get without it."""
+    m = inputs.metropolis_weights(inputs.ring_graph(n))
+    K, cols = 2, np.arange(d // 64 * 64, d)
+    rng = np.random.default_rng(n + d)
+    arrays = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c", "g_new")}
+    got = []
+    for bad in (False, True):
+        with Session(m, d, K, 0.2, 0.05, sigma=0.1, seed=3, external_gradient=mode == "external", algorithm=int(mode == "dpsgd")) as s:
+            for k, v in arrays.items():
+                if getattr(s, k) is not None:
+                    s.upload(k, v)
+            if bad:
+                s.x[cols % n, cols] = float("inf")
+            B.detag_set_step(s.state, 0)
+            s.step()
+            s.status()
+            got.append(s.download("x")[:, cols])
+    hears = np.abs((np.arange(n)[:, None] - cols[None, :] % n + n // 2) % n - n // 2) <= K
+    assert np.array_equal(np.isfinite(got[1]), ~hears)
+    assert worst_ratio(got[1][~hears], got[0][~hears].astype(np.float64)) <= 1.0
+
+
 def _runs(cols):
     ends = np.flatnonzero(np.diff(cols) != 1)
     return [(int(cols[a]), int(cols[b]) + 1) for a, b in zip(np.r_[0, ends + 1], np.r_[ends, len(cols) - 1])]
