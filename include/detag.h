@@ -319,7 +319,8 @@ int detag_status(detag_state* s, void* stream);
  * can be exercised without faulting, trapping or hanging the GPU.
  *
  * detag_debug_inject_stall: from now on the loading thread of every CTA of the tensor-path step kernels stops
- * issuing loads after `after_tiles` tiles, and every device-side wait gives up after `poll_limit` polls
+ * issuing loads after `after_tiles` tiles (where groups of warps load for themselves, 17 to 48 workers: the groups stop),
+ * and every device-side wait gives up after `poll_limit` polls
  * (16 .. 2^20; a poll suspends for at most about two microseconds).  The CTAs' waiters then time out one
  * after the other, set the status word and return; the launch ends normally and detag_status reports
  * DETAG_ERR_TIMEOUT.  The state arrays are left partly updated.  after_tiles < 0 restores normal operation

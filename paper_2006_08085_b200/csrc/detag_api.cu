@@ -460,7 +460,7 @@ bool small_ok(const StepParams& p) {
 // one per SM the integer path is ahead: 48, d = 9400 12.3 -> 13.9, d = 18000 16.4 -> 14.4 (40, d = 9400: 12.3 both).  The length is the
 // state's, not a staged chunk's: host-resident stepping gives the same bits.
 bool dense_step_ok(const detag_state* s, const StepParams& p, int variant) {
-  if (p.n <= detag::kMaxSmallWorkers || p.n > detag::kMaxDenseStepWorkers || p.stall_after >= 0 || p.poly == nullptr || p.d > 0x7fffffffLL) return false;
+  if (p.n <= detag::kMaxSmallWorkers || p.n > detag::kMaxDenseStepWorkers || p.poly == nullptr || p.d > 0x7fffffffLL) return false;
   if (p.mode == detag::kModeExternal ? p.n > 24 && p.n <= 32 : p.n > 40 && s->d <= 64LL * s->sm_count) return false;
   return variant == DETAG_VARIANT_DENSE || (variant == DETAG_VARIANT_CSR && s->variant_forced == DETAG_VARIANT_AUTO);
 }
@@ -819,10 +819,9 @@ int detag_step_many(detag_state* s, int count, void* stream) {
   if (!s->bound) return fail(s, DETAG_ERR_UNBOUND, "detag_step_many before detag_bind");
   if (count >= 2 && step_mode(s) == detag::kModeExternal)
     return fail(s, DETAG_ERR_ARG, "detag_step_many: caller-written gradients need one call per step");
-  // the fused kernels exist for the dense polynomial with n <= 32; the observer wants every step's tracker, the
-  // failure-detection self test the kernel with a loading thread
+  // the fused kernels exist for the dense polynomial with n <= 32; the observer wants every step's tracker
   if (count >= 2 && resolve_variant(s) == DETAG_VARIANT_DENSE && s->n <= 32 && s->y_obs == nullptr &&
-      step_mode(s) == detag::kModeDetag && s->stall_after < 0) {
+      step_mode(s) == detag::kModeDetag) {
     // A launch is cut off at kMaxFusedSteps so that no thread of the kernel waits on a peer for longer than its
     // bounded waits allow (a tile of 1024 steps takes some tens of milliseconds; the waits give up after seconds).
     constexpr int kMaxFusedSteps = 1024;
@@ -840,7 +839,8 @@ int detag_step_many(detag_state* s, int count, void* stream) {
         // while there are at most two slabs per SM.  us for ten steps, padded -> groups: 17 workers, d = 9000 26.6 -> 22.5,
         // d = 72 k 127 -> 71; 24, d = 9000 26.6 -> 23.9; 28, d = 18 k 39.0 -> 41.0, d = 36 k 68 -> 59; 32, d = 9000 26.6 -> 32.8, d = 18 k
         // 39 -> 43, d = 36 k 70 -> 66, d = 72 k 130 -> 128.
-        const bool padded = p.n > 24 && p.d <= 128LL * s->sm_count;
+        // (At most 16 get here for the self test of failure detection.)
+        const bool padded = p.n <= detag::kMaxSmallWorkers || (p.n > 24 && p.d <= 128LL * s->sm_count);
         const detag::TensorMapSet* maps = maps_for(s, padded ? kFamilyMma : kFamilyDense, p);
         if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
         e = padded ? detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream))

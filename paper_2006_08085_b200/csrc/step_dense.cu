@@ -51,8 +51,9 @@ __host__ __device__ constexpr int dense_threads(int R) { return dense_groups(R) 
 __host__ __device__ constexpr int dense_blocks(int R) { return (R + 1) / 2; }
 __host__ __device__ constexpr int dense_frag_bytes(int R) { return R * dense_blocks(R) * 32 * 8; }
 __host__ __device__ constexpr int dense_group_bytes(int R) { return (R <= 8 ? 6 : 5) * R * 1024; }
-// barriers, and slack to align the tiles to 1 KiB, at the end
+// barriers and counters, and slack to align the tiles to 1 KiB, at the end
 __host__ __device__ constexpr int dense_smem_bytes(int R) { return dense_groups(R) * dense_group_bytes(R) + dense_frag_bytes(R) + 128 + 1024; }
+static_assert(4 * (2 * 8 + 4 * 4) <= 128, "barrier area");
 static_assert(dense_smem_bytes(12) <= 232448 && dense_smem_bytes(8) <= 232448, "shared memory plan");
 
 struct DenseMaps {
@@ -93,8 +94,8 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
   double* const frag = reinterpret_cast<double*>(smem + kGroups * dense_group_bytes(R));  // [input step][output block][lane]
   uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + kGroups * dense_group_bytes(R) + dense_frag_bytes(R));
   uint64_t *const in_full = bars + 2 * group, *const tail_full = in_full + 1;
-  unsigned* const in_done = reinterpret_cast<unsigned*>(bars + 2 * kGroups) + 2 * group;
-  unsigned* const tail_done = in_done + 1;
+  unsigned* const in_done = reinterpret_cast<unsigned*>(bars + 2 * kGroups) + 4 * group;  // warps done, slabs asked for
+  unsigned *const tail_done = in_done + 1, *const in_asked = in_done + 2, *const tail_asked = in_done + 3;
   const int n = p.n;
   // operands x | y | (g), then what the results replace: (g -> g') | a -> x' | c -> y'; up to 32 workers g' has a place of its own
   float* const tx = tiles;
@@ -131,13 +132,20 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
   const int whole = static_cast<int>(p.d / kDS), slabs = static_cast<int>((p.d + kDS - 1) / kDS), stride = gridDim.x * kGroups;
   int slab = blockIdx.x + gridDim.x * group;
 
-  auto load_operands = [&](int s) {  // one thread
+  // Self test of failure detection: nothing is asked for beyond p.stall_after slabs of the block - in odd groups the inputs of
+  // the tail alone, so that both waits run out, the one with the next operands on their way.
+  auto withheld = [&](int k) { return p.stall_after >= 0 && group + static_cast<long long>(kGroups) * k >= p.stall_after; };
+  auto load_operands = [&](int s, int k) {  // one thread, for the group's k-th slab
+    if ((group & 1) == 0 && withheld(k)) return;
+    *in_asked = k + 1;
     bar_expect_tx(in_full, (1u + (kMode != kModeDpsgd) + kEarly) * kTileBytes);
     rows_load(tx, &maps.x, 2 * s, 0, in_full);
     if (kMode != kModeDpsgd) rows_load(ty, &maps.y, 2 * s, 0, in_full);
     if (kEarly) rows_load(tg, &maps.g, 2 * s, 0, in_full);
   };
-  auto load_tail = [&](int s) {
+  auto load_tail = [&](int s, int k) {
+    if (withheld(k)) return;
+    *tail_asked = k + 1;
     bar_expect_tx(tail_full, (1u + (kMode != kModeExternal) + !kEarly) * kTileBytes);
     if (!kEarly) rows_load(tg, &maps.g, 2 * s, 0, tail_full);
     rows_load(ta, &maps.a, 2 * s, 0, tail_full);
@@ -146,13 +154,13 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
   if (part == 0 && lane == 0) {
     bar_init(in_full, 1);
     bar_init(tail_full, 1);
-    *in_done = *tail_done = 0;
+    *in_done = *tail_done = *in_asked = *tail_asked = 0;
     fence_barrier_init();
     fence_async_shared();
     chain_wait();
     if (slab < whole) {
-      load_operands(slab);
-      load_tail(slab);
+      load_operands(slab, 0);
+      load_tail(slab, 0);
     }
   }
 #pragma unroll
@@ -174,7 +182,7 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
     if (owes) {
       store_wait_read();
       if (!ragged) {
-        load_tail(slab);
+        load_tail(slab, use);
       } else {
         bar_arrive(tail_full);
       }
@@ -286,7 +294,7 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
       }
       if (!kMany) {  // several steps write their results over the operands
         __syncwarp();
-        if (lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride);
+        if (lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride, use + 1);
       }
       // Normals, all before the wait where their registers allow it.  Two coordinates: lane q draws coordinate q % 2, quad
       // 2 h + q / 2, and entry s of what it gets in return is coordinate s % 2, quad 2 h + s / 2.  One: lane q draws quad 4 h + q.
@@ -388,7 +396,7 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
     // intermediate ones before the next operands that are loaded over them.
     fence_async_shared();
     __syncwarp();
-    if (kMany && lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride);
+    if (kMany && lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride, use + 1);
     if (!ragged) {
       if (lane == 0 && last_of(tail_done, kWarps)) {
         rows_store(&maps.g, 2 * slab, 0, t_gout);
@@ -399,10 +407,13 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
       }
     }
   }
-  if (!ok) {  // copies still in flight land in this CTA's shared memory: wait for them (bounded) before leaving
+  if (!ok) {
+    // Copies still in flight land in this CTA's shared memory: wait for the last that were asked for (bounded) before leaving.
+    // A warp that asks for more after this is still in its loop: it sees them land, or gets here itself.
     if (lane == 0) atomicExch(p.status, 1);
-    bar_wait(in_full, use & 1, limit);
-    bar_wait(tail_full, use & 1, limit);
+    const unsigned in = *const_cast<volatile unsigned*>(in_asked), tail = *const_cast<volatile unsigned*>(tail_asked);
+    if (in != 0) bar_wait(in_full, (in - 1) & 1, limit);
+    if (tail != 0) bar_wait(tail_full, (tail - 1) & 1, limit);
   }
   if (lane == 0) store_wait_all();
 }

@@ -1,5 +1,6 @@
 // Dense-polynomial DeTAG step on the FP64 tensor path (n <= 32), tiles padded to 32 workers: caller-written gradients of 25 to 32
-// workers, where it is ahead of step_dense.cu, and all steps under the self test of failure detection, which wants its waits.
+// workers, where it is ahead of step_dense.cu, and, under the self test of failure detection, which wants bounded waits, the
+// steps of at most 16.
 //
 // AG_K is linear, AG_K(z) = P z with P = P_K(M) built by the host in float64 from the matrix form of
 // Algorithm 3.  For a slab of coordinates the step is therefore two small dense contractions

@@ -90,6 +90,41 @@ def test_a_stalled_loader_times_out_every_waiter_and_the_state_recovers(n, d, K,
         assert rel_l2(s.download("y"), orc.folded_tracker(ref)) <= 1e-4
 
 
+@pytest.mark.parametrize("n,mode,after,many", [
+    (17, "detag", 0, False), (24, "start", 5, False), (32, "detag", 6, False), (24, "external", 1, False), (32, "dpsgd", 5, False),
+    (33, "detag", 1, False), (48, "start", 4, False), (48, "detag", 0, False), (40, "external", 4, False), (48, "dpsgd", 1, False),
+    (20, "detag", 5, True), (32, "start", 2, True),  # several steps per launch, loaded over the last one's
+    (16, "detag", 1, True)])                         # ... on the padded tiles
+def test_groups_that_get_no_more_slabs_time_out_and_the_state_recovers(n, mode, after, many):
+    """17 to 48 workers: groups of four or eight warps wait for operands and, separately, for the inputs of the tail; `after`
+    counts the slabs of a block of three or four groups.  Here some groups get no operands and others no inputs of the tail."""
+    d = 64 * 148 * 9 + 17
+    m, a, c, x0 = _case(n, d, n)
+    rng = np.random.default_rng(n + after)
+    start = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g") + (("g_new",) if mode == "external" else ())}
+    got = []
+    for stalled in (False, True):
+        with Session(m, d, 2, 0.2, 0.05, a, c, x0, 0.1, 7, gradient_point=int(mode == "start"), algorithm=int(mode == "dpsgd"),
+                     external_gradient=mode == "external") as s:
+            step = (lambda: s.step_many(3)) if many else s.step
+            if stalled:
+                B.detag_debug_inject_stall(s.state, after, 2048)
+                step()
+                with pytest.raises(B.DetagError) as e:
+                    s.status()
+                assert e.value.code == B.DETAG_ERR_TIMEOUT
+                B.detag_debug_inject_stall(s.state, -1, 0)
+                _rebind(s)
+            for k, v in start.items():
+                s.upload(k, v)
+            B.detag_set_step(s.state, 0)
+            step()
+            s.status()
+            got.append([s.download(k) for k in ("x", "y", "g")])
+    for k in range(3):
+        assert np.array_equal(got[0][k], got[1][k])
+
+
 def test_status_after_host_resident_stepping_needs_no_bind_and_sees_a_timeout():
     import torch
 
