@@ -13,7 +13,8 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // The next launch may begin (once every block has said so).  After chain_wait(): what it finds running is this launch alone.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Launch with that attribute; a cudaError_t value.
+// Launch with that attribute; a cudaError_t value.  The caller reports a failure, so it is not left behind as the runtime's last
+// error for whoever asks next.
 template <typename... P>
 int launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, const P&... args) {
   cudaLaunchConfig_t config = {};
@@ -26,7 +27,9 @@ int launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t
   chained.val.programmaticStreamSerializationAllowed = 1;
   config.attrs = &chained;
   config.numAttrs = 1;
-  return static_cast<int>(cudaLaunchKernelEx(&config, kernel, args...));
+  const cudaError_t e = cudaLaunchKernelEx(&config, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return static_cast<int>(e);
 }
 
 }  // namespace detag

@@ -69,3 +69,29 @@ def test_back_to_back_as_with_the_device_idle_between(case):
     for other in got[1:]:
         for k in ("x", "y", "g"):
             assert np.array_equal(got[0][k], other[k]), k
+
+
+@pytest.mark.parametrize("n", [8, 24, 60])
+def test_a_launch_that_fails_is_reported_once(n):
+    """A step on a stream whose capture was broken off fails at its launch; the next call knows nothing of it."""
+    import ctypes
+
+    import torch
+
+    cu = ctypes.CDLL("libcuda.so.1")
+    with _session(n, 4096, 2, "ring", B.DETAG_VARIANT_AUTO, "detag") as s:
+        s.step()
+        torch.cuda.synchronize()
+        handle = ctypes.c_void_p(torch.cuda.Stream().cuda_stream)
+        assert cu.cuStreamBeginCapture_v2(handle, 1) == 0   # thread-local
+        assert cu.cuStreamSynchronize(handle) != 0          # not allowed there: ends the capture
+        with pytest.raises(B.DetagError) as e:
+            B.detag_step(s.state, handle.value)
+        assert e.value.code == B.DETAG_ERR_CUDA
+        graph = ctypes.c_void_p()
+        assert cu.cuStreamEndCapture(handle, ctypes.byref(graph)) != 0
+        B.detag_init(s.state, handle.value)
+        B.detag_step(s.state, handle.value)
+        s.consensus_error()
+        torch.cuda.synchronize()
+        s.status()
