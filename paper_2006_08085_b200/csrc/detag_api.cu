@@ -456,12 +456,12 @@ bool small_ok(const StepParams& p) {
 // padded tiles (up to 32) or the integer tensor path -> that one: 17 workers, d = 3 M 582 -> 340; 24 569 -> 414; 28 572 -> 531; 32
 // 600 -> 580, d = 25.6 M 5030 -> 4805, printed timing, d = 3 M 790 -> 578; 33, d = 1 M 411 -> 272; 40 427 -> 292; 48 430 -> 393; D-PSGD
 // of 32, d = 3 M 415 -> 405, of 48, d = 1 M 444 -> 265; caller-written gradients of 24, d = 3 M 448 -> 410, of 48, d = 1 M 664 (rounds)
-// -> 391.  But caller-written gradients of 28 470 -> 496, of 32 498 -> 535; and from 41 workers on a slab takes long enough that with
-// one per SM the integer path is ahead: 48, d = 9400 12.3 -> 13.9, d = 18000 16.4 -> 14.4 (40, d = 9400: 12.3 both).  The length is the
-// state's, not a staged chunk's: host-resident stepping gives the same bits.
+// -> 391.  But caller-written gradients of 28 470 -> 496, of 32 498 -> 535.  At every length: with one slab per SM the integer path is
+// up to 0.25 us ahead (48, d = 9400 9.50 -> 9.67, D-PSGD 9.17 -> 7.69), but its sums are not the same bits, and a shard of the
+// coordinates gives what the whole gives.
 bool dense_step_ok(const detag_state* s, const StepParams& p, int variant) {
   if (p.n <= detag::kMaxSmallWorkers || p.n > detag::kMaxDenseStepWorkers || p.poly == nullptr || p.d > 0x7fffffffLL) return false;
-  if (p.mode == detag::kModeExternal ? p.n > 24 && p.n <= 32 : p.n > 40 && s->d <= 64LL * s->sm_count) return false;
+  if (p.mode == detag::kModeExternal && p.n > 24 && p.n <= 32) return false;
   return variant == DETAG_VARIANT_DENSE || (variant == DETAG_VARIANT_CSR && s->variant_forced == DETAG_VARIANT_AUTO);
 }
 

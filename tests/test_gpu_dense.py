@@ -65,6 +65,28 @@ def test_one_step_against_the_oracle(n, d, mode):
         assert worst_ratio(out["y"], y_gossip + g_ref - g_, extra=HALF_ULP32 * np.abs(g_ref)) <= 1.0
 
 
+@pytest.mark.parametrize("n", [20, 32, 41, 48])
+@pytest.mark.parametrize("mode", ["new", "start", "external", "dpsgd"])
+def test_a_shard_of_the_coordinates_gives_what_the_whole_gives(n, mode):
+    """Bit for bit, at lengths below and beyond a slab per SM."""
+    m = inputs.metropolis_weights(inputs.random_regular4_graph(n, n))
+    d, cut = 2 * ROUND + 100, ROUND - 60
+    rng = np.random.default_rng(n)
+    arrays = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c") + (("g_new",) if mode == "external" else ())}
+    got = []
+    for lo, hi in ((0, d), (0, cut), (cut, 2 * cut), (2 * cut, d)):
+        with Session(m, hi - lo, 4, 0.2, 0.05, sigma=0.1, seed=3, coord_offset=lo, gradient_point=int(mode == "start"),
+                     external_gradient=mode == "external", algorithm=int(mode == "dpsgd")) as s:
+            for k, v in arrays.items():
+                s.upload(k, v[:, lo:hi])
+            B.detag_set_step(s.state, 0)
+            s.step(3)
+            s.status()
+            got.append([s.download(k) for k in ("x", "y", "g")])
+    for k in range(3):
+        assert np.array_equal(got[0][k], np.concatenate([part[k] for part in got[1:]], axis=1))
+
+
 @pytest.mark.parametrize("n,bad", [(33, np.inf), (40, np.nan), (48, -np.inf)])
 @pytest.mark.parametrize("mode", ["new", "external", "dpsgd"])
 def test_what_is_not_finite_reaches_those_that_hear_of_it(n, bad, mode):
