@@ -7,8 +7,7 @@
 //   u_rad = (2 (r_even >> 9) + 1) * 2^-24 in (0,1),  u_ang = (r_odd >> 9) * 2^-23 in [0,1)
 //   rad = sqrt(-2 ln u_rad);  first = rad cos(2 pi u_ang);  second = rad sin(2 pi u_ang)
 // Both uniforms are exactly representable in float32 and are built with bit operations, no
-// integer-to-float conversion.  The logarithm is an own float32 routine (exponent split, degree-7
-// polynomial of ln(1+f)/..., relative error < 1.2e-7 over all 2^23 inputs); the square root uses the
+// integer-to-float conversion.  The logarithm is an own float32 routine (below); the square root uses the
 // reciprocal-square-root unit and sine/cosine the special-function unit on an argument reduced
 // exactly to [-pi, pi).  Resulting absolute error of a normal: about 1e-6 (1 + |xi|).
 #ifndef DETAG_NOISE_CUH
@@ -61,15 +60,23 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
 // 1 + (r >> 9) 2^-23: the exponent bits of 1.0 come in from above as the word is shifted, one instruction for both.
 __device__ __forceinline__ float one_to_two(uint32_t r) { return __uint_as_float(__funnelshift_r(r, 0x7fu, 9)); }
 
-// -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9, of two words.  The factor -2 is in the argument F = -2 f and in the coefficients,
-// scaled by powers of two: the bits are those of -2 times the logarithm.
+// -2 ln(u) for u = (2k+1) 2^-24, k = r >> 9, of two words, as Cody and Waite ("Software Manual for the Elementary Functions",
+// 1980) lay a logarithm out: u = m 2^e, ln u = e ln 2 + ln m with ln 2 in two parts.  Own choices:
+//  - m in [2/3, 4/3).  Of the intervals [c, 2 c) this is the one with the smallest largest |m - 1|: 1 - c = 2 c - 1.  m and u
+//    differ in their exponent fields alone, by e, so e is the exponent field of u's bits less the bits of c; m - 1 is exact.
+//  - The parts of ln 2 are its nearest float32 and the float32 next to what is left.  A fused multiply-add does not round e times
+//    either, so the upper part needs no room for e, and what both leave out is below 2^-53.
+//  - ln(1 + f) = f + f^2 r(f), r a degree-7 Chebyshev fit of (ln(1+f) - f) / f^2 on |f| <= 1/3.
+// Relative error over all 2^23 arguments: at most 9.9e-8, 2.9e-8 rms.  The factor -2 is in the argument F = -2 f and in the
+// coefficients, scaled by powers of two: the bits are those of -2 times the logarithm.
 __device__ __forceinline__ F2 neg2_ln_unit(uint32_t r0, uint32_t r1) {
   float u0, u1;
   unpack2(add2(pack2(one_to_two(r0), one_to_two(r1)), both(-0x1.fffffep-1f)), u0, u1);  // (2k+1) 2^-24, exact
   const int b0 = __float_as_int(u0), b1 = __float_as_int(u1);
-  const int e0 = (b0 - 0x3f2aaaab) & 0xff800000, e1 = (b1 - 0x3f2aaaab) & 0xff800000;   // u = m 2^e with m in [2/3, 4/3); here e 2^23
+  constexpr int kTwoThirds = 0x3f2aaaab, kExponent = static_cast<int>(0xff800000u);     // the float's bits; sign and exponent field
+  const int e0 = (b0 - kTwoThirds) & kExponent, e1 = (b1 - kTwoThirds) & kExponent;     // here e 2^23
   const F2 F = fma2(pack2(__int_as_float(b0 - e0), __int_as_float(b1 - e1)), both(-2.0f), both(2.0f));  // -2 f, f = m - 1, exact
-  // ln(1+f) = f + f^2 r(f) on |f| <= 1/3 (Chebyshev fit of (ln(1+f) - f)/f^2, degree 7); here -r(-F/2) / 2
+  // -r(-F/2) / 2
   F2 r7 = both(0.13756538927555084f * 0x1p-8f);
   r7 = fma2(r7, F, both(0.1504942923784256f * 0x1p-7f));
   r7 = fma2(r7, F, both(0.1405421793460846f * 0x1p-6f));
@@ -80,8 +87,10 @@ __device__ __forceinline__ F2 neg2_ln_unit(uint32_t r0, uint32_t r1) {
   r7 = fma2(r7, F, both(0.49999985098838806f * 0x1p-1f));
   F2 ln = fma2(mul2(F, F), r7, F);
   const F2 ef = pack2(__int2float_rn(e0), __int2float_rn(e1));                          // exact
-  ln = fma2(ef, both(-1.42860677e-06f * 0x1p-22f), ln);
-  return fma2(ef, both(-0.693145751953125f * 0x1p-22f), ln);
+  constexpr double kLn2 = 0.69314718055994530942;
+  constexpr float kUpper = static_cast<float>(kLn2), kLower = static_cast<float>(kLn2 - static_cast<double>(kUpper));
+  ln = fma2(ef, both(-kLower * 0x1p-22f), ln);
+  return fma2(ef, both(-kUpper * 0x1p-22f), ln);
 }
 
 // Approximate reciprocal square root of a normal number (rsqrtf() tests for subnormal arguments first).
