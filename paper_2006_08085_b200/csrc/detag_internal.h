@@ -56,6 +56,7 @@ struct StepParams {
   int mode;           // kModeDetag, kModeExternal or kModeDpsgd
   const float* g_ext; // kModeExternal: the caller's newest stochastic gradient, [n][ld]
   unsigned spin_limit;    // polls after which a device-side wait gives up
+  int operands_end, tails_end;  // step_dense.cu: slabs from here on are not asked for
   long long stall_after;  // failure-detection self test: a CTA's producer stops loading after this many tiles (< 0: off)
   int* status;
 };

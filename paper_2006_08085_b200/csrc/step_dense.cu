@@ -132,11 +132,7 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
   const int whole = static_cast<int>(p.d / kDS), slabs = static_cast<int>((p.d + kDS - 1) / kDS), stride = gridDim.x * kGroups;
   int slab = blockIdx.x + gridDim.x * group;
 
-  // Self test of failure detection: nothing is asked for beyond p.stall_after slabs of the block - in odd groups the inputs of
-  // the tail alone, so that both waits run out, the one with the next operands on their way.
-  auto withheld = [&](int k) { return p.stall_after >= 0 && group + static_cast<long long>(kGroups) * k >= p.stall_after; };
   auto load_operands = [&](int s, int k) {  // one thread, for the group's k-th slab
-    if ((group & 1) == 0 && withheld(k)) return;
     *in_asked = k + 1;
     bar_expect_tx(in_full, (1u + (kMode != kModeDpsgd) + kEarly) * kTileBytes);
     rows_load(tx, &maps.x, 2 * s, 0, in_full);
@@ -144,7 +140,6 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
     if (kEarly) rows_load(tg, &maps.g, 2 * s, 0, in_full);
   };
   auto load_tail = [&](int s, int k) {
-    if (withheld(k)) return;
     *tail_asked = k + 1;
     bar_expect_tx(tail_full, (1u + (kMode != kModeExternal) + !kEarly) * kTileBytes);
     if (!kEarly) rows_load(tg, &maps.g, 2 * s, 0, tail_full);
@@ -158,10 +153,8 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
     fence_barrier_init();
     fence_async_shared();
     chain_wait();
-    if (slab < whole) {
-      load_operands(slab, 0);
-      load_tail(slab, 0);
-    }
+    if (slab < p.operands_end) load_operands(slab, 0);
+    if (slab < p.tails_end) load_tail(slab, 0);
   }
 #pragma unroll
   for (int e = threadIdx.x; e < R * kBlocks * 32; e += dense_threads(R)) {  // while the first loads are on their way
@@ -181,9 +174,9 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
     if (!ragged) ok = bar_wait(in_full, use & 1, limit);
     if (owes) {
       store_wait_read();
-      if (!ragged) {
+      if (slab < p.tails_end) {
         load_tail(slab, use);
-      } else {
+      } else if (ragged) {
         bar_arrive(tail_full);
       }
       owes = false;
@@ -294,7 +287,7 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
       }
       if (!kMany) {  // several steps write their results over the operands
         __syncwarp();
-        if (lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride, use + 1);
+        if (lane == 0 && last_of(in_done, kWarps) && slab + stride < p.operands_end) load_operands(slab + stride, use + 1);
       }
       // Normals, all before the wait where their registers allow it.  Two coordinates: lane q draws coordinate q % 2, quad
       // 2 h + q / 2, and entry s of what it gets in return is coordinate s % 2, quad 2 h + s / 2.  One: lane q draws quad 4 h + q.
@@ -396,7 +389,7 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
     // intermediate ones before the next operands that are loaded over them.
     fence_async_shared();
     __syncwarp();
-    if (kMany && lane == 0 && last_of(in_done, kWarps) && slab + stride < whole) load_operands(slab + stride, use + 1);
+    if (kMany && lane == 0 && last_of(in_done, kWarps) && slab + stride < p.operands_end) load_operands(slab + stride, use + 1);
     if (!ragged) {
       if (lane == 0 && last_of(tail_done, kWarps)) {
         rows_store(&maps.g, 2 * slab, 0, t_gout);
@@ -421,10 +414,18 @@ __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const S
 typedef void (*DenseKernel)(const StepParams, const DenseMaps);
 
 template <int R>
-int launch_kernel(DenseKernel kernel, const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream) {
+int launch_kernel(DenseKernel kernel, StepParams p, const TensorMapSet& maps, int sm_count, cudaStream_t stream) {
   const int e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), dense_smem_bytes(R));
   if (e != 0) return e;
   const long long slabs = (p.d + kDS - 1) / kDS, grid = slabs < sm_count ? slabs : sm_count;
+  p.operands_end = p.tails_end = static_cast<int>(p.d / kDS);
+  // Self test of failure detection: a block's first stall_after slabs are loaded, of the others nothing or, if the number is odd,
+  // all but the tail's inputs - both waits can run out, the second with the next operands on their way.  The limits come from
+  // here because a test in the kernel, run once a slab by one thread, took 48 workers from 388 to 402 us (d = 1 M).
+  if (p.stall_after >= 0 && p.stall_after <= p.tails_end / grid) {
+    p.tails_end = static_cast<int>(p.stall_after * grid);
+    if (p.stall_after % 2 == 0) p.operands_end = p.tails_end;
+  }
   return launch_chained(kernel, static_cast<unsigned>(grid), dense_threads(R), dense_smem_bytes(R), stream, p, *reinterpret_cast<const DenseMaps*>(maps.bytes));
 }
 

@@ -97,7 +97,8 @@ def test_a_stalled_loader_times_out_every_waiter_and_the_state_recovers(n, d, K,
     (16, "detag", 1, True)])                         # ... on the padded tiles
 def test_groups_that_get_no_more_slabs_time_out_and_the_state_recovers(n, mode, after, many):
     """17 to 48 workers: groups of four or eight warps wait for operands and, separately, for the inputs of the tail; `after`
-    counts the slabs of a block of three or four groups.  Here some groups get no operands and others no inputs of the tail."""
+    counts the slabs of a block of three or four groups.  Beyond an even number there are no operands, beyond an odd one no inputs
+    of the tail."""
     d = 64 * 148 * 9 + 17
     m, a, c, x0 = _case(n, d, n)
     rng = np.random.default_rng(n + after)
