@@ -54,12 +54,13 @@ def test_a_wait_that_nothing_ends_gives_up_and_is_reported():
 
 
 @pytest.mark.parametrize("n,d,K,variant,after", [
-    # dense kernel, several slabs per CTA (the kernel for n <= 16 has no waits; under injection n <= 32 runs this one)
+    # padded tiles, several slabs per CTA (the kernel for n <= 16 has no waits; under injection this one runs)
     (16, 64 * 148 * 4 + 17, 3, B.DETAG_VARIANT_DENSE, 1),
     (16, 64 * 148 * 4 + 17, 3, B.DETAG_VARIANT_DENSE, 0),   # nothing is ever loaded
     (64, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_RING, 3),     # circulant band kernel
     (288, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_RING, 5),
-    (48, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # integer tensor path, two slabs' digits
+    (48, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # groups of warps
+    (56, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # integer tensor path, two slabs' digits
     (64, 64 * 148 * 3 + 5, 2, B.DETAG_VARIANT_TORUS, 2),    # block-circulant transform kernel
     (32, 64 * 148 * 3 + 5, 2, B.DETAG_VARIANT_TORUS, 0),
     (72, 64 * 148 * 2 + 5, 2, B.DETAG_VARIANT_DENSE, 1),    # ... one slab's digits
