@@ -426,7 +426,7 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
 }
 
-// The integer tensor path takes the dense and circulant products with 32 < n <= 256, and, where the choice is the
+// The integer tensor path takes the dense and circulant products with 48 < n <= 256, and, where the choice is the
 // library's, the rounds of such matrices too.  Circulant bands stay on their float64 kernel, which needs no test of the
 // operands; us per step, integer path -> that one: 64 workers, d = 2 M, K = 1 1099 -> 1035, K = 16 1020 -> 1035; 128, d = 1 M,
 // K = 1 1260 -> 1031, K = 16 1103 -> 1031; 224, d = 500 k, K = 16 1198 -> 927; 256, d = 1 M, K = 1 3157 -> 2032, K = 16
@@ -579,7 +579,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   if (n <= 64) s->poly = poly;  // what the small kernels and the torus analysis use
   analyse_circulant(s);
   analyse_torus(s);
-  if (n > 32 && n <= detag::kMaxSplitWorkers) {
+  if (n > detag::kMaxDenseStepWorkers && n <= detag::kMaxSplitWorkers) {
     const bool blocks = block_circulant(s);
     if (blocks) first_block_row(s, poly);
     if (!poly.empty()) detag::split_polynomial(n, poly, blocks, s->split);  // else: too many distinct blocks

@@ -118,7 +118,7 @@ int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
 bool build_maps_dense(const StepParams& p, TensorMapSet* maps);
 int launch_step_dense(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);
 int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);  // n <= 32, p.steps steps
-// polynomial on the integer tensor path (step_split.cu): 32 < n <= 256, DeTAG and D-PSGD steps
+// polynomial on the integer tensor path (step_split.cu): 48 < n <= 256, DeTAG and D-PSGD steps
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
 bool build_maps_split(const StepParams& p, TensorMapSet* maps);
 struct SplitDevice {  // the tables of a SplitPoly in the workspace
@@ -153,7 +153,7 @@ struct detag_state {
   // 8 x 8 polynomial blocks in MMA fragment order
   bool torus = false;
   std::vector<double> torus_frag;
-  detag::SplitPoly split;         // 32 < n <= 256: P_K(M) for the integer tensor path (empty: not taken)
+  detag::SplitPoly split;         // 48 < n <= 256: P_K(M) for the integer tensor path (empty: not taken)
   std::vector<unsigned char> image;  // the workspace up to the partial sums, as it is uploaded
   int variant_forced = DETAG_VARIANT_AUTO;
   int gradient_point = DETAG_GRADIENT_AT_NEW_MODEL;
