@@ -47,17 +47,18 @@ KERNEL_SOURCES = {
 }
 MEASURED_TRAFFIC = {
     # (kernel, mode): (source digest, bytes per wc)
-    ("small", "column"): ("26f1b4f3eccbed2b", 28.81),  # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1410 GB written / 16 M wc
-    ("dense", "product"): ("070f126e2d58dbf8", 31.22),  # cfg5 shape at d = 2 M: 1.2802 + 0.7177 GB / 64 M wc
-    ("torus", "torus8"): ("4ccde3daf94c6d39", 31.24),  # cfg3 shape at d = 1 M: 1.2801 + 0.7193 GB / 64 M wc
-    ("ring", "band"): ("a9f574115be24d04", 31.08),  # cfg4 shape at d = 200 k: 1.0275 + 0.5641 GB / 51.2 M wc
-    ("split", "digits"): ("70667638fd698bcb", 30.80),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4315 GB / 40 M wc
-    ("csr", "rounds"): ("b8924f0a1b9a670d", 30.67),  # 300-worker random graph at d = 100 k: 0.6017 + 0.3183 GB / 30 M wc
+    ("small", "column"): ("c6d0a442e7230680", 28.81),  # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1409 GB written / 16 M wc
+    ("dense", "product"): ("1d4428cc1d4b78f9", 31.21),  # cfg5 shape at d = 2 M: 1.2801 + 0.7177 GB / 64 M wc
+    ("torus", "torus8"): ("194904bdd0cabfdc", 31.23),  # cfg3 shape at d = 1 M: 1.2802 + 0.7185 GB / 64 M wc
+    ("ring", "band"): ("72c17745930c7df4", 31.09),  # cfg4 shape at d = 200 k: 1.0277 + 0.5641 GB / 51.2 M wc
+    ("split", "digits"): ("e2d36bcd79226d9b", 30.80),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4315 GB / 40 M wc
+    ("csr", "rounds"): ("8691108dc6578a76", 30.62),  # 300-worker random graph at d = 100 k: 0.6017 + 0.3169 GB / 30 M wc
 }
 
-# Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes) and that
-# pipe's peak: 64 multiply-adds per clock and SM (measured: 61 with m8n8k4 MMAs from 16 warps) x 148 SMs x max clock.
-FP64_FMA_PER_WC = {("dense", "product"): 64, ("ring", "band"): 80, ("torus", "torus8"): 26, ("torus", "torus4"): 28}
+# Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes; the dense product by its
+# worker count, fp64_fma_per_wc) and that pipe's peak: 64 multiply-adds per clock and SM (measured: 61 with m8n8k4 MMAs from 16
+# warps) x 148 SMs x max clock.
+FP64_FMA_PER_WC = {("ring", "band"): 80, ("torus", "torus8"): 26, ("torus", "torus4"): 28}
 VARIANT_NAMES = {1: "csr", 2: "dense", 3: "ring", 4: "torus"}
 FP64_FMA_PER_CLK_SM = 64
 SM_COUNT = 148
@@ -73,6 +74,12 @@ def kernel_key(variant: str, n: int):
     if variant == "torus":
         return ("torus", "torus8" if n == 64 else "torus4")
     return None
+
+
+def fp64_fma_per_wc(key, n: int):
+    if key == ("dense", "product"):  # inputs padded to 4 workers, outputs to 8
+        return 2 * ((n + 3) // 4 * 4) * ((n + 7) // 8 * 8) / n
+    return FP64_FMA_PER_WC.get(key)
 
 
 def source_digest(kernel: str) -> str:
@@ -289,9 +296,10 @@ def time_config(name: str, dev, args) -> dict:
            "achieved_gbs": achieved, "frac_of_measured_peak": achieved / peak,
            "frac_of_8TBps_nominal": achieved / 8000.0, "consensus_error_after_run": ce,
            "l2": "exceeds L2" if 20 * cfg.wc > 4 * 126e6 else "working set fits the 126 MB L2: not an HBM measurement"}
-    if key in FP64_FMA_PER_WC:
-        out["fp64_fma_per_wc"] = FP64_FMA_PER_WC[key]
-        out["fp64_pipe_frac"] = FP64_FMA_PER_WC[key] * out["value"] / (FP64_FMA_PER_CLK_SM * SM_COUNT * 1965e6)
+    fma = fp64_fma_per_wc(key, cfg.n)
+    if fma is not None:
+        out["fp64_fma_per_wc"] = fma
+        out["fp64_pipe_frac"] = fma * out["value"] / (FP64_FMA_PER_CLK_SM * SM_COUNT * 1965e6)
     traffic = measured_traffic_bytes(variant, cfg.n, cfg.wc)  # ncu DRAM bytes of a small case, scaled; None if stale
     out["traffic_bytes_per_step"] = traffic
     return out
@@ -579,10 +587,11 @@ def run_ours(args, rank: int, world: int, local_rank: int) -> None:
         traffic = measured_traffic_bytes(variant, cfg.n, cfg.wc)
         key = kernel_key(variant, cfg.n)
         fp64, fp64_peak = None, None
-        if key in FP64_FMA_PER_WC:  # second roofline: the FP64 pipe that carries both contractions
-            fma = FP64_FMA_PER_WC[key] * cfg.wc / (kernel_ms * 1e-3)
+        fma_per_wc = fp64_fma_per_wc(key, cfg.n)
+        if fma_per_wc is not None:  # second roofline: the FP64 pipe that carries both contractions
+            fma = fma_per_wc * cfg.wc / (kernel_ms * 1e-3)
             fp64_peak = FP64_FMA_PER_CLK_SM * SM_COUNT * (clocks.get("sm_max_mhz") or 1965) * 1e6
-            fp64 = {"fma_per_wc": FP64_FMA_PER_WC[key], "achieved_tfma_s": fma / 1e12, "peak_tfma_s": fp64_peak / 1e12,
+            fp64 = {"fma_per_wc": fma_per_wc, "achieved_tfma_s": fma / 1e12, "peak_tfma_s": fp64_peak / 1e12,
                     "frac": fma / fp64_peak, "peak_source": "64 FMA/clk/SM x 148 SMs x max SM clock"}
         line = {
             "metric": METRIC, "value": world * cfg.wc * args.steps / (total_ms_max * 1e-3), "unit": UNIT,
@@ -608,7 +617,7 @@ def run_ours(args, rank: int, world: int, local_rank: int) -> None:
             line["e2e"] = e2e
         if multi is not None:
             if fp64_peak is not None:
-                multi["fp64_tensor_pipe_frac"] = FP64_FMA_PER_WC[key] * multi["value"] / fp64_peak
+                multi["fp64_tensor_pipe_frac"] = fma_per_wc * multi["value"] / fp64_peak
             line["multi_step"] = multi
         if modes is not None:
             for v in modes.values():

@@ -54,8 +54,8 @@ enum {
   DETAG_ERR_SPECTRUM = -9        /* lambda >= 1: disconnected or bipartite graph, no valid eta */
 };
 
-/* Kernel variants of the gossip part of the step; all compute the same result.  The polynomial variants of 32 < n <= 256
-   workers run on the integer tensor path where its shared-memory plan holds P_K(M) (any matrix up to n = 128, beyond that
+/* Kernel variants of the gossip part of the step; all compute the same result.  Up to 48 workers the polynomial variants run in
+   float64 throughout.  Those of 48 < n <= 256 run on the integer tensor path where its shared-memory plan holds P_K(M) (any matrix up to n = 128, beyond that
    matrices whose 32 x 32 blocks depend on their distance only); coordinates in which an output may read operands far below
    the largest are summed in float64 instead, which takes up to five times as long when it concerns all of them (one or two
    rounds on sparse graphs, workers of very different magnitude).  Circulant bands run in float64 throughout.  What neither
@@ -64,7 +64,7 @@ enum {
   DETAG_VARIANT_AUTO = 0,  /* host cost model picks */
   DETAG_VARIANT_CSR = 1,   /* K rounds of neighbour-indexed sums over the CSR rows, slab staged on chip: any graph, n <= 1024.
                               Where AUTO resolves to it, the library still applies the rounds as one product with their
-                              polynomial if the integer tensor path takes it; forced, the rounds run as such */
+                              polynomial up to n = 48 or if the integer tensor path takes it; forced, the rounds run as such */
   DETAG_VARIANT_DENSE = 2, /* one product with the host-precomputed polynomial P_K(M), n <= 128 (any M) */
   DETAG_VARIANT_RING = 3,  /* circulant M (rings), n % 32 == 0, 64 <= n <= 1024: the circulant polynomial P_K(M), a band
                               while K * bandwidth <= 16, or any (n <= 256), e.g. at Theorem 3's phase length; a band's last

@@ -44,7 +44,8 @@ struct Vec<4> {
   typedef float4 Type;
 };
 
-// Blocks per SM the registers are planned for: what the five arrays' vectors and the sums need without spills.  More blocks
+// Blocks per SM the registers are planned for: what the five arrays' vectors and the sums need, but for 4 to 40 bytes that the
+// printed timing of 12 to 16 workers and the default step of 13 to 15 spill.  More blocks
 // at fewer registers lose (n = 16: above), fewer do not gain; many steps at n = 16 in 6 blocks 76 us for 68.
 constexpr int small_blocks(int R, int V, bool many) { return many ? 4 : R * V <= 8 ? 5 : R * V <= 12 ? 4 : 3; }
 
@@ -67,8 +68,9 @@ __global__ void __launch_bounds__(kSmallThreads, small_blocks(R, V, kMany)) step
   const bool noisy = kMode != kModeExternal && p.sigma != 0.0;
   const float* const pa = kMode == kModeExternal ? p.g_ext : p.a;
 
-  // ---- everything is asked for before anything is used.  Workers beyond n and coordinates beyond d count as zero; they read
-  // a row and a column that are there, so that no branch keeps the loads apart.
+  // ---- everything is asked for before anything is used.  Workers beyond n count as zero; they read a row that is there, so
+  // that no branch keeps the loads apart.  Coordinates beyond d take what the rows' padding or the warp's first column holds:
+  // they keep to themselves and are not stored.
   const long long at = inside ? j : first;
   auto load = [&](const float* base, float (&v)[R][V]) {
 #pragma unroll

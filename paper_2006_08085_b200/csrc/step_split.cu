@@ -1,5 +1,5 @@
 // DeTAG step with the polynomial P = P_K(M) applied on the fifth-generation tensor cores in exact integer arithmetic,
-// for any gossip matrix with 32 < n <= 256 whose distinct 32 x 32 blocks of P fit in shared memory.
+// for any gossip matrix with 48 < n <= 256 whose distinct 32 x 32 blocks of P fit in shared memory.
 //
 // AG_K(z) = P z.  The float64 tensor path (mma m8n8k4) bounds this product at 64 multiply-adds per clock and SM, which
 // for n = 100 is 3.3 times and for a dense n = 256 eight times the time of the step's HBM traffic.  Here both operands
@@ -85,8 +85,8 @@ constexpr int kPStageBytes = 3 * kPStageFloats * 4;  // g | a | c  ->  g' | x' |
 constexpr int kPScaleSlots = 4;     // slabs whose scales are kept: see the splitting warps
 constexpr int kPMaxGroups = 4, kPMaxStages = 2, kPMaxBlocks = 8;
 // Splitting and finishing warps.  Up to 128 workers two groups of four share the blocks of a slab: its splitting is a
-// serial chain (largest value, then digits) that one group needs 5.6 k cycles for at n = 48, as long as the slab's HBM
-// time.  Beyond, a slab's other stages take longer than its splitting, and the warps finish instead.
+// serial chain (largest value, then digits) that one group needed 5.6 k cycles for at n = 48, as long as the slab's HBM
+// time (such worker counts have left for step_dense.cu since; 64 workers 213 -> 185 us, d = 400 k).  Beyond, a slab's other stages take longer than its splitting, and the warps finish instead.
 __host__ __device__ constexpr int split_warps(bool big) { return big ? 4 : 8; }
 __host__ __device__ constexpr int finish_groups(bool big) { return big ? 4 : 3; }
 constexpr int kPThreads = 24 * 32;  // both: split_warps + 4 finish_groups + 4
