@@ -212,18 +212,22 @@ SmallKernel pick_small(const StepParams& p) {
 }
 
 template <int R, bool kFull>
-SmallKernel pick_many(const StepParams& p) {
+SmallKernel pick_many(const StepParams& p, bool wide) {
+  if (R == 1 && wide) return p.grad_at_start ? step_small_kernel<1, kFull, 4, kModeDetag, true, true> : step_small_kernel<1, kFull, 4, kModeDetag, false, true>;
   return p.grad_at_start ? step_small_kernel<R, kFull, 2, kModeDetag, true, true> : step_small_kernel<R, kFull, 2, kModeDetag, false, true>;
 }
 
 template <int R>
 int launch_small(const StepParams& p, int sm_count, cudaStream_t stream) {
   const bool many = p.steps > 1, full = p.n == 4 * R;
-  const SmallKernel kernel = many ? (full ? pick_many<R, true>(p) : pick_many<R, false>(p))
+  // Many steps: half as many coordinates to a warp, twice the warps to hide the chain of a step behind.  But with up to 4 workers a
+  // lane throws half of its Philox call away then: once every scheduler has a warp, four coordinates per lane (3 workers, twenty
+  // steps, two -> four: d = 4096 9.2 -> 10.2 us, 14 k 10.2 both, 32 k 14.3 -> 12.3, 150 k 40 -> 30, 1 M 233 -> 166).
+  const bool wide = !many || (R == 1 && p.d > 64LL * sm_count);
+  const SmallKernel kernel = many ? (full ? pick_many<R, true>(p, wide) : pick_many<R, false>(p, wide))
                                   : (full ? pick_small<R, true>(p) : pick_small<R, false>(p));
-  // Many steps: half as many coordinates to a warp, twice the warps to hide the chain of a step behind.  Short vectors: smaller
-  // blocks, so that every SM gets a share.
-  const int width = 8 * (many ? 2 : 4);
+  // Short vectors: smaller blocks, so that every SM gets a share.
+  const int width = wide ? 32 : 16;
   const long long warps = (p.d + width - 1) / width;
   const int per_block = warps >= 4LL * sm_count ? 4 : warps >= 2LL * sm_count ? 2 : 1;
   const unsigned grid = static_cast<unsigned>((warps + per_block - 1) / per_block);

@@ -58,6 +58,26 @@ def test_fused_steps_of_17_to_32_workers(n, d, count, where):
     test_fused_steps_equal_single_steps_bit_for_bit(n, d, 3, count, where)
 
 
+@pytest.mark.parametrize("n,d", [(1, 70), (3, 64 * 148), (4, 64 * 148 + 1), (3, 64 * 148 * 5 + 7), (4, 64 * 148 * 16 + 34)])
+@pytest.mark.parametrize("where", [B.DETAG_GRADIENT_AT_NEW_MODEL, B.DETAG_GRADIENT_AT_PHASE_START])
+def test_fused_steps_of_up_to_4_workers(n, d, where):
+    """Two coordinates per lane, and four beyond 64 per SM."""
+    m = inputs.csr_from_dense(np.ones((1, 1))) if n == 1 else inputs.metropolis_weights(inputs.ring_graph(n))
+    rng = np.random.default_rng(n + d)
+    state = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c")}
+    got = []
+    for fused in (False, True):
+        with Session(m, d, 2, 0.2, 0.05, sigma=0.1, seed=9, coord_offset=5, gradient_point=where) as s:
+            for k, v in state.items():
+                s.upload(k, v)
+            B.detag_set_step(s.state, 0)
+            s.step_many(3) if fused else s.step(3)
+            s.status()
+            got.append({k: s.download(k) for k in ("x", "y", "g")})
+    for k in ("x", "y", "g"):
+        assert np.array_equal(got[0][k], got[1][k]), k
+
+
 def test_fused_trajectory_against_the_oracle():
     n, d, K, steps = 16, 3_001, 4, 12
     m, eta, a, c, x0 = _case(n, d, 5)
