@@ -1,4 +1,5 @@
-// Several consecutive DeTAG steps in one launch (dense polynomial on the FP64 tensor path, n <= 32).
+// Several consecutive DeTAG steps in one launch (dense polynomial on the FP64 tensor path): 29 to 32 workers, 25 to 28 while there are
+// at most two slabs per SM, and at most 16 under the self test of failure detection.
 //
 // The step never mixes coordinates: each coordinate's n-vector of models, trackers and gradients evolves on its
 // own (the gossip mixes workers, the synthetic objective is diagonal, the noise is a pure function of
@@ -8,7 +9,7 @@
 // the kernel is the FP64 tensor pipe (64 multiply-adds per worker-coordinate and step) instead of HBM.
 //
 // Same roles, pipeline and arithmetic as the one-step kernel (step_mma.cu): the results are bit-identical to
-// `steps` launches of it.  Differences: the stage is kept for all steps and a tile's intermediate x', y', g' are
+// single steps, by whichever kernel.  Differences: the stage is kept for all steps and a tile's intermediate x', y', g' are
 // written back into the stage, into the warp's own eight columns (the B-fragment loads of the next step read
 // them there); only the last step writes the dense output tile that the TMA stores send out.  The noise index of
 // step i of the launch is t_noise + i.

@@ -94,8 +94,8 @@ def test_a_stalled_loader_times_out_every_waiter_and_the_state_recovers(n, d, K,
 @pytest.mark.parametrize("n,mode,after,many", [
     (17, "detag", 0, False), (24, "start", 5, False), (32, "detag", 6, False), (24, "external", 1, False), (32, "dpsgd", 5, False),
     (33, "detag", 1, False), (48, "start", 4, False), (48, "detag", 0, False), (40, "external", 4, False), (48, "dpsgd", 1, False),
-    (20, "detag", 5, True), (32, "start", 2, True),  # several steps per launch, loaded over the last one's
-    (16, "detag", 1, True)])                         # ... on the padded tiles
+    (20, "detag", 5, True), (28, "start", 2, True),    # several steps per launch, loaded over the last one's
+    (16, "detag", 1, True), (32, "start", 2, True)])   # ... on the padded tiles
 def test_groups_that_get_no_more_slabs_time_out_and_the_state_recovers(n, mode, after, many):
     """17 to 48 workers: groups of four or eight warps wait for operands and, separately, for the inputs of the tail; `after`
     counts the slabs of a block of three or four groups.  Beyond an even number there are no operands, beyond an odd one no inputs
