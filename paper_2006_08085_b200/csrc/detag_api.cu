@@ -836,12 +836,13 @@ int detag_step_many(detag_state* s, int count, void* stream) {
         e = detag::launch_step_small(p, s->sm_count, static_cast<cudaStream_t>(stream));
       } else {
         // Groups of four warps take a slab's steps in turn; the kernel with padded tiles puts eight warps on one, which is ahead
-        // while there are at most two slabs per SM, and where nothing is padded at every length.  us, padded -> groups, for ten steps:
-        // 17 workers, d = 9000 26.6 -> 22.5, d = 72 k 127 -> 71; 24, d = 9000 26.6 -> 23.9; 28, d = 18 k 39.0 -> 41.0, d = 36 k 68 -> 59;
-        // for twenty: 28, d = 1 M 3044 -> 2790; 32, d = 25 k 103 -> 97, d = 30 k 122 -> 124, d = 45 k 162 -> 179, d = 60 k 220 -> 217,
-        // d = 150 k 473 -> 486, d = 1 M 3077 -> 3171, printed timing, d = 150 k 482 -> 491.
+        // while there are at most two slabs per SM, and where nothing is padded beyond three, which the groups take side by side and
+        // its two in two turns.  us, padded -> groups, for ten steps: 17 workers, d = 9000 26.6 -> 22.5, d = 72 k 127 -> 71; 24, d = 9000
+        // 26.6 -> 23.9; 28, d = 18 k 39.0 -> 41.0, d = 36 k 68 -> 59; for twenty: 28, d = 1 M 3044 -> 2790; 32, d = 25 k 103 -> 97,
+        // d = 30 k 122 -> 124, d = 45 k 162 -> 179, d = 60 k 220 -> 217, d = 150 k 473 -> 486, d = 1 M 3077 -> 3171; printed timing,
+        // d = 150 k 482 -> 491.
         // (At most 16 get here for the self test of failure detection.)
-        const bool padded = p.n <= detag::kMaxSmallWorkers || p.n > 28 || (p.n > 24 && p.d <= 128LL * s->sm_count);
+        const bool padded = p.n <= detag::kMaxSmallWorkers || (p.n > 24 && p.d <= 128LL * s->sm_count) || (p.n > 28 && p.d > 192LL * s->sm_count);
         const detag::TensorMapSet* maps = maps_for(s, padded ? kFamilyMma : kFamilyDense, p);
         if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
         e = padded ? detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream))

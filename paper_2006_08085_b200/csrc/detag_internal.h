@@ -117,7 +117,7 @@ int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
 // dense product, groups of warps with a slab each (step_dense.cu): 16 < n <= 48, all modes
 bool build_maps_dense(const StepParams& p, TensorMapSet* maps);
 int launch_step_dense(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);
-int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);  // n <= 28, p.steps steps
+int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);  // n <= 32, p.steps steps
 // polynomial on the integer tensor path (step_split.cu): 48 < n <= 256, DeTAG and D-PSGD steps
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
 bool build_maps_split(const StepParams& p, TensorMapSet* maps);

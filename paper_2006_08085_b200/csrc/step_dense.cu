@@ -76,7 +76,7 @@ __device__ __forceinline__ void copy_bytes(float* to, const float* from, int byt
 }
 
 // R: workers per lane, n rounded up to 4 R.  kWide: the gradient in float64 instead of float32 at the rounded model.
-// kMany: p.steps iterations (DeTAG with the synthetic gradient, up to 28 workers): every lane's results take the places of its
+// kMany: p.steps iterations (DeTAG with the synthetic gradient, up to 32 workers): every lane's results take the places of its
 // own operands.
 template <int R, int kMode, bool kAtStart, bool kWide, bool kMany = false>
 __global__ void __launch_bounds__(dense_threads(R), 1) step_dense_kernel(const StepParams p, const __grid_constant__ DenseMaps maps) {
@@ -458,13 +458,14 @@ bool build_maps_dense(const StepParams& p, TensorMapSet* out) {
          make_half_map(&m.c, c, p.n, p.d, p.ld, rows);
 }
 
-// p.steps iterations, up to 28 workers.
+// p.steps iterations, up to 32 workers.
 int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream) {
-  if (p.n <= kMaxSmallWorkers || p.n > 28 || p.d <= 0 || p.d > 0x7fffffffLL || p.mode != kModeDetag) return static_cast<int>(cudaErrorInvalidValue);
+  if (p.n <= kMaxSmallWorkers || p.n > 32 || p.d <= 0 || p.d > 0x7fffffffLL || p.mode != kModeDetag) return static_cast<int>(cudaErrorInvalidValue);
   switch ((p.n + 3) / 4) {
     case 5: return launch_many<5>(p, maps, sm_count, stream);
     case 6: return launch_many<6>(p, maps, sm_count, stream);
-    default: return launch_many<7>(p, maps, sm_count, stream);
+    case 7: return launch_many<7>(p, maps, sm_count, stream);
+    default: return launch_many<8>(p, maps, sm_count, stream);
   }
 }
 

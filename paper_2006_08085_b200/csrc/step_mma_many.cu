@@ -1,5 +1,5 @@
-// Several consecutive DeTAG steps in one launch (dense polynomial on the FP64 tensor path): 29 to 32 workers, 25 to 28 while there are
-// at most two slabs per SM, and at most 16 under the self test of failure detection.
+// Several consecutive DeTAG steps in one launch (dense polynomial on the FP64 tensor path): 25 to 32 workers while there are at most
+// two slabs per SM, 29 to 32 beyond three too, and at most 16 under the self test of failure detection.
 //
 // The step never mixes coordinates: each coordinate's n-vector of models, trackers and gradients evolves on its
 // own (the gossip mixes workers, the synthetic objective is diagonal, the noise is a pure function of

@@ -53,7 +53,7 @@ def test_fused_steps_equal_single_steps_bit_for_bit(n, d, K, count, where):
     (25, 9001, 3), (28, 18_944, 2), (32, 257, 4),              # padded tiles where single steps run by groups of warps
     (17, 9001, 3), (23, 20_003, 3), (28, 20_003, 3),           # groups of warps, 5, 6 and 7 workers per lane
     (20, 64 * 148 * 9 + 35, 3), (28, 64 * 148 * 9 + 35, 2),    # several slabs per group, loaded over the last one's steps
-    (29, 20_003, 3), (32, 64 * 148 * 9 + 35, 2)])              # padded tiles, at every length
+    (29, 128 * 148 + 1, 3), (32, 192 * 148, 3), (31, 192 * 148 + 1, 2), (32, 64 * 148 * 9 + 35, 2)])  # 8 per lane, and padded again
 @pytest.mark.parametrize("where", [B.DETAG_GRADIENT_AT_NEW_MODEL, B.DETAG_GRADIENT_AT_PHASE_START])
 def test_fused_steps_of_17_to_32_workers(n, d, count, where):
     test_fused_steps_equal_single_steps_bit_for_bit(n, d, 3, count, where)
