@@ -47,7 +47,7 @@ KERNEL_SOURCES = {
 }
 MEASURED_TRAFFIC = {
     # (kernel, mode): (source digest, bytes per wc)
-    ("small", "column"): ("c6d0a442e7230680", 28.81),  # 16-worker ring at d = 1 M: 0.3200 GB read + 0.1409 GB written / 16 M wc
+    ("small", "column"): ("06300ac00a29f2b9", 28.79),  # 16-worker ring at d = 1 M: 0.3201 GB read + 0.1405 GB written / 16 M wc
     ("dense", "product"): ("1d4428cc1d4b78f9", 31.21),  # cfg5 shape at d = 2 M: 1.2801 + 0.7177 GB / 64 M wc
     ("torus", "torus8"): ("194904bdd0cabfdc", 31.23),  # cfg3 shape at d = 1 M: 1.2802 + 0.7185 GB / 64 M wc
     ("ring", "band"): ("72c17745930c7df4", 31.09),  # cfg4 shape at d = 200 k: 1.0277 + 0.5641 GB / 51.2 M wc
