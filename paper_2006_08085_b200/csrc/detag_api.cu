@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <utility>
 
 #include "detag_internal.h"
 #include "torus_basis.h"
@@ -18,7 +19,8 @@ namespace {
 size_t align_up(size_t v) { return (v + detag::kWsAlign - 1) / detag::kWsAlign * detag::kWsAlign; }
 
 struct WsLayout {
-  size_t status, result, row_ptr, col_idx, vals, poly, torus, split_blocks, split_exp, split_guard, split_poly, partials, total;
+  size_t status, result, row_ptr, col_idx, vals, poly, torus, partials, total;
+  struct { size_t weights, row_exp, guard, poly; } split, rows;
 };
 
 WsLayout ws_layout(const detag_state* s) {
@@ -37,14 +39,17 @@ WsLayout ws_layout(const detag_state* s) {
   off += align_up(s->poly.size() * sizeof(double));
   l.torus = off;
   off += align_up(s->torus_frag.size() * sizeof(double));
-  l.split_blocks = off;
-  off += align_up(s->split.blocks.size());
-  l.split_exp = off;
-  off += align_up(s->split.row_exp.size() * sizeof(int32_t));
-  l.split_guard = off;
-  off += align_up(s->split.guard.size() * sizeof(int32_t));
-  l.split_poly = off;
-  off += align_up(s->split.poly_t.size() * sizeof(double));
+  const std::pair<const detag::SplitPoly*, decltype(l.split)*> tables[2] = {{&s->split, &l.split}, {&s->rows, &l.rows}};
+  for (const auto& t : tables) {
+    t.second->weights = off;
+    off += align_up(t.first->weights.size());
+    t.second->row_exp = off;
+    off += align_up(t.first->row_exp.size() * sizeof(int32_t));
+    t.second->guard = off;
+    off += align_up(t.first->guard.size());
+    t.second->poly = off;
+    off += align_up(t.first->poly.size() * sizeof(double));
+  }
   l.partials = off;
   off += align_up(detag::kMaxPartials * sizeof(double));
   l.total = off;
@@ -289,7 +294,7 @@ StepParams make_params(const detag_state* s) {
   p.vals = s->d_vals;
   p.poly = s->d_poly;
   p.torus = s->d_torus;
-  p.split = s->d_split;
+  p.tables = s->d_tables;
   p.eta = s->eta;
   p.alpha = s->alpha;
   p.sigma = s->sigma;
@@ -360,7 +365,7 @@ int query_device(detag_state* s) {
 }
 
 // Kernel families that take tensor maps.
-enum { kFamilyMma = 1, kFamilyTorus = 2, kFamilyRing = 3, kFamilySplit = 4, kFamilyDense = 5 };
+enum { kFamilyMma = 1, kFamilyTorus = 2, kFamilyRing = 3, kFamilySplit = 4, kFamilyDense = 5, kFamilyRows = 6 };
 
 // Tensor maps for the buffers in `p`: built on first use, then found again by buffer addresses and sizes
 // (detag_step always hits; detag_step_host cycles through its two chunk slots and the ragged last chunk).
@@ -387,6 +392,7 @@ const detag::TensorMapSet* maps_for(detag_state* s, int family, const StepParams
                   : family == kFamilyRing ? detag::build_maps_ring(p, &en.maps)
                   : family == kFamilySplit ? detag::build_maps_split(p, &en.maps)
                   : family == kFamilyDense ? detag::build_maps_dense(p, &en.maps)
+                  : family == kFamilyRows  ? detag::build_maps_rows(p, &en.maps)
                                           : detag::build_maps_torus(p, &en.maps);
   if (!ok) return nullptr;
   en.family = family;
@@ -396,14 +402,17 @@ const detag::TensorMapSet* maps_for(detag_state* s, int family, const StepParams
   return &en.maps;
 }
 
-int launch_split(detag_state* s, const StepParams& p, bool wide, cudaStream_t stream) {
-  const detag::TensorMapSet* maps = maps_for(s, kFamilySplit, p);
+// The integer tensor path: lanes as coordinates, or (rows) as output workers.
+int launch_split(detag_state* s, const StepParams& p, bool rows, bool wide, cudaStream_t stream) {
+  const detag::TensorMapSet* maps = maps_for(s, rows ? kFamilyRows : kFamilySplit, p);
   if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
   const WsLayout l = ws_layout(s);
-  const detag::SplitDevice tables{p.split, reinterpret_cast<const int32_t*>(p.split + (l.split_exp - l.split_blocks)),
-                                  reinterpret_cast<const int32_t*>(p.split + (l.split_guard - l.split_blocks)),
-                                  reinterpret_cast<const double*>(p.split + (l.split_poly - l.split_blocks))};
-  const int e = detag::launch_step_split(p, *maps, s->split, tables, wide, s->sm_count, stream);
+  const auto& at = rows ? l.rows : l.split;
+  const unsigned char* base = p.tables;
+  const detag::SplitDevice tables{base + at.weights, reinterpret_cast<const int32_t*>(base + at.row_exp), base + at.guard,
+                                  reinterpret_cast<const double*>(base + at.poly)};
+  const int e = rows ? detag::launch_step_rows(p, *maps, s->rows, tables, wide, s->sm_count, stream)
+                     : detag::launch_step_split(p, *maps, s->split, tables, wide, s->sm_count, stream);
   return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
 }
 
@@ -419,7 +428,7 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   pt.a = p.a + first;
   pt.c = p.c + first;
   if (p.y_obs) pt.y_obs = p.y_obs + first;
-  if (!s->split.blocks.empty()) return launch_split(s, pt, false, stream);
+  if (!s->split.weights.empty() || !s->rows.weights.empty()) return launch_split(s, pt, s->split.weights.empty(), false, stream);
   const int rc = detag::plan_step_csr(pt, s->smem_optin);
   if (rc != DETAG_OK) return fail(s, rc, "graph too large for the shared-memory plan");
   const int e = detag::launch_step_csr(pt, s->sm_count, stream);
@@ -435,12 +444,38 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
 // in one.  Two launches -> one: 64 workers, K = 4, d = 9001 26 -> 16; 128, K = 4, d = 9001 39 -> 24, but K = 1, d = 20001
 // 61 -> 60; 256, K = 4, d = 4097 71 -> 43, but K = 1, d = 9001 70 -> 82.
 bool split_ok(const detag_state* s, const StepParams& p, int variant) {
-  if (s->split.blocks.empty() || p.mode == detag::kModeExternal || p.d > 0x7fffffffLL) return false;
+  if (p.d > 0x7fffffffLL) return false;
   if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
   if (variant == DETAG_VARIANT_DENSE) return true;
   if (variant != DETAG_VARIANT_RING) return false;
   // by the length of the state, not of a staged chunk: host-resident stepping gives the same bits
   return !ring_band(s) || (s->d % 64 != 0 && s->d <= (s->n <= 128 ? 2LL : 1LL) * 64 * s->sm_count);
+}
+
+// Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.1 -> 9.5, 20 k 31.9 -> 27.1,
+// 1 M 960 -> 880; 128, 40 k 53.0 -> 45.4; D-PSGD of 96, 10 k 17.5 -> 14.3, 1 M 709 -> 632, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
+// 5 k 12.3 -> 13.6; 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
+// calls whose blocks have at most 32 chunks of 32 coordinates to do.  What would run as rounds otherwise - caller-written gradients up to
+// 128 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Rounds -> here: caller-written,
+// 100 workers, d = 1 M 3177 -> 860, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 1034, 256 5327 -> 1832,
+// 180, K = 1, d = 72 k 225 against 230, ring of 144, K = 4, d = 8931 35.6 against 48.1.  Polynomials with few entries per row cost the
+// longer test of the operands, and more coordinates that fail it.  On short vectors rounds take their latency, one after the other:
+// caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
+bool rows_ok(const detag_state* s, const StepParams& p) {
+  if (s->rows.weights.empty()) return false;
+  const double d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * s->sm_count));
+  const double products = s->K * static_cast<double>(s->col_idx.size());
+  const bool sparse = s->rows.guard.size() > static_cast<size_t>(s->n);
+  if (p.mode == detag::kModeExternal) {
+    const double here = 9.0 + turns * (1.0 + 0.031 * p.n) * (sparse && p.n > 64 && p.n <= 96 ? 2.2 : 1.0);  // six warps for the test
+    const double rounds = std::fmax((0.0021 * p.n + 0.00099 * products) * d / 1000.0, 0.0155 * p.n * s->K);
+    return p.n <= 128 && here < std::fmax(8.0, 6.0 + rounds);
+  }
+  if (p.n <= 64) return turns <= 32.0;
+  if (p.n <= 96) return p.mode == detag::kModeDpsgd;
+  if (p.n <= 128) return true;
+  const double here = sparse ? 14.0 + 0.098 * p.n * turns : 10.0 + 0.065 * p.n * turns;
+  return here < std::fmax(std::fmax(8.0, 6.0 + 0.0068 * p.n * s->K), 1.25 * (0.024 * p.n + 0.00155 * products) * d / 2000.0);
 }
 
 // Up to 16 workers the step runs in registers, without staging.  us per step, tensor-path kernel with its stages and barriers
@@ -482,7 +517,11 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     e = detag::launch_step_dense(p, *maps, s->sm_count, stream);
     return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
   }
-  if (split_ok(s, p, variant)) return launch_split(s, p, variant == DETAG_VARIANT_CSR, stream);
+  if (split_ok(s, p, variant)) {
+    const bool rows = rows_ok(s, p);
+    if (rows || (!s->split.weights.empty() && p.mode != detag::kModeExternal))
+      return launch_split(s, p, rows, variant == DETAG_VARIANT_CSR, stream);
+  }
   // what the integer tensor path does not take although its variant promises it (a polynomial whose entries cannot be
   // scaled, e.g. under an absurd momentum) runs as rounds
   const bool as_rounds = (variant == DETAG_VARIANT_DENSE && p.n > 32) || (variant == DETAG_VARIANT_RING && !ring_band(s));
@@ -581,8 +620,13 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   analyse_torus(s);
   if (n > detag::kMaxDenseStepWorkers && n <= detag::kMaxSplitWorkers) {
     const bool blocks = block_circulant(s);
-    if (blocks) first_block_row(s, poly);
-    if (!poly.empty()) detag::split_polynomial(n, poly, blocks, s->split);  // else: too many distinct blocks
+    if (blocks) {
+      first_block_row(s, poly);
+    } else if (n > 128) {
+      gossip_polynomial(s, poly);
+    }
+    if (n <= 96 || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
+    if (n <= 128 || !blocks) detag::rows_polynomial(n, poly, blocks, s->rows);
   }
   s->map_cache.reserve(8);
   // the workspace's tables as they are uploaded, the cleared status block in front
@@ -596,10 +640,14 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   put(l.vals, s->vals.data(), s->vals.size() * sizeof(double));
   put(l.poly, s->poly.data(), s->poly.size() * sizeof(double));
   put(l.torus, s->torus_frag.data(), s->torus_frag.size() * sizeof(double));
-  put(l.split_blocks, s->split.blocks.data(), s->split.blocks.size());
-  put(l.split_exp, s->split.row_exp.data(), s->split.row_exp.size() * sizeof(int32_t));
-  put(l.split_guard, s->split.guard.data(), s->split.guard.size() * sizeof(int32_t));
-  put(l.split_poly, s->split.poly_t.data(), s->split.poly_t.size() * sizeof(double));
+  auto put_split = [&](const auto& at, const detag::SplitPoly& t) {
+    put(at.weights, t.weights.data(), t.weights.size());
+    put(at.row_exp, t.row_exp.data(), t.row_exp.size() * sizeof(int32_t));
+    put(at.guard, t.guard.data(), t.guard.size());
+    put(at.poly, t.poly.data(), t.poly.size() * sizeof(double));
+  };
+  put_split(l.split, s->split);
+  put_split(l.rows, s->rows);
   *out = s;
   return DETAG_OK;
 }
@@ -634,7 +682,7 @@ int detag_bind(detag_state* s, int64_t ld, float* x, float* y, float* g, const f
   s->d_vals = reinterpret_cast<double*>(base + l.vals);
   s->d_poly = s->poly.empty() ? nullptr : reinterpret_cast<double*>(base + l.poly);
   s->d_torus = s->torus_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.torus);
-  s->d_split = s->split.blocks.empty() ? nullptr : base + l.split_blocks;
+  s->d_tables = base;
   s->d_partials = reinterpret_cast<double*>(base + l.partials);
 
   e = cudaMemcpy(base, s->image.data(), s->image.size(), cudaMemcpyHostToDevice);  // status word and result cleared
@@ -911,7 +959,7 @@ int detag_step_host(detag_state* s, int64_t ld_host, float* x, float* y, float* 
   p.vals = reinterpret_cast<double*>(base + l.vals);
   p.poly = s->poly.empty() ? nullptr : reinterpret_cast<double*>(base + l.poly);
   p.torus = s->torus_frag.empty() ? nullptr : reinterpret_cast<double*>(base + l.torus);
-  p.split = s->split.blocks.empty() ? nullptr : base + l.split_blocks;
+  p.tables = base;
   p.status = status_word;
   p.y_obs = nullptr;
   p.t_noise = static_cast<uint32_t>(s->t + 1);

@@ -44,7 +44,7 @@ struct StepParams {
   const int32_t* col_idx;
   const double* vals;
   const double* poly;  // dense P_K(M), row-major n x n (null when n > 64)
-  const unsigned char* split;  // split kernel: digit blocks, row exponents, guard and P in the workspace (or null)
+  const unsigned char* tables;  // the workspace, for the integer tensor path's tables
   const double* torus; // block-circulant kernel: per-frequency 8 x 8 polynomial blocks in fragment order (or null)
   double eta;
   double alpha;
@@ -72,19 +72,19 @@ struct alignas(64) TensorMapSet {
   unsigned char bytes[8 * 128];
 };
 
-// P_K(M) as the split kernel (step_split.cu) takes it: the distinct 32 x 32 blocks of its base-256 digits, their table,
-// the exponent of every row's scale, the groups of inputs that tell when a coordinate's operands may share one scale, and P
-// itself (transposed).  Empty when the kernel does not take the matrix.
+// P_K(M) as a kernel of the integer tensor path takes it: its base-256 digits, the exponent of every row's scale, the groups of
+// inputs that tell when a coordinate's operands may share one scale, and P itself.  Empty when neither kernel takes the matrix.
 struct SplitPoly {
-  std::vector<unsigned char> blocks;
+  std::vector<unsigned char> weights;  // digits: tiles of 128 outputs x 32 inputs, or the distinct 32 x 32 blocks
   std::vector<int32_t> row_exp;
-  std::vector<double> poly_t;  // transposed, rows padded to a multiple of 16, their number to one of 32; or see circulant
-  std::vector<int32_t> guard;  // groups of guard_size inputs, as offsets into a staged column
+  std::vector<double> poly;  // in float64, padded; step_split.cu: transposed
+  std::vector<uint8_t> guard;  // groups of guard_size inputs
   int guard_size;
-  float guard_tau;       // each group's largest operand must be at least this share of the coordinate's largest
-  bool circulant;        // blocks depend on their distance only: poly_t holds output workers 0 .. 31
-  unsigned char id[64];  // [output block][input block] -> distinct block, 255: no digit of it is set
-  unsigned char reach[8];  // [output block], a bit per input block: some entry of P is not zero
+  float guard_tau;         // each group's largest operand must be at least this share of the coordinate's largest
+  bool circulant;          // the 32 x 32 blocks depend on their distance only: `poly` holds output workers 0 .. 31
+  unsigned char id[64];    // step_split.cu: [output block][input block] -> distinct block, 255: no digit of it is set
+  unsigned char used[2];   // step_rows.cu: [128 outputs], a bit per input block: a digit of its tile is set
+  unsigned char reach[8];  // [32 outputs], a bit per input block: some entry of P is not zero
 };
 
 // host helpers (spectral.cpp)
@@ -118,17 +118,25 @@ int launch_step_small(const StepParams& p, int sm_count, cudaStream_t stream);
 bool build_maps_dense(const StepParams& p, TensorMapSet* maps);
 int launch_step_dense(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);
 int launch_step_dense_many(const StepParams& p, const TensorMapSet& maps, int sm_count, cudaStream_t stream);  // n <= 32, p.steps steps
-// polynomial on the integer tensor path (step_split.cu): 48 < n <= 256, DeTAG and D-PSGD steps
+// polynomial on the integer tensor path, 48 < n <= 256
+void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& out);
+bool split_digits(int n, const std::vector<double>& poly, int rows, int wide, std::vector<int64_t>& digits, std::vector<int32_t>& row_exp);
+struct SplitDevice {  // the tables of a SplitPoly in the workspace
+  const void* weights;
+  const int32_t* row_exp;
+  const uint8_t* guard;
+  const double* poly;
+};
+// step_split.cu: lanes are coordinates; the distinct blocks have to fit in shared memory
 void split_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
 bool build_maps_split(const StepParams& p, TensorMapSet* maps);
-struct SplitDevice {  // the tables of a SplitPoly in the workspace
-  const void* blocks;
-  const int32_t* row_exp;
-  const int32_t* guard;
-  const double* poly_t;
-};
 int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& tables,
                       bool wide_gradient, int sm_count, cudaStream_t stream);
+// step_rows.cu: lanes are output workers; any matrix
+void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
+bool build_maps_rows(const StepParams& p, TensorMapSet* maps);
+int launch_step_rows(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& tables,
+                     bool wide_gradient, int sm_count, cudaStream_t stream);
 int launch_consensus_error(const StepParams& p, double* partials, double* result, int sm_count, cudaStream_t stream);
 int launch_init_external(const StepParams& p, int sm_count, cudaStream_t stream);  // y = g = g_ext
 int launch_expire_wait(int* status, unsigned polls, cudaStream_t stream);          // a wait nobody ends (self test)
@@ -153,7 +161,7 @@ struct detag_state {
   // 8 x 8 polynomial blocks in MMA fragment order
   bool torus = false;
   std::vector<double> torus_frag;
-  detag::SplitPoly split;         // 48 < n <= 256: P_K(M) for the integer tensor path (empty: not taken)
+  detag::SplitPoly split, rows;   // 48 < n <= 256: P_K(M) for the integer tensor path's two kernels (empty: not taken)
   std::vector<unsigned char> image;  // the workspace up to the partial sums, as it is uploaded
   int variant_forced = DETAG_VARIANT_AUTO;
   int gradient_point = DETAG_GRADIENT_AT_NEW_MODEL;
@@ -178,7 +186,7 @@ struct detag_state {
   double* d_vals = nullptr;
   double* d_poly = nullptr;
   double* d_torus = nullptr;
-  unsigned char* d_split = nullptr;  // blocks, row exponents, guard and P of `split`, one after the other (ws_layout)
+  const unsigned char* d_tables = nullptr;  // the workspace's beginning
   double* d_partials = nullptr;
 
   double sigma = 0.0;

@@ -1,0 +1,74 @@
+// What the two kernels of the integer tensor path share: how operands are scaled and split.
+#ifndef DETAG_DIGITS_CUH
+#define DETAG_DIGITS_CUH
+
+#include <cstdint>
+
+#include "packed.cuh"
+
+namespace detag {
+
+namespace {
+
+// As bits of a coordinate's largest magnitude.  Mantissas from 1.988 on count as the next power of two, so that five balanced digits
+// (at most 0x7F7F7F7F7F) hold every operand; maxima below 2^-90 leave the range of the float32 scale.
+constexpr unsigned kRoundUp = 0x18000u, kSmallest = 0x12800000u;
+
+// Digits of four workers' values x (+ rest, below an ulp of x): digit k of all four in d[k].  The value z scale, at most 31 bits before
+// the point, in two steps that float32 does exactly: its multiple of 2^14 next to it, and what is left in 1/256, each as the low bits
+// of 1.5 * 2^23 plus it.  With the 40-bit integer q of both, q + 0x0080808080 has the balanced digits as bytes, all but the top one
+// offset by 128.  No conversions: they run on a pipe a quarter as wide.
+template <bool kRest>
+__device__ __forceinline__ void digits_of(const F2 (&x)[2], const F2 (&rest)[2], float scale, uint32_t (&d)[5]) {
+  uint32_t z[4], f[4];
+#pragma unroll
+  for (int v = 0; v < 4; v += 2) {
+    const F2 high = fma2(x[v / 2], both(scale), both(206158430208.f));                          // 1.5 * 2^37
+    F2 left = fma2(x[v / 2], both(scale), sub2(both(206158430208.f), high));
+    if (kRest) left = fma2(rest[v / 2], both(scale), left);
+    const F2 low = fma2(left, both(256.f), both(12583040.f));                                   // 1.5 * 2^23 + 128
+    float h0, h1, f0, f1;
+    unpack2(high, h0, h1);
+    unpack2(low, f0, f1);
+    f[v] = __float_as_uint(f0);
+    f[v + 1] = __float_as_uint(f1);
+    z[v] = (__float_as_uint(h0) << 14) + ((f[v] >> 8) + (0x00808080u - 0x4B4000u));
+    z[v + 1] = (__float_as_uint(h1) << 14) + ((f[v + 1] >> 8) + (0x00808080u - 0x4B4000u));
+  }
+  const uint32_t ab = __byte_perm(z[0], z[1], 0x5140), cd = __byte_perm(z[2], z[3], 0x5140);
+  const uint32_t ef = __byte_perm(z[0], z[1], 0x7362), gh = __byte_perm(z[2], z[3], 0x7362);
+  d[0] = __byte_perm(__byte_perm(f[0], f[1], 0x0040), __byte_perm(f[2], f[3], 0x0040), 0x5410) ^ 0x80808080u;
+  d[1] = __byte_perm(ab, cd, 0x5410) ^ 0x80808080u;
+  d[2] = __byte_perm(ab, cd, 0x7632) ^ 0x80808080u;
+  d[3] = __byte_perm(ef, gh, 0x5410) ^ 0x80808080u;
+  d[4] = __byte_perm(ef, gh, 0x7632);
+}
+
+// Of four workers, `pitch` floats apart.
+__device__ __forceinline__ void four_digits(const float* src, int pitch, float scale, uint32_t (&d)[5]) {
+  const F2 x[2] = {pack2(src[0], src[pitch]), pack2(src[2 * pitch], src[3 * pitch])};
+  digits_of<false>(x, x, scale, d);
+}
+
+// Of the sums y + (g_new - g) of four workers, the three arrays `array` floats apart: both operations' roundings are added up exactly
+// (Knuth's two-sum) and rounded once, which leaves 2^-48 of the largest of the three.
+__device__ __forceinline__ void four_fold_digits(const float* src, int array, int pitch, float scale, uint32_t (&d)[5]) {
+  F2 x[2], rest[2];
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    const float* const at = src + 2 * v * pitch;
+    const F2 y = pack2(at[0], at[pitch]), b = pack2(at[array], at[array + pitch]), a = pack2(at[2 * array], at[2 * array + pitch]);
+    const F2 t = sub2(b, a), tb = sub2(t, b);                              // g_new - g, and the part of it that stands for -g
+    const F2 e1 = sub2(sub2(b, sub2(t, tb)), add2(a, tb));
+    x[v] = add2(y, t);
+    const F2 xt = sub2(x[v], y);
+    const F2 e2 = add2(sub2(y, sub2(x[v], xt)), sub2(t, xt));
+    rest[v] = add2(e1, e2);
+  }
+  digits_of<true>(x, rest, scale, d);
+}
+
+}  // namespace
+
+}  // namespace detag
+#endif  // DETAG_DIGITS_CUH

@@ -1,0 +1,132 @@
+// Host part of the integer tensor path (step_split.cu, step_rows.cu): the balanced base-256 digits of the gossip polynomial, and
+// the groups of inputs that tell which coordinates may share one scale.
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <vector>
+
+#include "detag_internal.h"
+
+namespace detag {
+
+// Groups of inputs for the test described in step_split.cu, for the n x n matrix whose first `rows` rows are given (the others
+// follow from the block structure).  For each theta and group size a greedy cover: take an output that no group serves yet
+// and add those of its inputs, one after the other, that keep the most other such outputs served.  Kept is the one with the
+// least expected work: reads of its groups against coordinates in float64, if operands were drawn alike (an operand is below
+// tau of the largest with a probability of about 2 tau, a group with its size's power of that) and, weighing less, if their
+// magnitudes were spread evenly over four decades.
+void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& out) {
+  constexpr int kWords = 4, kLevels = 7;
+  // level[i][j] = k: output i gives input j between 2^-k and 2^(1 - k) of its largest weight (0: all of it)
+  std::vector<uint8_t> level(static_cast<size_t>(n) * n, 255);
+  int terms = 1;
+  for (int i = 0; i < n; ++i) {
+    const double* row = &poly[static_cast<size_t>(i % rows) * n];
+    const int shift = i / rows * rows;  // rows beyond the given ones: the block structure moves them
+    double top = 0.0;
+    int count = 0;
+    for (int j = 0; j < n; ++j) {
+      top = std::fmax(top, std::fabs(row[j]));
+      count += row[j] != 0.0 ? 1 : 0;
+    }
+    terms = std::max(terms, count);
+    for (int j = 0; j < n; ++j) {
+      const double r = std::fabs(row[j]) / (0.999999 * top);
+      const int k = r >= 1.0 ? 0 : r >= 1.0 / (1 << (kLevels - 1)) ? -std::ilogb(r) : 255;
+      level[static_cast<size_t>(i) * n + (j + shift < n ? j + shift : j + shift - n)] = static_cast<uint8_t>(k);
+    }
+  }
+  const int stride = n % 2 == 0 ? n / 2 - (n % 4 == 0 ? 1 : 2) : n / 2;  // coprime to n: ties go to inputs far apart
+  double best = 1e300;
+  std::vector<uint64_t> readers(static_cast<size_t>(n) * kWords, 0);  // [input]: outputs that give it at least theta
+  std::vector<int> inputs;
+  std::vector<uint8_t> groups;
+  for (int k = 0; k < kLevels && best > 0.25 * n; ++k) {
+    const double tau = std::sqrt(static_cast<double>(terms)) / 4096.0 * (1 << k);
+    if (tau > 0.5) break;
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j)
+        if (level[static_cast<size_t>(i) * n + j] == k) readers[static_cast<size_t>(j) * kWords + i / 64] |= 1ull << (i % 64);
+    const double small = std::fmax(0.0, 1.0 - std::log2(1.0 / tau) / 13.3);
+    int largest = 32;  // of a group, as far as its outputs have such inputs
+    for (int size = 2; size <= 32 && size / 2 <= largest && best > 0.25 * n; size *= 2) {
+      uint64_t open[kWords] = {0, 0, 0, 0};
+      for (int i = 0; i < n; ++i) open[i / 64] |= 1ull << (i % 64);
+      groups.clear();
+      largest = 0;
+      double fail = 0.0, fail_spread = 0.0;
+      for (int i = 0; i < n && groups.size() <= 2 * static_cast<size_t>(n) && groups.size() < best; ++i) {
+        if ((open[i / 64] >> (i % 64) & 1) == 0) continue;
+        inputs.clear();
+        for (int v = 0, j = i; v < n; ++v, j = j + stride < n ? j + stride : j + stride - n)
+          if (level[static_cast<size_t>(i) * n + j] <= k) inputs.push_back(j);
+        uint64_t served[kWords];
+        std::copy(open, open + kWords, served);
+        int have = 0;
+        uint8_t last = 0;
+        double p = 1.0, p_spread = 1.0;
+        for (; have < size && have < static_cast<int>(inputs.size()); ++have, p *= 2.0 * tau, p_spread *= small) {
+          int pick = have, most = -1;
+          for (int v = have; v < static_cast<int>(inputs.size()); ++v) {
+            const uint64_t* r = &readers[static_cast<size_t>(inputs[v]) * kWords];
+            int count = 0;
+            for (int w = 0; w < kWords; ++w) count += __builtin_popcountll(served[w] & r[w]);
+            if (count > most) {
+              most = count;
+              pick = v;
+            }
+          }
+          std::swap(inputs[have], inputs[pick]);
+          const int j = inputs[have];
+          for (int w = 0; w < kWords; ++w) served[w] &= readers[static_cast<size_t>(j) * kWords + w];
+          last = static_cast<uint8_t>(j);
+          groups.push_back(last);
+        }
+        largest = std::max(largest, have);
+        for (; have < size; ++have) groups.push_back(last);
+        for (int w = 0; w < kWords; ++w) open[w] &= ~served[w];
+        fail += p;
+        fail_spread += p_spread;
+      }
+      const double work = groups.size() + n * (6000.0 * std::fmin(fail, 1.0) + 40.0 * std::fmin(fail_spread, 1.0));
+      if (groups.size() <= 2 * static_cast<size_t>(n) && work < best) {
+        best = work;
+        out.guard = groups;
+        out.guard_size = size;
+        out.guard_tau = static_cast<float>(tau);
+      }
+    }
+  }
+  if (out.guard.empty()) {  // nothing to tell the coordinates by: all in float64 (one input is as good as another)
+    out.guard.assign(2, 0);
+    out.guard_size = 2;
+    out.guard_tau = 2.f;
+  }
+}
+
+// Digits of the `rows` given rows of the n x n matrix, as bytes of 64-bit integers (`wide` per row, zeros beyond n), and the exponent
+// of every row's scale (rows beyond the given ones: the block structure repeats them).  False if an entry or a row cannot be scaled.
+bool split_digits(int n, const std::vector<double>& poly, int rows, int wide, std::vector<int64_t>& digits, std::vector<int32_t>& row_exp) {
+  constexpr long long kMaxDigits = 0x7F7F7F7F7FLL;  // largest integer with five balanced digits
+  digits.assign(static_cast<size_t>(rows) * wide, 0);
+  row_exp.assign(n, 0);
+  for (int i = 0; i < rows; ++i) {
+    const double* row = &poly[static_cast<size_t>(i) * n];
+    double top = 0.0;
+    for (int j = 0; j < n; ++j) {
+      const double v = std::fabs(row[j]);
+      if (!(v <= 1e30)) return false;  // also NaN
+      top = v > top ? v : top;
+    }
+    if (!(top >= 1e-30)) return false;
+    int e = std::ilogb(top);
+    if (std::nearbyint(std::ldexp(top, 38 - e)) > static_cast<double>(kMaxDigits)) ++e;
+    for (int k = i; k < n; k += rows) row_exp[k] = e - 30;
+    const double scale = std::ldexp(1.0, 38 - e);
+    for (int j = 0; j < n; ++j)
+      digits[static_cast<size_t>(i) * wide + j] = (std::llrint(row[j] * scale) + 0x8080808080LL) ^ 0x8080808080LL;
+  }
+  return true;
+}
+
+}  // namespace detag

@@ -64,6 +64,7 @@
 
 #include "chain.cuh"
 #include "detag_internal.h"
+#include "digits.cuh"
 #include "noise.cuh"
 #include "packed.cuh"
 #include "pipeline.cuh"
@@ -99,9 +100,6 @@ static_assert(digit_buffers(2) * 40 * 2 + accumulators(false) * kPAccColumns <= 
                   digit_buffers(4) * 40 * 4 + accumulators(false) * kPAccColumns <= kTmemColumns &&
                   digit_buffers(8) * 40 * 8 + accumulators(true) * kPAccColumns <= kTmemColumns,
               "tensor memory plan");
-constexpr long long kMaxDigits = 0x7F7F7F7F7FLL;  // largest integer with five balanced digits
-constexpr unsigned kRoundUp = 0x18000u;      // mantissas from 1.988 on count as the next power of two (see kMaxDigits)
-constexpr unsigned kSmallest = 0x12800000u;  // 2^-90: smaller maxima leave the range of the float32 scale
 constexpr size_t kPCtrlBytes = 640, kPSmemLimit = 232448;
 
 struct SplitMaps {
@@ -120,7 +118,7 @@ struct SplitTables {
   int circulant;
   int num_blocks;
   int nb;                  // 32-worker blocks per side
-  const int* guard;        // guard_groups x guard_size inputs, as offsets into a coordinate's staged column
+  const uint8_t* guard;    // guard_groups x guard_size inputs
   int guard_groups, guard_size;  // size 2 or a multiple of 4
   float guard_tau;
   uint64_t id[8];          // [output chunk], a byte per input block: distinct block, 255: no digit of it is set
@@ -229,36 +227,16 @@ __device__ __forceinline__ float group_low(const float* col, const int* guard, i
   return low;
 }
 
-// Digits of a block's 32 workers (zeros beyond n): digit 0 in w0, digit k in words 8 (k - 1) .. 8 k - 1 of w.  The value
-// z scale, at most 31 bits before the point, in two steps that float32 does exactly: its multiple of 2^14 next to it, and
-// what is left in 1/256, each as the low bits of 1.5 * 2^23 plus it.  With the 40-bit integer q of both, q + 0x0080808080
-// has the balanced digits as bytes, all but the top one offset by 128.  No conversions: they run on a pipe a quarter as wide.  No test per row:
+// Digits of a block's 32 workers (zeros beyond n): digit 0 in w0, digit k in words 8 (k - 1) .. 8 k - 1 of w.  No test per row:
 // the splitting is a serial chain, and so its loads and chains overlap.
 __device__ __forceinline__ void block_digits(const float* src, float scale, uint32_t (&w)[32], uint32_t (&w0)[8]) {
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
-    uint32_t z[4], f[4];
+    uint32_t d[5];
+    four_digits(src + 4 * u * kPS, kPS, scale, d);
+    w0[u] = d[0];
 #pragma unroll
-    for (int v = 0; v < 4; v += 2) {
-      const F2 x = pack2(src[(4 * u + v) * kPS], src[(4 * u + v + 1) * kPS]);
-      const F2 high = fma2(x, both(scale), both(206158430208.f));                          // 1.5 * 2^37
-      const F2 rest = fma2(x, both(scale), sub2(both(206158430208.f), high));
-      const F2 low = fma2(rest, both(256.f), both(12583040.f));                            // 1.5 * 2^23 + 128
-      float h0, h1, f0, f1;
-      unpack2(high, h0, h1);
-      unpack2(low, f0, f1);
-      f[v] = __float_as_uint(f0);
-      f[v + 1] = __float_as_uint(f1);
-      z[v] = (__float_as_uint(h0) << 14) + ((f[v] >> 8) + (0x00808080u - 0x4B4000u));
-      z[v + 1] = (__float_as_uint(h1) << 14) + ((f[v + 1] >> 8) + (0x00808080u - 0x4B4000u));
-    }
-    const uint32_t ab = __byte_perm(z[0], z[1], 0x5140), cd = __byte_perm(z[2], z[3], 0x5140);
-    const uint32_t ef = __byte_perm(z[0], z[1], 0x7362), gh = __byte_perm(z[2], z[3], 0x7362);
-    w0[u] = __byte_perm(__byte_perm(f[0], f[1], 0x0040), __byte_perm(f[2], f[3], 0x0040), 0x5410) ^ 0x80808080u;
-    w[u] = __byte_perm(ab, cd, 0x5410) ^ 0x80808080u;
-    w[8 + u] = __byte_perm(ab, cd, 0x7632) ^ 0x80808080u;
-    w[16 + u] = __byte_perm(ef, gh, 0x5410) ^ 0x80808080u;
-    w[24 + u] = __byte_perm(ef, gh, 0x7632);
+    for (int k = 1; k < 5; ++k) w[8 * (k - 1) + u] = d[k];
   }
 }
 
@@ -307,7 +285,8 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     uint4* dst = reinterpret_cast<uint4*>(smem + plan.blocks_at);
     for (int e = tid; e < tb.num_blocks * (kPBlockBytes / 16); e += blockDim.x) dst[e] = src[e];
     for (int e = tid; e < 256; e += blockDim.x) row_scale[e] = __hiloint2double((1023 + (e < n ? tb.row_exp[e] : 0)) << 20, 0);
-    for (int e = tid; e < tb.guard_groups * tb.guard_size; e += blockDim.x) guard[e] = tb.guard[e];
+    for (int e = tid; e < tb.guard_groups * tb.guard_size; e += blockDim.x)  // as offsets into a coordinate's staged column
+      guard[e] = tb.guard[e] / kPChunk * (2 * kPTileFloats) + tb.guard[e] % kPChunk * kPS;
   }
   if (tid == 0) {
     bar_init(xy_full, 1);
@@ -830,100 +809,6 @@ SplitKernel pick_split(const StepParams& p, bool wide) {
 
 }  // namespace
 
-// Groups of inputs for the test described at the top, for the n x n matrix whose first `rows` rows are given (the others
-// follow from the block structure).  For each theta and group size a greedy cover: take an output that no group serves yet
-// and add those of its inputs, one after the other, that keep the most other such outputs served.  Kept is the one with the
-// least expected work: reads of its groups against coordinates in float64, if operands were drawn alike (an operand is below
-// tau of the largest with a probability of about 2 tau, a group with its size's power of that) and, weighing less, if their
-// magnitudes were spread evenly over four decades.
-void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& out) {
-  constexpr int kWords = 4, kLevels = 7;
-  // level[i][j] = k: output i gives input j between 2^-k and 2^(1 - k) of its largest weight (0: all of it)
-  std::vector<uint8_t> level(static_cast<size_t>(n) * n, 255);
-  int terms = 1;
-  for (int i = 0; i < n; ++i) {
-    const double* row = &poly[static_cast<size_t>(i % rows) * n];
-    const int shift = i / rows * rows;  // rows beyond the given ones: the block structure moves them
-    double top = 0.0;
-    int count = 0;
-    for (int j = 0; j < n; ++j) {
-      top = std::fmax(top, std::fabs(row[j]));
-      count += row[j] != 0.0 ? 1 : 0;
-    }
-    terms = std::max(terms, count);
-    for (int j = 0; j < n; ++j) {
-      const double r = std::fabs(row[j]) / (0.999999 * top);
-      const int k = r >= 1.0 ? 0 : r >= 1.0 / (1 << (kLevels - 1)) ? -std::ilogb(r) : 255;
-      level[static_cast<size_t>(i) * n + (j + shift < n ? j + shift : j + shift - n)] = static_cast<uint8_t>(k);
-    }
-  }
-  const int stride = n % 2 == 0 ? n / 2 - (n % 4 == 0 ? 1 : 2) : n / 2;  // coprime to n: ties go to inputs far apart
-  double best = 1e300;
-  std::vector<uint64_t> readers(static_cast<size_t>(n) * kWords, 0);  // [input]: outputs that give it at least theta
-  std::vector<int> inputs;
-  std::vector<int32_t> groups;
-  for (int k = 0; k < kLevels && best > 0.25 * n; ++k) {
-    const double tau = std::sqrt(static_cast<double>(terms)) / 4096.0 * (1 << k);
-    if (tau > 0.5) break;
-    for (int i = 0; i < n; ++i)
-      for (int j = 0; j < n; ++j)
-        if (level[static_cast<size_t>(i) * n + j] == k) readers[static_cast<size_t>(j) * kWords + i / 64] |= 1ull << (i % 64);
-    const double small = std::fmax(0.0, 1.0 - std::log2(1.0 / tau) / 13.3);
-    int largest = 32;  // of a group, as far as its outputs have such inputs
-    for (int size = 2; size <= 32 && size / 2 <= largest && best > 0.25 * n; size *= 2) {
-      uint64_t open[kWords] = {0, 0, 0, 0};
-      for (int i = 0; i < n; ++i) open[i / 64] |= 1ull << (i % 64);
-      groups.clear();
-      largest = 0;
-      double fail = 0.0, fail_spread = 0.0;
-      for (int i = 0; i < n && groups.size() <= 2 * static_cast<size_t>(n) && groups.size() < best; ++i) {
-        if ((open[i / 64] >> (i % 64) & 1) == 0) continue;
-        inputs.clear();
-        for (int v = 0, j = i; v < n; ++v, j = j + stride < n ? j + stride : j + stride - n)
-          if (level[static_cast<size_t>(i) * n + j] <= k) inputs.push_back(j);
-        uint64_t served[kWords];
-        std::copy(open, open + kWords, served);
-        int have = 0, last = 0;
-        double p = 1.0, p_spread = 1.0;
-        for (; have < size && have < static_cast<int>(inputs.size()); ++have, p *= 2.0 * tau, p_spread *= small) {
-          int pick = have, most = -1;
-          for (int v = have; v < static_cast<int>(inputs.size()); ++v) {
-            const uint64_t* r = &readers[static_cast<size_t>(inputs[v]) * kWords];
-            int count = 0;
-            for (int w = 0; w < kWords; ++w) count += __builtin_popcountll(served[w] & r[w]);
-            if (count > most) {
-              most = count;
-              pick = v;
-            }
-          }
-          std::swap(inputs[have], inputs[pick]);
-          const int j = inputs[have];
-          for (int w = 0; w < kWords; ++w) served[w] &= readers[static_cast<size_t>(j) * kWords + w];
-          last = j / kPChunk * (2 * kPTileFloats) + j % kPChunk * kPS;
-          groups.push_back(last);
-        }
-        largest = std::max(largest, have);
-        for (; have < size; ++have) groups.push_back(last);
-        for (int w = 0; w < kWords; ++w) open[w] &= ~served[w];
-        fail += p;
-        fail_spread += p_spread;
-      }
-      const double work = groups.size() + n * (6000.0 * std::fmin(fail, 1.0) + 40.0 * std::fmin(fail_spread, 1.0));
-      if (groups.size() <= 2 * static_cast<size_t>(n) && work < best) {
-        best = work;
-        out.guard = groups;
-        out.guard_size = size;
-        out.guard_tau = static_cast<float>(tau);
-      }
-    }
-  }
-  if (out.guard.empty()) {  // nothing to tell the coordinates by: all in float64 (one input is as good as another)
-    out.guard.assign(2, 0);
-    out.guard_size = 2;
-    out.guard_tau = 2.f;
-  }
-}
-
 // Digits of P: distinct 32 x 32 blocks, their table and the rows' exponents.  `poly`: the n x n matrix, or (circulant: the
 // blocks depend on their distance only) its first 32 rows.  Leaves `out` empty when the kernel does not take the matrix:
 // n outside 33 .. 256, an entry or a row that cannot be scaled, too many distinct blocks.
@@ -931,24 +816,10 @@ void split_polynomial(int n, const std::vector<double>& poly, bool circulant, Sp
   out = SplitPoly{};
   if (n <= 32 || n > 256 || encode_tiled_fn() == nullptr) return;
   const int nb = (n + kPChunk - 1) / kPChunk, rows = circulant ? kPChunk : n, wide = nb * kPChunk;
-  std::vector<int64_t> digits(static_cast<size_t>(circulant ? 1 : nb) * kPChunk * wide, 0);  // balanced digits as bytes
-  std::vector<int32_t> row_exp(n);
-  for (int i = 0; i < rows; ++i) {
-    const double* row = &poly[static_cast<size_t>(i) * n];
-    double top = 0.0;
-    for (int j = 0; j < n; ++j) {
-      const double v = std::fabs(row[j]);
-      if (!(v <= 1e30)) return;  // also NaN
-      top = v > top ? v : top;
-    }
-    if (!(top >= 1e-30)) return;
-    int e = std::ilogb(top);
-    if (std::nearbyint(std::ldexp(top, 38 - e)) > static_cast<double>(kMaxDigits)) ++e;
-    for (int k = i; k < n; k += rows) row_exp[k] = e - 30;
-    const double scale = std::ldexp(1.0, 38 - e);
-    for (int j = 0; j < n; ++j)
-      digits[static_cast<size_t>(i) * wide + j] = (std::llrint(row[j] * scale) + 0x8080808080LL) ^ 0x8080808080LL;
-  }
+  std::vector<int64_t> digits;
+  std::vector<int32_t> row_exp;
+  if (!split_digits(n, poly, rows, wide, digits, row_exp)) return;
+  digits.resize(static_cast<size_t>(circulant ? 1 : nb) * kPChunk * wide, 0);
   SplitPoly made{};
   split_guard(n, poly, rows, made);
   std::vector<unsigned char> blocks;
@@ -988,10 +859,10 @@ void split_polynomial(int n, const std::vector<double>& poly, bool circulant, Sp
         made.reach[c] |= static_cast<unsigned char>((made.reach[0] >> ((kb - c + nb) % nb) & 1) << kb);
       }
   const size_t pitch = circulant ? kPChunk : static_cast<size_t>((n + kPUnit - 1) / kPUnit) * kPUnit;
-  made.poly_t.assign(wide * pitch, 0.0);
+  made.poly.assign(wide * pitch, 0.0);
   for (int i = 0; i < rows; ++i)
-    for (int j = 0; j < n; ++j) made.poly_t[j * pitch + i] = poly[static_cast<size_t>(i) * n + j];
-  made.blocks.swap(blocks);
+    for (int j = 0; j < n; ++j) made.poly[j * pitch + i] = poly[static_cast<size_t>(i) * n + j];
+  made.weights.swap(blocks);
   made.row_exp.swap(row_exp);
   made.circulant = circulant;
   out = std::move(made);
@@ -1014,19 +885,19 @@ bool build_maps_split(const StepParams& p, TensorMapSet* out) {
 
 int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& dev, bool wide,
                       int sm_count, cudaStream_t stream) {
-  if (p.mode == kModeExternal || poly.blocks.empty()) return static_cast<int>(cudaErrorInvalidValue);
+  if (p.mode == kModeExternal || poly.weights.empty()) return static_cast<int>(cudaErrorInvalidValue);
   p.S = kPS;
   p.num_slabs = (p.d + kPS - 1) / kPS;
   SplitTables tb{};
-  tb.blocks = static_cast<const uint4*>(dev.blocks);
+  tb.blocks = static_cast<const uint4*>(dev.weights);
   tb.row_exp = dev.row_exp;
-  tb.poly_t = dev.poly_t;
+  tb.poly_t = dev.poly;
   tb.guard = dev.guard;
   tb.guard_size = poly.guard_size;
   tb.guard_groups = static_cast<int>(poly.guard.size()) / poly.guard_size;
   tb.guard_tau = poly.guard_tau;
   tb.circulant = poly.circulant ? 1 : 0;
-  tb.num_blocks = static_cast<int>(poly.blocks.size() / kPBlockBytes);
+  tb.num_blocks = static_cast<int>(poly.weights.size() / kPBlockBytes);
   tb.nb = (p.n + kPChunk - 1) / kPChunk;
   std::memcpy(tb.id, poly.id, sizeof tb.id);
   std::memcpy(tb.reach, poly.reach, sizeof tb.reach);

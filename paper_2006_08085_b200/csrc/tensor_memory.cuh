@@ -79,6 +79,17 @@ __device__ __forceinline__ void mma_i8(uint32_t d, uint32_t a, uint64_t b, uint3
       : "memory");
 }
 
+// The same with A[128][32 bytes] in shared memory.
+__device__ __forceinline__ void mma_i8_shared(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, unsigned accumulate, bool leader) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %4, 0;\n\t"
+      "setp.ne.u32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(leader ? 1u : 0u)
+      : "memory");
+}
+
 // The barrier gets one arrival when every MMA the leader has issued so far is complete.
 __device__ __forceinline__ void mma_commit(uint64_t* bar, bool leader) {
   asm volatile(

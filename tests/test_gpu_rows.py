@@ -1,0 +1,114 @@
+"""The integer tensor path with output workers as lanes (step_rows.cu): the sizes at which its plan changes (64, 128 workers, planes of
+the polynomial in tensor memory or through a ring), caller-written gradients, coordinates summed in float64."""
+import numpy as np
+import pytest
+
+from paper_2006_08085_b200 import build, inputs
+from paper_2006_08085_b200.session import Session
+from test_gpu_split import (_graph, _polynomial, _unequal, test_dpsgd as dpsgd, test_every_result_is_as_precise_as_what_it_reads as precision,
+                            test_one_step_against_the_oracle as one_step, test_what_is_not_finite_stays_in_reach as not_finite)
+
+pytestmark = pytest.mark.gpu
+
+CHUNKS = 32 * 148  # one chunk of 32 coordinates per block
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+# below, at and beyond a chunk, one and several per block and (beyond 16 per block) chunks in pairs; odd numbers of chunks
+@pytest.mark.parametrize("n,d,K,kind,at_start", [
+    (49, 31, 3, "regular4", False), (64, 33, 4, "ring", True), (64, 17 * CHUNKS + 33, 3, "regular4", False), (65, 3 * CHUNKS + 5, 3, "path", False),
+    (97, 17 * CHUNKS + 2, 4, "regular4", True), (128, 18 * CHUNKS + 31, 5, "regular4", False),
+    (129, 65, 4, "ring", False), (130, 3 * CHUNKS + 5, 6, "path", False), (150, 5 * CHUNKS + 67, 2, "regular4", True), (161, 130, 7, "directed", False),
+    (200, 63, 12, "regular4", False), (255, 2 * CHUNKS + 3, 9, "ring", True), (256, 17 * CHUNKS + 66, 5, "regular4", False)])
+def test_one_step(n, d, K, kind, at_start):
+    one_step(n, d, K, kind, at_start)
+
+
+@pytest.mark.parametrize("kind,n", [("regular4", 144), ("ring", 181), ("regular4", 256)])
+@pytest.mark.parametrize("K", [3, 16])
+def test_precision_beyond_128_workers(kind, n, K):
+    precision(kind, n, K)
+
+
+def test_dpsgd_and_infinities_beyond_128_workers():
+    dpsgd(171, 5 * CHUNKS + 9)
+    not_finite(171, np.inf)
+
+
+@pytest.mark.parametrize("n,d,K,kind", [(49, 1, 1, "regular4"), (50, 35, 2, "ring"), (64, 2 * CHUNKS + 34, 4, "regular4"), (65, 97, 6, "path"),
+                                        (100, 5 * CHUNKS + 7, 2, "regular4"), (128, 17 * CHUNKS + 33, 9, "regular4")])
+def test_caller_written_gradients(n, d, K, kind):
+    """x' = P x - alpha y', y' = P (y + g_new - g), g' = g_new: two steps, the second with operands of unequal size.  Bound: half an
+    ulp of what is stored, and as much again relative to the magnitudes that the result reads for the sums; the folded operand itself
+    carries 2^-40 of its three parts."""
+    eta, alpha = 0.2, 0.05
+    m = _graph(kind, n)
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(n + d)
+    zero = np.zeros((n, d), np.float32)
+    cols = slice(0, d) if d <= 5000 else np.unique(np.concatenate([np.arange(200), np.arange(d - 200, d), rng.integers(0, d, 400)]))
+    with Session(m, d, K, eta, alpha, zero, zero, zero, external_gradient=True, observe_gossip=True) as s:
+        for pattern in ("alike", "log-uniform"):
+            state = {"x": _unequal(pattern, n, d, rng), "y": _unequal(pattern, n, d, rng), "g": (30 * rng.standard_normal((n, d))).astype(np.float32),
+                     "g_new": (30 * rng.standard_normal((n, d))).astype(np.float32)}
+            for k, v in state.items():
+                s.upload(k, v)
+            s.step()
+            s.status()
+            got = {k: s.download(k)[:, cols].astype(np.float64) for k in ("x", "y", "g", "y_gossip")}
+            x, y, g, gn = (state[k][:, cols].astype(np.float64) for k in ("x", "y", "g", "g_new"))
+            z, parts = y + gn - g, np.abs(y) + np.abs(gn) + np.abs(g)
+            yt = P @ z
+            of_y = 2.0 ** -24 * (np.abs(yt) + np.abs(P) @ np.abs(z)) + 2.0 ** -40 * (np.abs(P) @ parts) + 1e-45
+            xt = P @ x - alpha * yt
+            of_x = 2.0 ** -24 * (np.abs(xt) + np.abs(P) @ np.abs(x)) + alpha * of_y + 1e-45
+            assert (np.abs(got["y"] - yt) <= of_y).all()
+            assert (np.abs(got["x"] - xt) <= of_x).all()
+            assert np.array_equal(got["g"], gn) and np.array_equal(got["y_gossip"], got["y"])
+
+
+def test_caller_written_gradients_that_are_not_finite():
+    n, d, K, eta = 70, 40, 2, 0.2
+    m = _graph("ring", n)
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(7)
+    zero = np.zeros((n, d), np.float32)
+    y, g, gn = (rng.standard_normal((n, d)).astype(np.float32) for _ in range(3))
+    gn[9, 35] = np.inf
+    with Session(m, d, K, eta, 0.0, zero, zero, zero, external_gradient=True) as s:
+        for k, v in (("y", y), ("g", g), ("g_new", gn)):
+            s.upload(k, v)
+        s.step()
+        s.status()
+        got, g_out = s.download("y"), s.download("g")
+    reached = P[:, 9] != 0.0
+    assert not np.isfinite(got[reached, 35]).any()
+    keep = np.ones((n, d), bool)
+    keep[reached, 35] = False
+    gn0 = np.where(np.isfinite(gn), gn, 0.0).astype(np.float64)
+    want = P @ (y.astype(np.float64) + gn0 - g)
+    assert (np.abs(got - want)[keep] <= 1e-5 * (1.0 + np.abs(want[keep]))).all()
+    assert np.array_equal(g_out, gn)
+
+
+@pytest.mark.parametrize("n,mode", [(60, "detag"), (90, "dpsgd"), (100, "detag"), (144, "detag"), (100, "external")])
+def test_rows_further_apart_give_the_same_bits(n, mode):
+    from paper_2006_08085_b200 import binding as B
+    d, m = 3 * CHUNKS + 3, _graph("regular4", n)
+    rng = np.random.default_rng(n)
+    state = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c", "g_new")}
+    got = []
+    for ld in (None, (d + 3) // 4 * 4 + 20):
+        with Session(m, d, 6, 0.2, 0.01, sigma=0.1, seed=5, ld=ld, external_gradient=mode == "external",
+                     algorithm=B.DETAG_ALGORITHM_DPSGD if mode == "dpsgd" else B.DETAG_ALGORITHM_DETAG) as s:
+            for k, v in state.items():
+                if k != "g_new" or mode == "external":
+                    s.upload(k, v)
+            s.step(2)
+            s.status()
+            got.append({k: s.download(k) for k in ("x", "y", "g")})
+    assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])
