@@ -416,8 +416,10 @@ int launch_split(detag_state* s, const StepParams& p, bool rows, bool wide, cuda
   return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
 }
 
-// The columns from `first` on, which the circulant kernel leaves (it takes whole 64-coordinate slabs), in the same call:
-// through the integer tensor path where that takes the matrix (one slab), else through the generic rounds kernel.
+// The columns from `first` on, which the circulant kernel leaves (it takes whole 64-coordinate slabs), in the same call, beside
+// it (64-ring, K = 4, d = 14001 21.3 -> 14.6 us in one launch, 256, d = 60001 188 -> 168 in two): through the integer tensor path up to
+// 128 workers (one chunk or two 8 .. 11 us), beyond as rounds while their latency is the smaller one (256 workers 6 us and 1.7 a round,
+// step_split.cu's slab 38).
 int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cudaStream_t stream) {
   StepParams pt = p;
   pt.d = p.d - first;
@@ -428,7 +430,9 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   pt.a = p.a + first;
   pt.c = p.c + first;
   if (p.y_obs) pt.y_obs = p.y_obs + first;
-  if (!s->split.weights.empty() || !s->rows.weights.empty()) return launch_split(s, pt, s->split.weights.empty(), false, stream);
+  pt.beside = first > 0 ? 1 : 0;
+  if (p.n <= 128 && !s->rows.weights.empty()) return launch_split(s, pt, true, false, stream);
+  if (!s->split.weights.empty() && 6.0 + 0.0068 * p.n * s->K > 0.15 * p.n) return launch_split(s, pt, false, false, stream);
   const int rc = detag::plan_step_csr(pt, s->smem_optin);
   if (rc != DETAG_OK) return fail(s, rc, "graph too large for the shared-memory plan");
   const int e = detag::launch_step_csr(pt, s->sm_count, stream);
@@ -439,24 +443,27 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
 // library's, the rounds of such matrices too.  Circulant bands stay on their float64 kernel, which needs no test of the
 // operands; us per step, integer path -> that one: 64 workers, d = 2 M, K = 1 1099 -> 1035, K = 16 1020 -> 1035; 128, d = 1 M,
 // K = 1 1260 -> 1031, K = 16 1103 -> 1031; 224, d = 500 k, K = 16 1198 -> 927; 256, d = 1 M, K = 1 3157 -> 2032, K = 16
-// 2620 -> 2032; 256, d = 4096 82 -> 30.  Unless d is ragged and short:
-// the columns beyond the last whole slab are a second launch, a slab's latency long, where the integer path takes everything
-// in one.  Two launches -> one: 64 workers, K = 4, d = 9001 26 -> 16; 128, K = 4, d = 9001 39 -> 24, but K = 1, d = 20001
-// 61 -> 60; 256, K = 4, d = 4097 71 -> 43, but K = 1, d = 9001 70 -> 82.
+// 2620 -> 2032; 256, d = 4096 82 -> 30.  Unless d is ragged, up to 128 workers, and so short that one launch takes less than two side by
+// side: 64 workers, K = 4, d = 3001 13.8 -> 9.6, 60001 50.4 -> 40.5, but 200001 125 -> 129; 128, 3001 15.3 -> 12.4, but 9001 15.9 -> 18.7; 256, 3001
+// 42.8 -> 67.  Or, up to 128 workers, the band is nearly as wide as the float64 kernel takes, so that the test is short (float64 -> integer):
+// 64, K = 12, d = 60032 42.1 -> 35.5; 96, K = 16, 200001 174 -> 157, 1 M 769 -> 751, but K = 12 768 -> 778; 128, K = 16, 60001 80.6 -> 62.8; D-PSGD of
+// 128, K = 12, 1 M 1011 -> 847; narrower: 96, K = 4, 1 M 769 against 808, K = 8 769 against 792.
 bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   if (p.d > 0x7fffffffLL) return false;
   if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
   if (variant == DETAG_VARIANT_DENSE) return true;
   if (variant != DETAG_VARIANT_RING) return false;
+  if (!ring_band(s)) return true;
   // by the length of the state, not of a staged chunk: host-resident stepping gives the same bits
-  return !ring_band(s) || (s->d % 64 != 0 && s->d <= (s->n <= 128 ? 2LL : 1LL) * 64 * s->sm_count);
+  if (s->n <= 128 && s->half_band >= 12 && (p.mode == detag::kModeDpsgd || s->d <= 128LL * 32 * s->sm_count)) return true;
+  return s->d % 64 != 0 && s->d <= (s->n <= 64 ? 20LL : s->n <= 128 ? 1LL : 0LL) * 32 * s->sm_count;
 }
 
 // Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.1 -> 9.5, 20 k 31.9 -> 27.1,
 // 1 M 960 -> 880; 128, 40 k 53.0 -> 45.4; D-PSGD of 96, 10 k 17.5 -> 14.3, 1 M 709 -> 632, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
 // 5 k 12.3 -> 13.6; 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
 // calls whose blocks have at most 32 chunks of 32 coordinates to do.  What would run as rounds otherwise - caller-written gradients up to
-// 128 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Rounds -> here: caller-written,
+// 192 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Rounds -> here: caller-written,
 // 100 workers, d = 1 M 3177 -> 860, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 1034, 256 5327 -> 1832,
 // 180, K = 1, d = 72 k 225 against 230, ring of 144, K = 4, d = 8931 35.6 against 48.1.  Polynomials with few entries per row cost the
 // longer test of the operands, and more coordinates that fail it.  On short vectors rounds take their latency, one after the other:
@@ -467,13 +474,15 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
   const double products = s->K * static_cast<double>(s->col_idx.size());
   const bool sparse = s->rows.guard.size() > static_cast<size_t>(s->n);
   if (p.mode == detag::kModeExternal) {
-    const double here = 9.0 + turns * (1.0 + 0.031 * p.n) * (sparse && p.n > 64 && p.n <= 96 ? 2.2 : 1.0);  // six warps for the test
+    const double here = p.n > 128 ? 10.0 + 0.065 * p.n * turns * (sparse ? 1.5 : 1.0)
+                                  : 9.0 + turns * (1.0 + 0.031 * p.n) * (sparse && p.n > 64 && p.n <= 96 ? 2.2 : 1.0);  // six warps for the test
     const double rounds = std::fmax((0.0021 * p.n + 0.00099 * products) * d / 1000.0, 0.0155 * p.n * s->K);
-    return p.n <= 128 && here < std::fmax(8.0, 6.0 + rounds);
+    return here < std::fmax(8.0, 6.0 + rounds) && detag::rows_take_external(s->rows);
   }
   if (p.n <= 64) return turns <= 32.0;
   if (p.n <= 96) return p.mode == detag::kModeDpsgd;
   if (p.n <= 128) return true;
+  if (!s->split.weights.empty()) return false;
   const double here = sparse ? 14.0 + 0.098 * p.n * turns : 10.0 + 0.065 * p.n * turns;
   return here < std::fmax(std::fmax(8.0, 6.0 + 0.0068 * p.n * s->K), 1.25 * (0.024 * p.n + 0.00155 * products) * d / 2000.0);
 }
@@ -626,7 +635,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
       gossip_polynomial(s, poly);
     }
     if (n <= 96 || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
-    if (n <= 128 || !blocks) detag::rows_polynomial(n, poly, blocks, s->rows);
+    if (n <= 192 || !blocks) detag::rows_polynomial(n, poly, blocks, s->rows);
   }
   s->map_cache.reserve(8);
   // the workspace's tables as they are uploaded, the cleared status block in front

@@ -57,6 +57,7 @@ struct StepParams {
   const float* g_ext; // kModeExternal: the caller's newest stochastic gradient, [n][ld]
   unsigned spin_limit;    // polls after which a device-side wait gives up
   int operands_end, tails_end;  // step_dense.cu: slabs from here on are not asked for
+  int beside;             // this launch's columns are not the ones of the launch before it (chain.cuh)
   long long stall_after;  // failure-detection self test: a CTA's producer stops loading after this many tiles (< 0: off)
   int* status;
 };
@@ -134,6 +135,7 @@ int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& p
                       bool wide_gradient, int sm_count, cudaStream_t stream);
 // step_rows.cu: lanes are output workers; any matrix
 void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
+bool rows_take_external(const SplitPoly& poly);
 bool build_maps_rows(const StepParams& p, TensorMapSet* maps);
 int launch_step_rows(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& tables,
                      bool wide_gradient, int sm_count, cudaStream_t stream);

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepPara
     cols = s_col;
     __syncthreads();  // the tables are read right below
   }
-  chain_wait();
+  if (p.beside == 0) chain_wait();
   chain_next();
   // item = ((row quad * 4 + row within quad) * groups + coordinate group): a row's threads side by side, the four
   // rows of a Philox call `groups` lanes apart in one warp (groups is a power of two, at most 8)
@@ -267,6 +267,7 @@ __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepPara
       }
     }
   }
+  if (p.beside != 0) chain_wait();
 }
 
 }  // namespace

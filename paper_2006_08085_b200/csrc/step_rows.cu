@@ -1,6 +1,6 @@
 // DeTAG step with the polynomial P = P_K(M) in exact integer arithmetic on the fifth-generation tensor cores, like step_split.cu (whose
 // head explains the digits, the scales and the test that sends a coordinate to float64), with the output workers as lanes: any matrix
-// of 49 to 256 workers, and caller-written gradients up to 128.
+// of 49 to 256 workers, caller-written gradients up to 192.
 //
 // A unit of work is a chunk of 32 coordinates.  A of the MMA is a digit plane of P (128 output workers x 32 inputs), B the digits
 // of the chunk's models and trackers, 64 columns per digit, digit by digit: plane l meets the digits 4 - l .. 4 in one instruction (N up to
@@ -303,7 +303,7 @@ __device__ __noinline__ void exact_sums(const float* z, const double* poly, unsi
   }
 }
 
-// kMode: caller-written gradients (kModeExternal) up to 128 workers.  kWide: the gradient in float64 (the precision of the rounds kernel, in whose place
+// kWide: the gradient in float64 (the precision of the rounds kernel, in whose place
 // the call runs) instead of float32 at the rounded model (the other tensor-path kernels').  kRows: 64, 96, 128 or 256, n rounded up.
 // kAtStart: the gradient at the model the step started from.
 template <int kMode, bool kWide, int kRows, bool kAtStart>
@@ -396,7 +396,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
     __syncthreads();
     tmem_fence_after();
   }
-  chain_wait();
+  if (p.beside == 0) chain_wait();
   chain_next();
 
   // This CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ... of 1 << chunk_shift chunks; unit v = chunk number * H + half
@@ -874,6 +874,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
     __syncwarp();
   }
   }
+  if (p.beside != 0) chain_wait();
   tmem_fence_before();
   __syncthreads();
   if (warp == kPMmaWarp) {
@@ -893,7 +894,7 @@ RowsKernel pick_rows(const StepParams& p, bool wide) {
 
 template <int kRows>
 RowsKernel pick_rows(const StepParams& p, bool wide) {
-  if (kRows <= kPRows && p.mode == kModeExternal) return step_rows_kernel<kModeExternal, false, kRows <= kPRows ? kRows : kPRows, false>;
+  if (p.mode == kModeExternal) return step_rows_kernel<kModeExternal, false, kRows, false>;
   return p.grad_at_start != 0 ? pick_rows<kRows, true>(p, wide) : pick_rows<kRows, false>(p, wide);
 }
 
@@ -951,6 +952,11 @@ void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, Spl
   out = std::move(made);
 }
 
+// Four arrays are staged for caller-written gradients: up to 192 workers.
+bool rows_take_external(const SplitPoly& poly) {
+  return !poly.weights.empty() && rows_plan(static_cast<int>(poly.row_exp.size()), kModeExternal, static_cast<int>(poly.guard.size())).bytes != 0;
+}
+
 bool build_maps_rows(const StepParams& p, TensorMapSet* out) {
   RowsMaps& m = *reinterpret_cast<RowsMaps*>(out->bytes);
   const float* y = p.mode == kModeDpsgd ? p.x : p.y;  // D-PSGD has no tracker: those maps are never used
@@ -974,7 +980,7 @@ bool build_maps_rows(const StepParams& p, TensorMapSet* out) {
 
 int launch_step_rows(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& dev, bool wide,
                       int sm_count, cudaStream_t stream) {
-  if (poly.weights.empty() || (p.mode == kModeExternal && p.n > kPRows)) return static_cast<int>(cudaErrorInvalidValue);
+  if (poly.weights.empty()) return static_cast<int>(cudaErrorInvalidValue);
   RowsTables tb{};
   tb.tiles = static_cast<const unsigned char*>(dev.weights);
   tb.row_exp = dev.row_exp;

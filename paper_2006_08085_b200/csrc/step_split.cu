@@ -314,7 +314,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   tmem_fence_before();
   __syncthreads();
   tmem_fence_after();
-  chain_wait();
+  if (p.beside == 0) chain_wait();
   chain_next();
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
   if (tid == 0 && *tmem_slot != 0) atomicExch(p.status, 2);
@@ -790,6 +790,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     }
     __syncwarp();
   }
+  if (p.beside != 0) chain_wait();
   tmem_fence_before();
   __syncthreads();
   if (warp == kMmaWarp) {

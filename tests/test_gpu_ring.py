@@ -95,3 +95,23 @@ def test_what_is_not_finite_stays_in_reach(n, worker, K, bad):
             keep[reached, 64] = False  # x' = P x - 0 * P y
         z[worker, col] = 0.0
         assert worst_ratio(got[name][keep], (P @ z.astype(np.float64))[keep]) <= 1.0, name
+
+
+@pytest.mark.parametrize("n,d,K", [(128, 64 * 200 + 3, 4), (160, 65, 3), (192, 64 * 150 + 33, 16), (256, 3001, 2), (288, 1000, 5)])
+def test_ragged_steps_in_a_row_give_the_bits_of_steps_one_by_one(n, d, K):
+    """The columns beyond the last whole slab are a launch of their own that runs beside the band's."""
+    m = inputs.metropolis_weights(inputs.ring_graph(n))
+    rng = np.random.default_rng(n)
+    state = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c")}
+    got = []
+    for together in (False, True):
+        with Session(m, d, K, 0.2, 0.01, sigma=0.1, seed=9) as s:
+            for k, v in state.items():
+                s.upload(k, v)
+            for _ in range(12):
+                s.step()
+                if not together:
+                    s.torch.cuda.synchronize()
+            s.status()
+            got.append({k: s.download(k) for k in ("x", "y", "g")})
+    assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])

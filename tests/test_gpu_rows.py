@@ -40,7 +40,8 @@ def test_dpsgd_and_infinities_beyond_128_workers():
 
 
 @pytest.mark.parametrize("n,d,K,kind", [(49, 1, 1, "regular4"), (50, 35, 2, "ring"), (64, 2 * CHUNKS + 34, 4, "regular4"), (65, 97, 6, "path"),
-                                        (100, 5 * CHUNKS + 7, 2, "regular4"), (128, 17 * CHUNKS + 33, 9, "regular4")])
+                                        (100, 5 * CHUNKS + 7, 2, "regular4"), (128, 17 * CHUNKS + 33, 9, "regular4"), (129, 3 * CHUNKS + 35, 7, "path"),
+                                        (160, 2 * CHUNKS + 1, 40, "ring"), (192, 4 * CHUNKS + 33, 6, "regular4"), (193, 65, 6, "regular4")])
 def test_caller_written_gradients(n, d, K, kind):
     """x' = P x - alpha y', y' = P (y + g_new - g), g' = g_new: two steps, the second with operands of unequal size.  Bound: half an
     ulp of what is stored, and as much again relative to the magnitudes that the result reads for the sums; the folded operand itself
