@@ -463,7 +463,10 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
 // 1 M 960 -> 880; 128, 40 k 53.0 -> 45.4; D-PSGD of 96, 10 k 17.5 -> 14.3, 1 M 709 -> 632, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
 // 5 k 12.3 -> 13.6; 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
 // calls whose blocks have at most 32 chunks of 32 coordinates to do.  What would run as rounds otherwise - caller-written gradients up to
-// 192 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Rounds -> here: caller-written,
+// 192 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Block-circulant
+// matrices beyond 160 workers come here while P is dense and calls are not the longest (lanes as coordinates -> here: 256-ring, K = 40, d = 4 k
+// 34.6 -> 21.9, 60 k 285 -> 207, 16 x 16 torus, 19 k 88.5 -> 77.2, but K = 196, 200 k 577 -> 594, D-PSGD, 300 k 694 -> 775; torus, K = 2, 500 k 1152 -> 1202),
+// all with a chunk per block at most.  Rounds -> here: caller-written,
 // 100 workers, d = 1 M 3177 -> 860, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 1034, 256 5327 -> 1832,
 // 180, K = 1, d = 72 k 225 against 230, ring of 144, K = 4, d = 8931 35.6 against 48.1.  Polynomials with few entries per row cost the
 // longer test of the operands, and more coordinates that fail it.  On short vectors rounds take their latency, one after the other:
@@ -480,9 +483,11 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
     return here < std::fmax(8.0, 6.0 + rounds) && detag::rows_take_external(s->rows);
   }
   if (p.n <= 64) return turns <= 32.0;
-  if (p.n <= 96) return p.mode == detag::kModeDpsgd;
-  if (p.n <= 128) return true;
-  if (!s->split.weights.empty()) return false;
+  if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd && (turns <= 64.0 || !sparse));
+  if (!s->split.weights.empty()) {
+    const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
+    return turns <= (p.n <= 160 ? 1.0 : p.mode == detag::kModeDpsgd ? 4.0 : dense ? 40.0 : 1.0);
+  }
   const double here = sparse ? 14.0 + 0.098 * p.n * turns : 10.0 + 0.065 * p.n * turns;
   return here < std::fmax(std::fmax(8.0, 6.0 + 0.0068 * p.n * s->K), 1.25 * (0.024 * p.n + 0.00155 * products) * d / 2000.0);
 }
@@ -635,7 +640,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
       gossip_polynomial(s, poly);
     }
     if (n <= 96 || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
-    if (n <= 192 || !blocks) detag::rows_polynomial(n, poly, blocks, s->rows);
+    detag::rows_polynomial(n, poly, blocks, s->rows);
   }
   s->map_cache.reserve(8);
   // the workspace's tables as they are uploaded, the cleared status block in front

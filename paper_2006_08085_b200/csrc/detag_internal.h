@@ -73,6 +73,13 @@ struct alignas(64) TensorMapSet {
   unsigned char bytes[8 * 128];
 };
 
+// Tiles (128 outputs x 32 inputs) of the polynomial that the MMAs take for either half of the outputs.
+struct RowsTiles {
+  uint32_t order[2], place[2];  // four bits each: input block; where it stays in tensor memory, 15: it travels
+  int count[2], residents;
+  unsigned char resident[4];    // half << 4 | input block
+};
+
 // P_K(M) as a kernel of the integer tensor path takes it: its base-256 digits, the exponent of every row's scale, the groups of
 // inputs that tell when a coordinate's operands may share one scale, and P itself.  Empty when neither kernel takes the matrix.
 struct SplitPoly {
@@ -84,7 +91,7 @@ struct SplitPoly {
   float guard_tau;         // each group's largest operand must be at least this share of the coordinate's largest
   bool circulant;          // the 32 x 32 blocks depend on their distance only: `poly` holds output workers 0 .. 31
   unsigned char id[64];    // step_split.cu: [output block][input block] -> distinct block, 255: no digit of it is set
-  unsigned char used[2];   // step_rows.cu: [128 outputs], a bit per input block: a digit of its tile is set
+  RowsTiles use;           // step_rows.cu beyond 128 workers
   unsigned char reach[8];  // [32 outputs], a bit per input block: some entry of P is not zero
 };
 

@@ -6,9 +6,10 @@
 // of the chunk's models and trackers, 64 columns per digit, digit by digit: plane l meets the digits 4 - l .. 4 in one instruction (N up to
 // 256; five digits take two), whose sums all start at the same column of the accumulators, weight 4 first.  Six instructions per
 // 32 inputs serve 128 output workers and both arrays; with coordinates as lanes it is twenty for the same chunk.  Up to 128 workers P
-// stays in tensor memory (160 of its columns beside 320 of accumulators); beyond, two halves of the outputs take turns on the accumulators
-// and P comes from L2 through a ring, whole tiles of five planes at a time where there is room for two (waiting for single planes
-// the MMA warp took 290 .. 440 cycles each).
+// stays in tensor memory (160 of its columns beside 320 of accumulators); beyond, two halves of the outputs take turns on the accumulators,
+// four tiles of P stay in tensor memory - of a block-circulant matrix four that both halves use, half of all there is to do - and the
+// others come from L2 through a ring, whole tiles of five planes at a time where there is room for two (waiting for single planes
+// the MMA warp took 290 .. 440 cycles each; without the four, 256-ring, K = 40, d = 19 k 119 -> 85 us).
 //
 // A lane has model and tracker sums of its worker, eight coordinates in a row: the element-wise tail is its own, reads and writes
 // shared memory in 16-byte pieces (128-byte swizzle, no conflicts), and a Philox call's four workers are four neighbouring lanes, which
@@ -26,8 +27,9 @@
 // the power cap (1.5 .. 1.7 GHz on long vectors), and beyond a row pitch of 2 MB by rows travelling in pieces of 128 bytes: loads
 // and stores alone then reach 0.68 of the copy rate (0.85 below that pitch), where 256-byte pieces reach 0.84.  us per step,
 // step_split.cu -> here: 100 workers, d = 2 k 13.1 -> 9.5, 20 k 31.9 -> 27.1, 1 M 960 -> 880; 128, 1 M 1074 -> 1067; D-PSGD of 128, 1 M 979 -> 832;
-// rounds -> here: 144, K = 6, d = 500 k 3396 -> 1034, 256 5327 -> 1832 (waiting for P: 24 k of 32 k cycles a chunk, resident 13 k); caller-written
-// gradients, 100 workers, d = 1 M 3177 -> 860.
+// 256-ring, K = 40, d = 4 k 34.6 -> 21.9, 60 k 285 -> 207; rounds -> here: 144, K = 6,
+// d = 500 k 3396 -> 1003, 256 5327 -> 1650 (waiting for P; all of it at hand would be 1250); caller-written gradients, 100 workers, d = 1 M
+// 3177 -> 860.
 //
 // Measured without gain: asking for 256-byte pieces in L2 ahead of the loads 917 -> 1200 us (128 workers, loads and stores alone); sums
 // read sixteen columns at a time 966 -> 1043 (spills); normals drawn before the sums, or by half of the groups before, 1690 -> 1815, 1905
@@ -96,8 +98,7 @@ struct RowsTables {
   const uint8_t* guard;    // guard_groups x guard_size inputs
   int guard_groups, guard_size;  // size 2 or a multiple of 4
   float guard_tau;
-  uint32_t order[2];       // [output half]: input blocks with a digit in their tile, four bits each
-  int tiles_used[2];       // how many
+  RowsTiles use;           // beyond 128 workers: which tiles, in which order, from where
   int plane_bytes[2], half_at;  // [output half]: a plane of the rows there are; where the second half's tiles begin
   uint8_t reach[8];        // [32 outputs], a bit per input block: some entry of P itself is not zero
 };
@@ -243,9 +244,11 @@ __device__ __forceinline__ float group_low(Value value, const uint8_t* guard, in
 }
 
 // A warp's 32 output workers x 8 coordinates in float64, from the operands themselves: of the model where one of bits 0 .. 7 of
-// `which` is set, of the tracker (fold: with the caller's gradients, y + g_new - g) for bits 8 .. 15.  z: [array][input worker][32] at the first of the coordinates.  poly: rows of P
-// of these workers (circulant: of the first 32, block `b` of whose columns is block (b + c) mod nb here).  Rare, and so out of the
-// way of the main path's registers.
+// `which` is set, of the tracker (fold: with the caller's gradients, y + g_new - g) for bits 8 .. 15.  z: [array][input worker][32] at
+// the first of the coordinates.  poly: rows of P of these workers (circulant: of the first 32, block `b` of whose columns is block
+// (b + c) mod nb here).  Rare, and so out of the way of the main path's registers, on which its own tell all the same: with sixteen
+// entries of P in flight instead of eight the main path took 1824 us for 1651 (100 workers, d = 2 M).  Bound by the latency of P from L2: with
+// every coordinate here 100 workers, K = 2, d = 1 M 906 -> 5004 us (6786 with an array at a time).
 __device__ __noinline__ void exact_sums(const float* z, const double* poly, unsigned which, bool fold, int circulant, int c, int nb, unsigned reach, double* out) {
   const int lane = threadIdx.x & 31, pitch = nb * kPBlock;
   const int stride = nb * kPBlock * kPS;
@@ -254,51 +257,66 @@ __device__ __noinline__ void exact_sums(const float* z, const double* poly, unsi
     if (fold && array != 0) v += static_cast<double>(at[stride]) - static_cast<double>(at[2 * stride]);
     return v;
   };
+  const bool model = (which & 0xffu) != 0, tracker = which >> 8 != 0;
+  // Products on the float64 tensor path: four tiles of eight output workers (M) by eight coordinates (N)
+  double sum[2][4][2];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) sum[i >> 3][i >> 1 & 3][i & 1] = 0.0;
+  for (int b = 0; b < nb; ++b) {
+    if ((reach >> b & 1) == 0) continue;  // a zero block of P
+    const int pb = !circulant ? b : b >= c ? b - c : b - c + nb;
+    const double* const pw = poly + static_cast<size_t>(lane >> 2) * pitch + kPBlock * pb + (lane & 3);
+    const float* const zb = z + (kPBlock * b + (lane & 3)) * kPS + (lane >> 2);
 #pragma unroll 1
-  for (int array = 0; array < 2; ++array, z += nb * kPBlock * kPS, out += 8, which >>= 8) {
-    if ((which & 0xffu) == 0) continue;
-    // Products on the float64 tensor path: four tiles of eight output workers (M) by eight coordinates (N)
-    double sum[4][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-    for (int b = 0; b < nb; ++b) {
-      if ((reach >> b & 1) == 0) continue;  // a zero block of P
-      const int pb = !circulant ? b : b >= c ? b - c : b - c + nb;
-      const double* const pw = poly + static_cast<size_t>(lane >> 2) * pitch + kPBlock * pb + (lane & 3);
-      const float* const zb = z + (kPBlock * b + (lane & 3)) * kPS + (lane >> 2);
+    for (int h = 0; h < kPBlock; h += 16) {
 #pragma unroll 2
-      for (int s = 0; s < 8; ++s) {
-        const double v = value(array, zb + 4 * s * kPS);
+      for (int s = 0; s < 4; ++s) {
+        const float* const at = zb + (h + 4 * s) * kPS;
+        double w[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) dmma(sum[t], __ldg(pw + static_cast<size_t>(8 * t) * pitch + 4 * s), v);
-      }
-    }
-    // lane l has tiles' rows l / 4, coordinates 2 (l % 4) + e; it wants row l, i.e. row l % 8 of tile l / 8
-    bool finite = true;
+        for (int t = 0; t < 4; ++t) w[t] = __ldg(pw + static_cast<size_t>(8 * t) * pitch + h + 4 * s);
+        if (model) {
+          const double v = value(0, at);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      double mine = 0.0;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const double v = __shfl_sync(0xffffffffu, sum[t][u & 1], 4 * (lane & 7) + (u >> 1));
-        if ((lane >> 3) == t) mine = v;
-      }
-      finite = finite && (__double2hiint(mine) & 0x7ff00000) != 0x7ff00000;
-      out[u] = mine;
-    }
-    if (__any_sync(0xffffffffu, !finite)) {
-      // Infinities or NaN among the operands: a lane sums its own worker, without the zeros of P, which the products above turn
-      // into NaN.
-#pragma unroll 1
-      for (int u = 0; u < 8; ++u) {
-        double own = 0.0;
-        for (int b = 0; b < nb; ++b) {
-          if ((reach >> b & 1) == 0) continue;
-          const int pb = !circulant ? b : b >= c ? b - c : b - c + nb;
-          const double* const pw = poly + static_cast<size_t>(lane) * pitch + kPBlock * pb;
-          for (int w = 0; w < kPBlock; ++w)
-            if (pw[w] != 0.0) own = fma(pw[w], value(array, z + (kPBlock * b + w) * kPS + u), own);
+          for (int t = 0; t < 4; ++t) dmma(sum[0][t], w[t], v);
         }
-        out[u] = own;
+        if (tracker) {
+          const double v = value(1, at + stride);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) dmma(sum[1][t], w[t], v);
+        }
       }
+    }
+  }
+  // lane l has tiles' rows l / 4, coordinates 2 (l % 4) + e; it wants row l, i.e. row l % 8 of tile l / 8
+  bool finite = true;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    double mine = 0.0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const double v = __shfl_sync(0xffffffffu, sum[u >> 3][t][u & 1], 4 * (lane & 7) + (u >> 1 & 3));
+      if ((lane >> 3) == t) mine = v;
+    }
+    finite = finite && (__double2hiint(mine) & 0x7ff00000) != 0x7ff00000;
+    out[u] = mine;
+  }
+  if (__any_sync(0xffffffffu, !finite)) {
+    // Infinities or NaN among the operands: a lane sums its own worker, without the zeros of P, which the products above turn
+    // into NaN.
+#pragma unroll 1
+    for (int u = 0; u < 16; ++u) {
+      if (!(u < 8 ? model : tracker)) continue;
+      const int array = u >> 3;
+      double own = 0.0;
+      for (int b = 0; b < nb; ++b) {
+        if ((reach >> b & 1) == 0) continue;
+        const int pb = !circulant ? b : b >= c ? b - c : b - c + nb;
+        const double* const pw = poly + static_cast<size_t>(lane) * pitch + kPBlock * pb;
+        for (int w = 0; w < kPBlock; ++w)
+          if (pw[w] != 0.0) own = fma(pw[w], value(array, z + array * stride + (kPBlock * b + w) * kPS + (u & 7)), own);
+      }
+      out[u] = own;
     }
   }
 }
@@ -379,23 +397,29 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
   const bool ours = *tmem_slot == 0;
   if (tid == 0 && !ours) atomicExch(p.status, 2);
-  if (!kTwo) {  // P into tensor memory: thread = output worker = tensor memory lane
-    if (ours && warp >= kPFinishWarp && warp < kPFinishWarp + 4) {
-      const int row = (warp & 3) * 32 + lane;
-      const unsigned char* src = tb.tiles + (row % (kRows == 64 ? 64 : kPRows) >> 3) * 256 + (row & 7) * 16;
-      const uint32_t to = tmem + kPPolyColumn + (static_cast<uint32_t>(warp & 3) << 21);
-#pragma unroll 4
-      for (int q = 0; q < nb * kPDigits; ++q, src += kPPlaneBytes) {
-        const uint4 a = __ldg(reinterpret_cast<const uint4*>(src)), b = __ldg(reinterpret_cast<const uint4*>(src + 128));
+  // P into tensor memory, all of it or four tiles: thread = output worker = tensor memory lane
+  if (ours && warp >= kPFinishWarp && warp < kPFinishWarp + 4) {
+    const int row = (warp & 3) * 32 + lane, at = (row % (kRows == 64 ? 64 : kPRows) >> 3) * 256 + (row & 7) * 16;
+    uint32_t to = tmem + kPPolyColumn + (static_cast<uint32_t>(warp & 3) << 21);
+    for (int t = 0; t < (kTwo ? tb.use.residents : nb); ++t) {
+      const int half = kTwo ? tb.use.resident[t] >> 4 : 0, plane = kTwo ? tb.plane_bytes[half] : kPPlaneBytes;
+      const unsigned char* src = tb.tiles + half * tb.half_at + static_cast<size_t>(kTwo ? tb.use.resident[t] & 15 : t) * kPDigits * plane + at;
+#pragma unroll
+      for (int q = 0; q < kPDigits; ++q, src += plane, to += 8) {
+        uint4 a = make_uint4(0, 0, 0, 0), b = a;  // a plane of the second half ends with its workers
+        if (!kTwo || at < plane) {
+          a = __ldg(reinterpret_cast<const uint4*>(src));
+          b = __ldg(reinterpret_cast<const uint4*>(src + 128));
+        }
         const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        tmem_store8(to + q * 8, w);
+        tmem_store8(to, w);
       }
-      tmem_wait_store();
     }
-    tmem_fence_before();
-    __syncthreads();
-    tmem_fence_after();
+    tmem_wait_store();
   }
+  tmem_fence_before();
+  __syncthreads();
+  tmem_fence_after();
   if (p.beside == 0) chain_wait();
   chain_next();
 
@@ -701,6 +725,16 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
     // The whole warp walks the loop, one lane issues: operands computed in uniform control flow stay in uniform registers.
     const uint64_t dig_base = mma_operand(s_addr(dig_mem), 256, 128), ring_base = mma_operand(s_addr(smem + plan.ring_at), 256, 128);
     const bool leader = lane == 0;
+    constexpr uint64_t kDigit = kPDigitBytes / 16;
+    // A tile in tensor memory: plane l of P with the digits 4 - l .. 4 of z -> weights 4 .. 4 + l
+    auto six = [&](uint32_t a, uint64_t b, unsigned add) {
+      mma_i8(tmem, a, b, mma_i8_desc(3 * kPColumns), add, leader);
+      mma_i8(tmem + 3 * kPColumns, a, b + 3 * kDigit, mma_i8_desc(2 * kPColumns), add, leader);
+      mma_i8(tmem, a + 8, b + kDigit, mma_i8_desc(4 * kPColumns), 1u, leader);
+      mma_i8(tmem, a + 16, b + 2 * kDigit, mma_i8_desc(3 * kPColumns), 1u, leader);
+      mma_i8(tmem, a + 24, b + 3 * kDigit, mma_i8_desc(2 * kPColumns), 1u, leader);
+      mma_i8(tmem, a + 32, b + 4 * kDigit, mma_i8_desc(kPColumns), 1u, leader);
+    };
     bool ok = true;
     int buf = 0, use = 0, slot = 0, round = 0;
     for (int k = 0, v = 0; k < chunks && ok; ++k) {
@@ -712,23 +746,21 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
         unsigned add = 0;  // the first plane clears the accumulators
         uint64_t b = dig_base + buf * nb * (kPBlockBytes / 16);
         uint32_t a = tmem + kPPolyColumn;
-        constexpr uint64_t kDigit = kPDigitBytes / 16;
-        // plane l of P with the digits 4 - l .. 4 of z -> weights 4 .. 4 + l
         if (!kTwo) {
           for (int kb = 0; kb < nb; ++kb, b += kPBlockBytes / 16, a += kPDigits * 8) {
-            mma_i8(tmem, a, b, mma_i8_desc(3 * kPColumns), add, leader);
-            mma_i8(tmem + 3 * kPColumns, a, b + 3 * kDigit, mma_i8_desc(2 * kPColumns), add, leader);
-            mma_i8(tmem, a + 8, b + kDigit, mma_i8_desc(4 * kPColumns), 1u, leader);
-            mma_i8(tmem, a + 16, b + 2 * kDigit, mma_i8_desc(3 * kPColumns), 1u, leader);
-            mma_i8(tmem, a + 24, b + 3 * kDigit, mma_i8_desc(2 * kPColumns), 1u, leader);
-            mma_i8(tmem, a + 32, b + 4 * kDigit, mma_i8_desc(kPColumns), 1u, leader);
+            six(a, b, add);
             add = 1;
           }
         } else {
           const int plane = tb.plane_bytes[half] / 16;
-          uint32_t order = tb.order[half];
-          for (int t = 0; t < tb.tiles_used[half] && ok; ++t, order >>= 4) {
+          uint32_t order = tb.use.order[half], place = tb.use.place[half];
+          for (int t = 0; t < tb.use.count[half] && ok; ++t, order >>= 4, place >>= 4) {
             const uint64_t bt = b + (order & 15) * (kPBlockBytes / 16);
+            if ((place & 15) != 15) {  // in tensor memory
+              six(a + (place & 15) * (kPDigits * 8), bt, add);
+              add = 1;
+              continue;
+            }
             uint64_t at = 0;
             int in_unit = 0;
 #pragma unroll
@@ -852,8 +884,9 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
       bool ok = true;
       for (int v = 0; v < total && ok; ++v) {
         const int half = v % H, plane = tb.plane_bytes[half];
-        for (int t = 0; t < tb.tiles_used[half] && ok; ++t) {
-          const unsigned char* src = tb.tiles + half * tb.half_at + static_cast<size_t>(tb.order[half] >> (4 * t) & 15) * kPDigits * plane;
+        for (int t = 0; t < tb.use.count[half] && ok; ++t) {
+          if ((tb.use.place[half] >> (4 * t) & 15) != 15) continue;
+          const unsigned char* src = tb.tiles + half * tb.half_at + static_cast<size_t>(tb.use.order[half] >> (4 * t) & 15) * kPDigits * plane;
           for (int left = kPDigits; left > 0; left -= plan.unit, src += plan.unit * plane) {
             if (round > 0) ok = bar_wait(&ring_empty[slot], (round - 1) & 1, limit);
             if (!ok) break;
@@ -912,6 +945,51 @@ bool make_swizzled_map(CUtensorMap* m, const float* base, int n, long long d, lo
 
 }  // namespace
 
+namespace {
+
+// Which tiles the MMAs of a half take: those with a digit, the ones that stay in tensor memory (four, first those that both halves
+// use, as in a block-circulant matrix) between those that travel, which thus have the time of two.
+void place_tiles(int n, int nb, const unsigned (&used)[2], SplitPoly& made) {
+  constexpr int kResidents = 4, kTravels = 15;
+  auto tile = [&](int half, int b) {
+    return &made.weights[static_cast<size_t>(half) * nb * kPDigits * kPPlaneBytes + static_cast<size_t>(b) * kPDigits * plane_bytes(n, half)];
+  };
+  int twin[8], place[2][8];
+  for (int b = 0; b < nb; ++b) {
+    twin[b] = -1;
+    place[0][b] = place[1][b] = kTravels;
+    for (int c = 0; c < nb && plane_bytes(n, 0) == plane_bytes(n, 1) && (used[0] >> b & 1); ++c)
+      if (std::memcmp(tile(0, b), tile(1, c), kPDigits * kPPlaneBytes) == 0) twin[b] = c;
+  }
+  RowsTiles& t = made.use;
+  auto keep = [&](int half, int b) {
+    if (t.residents == kResidents || !(used[half] >> b & 1) || place[half][b] != kTravels) return;
+    place[half][b] = t.residents;
+    if (half == 0 && twin[b] >= 0) place[1][twin[b]] = t.residents;
+    t.resident[t.residents++] = static_cast<unsigned char>(half << 4 | b);
+  };
+  for (int b = 0; b < nb; ++b)
+    if (twin[b] >= 0) keep(0, b);
+  for (int b = 0; b < nb; ++b)
+    for (int half = 0; half < 2; ++half) keep(half, b);
+  for (int half = 0; half < 2; ++half) {
+    int left[2] = {0, 0}, next[2] = {0, 0};  // travelling, staying
+    for (int b = 0; b < nb; ++b)
+      if (used[half] >> b & 1) ++left[place[half][b] == kTravels ? 0 : 1];
+    for (int turn = 0; left[0] + left[1] > 0; ++turn) {
+      const int kind = left[0] == 0 ? 1 : left[1] == 0 ? 0 : turn & 1;
+      int& b = next[kind];
+      while (!(used[half] >> b & 1) || (place[half][b] == kTravels ? 0 : 1) != kind) ++b;
+      t.order[half] |= static_cast<uint32_t>(b) << (4 * t.count[half]);
+      t.place[half] |= static_cast<uint32_t>(place[half][b]) << (4 * t.count[half]++);
+      ++b;
+      --left[kind];
+    }
+  }
+}
+
+}  // namespace
+
 // Digits of P, the rows' exponents, which of its parts are zero.  `poly`: the n x n matrix, or (circulant: the
 // blocks depend on their distance only) its first 32 rows.  Leaves `out` empty when the kernel does not take the matrix:
 // n outside 33 .. 256, an entry or a row that cannot be scaled.
@@ -924,6 +1002,7 @@ void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, Spl
   if (!split_digits(n, poly, rows, wide, digits, made.row_exp)) return;
   split_guard(n, poly, rows, made);
   if (rows_plan(n, kModeDetag, static_cast<int>(made.guard.size())).bytes == 0) return;
+  unsigned used[2] = {0, 0};
   made.weights.assign(static_cast<size_t>(halves) * nb * kPDigits * kPPlaneBytes, 0);
   for (int i = 0; i < n; ++i) {
     const int half = i / kPRows, r = i % kPRows, shift = circulant ? i / kPBlock : 0;  // block row c: block row 0, c blocks further
@@ -942,9 +1021,10 @@ void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, Spl
         if (v != 0)
           for (int l = 0; l < kPDigits; ++l) at[(kPDigits - 1 - l) * plane + (w / 16) * 128 + w % 16] = static_cast<unsigned char>(v >> (8 * l));
       }
-      if (any != 0) made.used[half] |= static_cast<unsigned char>(1u << b);
+      if (any != 0) used[half] |= 1u << b;
     }
   }
+  if (halves == 2) place_tiles(n, nb, used, made);
   const int padded = circulant ? kPBlock : wide;
   made.poly.assign(static_cast<size_t>(padded) * wide, 0.0);
   for (int i = 0; i < rows; ++i) std::copy(&poly[static_cast<size_t>(i) * n], &poly[static_cast<size_t>(i) * n] + n, &made.poly[static_cast<size_t>(i) * wide]);
@@ -992,11 +1072,8 @@ int launch_step_rows(StepParams p, const TensorMapSet& maps, const SplitPoly& po
   tb.circulant = poly.circulant ? 1 : 0;
   tb.nb = (p.n + kPBlock - 1) / kPBlock;
   tb.half_at = tb.nb * kPDigits * kPPlaneBytes;
-  for (int half = 0; half < 2; ++half) {
-    tb.plane_bytes[half] = plane_bytes(p.n, half);
-    for (int kb = 0; kb < tb.nb; ++kb)
-      if (poly.used[half] >> kb & 1) tb.order[half] |= static_cast<uint32_t>(kb) << (4 * tb.tiles_used[half]++);
-  }
+  for (int half = 0; half < 2; ++half) tb.plane_bytes[half] = plane_bytes(p.n, half);
+  tb.use = poly.use;
   std::memcpy(tb.reach, poly.reach, sizeof tb.reach);
   RowsPlan plan = rows_plan(p.n, p.mode, static_cast<int>(poly.guard.size()));
   if (plan.bytes == 0) return static_cast<int>(cudaErrorInvalidValue);
