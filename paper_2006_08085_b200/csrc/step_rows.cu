@@ -70,7 +70,7 @@ constexpr int kPMmaWarp = kPSplitWarps, kPLoadXYWarp = kPMmaWarp + 1, kPTailWarp
               kPFinishWarp = kPMmaWarp + 4;  // the one before it fetches P
 constexpr int kPThreads = (kPSplitWarps + 4 + kPFinishWarps) * 32;
 // Registers: 72 per thread at launch; what the issuing and the splitting warps give up goes to the finishing ones.
-constexpr int kPLaunchRegisters = 72, kPSplitRegisters = 56, kPIssueRegisters = 32, kPFinishRegisters = 88;
+constexpr int kPLaunchRegisters = 72, kPSplitRegisters = 48, kPIssueRegisters = 24, kPFinishRegisters = 96;
 static_assert(kPSplitWarps * kPSplitRegisters + 4 * kPIssueRegisters + kPFinishWarps * kPFinishRegisters <= kPThreads / 32 * kPLaunchRegisters,
               "register split");
 // Tensor memory: the accumulators; up to 128 workers the digit planes of P, eight columns each, behind them.
