@@ -10,9 +10,6 @@ namespace detag {
 
 // The launches before this one are complete.  Every thread that reads or writes state passes it.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// A launch that touches only what the one before it leaves alone (`beside`: the last columns of a band) runs next to it: the launches
-// before that one are complete when it starts, for that one has waited for them before it let this one begin.  It waits at its end
-// instead, so that whoever waits for it has waited for both.
 // The next launch may begin (once every block has said so).  After chain_wait(): what it finds running is this launch alone.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -57,7 +57,10 @@ struct StepParams {
   const float* g_ext; // kModeExternal: the caller's newest stochastic gradient, [n][ld]
   unsigned spin_limit;    // polls after which a device-side wait gives up
   int operands_end, tails_end;  // step_dense.cu: slabs from here on are not asked for
-  int beside;             // this launch's columns are not the ones of the launch before it (chain.cuh)
+  // This launch's columns are not the ones of the launch before it (the last columns of a band): it runs beside that one.  The launches
+  // before that are complete when it starts, for that one has waited for them before it let this one begin (chain.cuh); it waits at
+  // its end instead, so that whoever waits for it has waited for both.
+  int beside;
   long long stall_after;  // failure-detection self test: a CTA's producer stops loading after this many tiles (< 0: off)
   int* status;
 };
