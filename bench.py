@@ -39,7 +39,8 @@ BYTES_PER_WC = 32  # read x, y, g, a, c + write x, y, g, float32 each: the fused
 # sources the capture was taken on: a changed kernel reports null until it is captured again.
 KERNEL_SOURCES = {
     "small": ("step_small.cu", "noise.cuh", "packed.cuh", "pipeline.cuh", "chain.cuh"),
-    "split": ("step_split.cu", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
+    "split": ("step_split.cu", "digits.cuh", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
+    "rows": ("step_rows.cu", "digits.cuh", "tensor_memory.cuh", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
     "dense": ("step_dense.cu", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
     "ring": ("step_ring.cu", "pipeline.cuh", "noise.cuh", "packed.cuh", "chain.cuh"),
     "csr": ("step_csr.cu", "noise.cuh", "packed.cuh", "chain.cuh"),
@@ -66,6 +67,8 @@ SM_COUNT = 148
 
 def kernel_key(variant: str, n: int):
     if variant == "dense":
+        if n > 96:
+            return ("rows", "digits")
         return ("small", "column") if n <= 16 else ("dense", "product") if n <= 48 else ("split", "digits")
     if variant == "ring":
         return ("ring", "band")  # K times the bandwidth at most 16, as in the configurations

@@ -482,7 +482,7 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
     const double rounds = std::fmax((0.0021 * p.n + 0.00099 * products) * d / 1000.0, 0.0155 * p.n * s->K);
     return here < std::fmax(8.0, 6.0 + rounds) && detag::rows_take_external(s->rows);
   }
-  if (p.n <= 64) return turns <= 32.0;
+  if (p.n <= 64) return turns <= 32.0 || s->split.weights.empty();
   if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd && (turns <= 64.0 || !sparse));
   if (!s->split.weights.empty()) {
     const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
@@ -633,14 +633,18 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   analyse_circulant(s);
   analyse_torus(s);
   if (n > detag::kMaxDenseStepWorkers && n <= detag::kMaxSplitWorkers) {
+    // tables for whichever of the two kernels may be asked (rows_ok); those of step_rows.cu take 1 .. 3 ms to make beyond 128 workers
+    // and are left out where calls will surely not use them
     const bool blocks = block_circulant(s);
+    const double products = static_cast<double>(K) * nnz, rounds = std::fmax(0.0155 * n * K, 0.625e-3 * (0.024 * n + 0.00155 * products) * static_cast<double>(d));
+    const bool rows = n <= 128 || (blocks ? n <= 192 || d <= 40LL * 32 * 160 : 10.0 + 0.065 * n < 1.5 * (8.0 + rounds));
     if (blocks) {
       first_block_row(s, poly);
-    } else if (n > 128) {
+    } else if (n > 128 && rows) {
       gossip_polynomial(s, poly);
     }
-    if (n <= 96 || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
-    detag::rows_polynomial(n, poly, blocks, s->rows);
+    if ((n <= 96 && (n > 64 || d > 32LL * 32 * 100)) || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
+    if (rows) detag::rows_polynomial(n, poly, blocks, s->split, s->rows);
   }
   s->map_cache.reserve(8);
   // the workspace's tables as they are uploaded, the cleared status block in front

@@ -144,7 +144,7 @@ bool build_maps_split(const StepParams& p, TensorMapSet* maps);
 int launch_step_split(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& tables,
                       bool wide_gradient, int sm_count, cudaStream_t stream);
 // step_rows.cu: lanes are output workers; any matrix
-void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out);
+void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, const SplitPoly& other, SplitPoly& out);
 bool rows_take_external(const SplitPoly& poly);
 bool build_maps_rows(const StepParams& p, TensorMapSet* maps);
 int launch_step_rows(StepParams p, const TensorMapSet& maps, const SplitPoly& poly, const SplitDevice& tables,

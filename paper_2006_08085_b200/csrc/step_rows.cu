@@ -993,14 +993,20 @@ void place_tiles(int n, int nb, const unsigned (&used)[2], SplitPoly& made) {
 // Digits of P, the rows' exponents, which of its parts are zero.  `poly`: the n x n matrix, or (circulant: the
 // blocks depend on their distance only) its first 32 rows.  Leaves `out` empty when the kernel does not take the matrix:
 // n outside 33 .. 256, an entry or a row that cannot be scaled.
-void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, SplitPoly& out) {
+void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, const SplitPoly& other, SplitPoly& out) {
   out = SplitPoly{};
   if (n <= 32 || n > 256 || encode_tiled_fn() == nullptr) return;
   const int nb = (n + kPBlock - 1) / kPBlock, rows = circulant ? kPBlock : n, wide = nb * kPBlock, halves = n > kPRows ? 2 : 1;
   std::vector<int64_t> digits;
   SplitPoly made{};
   if (!split_digits(n, poly, rows, wide, digits, made.row_exp)) return;
-  split_guard(n, poly, rows, made);
+  if (other.guard.empty()) {
+    split_guard(n, poly, rows, made);
+  } else {  // the other kernel's tables have been made
+    made.guard = other.guard;
+    made.guard_size = other.guard_size;
+    made.guard_tau = other.guard_tau;
+  }
   if (rows_plan(n, kModeDetag, static_cast<int>(made.guard.size())).bytes == 0) return;
   unsigned used[2] = {0, 0};
   made.weights.assign(static_cast<size_t>(halves) * nb * kPDigits * kPPlaneBytes, 0);

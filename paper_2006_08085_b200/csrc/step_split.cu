@@ -1,5 +1,7 @@
 // DeTAG step with the polynomial P = P_K(M) applied on the fifth-generation tensor cores in exact integer arithmetic,
-// for any gossip matrix with 48 < n <= 256 whose distinct 32 x 32 blocks of P fit in shared memory.
+// for gossip matrices with 48 < n <= 256 whose distinct 32 x 32 blocks of P fit in shared memory.  Its other kernel, step_rows.cu,
+// takes the others and what it is faster at (rows_ok in detag_api.cu): left here are the DeTAG step of 65 to 96 workers, long vectors up
+// to 64, long vectors of block-circulant matrices beyond 128.
 //
 // AG_K(z) = P z.  The float64 tensor path (mma m8n8k4) bounds this product at 64 multiply-adds per clock and SM, which
 // for n = 100 is 3.3 times and for a dense n = 256 eight times the time of the step's HBM traffic.  Here both operands
@@ -12,7 +14,7 @@
 //
 // That scale is the coordinate's; an output that reads no operand near the largest must not inherit its error.  The host
 // therefore chooses groups of inputs such that every output gives every input of one of the groups at least `theta` of its
-// largest weight (split_guard below).  If the largest operand of each group is at least tau of the coordinate's largest,
+// largest weight (split_guard in split_poly.cpp).  If the largest operand of each group is at least tau of the coordinate's largest,
 // every sum of magnitudes sum_j |P_ij z_j| is at least theta tau of largest weight times largest operand, and
 // tau = 2^-12 sqrt(m) / theta keeps the error below 2^-24 of that sum by more than five standard deviations (largest found on
 // rings, tori and random graphs of 36 .. 256 workers, magnitudes spread in various ways: a fifth of it).  A coordinate that fails the test - or holds infinities, NaN or values outside
@@ -40,7 +42,7 @@
 //
 // Bound by the issue slots and the latency of what the six warps of a scheduler do, at a dense n = 256 by the MMAs, which take
 // turns with splitting and with reading the one accumulator there is room for.  us per step, the float64 kernels this one
-// replaced -> now: 100 workers, d = 2 M 3518 -> 1880; 256-ring at K = 196, d = 200 k 1940 -> 607; 16 x 16 torus, d = 500 k
+// replaced -> now: 100 workers, d = 2 M 3518 -> 1880 (step_rows.cu 1670 .. 1800); 256-ring at K = 196, d = 200 k 1940 -> 607; 16 x 16 torus, d = 500 k
 // 8992 -> 1470.  (Four digits and four accumulators took 1680, 566 and 1420 when this took 2060, 640 and 1640, but left 2^-31 of the
 // coordinate's largest operand in every result.)  From those figures it came by fewer instructions in the finishing and more
 // registers for it: the scale of a coordinate sits in the number that joins the sums, a row's scale is one factor of x~ - alpha y~
