@@ -461,7 +461,7 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
 
 // Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.1 -> 9.5, 20 k 31.9 -> 27.1,
 // 1 M 960 -> 880; 128, 40 k 53.0 -> 45.4; D-PSGD of 96, 10 k 17.5 -> 14.3, 1 M 709 -> 632, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
-// 5 k 12.3 -> 13.6; 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
+// 8 k 12.4 -> 14.4, 300 k 224 -> 234, only the shortest of these better (96, 3000 11.7 -> 10.9, K = 1, 700 12.8 -> 11.4); 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
 // calls whose blocks have at most 32 chunks of 32 coordinates to do.  What would run as rounds otherwise - caller-written gradients up to
 // 192 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Block-circulant
 // matrices beyond 160 workers come here while P is dense and calls are not the longest (lanes as coordinates -> here: 256-ring, K = 40, d = 4 k
@@ -483,7 +483,7 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
     return here < std::fmax(8.0, 6.0 + rounds) && detag::rows_take_external(s->rows);
   }
   if (p.n <= 64) return turns <= 32.0 || s->split.weights.empty();
-  if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd && (turns <= 64.0 || !sparse));
+  if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd ? turns <= 64.0 || !sparse : s->d <= 24LL * s->sm_count);
   if (!s->split.weights.empty()) {
     const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
     return turns <= (p.n <= 160 ? 1.0 : p.mode == detag::kModeDpsgd ? 4.0 : dense ? 40.0 : 1.0);

@@ -51,14 +51,15 @@ void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& ou
   const int stride = n % 2 == 0 ? n / 2 - (n % 4 == 0 ? 1 : 2) : n / 2;  // coprime to n: ties go to inputs far apart
   double best = 1e300;
   std::vector<uint64_t> readers(static_cast<size_t>(n) * kWords, 0);  // [input]: outputs that give it at least theta
-  std::vector<int> inputs;
-  std::vector<uint8_t> groups;
+  std::vector<int> inputs, have_list(n);
+  std::vector<uint8_t> groups, list(static_cast<size_t>(n) * n);  // [output]: its inputs of at least theta, once they have been asked for
   for (int k = 0; k < kLevels && best > 0.25 * n; ++k) {
     const double tau = std::sqrt(static_cast<double>(terms)) / 4096.0 * (1 << k);
     if (tau > 0.5) break;
     for (int i = 0; i < n; ++i)
       for (int j = 0; j < n; ++j)
         if (level[static_cast<size_t>(i) * n + j] == k) readers[static_cast<size_t>(j) * kWords + i / 64] |= 1ull << (i % 64);
+    std::fill(have_list.begin(), have_list.end(), -1);
     const double small = std::fmax(0.0, 1.0 - std::log2(1.0 / tau) / 13.3);
     int largest = 32;  // of a group, as far as its outputs have such inputs
     for (int size = 2; size <= 32 && size / 2 <= largest && best > 0.25 * n; size *= 2) {
@@ -72,9 +73,13 @@ void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& ou
       double fail = 0.0, fail_spread = 0.0;
       for (int i = 0; i < n && groups.size() <= 2 * static_cast<size_t>(n) && groups.size() < best; ++i) {
         if ((open[i / 64] >> (i % 64) & 1) == 0) continue;
-        inputs.clear();
-        for (int v = 0, j = i; v < n; ++v, j = j + stride < n ? j + stride : j + stride - n)
-          if (level[static_cast<size_t>(i) * n + j] <= k) inputs.push_back(j);
+        uint8_t* const of = &list[static_cast<size_t>(i) * n];
+        if (have_list[i] < 0) {
+          have_list[i] = 0;
+          for (int v = 0, j = i; v < n; ++v, j = j + stride < n ? j + stride : j + stride - n)
+            if (level[static_cast<size_t>(i) * n + j] <= k) of[have_list[i]++] = static_cast<uint8_t>(j);
+        }
+        inputs.assign(of, of + have_list[i]);
         uint64_t served[kWords];
         std::copy(open, open + kWords, served);
         int have = 0;
