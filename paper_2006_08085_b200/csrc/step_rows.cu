@@ -425,8 +425,8 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
 
   // This CTA takes slabs blockIdx.x, blockIdx.x + gridDim.x, ... of 1 << chunk_shift chunks; unit v = chunk number * H + half
   const int shift = plan.chunk_shift;
-  auto chunk_col = [&](int k) {
-    return (((static_cast<long long>(blockIdx.x) + static_cast<long long>(k >> shift) * gridDim.x) << shift) + (k & ((1 << shift) - 1))) * kPS;
+  auto chunk_col = [&](int k) {  // below 2^31 + 64 in 32 bits
+    return static_cast<long long>((((blockIdx.x + static_cast<unsigned>(k >> shift) * gridDim.x) << shift) + (k & ((1 << shift) - 1))) * kPS);
   };
   int chunks = ours && blockIdx.x < p.num_slabs ? static_cast<int>((p.num_slabs - blockIdx.x + gridDim.x - 1) / gridDim.x) << shift : 0;
   while (chunks > 0 && chunk_col(chunks - 1) >= p.d) --chunks;
@@ -560,7 +560,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
     const int d = static_cast<int>(p.d), d_tma = d & ~3;  // columns below d_tma are written by the TMA stores
     const int stage_floats = plan.outs * plan.rows * kPS, raw_floats = plan.ins * nb * kPBlock * kPS;
     const int at0 = ((2 * part) ^ (row & 7)) << 2, at1 = at0 ^ 4;
-    int st = set, st_phase = 0, raw = set;
+    int st = set, st_phase = 0, raw = set, power = row_exp[row] << 20;
     if (kCopies == 2 && set >= plan.stages) st = 0, st_phase = 1;
     if (kCopies == 2 && set >= plan.raws) raw = 0;
     bool ok = true;
@@ -586,7 +586,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
             exact_sums(raw_mem + raw * raw_floats + kPGroup * part, rows, exact, kMode == kModeExternal, tb.circulant, c, nb, tb.reach[c], in_full);
           }
           const int* const magic = magics + slot * kPColumns + 2 * kPGroup * part;
-          const int power = row_exp[w] << 20;
+          if (kTwo) power = row_exp[w] << 20;
           take_sums<kTwo>(acc, magic, power, sums);
           if (kMode != kModeDpsgd) take_sums<kTwo>(acc + kPGroup, magic + kPGroup, power, sums + 8);
           if (__builtin_expect(exact != 0, 0)) {
