@@ -53,7 +53,7 @@ MEASURED_TRAFFIC = {
     ("torus", "torus8"): ("194904bdd0cabfdc", 31.23),  # cfg3 shape at d = 1 M: 1.2802 + 0.7185 GB / 64 M wc
     ("ring", "band"): ("72c17745930c7df4", 31.09),  # cfg4 shape at d = 200 k: 1.0277 + 0.5641 GB / 51.2 M wc
     ("split", "digits"): ("feb6f88094eb2145", 31.05),  # 16 x 16 torus at d = 200 k: 1.0200 + 0.5698 GB / 51.2 M wc
-    ("rows", "digits"): ("d2474d191defd66b", 30.78),  # 100-worker random graph at d = 400 k: 0.8006 + 0.4306 GB / 40 M wc
+    ("rows", "digits"): ("6ddfc9a5b7574d81", 30.80),  # 100-worker random graph at d = 400 k: 0.8007 + 0.4312 GB / 40 M wc
     ("csr", "rounds"): ("57f2704a52f61fcf", 30.61),  # 300-worker random graph at d = 100 k: 0.6017 + 0.3165 GB / 30 M wc
 }
 

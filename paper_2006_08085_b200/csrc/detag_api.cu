@@ -459,15 +459,15 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   return s->d % 64 != 0 && s->d <= (s->n <= 64 ? 20LL : s->n <= 128 ? 1LL : 0LL) * 32 * s->sm_count;
 }
 
-// Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.1 -> 9.5, 20 k 31.9 -> 27.1,
-// 1 M 960 -> 880; 128, 40 k 53.0 -> 45.4; D-PSGD of 96, 10 k 17.5 -> 14.3, 1 M 709 -> 632, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
+// Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0,
+// 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7; D-PSGD of 96, 10 k 17.5 -> 14.5, 1 M 707 -> 639, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
 // 8 k 12.4 -> 14.4, 300 k 224 -> 234, only the shortest of these better (96, 3000 11.7 -> 10.9, K = 1, 700 12.8 -> 11.4); 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
 // calls whose blocks have at most 32 chunks of 32 coordinates to do.  What would run as rounds otherwise - caller-written gradients up to
 // 192 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Block-circulant
 // matrices beyond 160 workers come here while P is dense and calls are not the longest (lanes as coordinates -> here: 256-ring, K = 40, d = 4 k
 // 34.6 -> 21.9, 60 k 285 -> 207, 16 x 16 torus, 19 k 88.5 -> 77.2, but K = 196, 200 k 577 -> 594, D-PSGD, 300 k 694 -> 775; torus, K = 2, 500 k 1152 -> 1202),
 // all with a chunk per block at most.  Rounds -> here: caller-written,
-// 100 workers, d = 1 M 3177 -> 860, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 1034, 256 5327 -> 1832,
+// 100 workers, d = 1 M 3177 -> 895, 20 k 76 -> 28, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 984, 256 5327 -> 1680,
 // 180, K = 1, d = 72 k 225 against 230, ring of 144, K = 4, d = 8931 35.6 against 48.1.  Polynomials with few entries per row cost the
 // longer test of the operands, and more coordinates that fail it.  On short vectors rounds take their latency, one after the other:
 // caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.

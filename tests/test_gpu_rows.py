@@ -113,3 +113,35 @@ def test_rows_further_apart_give_the_same_bits(n, mode):
             s.status()
             got.append({k: s.download(k) for k in ("x", "y", "g")})
     assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])
+
+
+@pytest.mark.parametrize("n,mode,after", [(60, "detag", 0), (60, "detag", 3), (90, "dpsgd", 2), (100, "detag", 1), (100, "external", 2), (144, "detag", 1),
+                                          (144, "detag", 4), (150, "external", 2)])
+def test_loads_that_stop_time_out_and_the_state_recovers(n, mode, after):
+    """Some of a block's chunks are loaded, the others are not: every wait gives up and the launch ends; after re-binding the state steps
+    to the bits of one that was never disturbed."""
+    from paper_2006_08085_b200 import binding as B
+    from test_gpu_failure_detection import _rebind
+    d, m = 4 * CHUNKS + 5, _graph("regular4", n)
+    rng = np.random.default_rng(n + after)
+    state = {k: rng.standard_normal((n, d)).astype(np.float32) for k in ("x", "y", "g", "a", "c", "g_new")}
+    got = []
+    for stalled in (False, True):
+        with Session(m, d, 6, 0.2, 0.01, sigma=0.1, seed=5, external_gradient=mode == "external",
+                     algorithm=B.DETAG_ALGORITHM_DPSGD if mode == "dpsgd" else B.DETAG_ALGORITHM_DETAG) as s:
+            if stalled:
+                B.detag_debug_inject_stall(s.state, after, 2048)
+                s.step()
+                with pytest.raises(B.DetagError) as e:
+                    s.status()
+                assert e.value.code == B.DETAG_ERR_TIMEOUT
+                B.detag_debug_inject_stall(s.state, -1, 0)
+                _rebind(s)
+            for k, v in state.items():
+                if k != "g_new" or mode == "external":
+                    s.upload(k, v)
+            B.detag_set_step(s.state, 0)
+            s.step()
+            s.status()
+            got.append({k: s.download(k) for k in ("x", "y", "g")})
+    assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])
