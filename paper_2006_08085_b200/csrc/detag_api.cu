@@ -486,6 +486,8 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
   if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd ? turns <= 64.0 || !sparse : s->d <= 24LL * s->sm_count);
   if (!s->split.weights.empty()) {
     const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
+    // two chunks a block are one slab of 64 coordinates there (12 x 16 torus, d = 4863 24.0 against 27.5, but 256-ring, K = 40, d = 9 k 85 -> 38)
+    if (p.n <= 192 && turns > 1.0 && turns <= 2.0) return false;
     return turns <= (p.n <= 160 ? 1.0 : p.mode == detag::kModeDpsgd ? 4.0 : dense ? 40.0 : 1.0);
   }
   const double here = sparse ? 14.0 + 0.098 * p.n * turns : 10.0 + 0.065 * p.n * turns;
