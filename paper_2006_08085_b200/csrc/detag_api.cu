@@ -449,7 +449,7 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
 // 64, K = 12, d = 60032 42.1 -> 35.5; 96, K = 16, 200001 174 -> 157, 1 M 769 -> 751, but K = 12 768 -> 778; 128, K = 16, 60001 80.6 -> 62.8; D-PSGD of
 // 128, K = 12, 1 M 1011 -> 847; narrower: 96, K = 4, 1 M 769 against 808, K = 8 769 against 792.
 bool split_ok(const detag_state* s, const StepParams& p, int variant) {
-  if (p.d > 0x7fffffffLL) return false;
+  if ((s->split.weights.empty() && s->rows.weights.empty()) || p.d > 0x7fffffffLL) return false;
   if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
   if (variant == DETAG_VARIANT_DENSE) return true;
   if (variant != DETAG_VARIANT_RING) return false;
@@ -636,10 +636,11 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   analyse_torus(s);
   if (n > detag::kMaxDenseStepWorkers && n <= detag::kMaxSplitWorkers) {
     // tables for whichever of the two kernels may be asked (rows_ok); those of step_rows.cu take 1 .. 3 ms to make beyond 128 workers
-    // and are left out where calls will surely not use them
+    // and are left out where calls will surely not use them: both sides of rows_ok's estimates with a margin, and at 160 SMs
+    // (detag_create of 254 workers, K = 3, d = 374 3.4 ms -> 0.02 and 0.85 MB less of workspace)
     const bool blocks = block_circulant(s);
     const double products = static_cast<double>(K) * nnz, rounds = std::fmax(0.0155 * n * K, 0.625e-3 * (0.024 * n + 0.00155 * products) * static_cast<double>(d));
-    const bool rows = n <= 128 || (blocks ? n <= 192 || d <= 40LL * 32 * 160 : 10.0 + 0.065 * n < 1.5 * (8.0 + rounds));
+    const bool rows = n <= 128 || (blocks ? n <= 192 || d <= 40LL * 32 * 160 : 10.0 + 0.065 * n * std::ceil(static_cast<double>(d) / (32 * 160)) < 1.25 * (8.0 + rounds));
     if (blocks) {
       first_block_row(s, poly);
     } else if (n > 128 && rows) {
