@@ -14,7 +14,7 @@ namespace {
 // (at most 0x7F7F7F7F7F) hold every operand; maxima below 2^-90 leave the range of the float32 scale.
 constexpr unsigned kRoundUp = 0x18000u, kSmallest = 0x12800000u;
 
-// Digits of four workers' values x (+ rest, below an ulp of x): digit k of all four in d[k].  The value z scale, at most 31 bits before
+// Digits of four workers' values x (+ rest, below 2^-18 of the coordinate's largest): digit k of all four in d[k].  The value z scale, at most 31 bits before
 // the point, in two steps that float32 does exactly: its multiple of 2^14 next to it, and what is left in 1/256, each as the low bits
 // of 1.5 * 2^23 plus it.  With the 40-bit integer q of both, q + 0x0080808080 has the balanced digits as bytes, all but the top one
 // offset by 128.  No conversions: they run on a pipe a quarter as wide.
@@ -50,20 +50,35 @@ __device__ __forceinline__ void four_digits(const float* src, int pitch, float s
   digits_of<false>(x, x, scale, d);
 }
 
-// Of the sums y + (g_new - g) of four workers, the three arrays `array` floats apart: both operations' roundings are added up exactly
-// (Knuth's two-sum) and rounded once, which leaves 2^-48 of the largest of the three.
+// y + (g_new - g) (Algorithm 2's tracker update) as a float32 next to it: what the difference rounds off (Knuth's two-sum) is added again.  The
+// sum may be far below its parts - all of it may be what was rounded off - but then y + fl(g_new - g) is exact (Sterbenz: the two are
+// within a factor of two of one another), and the result is the sum rounded once; otherwise it is off by some ulps.
+__device__ __forceinline__ float fold_value(float y, float g_new, float g) {
+  const float t = g_new - g, tb = t - g_new;  // tb: the part of t that stands for -g
+  return (y + t) + ((g_new - (t - tb)) - (g + tb));
+}
+
+// Digits of the sums y + (g_new - g) of four workers, the three arrays `array` floats apart: x = fl(y + fl(g_new - g)) and both roundings'
+// errors e1, e2 (exact).  Where the parts cancel e1 + e2 is exact too (e2 = 0), and elsewhere below 2^-22 of x, so that x and their sum
+// rounded once are the sum to 2^-46 of itself.  digits_of wants the latter below 2^-18 of the coordinate's largest: kCancels where
+// that is not known, and then the two are normalised (x becomes the float32 next to the sum; |e1 + e2| <= |x|, or x = 0).
+template <bool kCancels>
 __device__ __forceinline__ void four_fold_digits(const float* src, int array, int pitch, float scale, uint32_t (&d)[5]) {
   F2 x[2], rest[2];
 #pragma unroll
   for (int v = 0; v < 2; ++v) {
     const float* const at = src + 2 * v * pitch;
     const F2 y = pack2(at[0], at[pitch]), b = pack2(at[array], at[array + pitch]), a = pack2(at[2 * array], at[2 * array + pitch]);
-    const F2 t = sub2(b, a), tb = sub2(t, b);                              // g_new - g, and the part of it that stands for -g
+    const F2 t = sub2(b, a), tb = sub2(t, b);
     const F2 e1 = sub2(sub2(b, sub2(t, tb)), add2(a, tb));
     x[v] = add2(y, t);
     const F2 xt = sub2(x[v], y);
-    const F2 e2 = add2(sub2(y, sub2(x[v], xt)), sub2(t, xt));
-    rest[v] = add2(e1, e2);
+    rest[v] = add2(e1, add2(sub2(y, sub2(x[v], xt)), sub2(t, xt)));
+    if (kCancels) {
+      const F2 s = add2(x[v], rest[v]);
+      rest[v] = sub2(rest[v], sub2(s, x[v]));
+      x[v] = s;
+    }
   }
   digits_of<true>(x, rest, scale, d);
 }

@@ -21,14 +21,15 @@
 // quarter, which only one of the SM's schedulers reaches, has nothing to finish; there that scheduler's warps do the splitting (96
 // workers, d = 1 M 801 -> 782 us).
 //
-// Caller-written gradients: y + (g_new - g) is split as the float32 sum and what it rounds off; g' = g_new is stored from the staged rows.
+// Caller-written gradients: y + (g_new - g) is split as the float32 sum and what it rounds off, normalised where the three cancel (a loop of
+// its own for each: with the choice inside the unrolled one 100 workers, d = 1 M 862 -> 930 us); g' = g_new is stored from the staged rows.
 //
 // Bound by issue slots and latency of the finishing warps (137 instructions per worker-coordinate of 128 lanes, 0.6 of the slots), by
 // the power cap (1.5 .. 1.7 GHz on long vectors), and beyond a row pitch of 2 MB by rows travelling in pieces of 128 bytes: loads
 // and stores alone then reach 0.68 of the copy rate (0.85 below that pitch), where 256-byte pieces reach 0.84.  us per step,
 // step_split.cu -> here: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0, 300 k 283 -> 262, 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7, 1 M 1063 -> 1044;
 // D-PSGD of 128, 1 M 966 -> 828; 256-ring, K = 40, d = 4 k 34.6 -> 21.9, 60 k 285 -> 207; rounds -> here: 144, K = 6, d = 500 k 3396 -> 984, 256
-// 5327 -> 1680 (waiting for P; all of it at hand would be 1250); caller-written gradients, 100 workers, d = 1 M 3177 -> 895, 20 k 76 -> 28.
+// 5327 -> 1680 (waiting for P; all of it at hand would be 1250); caller-written gradients, 100 workers, d = 1 M 3177 -> 862, 20 k 76 -> 27.
 //
 // Measured without gain: asking for 256-byte pieces in L2 ahead of the loads 917 -> 1200 us (128 workers, loads and stores alone); sums
 // read sixteen columns at a time 966 -> 1043 (spills); normals drawn before the sums, or by half of the groups before, 1690 -> 1815, 1905
@@ -458,20 +459,47 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
       }
       auto value = [&](int w) {
         const float* const at = col + w * kPS;
-        return kMode == kModeExternal && fold ? at[0] + (at[array_floats] - at[2 * array_floats]) : at[0];
+        return fold ? at[0] + (at[array_floats] - at[2 * array_floats]) : at[0];
       };
       // largest magnitude, and the smallest of the largest magnitudes of the guard's groups
       float top_f = 0.f, low_f = __uint_as_float(0x7f800000u);
       if (!idle) {
+        float change = 0.f;  // largest |g_new - g|
+        auto largest = [&](auto four) {  // `four`: of four workers
 #pragma unroll 1
-        for (int h = part; h < halves; h += kParts) {
-          float m[4];
+          for (int h = part; h < halves; h += kParts) {
+            float m[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            m[i] = max_abs3(max_abs3(value(16 * h + 4 * i), value(16 * h + 4 * i + 1), value(16 * h + 4 * i + 2)), value(16 * h + 4 * i + 3), 0.f);
-          top_f = max_abs3(max_abs3(m[0], m[1], m[2]), m[3], top_f);
+            for (int i = 0; i < 4; ++i) {
+              float v[4];
+              four(col + (16 * h + 4 * i) * kPS, v);
+              m[i] = max_abs3(max_abs3(v[0], v[1], v[2]), v[3], 0.f);
+            }
+            top_f = max_abs3(max_abs3(m[0], m[1], m[2]), m[3], top_f);
+          }
+        };
+        if (fold) {
+          largest([&](const float* at, float (&v)[4]) {
+            float t[4];
+#pragma unroll
+            for (int u = 0; u < 4; u += 2) {
+              const float *const p0 = at + u * kPS, *const p1 = p0 + kPS;
+              const F2 delta = sub2(pack2(p0[array_floats], p1[array_floats]), pack2(p0[2 * array_floats], p1[2 * array_floats]));
+              unpack2(delta, t[u], t[u + 1]);
+              unpack2(add2(pack2(p0[0], p1[0]), delta), v[u], v[u + 1]);
+            }
+            change = max_abs3(max_abs3(change, t[0], t[1]), t[2], t[3]);
+          });
+        } else {
+          largest([&](const float* at, float (&v)[4]) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = at[u * kPS];
+          });
         }
         low_f = group_low(value, guard, tb.guard_groups, tb.guard_size, part, kParts);
+        // These sums lack what their two roundings leave out, 2^-24 of the difference and of themselves: below 2^-18 of the largest of
+        // them while that is 2^-5 of the largest difference.  Else every warp looks anew, below.
+        if (fold && change * 0x1p-5f > top_f) low_f = -1.f;
       }
       float2* const mx = maxima + (k & 1) * 4 * kPColumns + column;  // read again two chunks later, behind the next hand-over
       mx[part * kPColumns] = make_float2(top_f, low_f);
@@ -484,6 +512,14 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
         const float2 other = mx[i * kPColumns];
         top_f = max_abs3(top_f, other.x, 0.f);
         low_f = fminf(low_f, other.y);
+      }
+      const bool cancels = fold && __any_sync(0xffffffffu, low_f < 0.f);  // the same in all warps of the array
+      if (cancels) {
+        auto sum = [&](int w) { return fold_value(col[w * kPS], col[w * kPS + array_floats], col[w * kPS + 2 * array_floats]); };
+        top_f = 0.f;
+#pragma unroll 2
+        for (int w = 0; w < 16 * halves; w += 2) top_f = max_abs3(sum(w), sum(w + 1), top_f);
+        low_f = group_low(sum, guard, tb.guard_groups, tb.guard_size, 0, 1);
       }
       const unsigned top = __float_as_uint(top_f);
       // as float bits: not finite, too small for the scale; an output may read nothing near the largest operand
@@ -500,21 +536,23 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
         if (lane == 0) flags[slot * 2 + array] = exact_lanes;
       }
       if (!idle) {
+        auto split_all = [&](auto four) {
 #pragma unroll 1
-        for (int h = part; h < halves; h += kParts) {
-          uint32_t d[4][kPDigits];
+          for (int h = part; h < halves; h += kParts) {
+            uint32_t d[4][kPDigits];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float* const src = col + (h * 16 + 4 * u) * kPS;
-            if (kMode == kModeExternal && fold) {
-              four_fold_digits(src, array_floats, kPS, scale, d[u]);
-            } else {
-              four_digits(src, kPS, scale, d[u]);
-            }
+            for (int u = 0; u < 4; ++u) four(col + (h * 16 + 4 * u) * kPS, d[u]);
+            unsigned char* const at = to + (buf * nb + (h >> 1)) * kPBlockBytes + (h & 1) * 128;
+#pragma unroll
+            for (int q = 0; q < kPDigits; ++q) *reinterpret_cast<uint4*>(at + q * kPDigitBytes) = make_uint4(d[0][q], d[1][q], d[2][q], d[3][q]);
           }
-          unsigned char* const at = to + (buf * nb + (h >> 1)) * kPBlockBytes + (h & 1) * 128;
-#pragma unroll
-          for (int q = 0; q < kPDigits; ++q) *reinterpret_cast<uint4*>(at + q * kPDigitBytes) = make_uint4(d[0][q], d[1][q], d[2][q], d[3][q]);
+        };
+        if (cancels) {
+          split_all([&](const float* src, uint32_t (&d)[kPDigits]) { four_fold_digits<true>(src, array_floats, kPS, scale, d); });
+        } else if (fold) {
+          split_all([&](const float* src, uint32_t (&d)[kPDigits]) { four_fold_digits<false>(src, array_floats, kPS, scale, d); });
+        } else {
+          split_all([&](const float* src, uint32_t (&d)[kPDigits]) { four_digits(src, kPS, scale, d); });
         }
       }
       fence_async_shared();  // the MMAs read the digits through the asynchronous proxy

@@ -72,6 +72,58 @@ def test_caller_written_gradients(n, d, K, kind):
             assert np.array_equal(got["g"], gn) and np.array_equal(got["y_gossip"], got["y"])
 
 
+@pytest.mark.parametrize("n,kind", [(60, "regular4"), (90, "regular4"), (128, "regular4"), (160, "ring"), (192, "regular4")])
+@pytest.mark.parametrize("K", [1, 2, 6])
+def test_caller_written_gradients_whose_fold_cancels(n, kind, K):
+    """y + g_new - g far below its parts: the first step after detag_init (y = g) where gradients have fallen.  The bound knows the sum z
+    alone: half an ulp of what is stored and as much again of the magnitudes read, nothing of the three parts (of which float64 itself
+    loses 2^-53, here some 2^-28 of the sum)."""
+    d, eta, alpha = 3 * CHUNKS + 35, 0.2, 0.05
+    m = _graph(kind, n)
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(n + K)
+    cols = np.unique(np.concatenate([np.arange(140), np.arange(d - 140, d), rng.integers(0, d, 500)]))
+    f = np.float32
+    x, y, g, gn = (rng.standard_normal((n, d), dtype=f) for _ in range(4))
+    y[:] = g
+    kind_of = np.arange(d) % 14
+    for k in range(9):  # gradients that fall by 2^0, 2^-3, .. 2^-24
+        gn[:, kind_of == k] *= f(2.0 ** (-3 * k))
+    outlier = np.ix_([n // 3], np.flatnonzero(kind_of == 9))  # one worker's gradient was large, the others are what they were
+    g[outlier] *= f(1e6)
+    y[outlier] = g[outlier]
+    at = kind_of == 10  # the float32 sum is zero at every worker, the exact one is not
+    y[:, at] = g[:, at] = f(1.0) + rng.random((n, at.sum()), dtype=f)
+    gn[:, at] = np.copysign(f(2.0 ** -25) * (f(1.0) + rng.random((n, at.sum()), dtype=f)), gn[:, at])
+    at = kind_of == 11  # all but cancels
+    y[:, at] *= f(1.0) + f(2.0 ** -20) * rng.standard_normal((n, at.sum()), dtype=f)
+    gn[:, at] *= f(2.0 ** -14)
+    at = kind_of == 12  # the gradients cancel, the tracker is small
+    gn[:, at] = g[:, at] * (f(1.0) + f(2.0 ** -18) * rng.standard_normal((n, at.sum()), dtype=f))
+    y[:, at] = f(2.0 ** -20) * rng.standard_normal((n, at.sum()), dtype=f)
+    at = kind_of == 13  # the tracker cancels the new gradient
+    y[:, at] = -gn[:, at]
+    g[:, at] *= f(2.0 ** -24)
+    zero = np.zeros((n, d), f)
+    with Session(m, d, K, eta, alpha, zero, zero, zero, external_gradient=True) as s:
+        for k, v in (("x", x), ("y", y), ("g", g), ("g_new", gn)):
+            s.upload(k, v)
+        s.step()
+        s.status()
+        got = {k: s.download(k)[:, cols].astype(np.float64) for k in ("x", "y", "g")}
+    wide = np.longdouble
+    z = (y[:, cols].astype(wide) - g[:, cols].astype(wide) + gn[:, cols].astype(wide)).astype(np.float64)
+    x = x[:, cols].astype(np.float64)
+    yt = P @ z
+    of_y = 2.0 ** -24 * (np.abs(yt) + np.abs(P) @ np.abs(z)) + 1e-45
+    xt = P @ x - alpha * yt
+    of_x = 2.0 ** -24 * (np.abs(xt) + np.abs(P) @ np.abs(x)) + alpha * of_y + 1e-45
+    worst = [float((np.abs(got["y"] - yt) / of_y)[:, cols % 14 == k].max()) for k in range(14)]
+    assert max(worst) <= 1.0, [round(v, 2) for v in worst]
+    assert (np.abs(got["x"] - xt) <= of_x).all()
+    assert np.array_equal(got["g"], gn[:, cols])
+
+
 def test_caller_written_gradients_that_are_not_finite():
     n, d, K, eta = 70, 40, 2, 0.2
     m = _graph("ring", n)
