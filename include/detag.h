@@ -329,9 +329,14 @@ int detag_status(detag_state* s, void* stream);
  * detag_debug_expire_wait: launches one thread that waits, through the same bounded wait, on a barrier that
  * nothing ever arrives at, with a limit of `polls` polls (1 .. 2^20); it gives up, sets the workspace's status
  * word and returns.  Asynchronous.  Errors: ARG, UNBOUND, CUDA.
+ *
+ * detag_debug_kernel: file name (without its ending) of the kernel that the last detag_step, detag_step_many or detag_step_host call launched
+ * for this state (part 0), or of the one that took a band's last coordinates in the same call (part 1); "" if none.  Static text, host only:
+ * so that a test can hold a case to the kernel it was written for.
  */
 int detag_debug_inject_stall(detag_state* s, int64_t after_tiles, uint32_t poll_limit);
 int detag_debug_expire_wait(detag_state* s, uint32_t polls, void* stream);
+const char* detag_debug_kernel(const detag_state* s, int part);
 
 /* Text of the last error on this state ("" if none).  Owned by the state. */
 const char* detag_last_error(const detag_state* s);

@@ -69,6 +69,7 @@ SIGNATURES = {
     "detag_set_gradient_source": (ctypes.c_int, [_P, ctypes.c_int, _P]),
     "detag_debug_inject_stall": (ctypes.c_int, [_P, ctypes.c_int64, ctypes.c_uint32]),
     "detag_debug_expire_wait": (ctypes.c_int, [_P, ctypes.c_uint32, _P]),
+    "detag_debug_kernel": (ctypes.c_char_p, [_P, ctypes.c_int]),
     "detag_zero_chain_gradient": (ctypes.c_int, [ctypes.c_int, ctypes.c_int64, ctypes.c_int64, _P, _P, ctypes.c_double,
                                                  ctypes.c_double, ctypes.c_double, ctypes.c_uint64, ctypes.c_int64, _P, _P]),
     "detag_phase_length": (ctypes.c_int, [ctypes.c_int, ctypes.c_double, ctypes.c_double, ctypes.c_double,
@@ -222,6 +223,11 @@ def detag_debug_inject_stall(state, after_tiles: int, poll_limit: int = 2048) ->
 
 def detag_debug_expire_wait(state, polls: int, stream=None) -> None:
     _check(lib().detag_debug_expire_wait(state, int(polls), _stream_handle(stream)), "detag_debug_expire_wait", state)
+
+
+def detag_debug_kernel(state, part: int = 0) -> str:
+    """Kernel the last step launched (part 0), or the one of a band's last coordinates (part 1); "" if none."""
+    return lib().detag_debug_kernel(state, int(part)).decode()
 
 
 def detag_zero_chain_gradient(n: int, d: int, ld: int, x, g_out, lam: float, gain: float, p: float, seed: int, t: int,

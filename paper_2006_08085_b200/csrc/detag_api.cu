@@ -411,6 +411,7 @@ int launch_split(detag_state* s, const StepParams& p, bool rows, bool wide, cuda
   const unsigned char* base = p.tables;
   const detag::SplitDevice tables{base + at.weights, reinterpret_cast<const int32_t*>(base + at.row_exp), base + at.guard,
                                   reinterpret_cast<const double*>(base + at.poly)};
+  s->launched[p.beside] = rows ? "step_rows" : "step_split";
   const int e = rows ? detag::launch_step_rows(p, *maps, s->rows, tables, wide, s->sm_count, stream)
                      : detag::launch_step_split(p, *maps, s->split, tables, wide, s->sm_count, stream);
   return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
@@ -433,6 +434,7 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   pt.beside = first > 0 ? 1 : 0;
   if (p.n <= 128 && !s->rows.weights.empty()) return launch_split(s, pt, true, false, stream);
   if (!s->split.weights.empty() && 6.0 + 0.0068 * p.n * s->K > 0.15 * p.n) return launch_split(s, pt, false, false, stream);
+  s->launched[pt.beside] = "step_csr";
   const int rc = detag::plan_step_csr(pt, s->smem_optin);
   if (rc != DETAG_OK) return fail(s, rc, "graph too large for the shared-memory plan");
   const int e = detag::launch_step_csr(pt, s->sm_count, stream);
@@ -519,6 +521,7 @@ bool dense_step_ok(const detag_state* s, const StepParams& p, int variant) {
 // Picks the kernel variant, plans it for the sizes in `p` and launches it.
 int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   int e = 0;
+  s->launched[0] = s->launched[1] = "";
   const int variant = resolve_variant(s);
   if (!variant_runs_mode(s, variant))
     return fail(s, DETAG_ERR_UNSUPPORTED,
@@ -530,6 +533,7 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   if (dense_step_ok(s, p, variant)) {
     const detag::TensorMapSet* maps = maps_for(s, kFamilyDense, p);
     if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+    s->launched[0] = "step_dense";
     e = detag::launch_step_dense(p, *maps, s->sm_count, stream);
     return e != 0 ? fail_cuda(s, e, "step kernel launch") : DETAG_OK;
   }
@@ -544,11 +548,13 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
   switch (as_rounds ? DETAG_VARIANT_CSR : variant) {
     case DETAG_VARIANT_DENSE: {
       if (small_ok(p)) {
+        s->launched[0] = "step_small";
         e = detag::launch_step_small(p, s->sm_count, stream);
         break;
       }
       const detag::TensorMapSet* maps = maps_for(s, kFamilyMma, p);
       if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+      s->launched[0] = "step_mma";
       e = detag::launch_step_mma(p, *maps, s->sm_count, stream);
       break;
     }
@@ -559,6 +565,7 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
         pm.d = d_main;
         const detag::TensorMapSet* maps = maps_for(s, kFamilyRing, pm);
         if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+        s->launched[0] = "step_ring";
         e = detag::launch_step_ring(pm, *maps, s->band, s->sm_count, stream);
         if (e != 0) return fail_cuda(s, e, "step kernel launch");
       }
@@ -571,11 +578,13 @@ int launch_step(detag_state* s, StepParams& p, cudaStream_t stream) {
     case DETAG_VARIANT_TORUS: {
       const detag::TensorMapSet* maps = maps_for(s, kFamilyTorus, p);
       if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+      s->launched[0] = "step_torus";
       e = detag::launch_step_torus(p, *maps, p.torus, s->sm_count, stream);
       break;
     }
     case DETAG_VARIANT_CSR:
     default: {
+      s->launched[0] = "step_csr";
       const int rc = detag::plan_step_csr(p, s->smem_optin);
       if (rc != DETAG_OK) return fail(s, rc, "graph too large for the shared-memory plan");
       e = detag::launch_step_csr(p, s->sm_count, stream);
@@ -901,7 +910,9 @@ int detag_step_many(detag_state* s, int count, void* stream) {
       p.steps = now;
       if (!p.a || !p.c) return fail(s, DETAG_ERR_UNBOUND, "the synthetic gradient needs the objective arrays a and c");
       int e;
+      s->launched[1] = "";
       if (small_ok(p)) {
+        s->launched[0] = "step_small";
         e = detag::launch_step_small(p, s->sm_count, static_cast<cudaStream_t>(stream));
       } else {
         // Groups of four warps take a slab's steps in turn; the kernel with padded tiles puts eight warps on one, which is ahead
@@ -914,6 +925,7 @@ int detag_step_many(detag_state* s, int count, void* stream) {
         const bool padded = p.n <= detag::kMaxSmallWorkers || (p.n > 24 && p.d <= 128LL * s->sm_count) || (p.n > 28 && p.d > 192LL * s->sm_count);
         const detag::TensorMapSet* maps = maps_for(s, padded ? kFamilyMma : kFamilyDense, p);
         if (!maps) return fail(s, DETAG_ERR_CUDA, "tensor map encoding failed");
+        s->launched[0] = padded ? "step_mma_many" : "step_dense";
         e = padded ? detag::launch_step_mma_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream))
                    : detag::launch_step_dense_many(p, *maps, s->sm_count, static_cast<cudaStream_t>(stream));
       }
@@ -1062,6 +1074,8 @@ int detag_status(detag_state* s, void* stream) {
   s->d_status_host = nullptr;  // read and clean: the staging area is not referred to again until the next host step
   return DETAG_OK;
 }
+
+const char* detag_debug_kernel(const detag_state* s, int part) { return s && (part == 0 || part == 1) ? s->launched[part] : ""; }
 
 const char* detag_last_error(const detag_state* s) { return s ? s->err.c_str() : ""; }
 

@@ -182,6 +182,7 @@ struct detag_state {
   const float* g_ext = nullptr;
   unsigned spin_limit = 1u << 20;
   long long stall_after = -1;
+  const char* launched[2] = {"", ""};  // detag_debug_kernel
 
   bool bound = false;
   long long ld = 0;

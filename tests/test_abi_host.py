@@ -116,6 +116,7 @@ def test_state_accessors_without_device():
         assert B.detag_get_step(st) == 0
         B.detag_set_step(st, 7)
         assert B.detag_get_step(st) == 7
+        assert B.detag_debug_kernel(st) == B.detag_debug_kernel(st, 1) == B.detag_debug_kernel(st, 2) == ""  # no step yet
         B.detag_set_noise(st, 0.1, 3)
         assert B.detag_get_variant(st) in (B.DETAG_VARIANT_CSR, B.DETAG_VARIANT_DENSE, B.DETAG_VARIANT_RING)
         with pytest.raises(B.DetagError) as e:
