@@ -322,7 +322,8 @@ __device__ __noinline__ void exact_sums(const float* z, const double* poly, unsi
 }
 
 // kWide: the gradient in float64 (the precision of the rounds kernel, in whose place
-// the call runs) instead of float32 at the rounded model (the other tensor-path kernels').  kRows: 64, 96, 128 or 256, n rounded up.
+// the call runs; beyond 128 workers, where it would run there, sigma xi in float64 too) instead of float32 at the rounded model (the other
+// tensor-path kernels').  kRows: 64, 96, 128 or 256, n rounded up.
 // kAtStart: the gradient at the model the step started from.
 template <int kMode, bool kWide, int kRows, bool kAtStart>
 __global__ void __launch_bounds__(kPThreads, 1)
@@ -592,6 +593,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
     const int row = (kCopies == 2 ? quarter & 1 : quarter) * 32 + lane, part = kCopies == 2 ? 2 * (group & 1) + (quarter >> 1) : group;
     const uint32_t acc = tmem + (static_cast<uint32_t>(quarter) << 21) + 2 * kPGroup * part;
     const double alpha = p.alpha;
+    constexpr bool kWideNoise = kWide && kTwo;
     const float sigma = static_cast<float>(p.sigma);
     const bool noisy = kMode != kModeExternal && p.sigma != 0.0;
     const int d = static_cast<int>(p.d), d_tma = d & ~3;  // columns below d_tma are written by the TMA stores
@@ -642,7 +644,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
             float t[4];
-            normal_quad(p.round_key, jn + 4 * i, static_cast<uint32_t>(w >> 2), p.t_noise, sigma, t);
+            normal_quad(p.round_key, jn + 4 * i, static_cast<uint32_t>(w >> 2), p.t_noise, kWideNoise ? 1.f : sigma, t);
             transpose_quad(t, lane & 3);
 #pragma unroll
             for (int u = 0; u < 4; ++u) xi[4 * i + u] = t[u];
@@ -706,7 +708,8 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
               if (kWide) {
 #pragma unroll
                 for (int e = u; e < u + 2; ++e)
-                  go[e] = static_cast<float>(fma(static_cast<double>(av[e]), (kAtStart ? static_cast<double>(from[e]) : sums[e]) - static_cast<double>(cv[e]), static_cast<double>(xi[e])));
+                  go[e] = static_cast<float>(fma(static_cast<double>(av[e]), (kAtStart ? static_cast<double>(from[e]) : sums[e]) - static_cast<double>(cv[e]),
+                                                    kWideNoise ? static_cast<double>(sigma) * static_cast<double>(xi[e]) : static_cast<double>(xi[e])));
               } else {
                 unpack2(fma2(pack2(av[u], av[u + 1]), sub2(pack2(from[u], from[u + 1]), pack2(cv[u], cv[u + 1])), pack2(xi[u], xi[u + 1])), go[u], go[u + 1]);
               }

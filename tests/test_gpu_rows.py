@@ -197,3 +197,24 @@ def test_loads_that_stop_time_out_and_the_state_recovers(n, mode, after):
             s.status()
             got.append({k: s.download(k) for k in ("x", "y", "g")})
     assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])
+
+
+@pytest.mark.parametrize("n,mode", [(144, "detag"), (200, "start"), (256, "dpsgd")])
+def test_the_gradient_beyond_128_workers_is_the_rounds(n, mode):
+    """Matrices without block structure: a o (x' - c) + sigma xi in float64, rounded once, as on the rounds kernel.  The models differ by the
+    fixed point's 1e-11 before they are rounded, which tips a few gradients in 10^5; a float32 product sigma xi tips one in five."""
+    from paper_2006_08085_b200 import binding as B
+    d, K, m = 5 * CHUNKS + 7, 6, _graph("regular4", n)
+    rng = np.random.default_rng(n)
+    state = {k: rng.standard_normal((n, d), dtype=np.float32) for k in ("x", "y", "g", "a", "c")}
+    got = []
+    for variant in (B.DETAG_VARIANT_AUTO, B.DETAG_VARIANT_CSR):
+        with Session(m, d, K, 0.2, 0.01, sigma=0.3, seed=5, variant=variant, gradient_point=int(mode == "start"),
+                     algorithm=int(mode == "dpsgd")) as s:
+            for k, v in state.items():
+                s.upload(k, v)
+            s.step()
+            s.status()
+            got.append((s.download("g"), B.detag_debug_kernel(s.state)))
+    assert [name for _, name in got] == ["step_rows", "step_csr"]
+    assert np.count_nonzero(got[0][0] != got[1][0]) <= 2e-4 * n * d
