@@ -419,8 +419,8 @@ int launch_split(detag_state* s, const StepParams& p, bool rows, bool wide, cuda
 
 // The columns from `first` on, which the circulant kernel leaves (it takes whole 64-coordinate slabs), in the same call, beside
 // it (64-ring, K = 4, d = 14001 21.3 -> 14.6 us in one launch, 256, d = 60001 188 -> 168 in two): through the integer tensor path up to
-// 128 workers (one chunk or two 8 .. 11 us), beyond as rounds while their latency is the smaller one (256 workers 6 us and 1.7 a round,
-// step_split.cu's slab 38).
+// 128 workers (one chunk or two 8 .. 11 us), beyond as rounds, whose latency is the smaller one (256 workers 6 us and 1.7 a round,
+// step_split.cu's slab 38), and so where the caller asked for the circulant kernel, which runs in float64 throughout.
 int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cudaStream_t stream) {
   StepParams pt = p;
   pt.d = p.d - first;
@@ -432,8 +432,7 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
   pt.c = p.c + first;
   if (p.y_obs) pt.y_obs = p.y_obs + first;
   pt.beside = first > 0 ? 1 : 0;
-  if (p.n <= 128 && !s->rows.weights.empty()) return launch_split(s, pt, true, false, stream);
-  if (!s->split.weights.empty() && 6.0 + 0.0068 * p.n * s->K > 0.15 * p.n) return launch_split(s, pt, false, false, stream);
+  if (p.n <= 128 && !s->rows.weights.empty() && s->variant_forced == DETAG_VARIANT_AUTO) return launch_split(s, pt, true, false, stream);
   s->launched[pt.beside] = "step_csr";
   const int rc = detag::plan_step_csr(pt, s->smem_optin);
   if (rc != DETAG_OK) return fail(s, rc, "graph too large for the shared-memory plan");
@@ -445,20 +444,20 @@ int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cu
 // library's, the rounds of such matrices too.  Circulant bands stay on their float64 kernel, which needs no test of the
 // operands; us per step, integer path -> that one: 64 workers, d = 2 M, K = 1 1099 -> 1035, K = 16 1020 -> 1035; 128, d = 1 M,
 // K = 1 1260 -> 1031, K = 16 1103 -> 1031; 224, d = 500 k, K = 16 1198 -> 927; 256, d = 1 M, K = 1 3157 -> 2032, K = 16
-// 2620 -> 2032; 256, d = 4096 82 -> 30.  Unless d is ragged, up to 128 workers, and so short that one launch takes less than two side by
-// side: 64 workers, K = 4, d = 3001 13.8 -> 9.6, 60001 50.4 -> 40.5, but 200001 125 -> 129; 128, 3001 15.3 -> 12.4, but 9001 15.9 -> 18.7; 256, 3001
-// 42.8 -> 67.  Or, up to 128 workers, the band is nearly as wide as the float64 kernel takes, so that the test is short (float64 -> integer):
-// 64, K = 12, d = 60032 42.1 -> 35.5; 96, K = 16, 200001 174 -> 157, 1 M 769 -> 751, but K = 12 768 -> 778; 128, K = 16, 60001 80.6 -> 62.8; D-PSGD of
-// 128, K = 12, 1 M 1011 -> 847; narrower: 96, K = 4, 1 M 769 against 808, K = 8 769 against 792.
+// 2620 -> 2032; 256, d = 4096 82 -> 30.  (Bands of half-width 12 to 16 of up to 128 workers gain on the integer path with operands alike -
+// 64, K = 12, d = 60 k 47 -> 45, 128, K = 16 105 -> 73 - and lose with operands spread over four decades: 47 -> 163, 119 -> 272.)
+// Unless the choice is the library's and d is ragged, up to 128 workers, and so short that one launch takes less than two side by
+// side: 64 workers, K = 4, d = 3001 13.8 -> 9.6; 128, 3001 15.3 -> 12.4, but 9001 15.9 -> 18.7; 256, 3001
+// 42.8 -> 67.  Longer ones of 64 would gain too, with operands alike (d = 60001 50.4 -> 40.5; spread 69 -> 172).
 bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   if ((s->split.weights.empty() && s->rows.weights.empty()) || p.d > 0x7fffffffLL) return false;
   if (variant == DETAG_VARIANT_CSR) return s->variant_forced == DETAG_VARIANT_AUTO;
   if (variant == DETAG_VARIANT_DENSE) return true;
   if (variant != DETAG_VARIANT_RING) return false;
   if (!ring_band(s)) return true;
+  if (s->variant_forced != DETAG_VARIANT_AUTO) return false;
   // by the length of the state, not of a staged chunk: host-resident stepping gives the same bits
-  if (s->n <= 128 && s->half_band >= 12 && (p.mode == detag::kModeDpsgd || s->d <= 128LL * 32 * s->sm_count)) return true;
-  return s->d % 64 != 0 && s->d <= (s->n <= 64 ? 20LL : s->n <= 128 ? 1LL : 0LL) * 32 * s->sm_count;
+  return s->d % 64 != 0 && s->d <= (s->n <= 64 ? 4LL : s->n <= 128 ? 1LL : 0LL) * 32 * s->sm_count;
 }
 
 // Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0,

@@ -115,3 +115,42 @@ def test_ragged_steps_in_a_row_give_the_bits_of_steps_one_by_one(n, d, K):
             s.status()
             got.append({k: s.download(k) for k in ("x", "y", "g")})
     assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])
+
+
+@pytest.mark.parametrize("n,d,K,mode", [(64, 3 * 64 + 5, 16, "new"), (64, SLABS - 3, 4, "start"), (96, 2 * SLABS + 64, 14, "new"), (128, SLABS + 33, 16, "dpsgd"),
+                                        (160, 131, 16, "new")])
+def test_the_variant_chosen_by_name_runs_in_float64_throughout(n, d, K, mode):
+    """Every sum is a float64 one rounded once, whatever the width of the band and the length: also where the sum cancels to a
+    hundred-thousandth of what it reads, of which fixed point of 39 bits would leave an error of 2^-21."""
+    m, eta = _matrix("ring", n), 0.2
+    prev, w = np.eye(n), m.to_dense()
+    P = prev
+    for _ in range(K):
+        prev, P = P, (1.0 + eta) * w @ P - eta * prev
+    x, y = np.random.default_rng(n + d).standard_normal((2, n, d)).astype(np.float32)
+    zero = np.zeros((n, d), np.float32)
+    with Session(m, d, K, eta, 0.0, zero, zero, x, observe_gossip=mode != "dpsgd", variant=B.DETAG_VARIANT_RING, gradient_point=int(mode == "start"),
+                 algorithm=int(mode == "dpsgd")) as s:
+        s.upload("y", y)
+        s.step()
+        s.status()
+        got = {"x": (s.download("x"), x)}
+        if mode != "dpsgd":
+            got["y"] = (s.download("y_gossip"), y)
+        ran = [B.detag_debug_kernel(s.state, part) for part in (0, 1)]
+    assert ran == ["step_ring", "step_csr" if d % 64 != 0 else ""]
+    for name, (have, z) in got.items():
+        want, reads = P @ z.astype(np.float64), np.abs(P) @ np.abs(z.astype(np.float64))
+        bound = 2.0 ** -24 * np.abs(want) + 2.0 ** -46 * reads + 1e-45
+        assert (np.abs(have - want) <= bound).all(), name
+
+
+@pytest.mark.parametrize("n,d,K,algorithm,ran", [
+    (64, 60_032, 12, 0, ("step_ring", "")), (96, 200_001, 16, 0, ("step_ring", "step_rows")), (128, 60_001, 16, 0, ("step_ring", "step_rows")),
+    (128, 4096, 16, 1, ("step_ring", "")), (256, 3_001, 4, 0, ("step_ring", "step_csr")), (64, 4 * 32 * 148 + 1, 4, 0, ("step_ring", "step_rows")),
+    (64, 3_001, 4, 0, ("step_rows", "")), (128, 3_001, 16, 0, ("step_rows", "")), (128, 32 * 148 + 1, 4, 1, ("step_ring", "step_rows"))])
+def test_bands_stay_in_float64_but_for_the_last_columns_and_short_ragged_calls(n, d, K, algorithm, ran):
+    with Session(_matrix("ring", n), d, K, 0.2, 0.01, algorithm=algorithm) as s:
+        s.step()
+        s.status()
+        assert tuple(B.detag_debug_kernel(s.state, part) for part in (0, 1)) == ran
