@@ -460,39 +460,65 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
   return s->d % 64 != 0 && s->d <= (s->n <= 64 ? 4LL : s->n <= 128 ? 1LL : 0LL) * 32 * s->sm_count;
 }
 
+// Whether step_rows.cu takes less than the rounds: caller-written gradients up to 192 workers, beyond 128 matrices without block
+// structure.  Estimates of both in us (`sms`: as if on that many SMs; before the tables are made with their best case).  Rounds -> there, operands alike: caller-written,
+// 100 workers, K = 6, d = 1 M 3177 -> 862, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 984,
+// 256, K = 12, d = 200 k 3830 -> 750, ring of 144, K = 4, d = 8931 35.6 against 48.1.  On short vectors rounds take their latency, one after the other:
+// caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
+// The rounds do not care how operands differ, and there what cannot share a scale is summed in float64 at up to five times the time (22 us more
+// per turn of the SMs at 100 workers, 61 at 256).  So the estimate is for operands spread over four decades (a tenth is allowed): few rounds on sparse graphs
+// then stay rounds, which alike would gain.  Alike / spread over four / over eight decades against rounds: caller-written, 100, d = 1 M, K = 2
+// 1323 / 5380 / 6348 against 1638, K = 4 1118 / 3392 / 4972 against 2402, but K = 6 923 / 1265 / 3321 against 3175; 144, d = 500 k, K = 6 894 / 2580 / 4251
+// against 3100; 256, d = 200 k, K = 4 719 / 3335 / 3338 against 1591, K = 6 731 / 2767 / 3215 against 2137, but K = 12 745 / 1157 / 2724 against 3827.
+bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
+  const detag::SplitPoly& t = s->rows;
+  const double n = s->n, d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * sms));
+  const double products = s->K * static_cast<double>(s->col_idx.size());
+  const bool sparse = t.guard.size() > static_cast<size_t>(s->n);
+  int reach = 0;  // 32 x 32 blocks that the float64 path goes through, per 32 outputs
+  for (unsigned char r : t.reach) reach += __builtin_popcount(r);
+  const double blocks = reach / std::ceil(n / 32.0);
+  double here, unequal, rounds, latency;
+  if (mode == detag::kModeExternal) {
+    here = n > 128 ? 10.0 + 0.065 * n * turns * (sparse ? 1.5 : 1.0)
+                   : 9.0 + turns * (1.0 + 0.031 * n) * (sparse && n > 64 && n <= 96 ? 2.2 : 1.0);  // six warps for the test
+    unequal = t.unequal * (n > 128 ? 20.0 + 2.4 * blocks : 5.5 * blocks);
+    rounds = 6.0 + (n > 128 ? 1.2 + 0.003 * n + 0.00105 * products : 0.0021 * n + 0.00099 * products) * d / 1000.0;
+    latency = 6.0 + 0.0155 * n * s->K;
+  } else {
+    here = sparse ? 14.0 + 0.098 * n * turns : 10.0 + 0.065 * n * turns;
+    unequal = t.unequal * (3.5 + 7.2 * blocks);
+    rounds = (1.35 + 0.004 * n + 0.0011 * products) * d / 1000.0;
+    latency = 6.0 + 0.0068 * n * s->K;
+    if (mode == detag::kModeDpsgd) {  // one array
+      unequal = (1.0 - std::sqrt(1.0 - t.unequal)) * 0.75 * (3.5 + 7.2 * blocks);
+      rounds *= 0.64;
+    }
+  }
+  rounds = std::fmax(std::fmax(rounds, latency), 8.0);
+  return here < rounds && here + unequal * d / (32.0 * sms) < 1.1 * rounds;
+}
+
 // Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0,
 // 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7; D-PSGD of 96, 10 k 17.5 -> 14.5, 1 M 707 -> 639, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
-// 8 k 12.4 -> 14.4, 300 k 224 -> 234, only the shortest of these better (96, 3000 11.7 -> 10.9, K = 1, 700 12.8 -> 11.4); 64, 10 k 12.9 -> 11.0, 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore
-// calls whose blocks have at most 32 chunks of 32 coordinates to do.  What would run as rounds otherwise - caller-written gradients up to
-// 192 workers, beyond 128 matrices without block structure - runs here if an estimate of both says so.  Block-circulant
+// 8 k 12.4 -> 14.4, 300 k 224 -> 234, only the shortest of these better (96, 3000 11.7 -> 10.9, K = 1, 700 12.8 -> 11.4); 64, 10 k 12.9 -> 11.0,
+// 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore calls whose blocks have at most 32 chunks of
+// 32 coordinates to do.  What would run as rounds otherwise runs here if rows_beat_rounds says so.  Block-circulant
 // matrices beyond 160 workers come here while P is dense and calls are not the longest (lanes as coordinates -> here: 256-ring, K = 40, d = 4 k
 // 34.6 -> 21.9, 60 k 285 -> 207, 16 x 16 torus, 19 k 88.5 -> 77.2, but K = 196, 200 k 577 -> 594, D-PSGD, 300 k 694 -> 775; torus, K = 2, 500 k 1152 -> 1202),
-// all with a chunk per block at most.  Rounds -> here: caller-written,
-// 100 workers, d = 1 M 3177 -> 895, 20 k 76 -> 28, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 984, 256 5327 -> 1680,
-// 180, K = 1, d = 72 k 225 against 230, ring of 144, K = 4, d = 8931 35.6 against 48.1.  Polynomials with few entries per row cost the
-// longer test of the operands, and more coordinates that fail it.  On short vectors rounds take their latency, one after the other:
-// caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
+// all with a chunk per block at most.
 bool rows_ok(const detag_state* s, const StepParams& p) {
   if (s->rows.weights.empty()) return false;
-  const double d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * s->sm_count));
-  const double products = s->K * static_cast<double>(s->col_idx.size());
+  if (p.mode == detag::kModeExternal) return detag::rows_take_external(s->rows) && rows_beat_rounds(s, p.mode, s->sm_count);
+  const double turns = std::ceil(static_cast<double>(s->d) / (32.0 * s->sm_count));
   const bool sparse = s->rows.guard.size() > static_cast<size_t>(s->n);
-  if (p.mode == detag::kModeExternal) {
-    const double here = p.n > 128 ? 10.0 + 0.065 * p.n * turns * (sparse ? 1.5 : 1.0)
-                                  : 9.0 + turns * (1.0 + 0.031 * p.n) * (sparse && p.n > 64 && p.n <= 96 ? 2.2 : 1.0);  // six warps for the test
-    const double rounds = std::fmax((0.0021 * p.n + 0.00099 * products) * d / 1000.0, 0.0155 * p.n * s->K);
-    return here < std::fmax(8.0, 6.0 + rounds) && detag::rows_take_external(s->rows);
-  }
   if (p.n <= 64) return turns <= 32.0 || s->split.weights.empty();
   if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd ? turns <= 64.0 || !sparse : s->d <= 24LL * s->sm_count);
-  if (!s->split.weights.empty()) {
-    const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
-    // two chunks a block are one slab of 64 coordinates there (12 x 16 torus, d = 4863 24.0 against 27.5, but 256-ring, K = 40, d = 9 k 85 -> 38)
-    if (p.n <= 192 && turns > 1.0 && turns <= 2.0) return false;
-    return turns <= (p.n <= 160 ? 1.0 : p.mode == detag::kModeDpsgd ? 4.0 : dense ? 40.0 : 1.0);
-  }
-  const double here = sparse ? 14.0 + 0.098 * p.n * turns : 10.0 + 0.065 * p.n * turns;
-  return here < std::fmax(std::fmax(8.0, 6.0 + 0.0068 * p.n * s->K), 1.25 * (0.024 * p.n + 0.00155 * products) * d / 2000.0);
+  if (s->split.weights.empty()) return rows_beat_rounds(s, p.mode, s->sm_count);
+  const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
+  // two chunks a block are one slab of 64 coordinates there (12 x 16 torus, d = 4863 24.0 against 27.5, but 256-ring, K = 40, d = 9 k 85 -> 38)
+  if (p.n <= 192 && turns > 1.0 && turns <= 2.0) return false;
+  return turns <= (p.n <= 160 ? 1.0 : p.mode == detag::kModeDpsgd ? 4.0 : dense ? 40.0 : 1.0);
 }
 
 // Up to 16 workers the step runs in registers, without staging.  us per step, tensor-path kernel with its stages and barriers
@@ -644,11 +670,13 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   analyse_torus(s);
   if (n > detag::kMaxDenseStepWorkers && n <= detag::kMaxSplitWorkers) {
     // tables for whichever of the two kernels may be asked (rows_ok); those of step_rows.cu take 1 .. 3 ms to make beyond 128 workers
-    // and are left out where calls will surely not use them: both sides of rows_ok's estimates with a margin, and at 160 SMs
-    // (detag_create of 254 workers, K = 3, d = 374 3.4 ms -> 0.02 and 0.85 MB less of workspace)
-    const bool blocks = block_circulant(s);
-    const double products = static_cast<double>(K) * nnz, rounds = std::fmax(0.0155 * n * K, 0.625e-3 * (0.024 * n + 0.00155 * products) * static_cast<double>(d));
-    const bool rows = n <= 128 || (blocks ? n <= 192 || d <= 40LL * 32 * 160 : 10.0 + 0.065 * n * std::ceil(static_cast<double>(d) / (32 * 160)) < 1.25 * (8.0 + rounds));
+    // and are left out where no call would use them on a device of up to 160 SMs (detag_create of 254 workers, K = 3, d = 374 3.4 ms -> 0.02
+    // and 0.85 MB less of workspace)
+    auto used = [&]() {
+      return rows_beat_rounds(s, detag::kModeDetag, 160) || rows_beat_rounds(s, detag::kModeDpsgd, 160) ||
+             (n <= 192 && rows_beat_rounds(s, detag::kModeExternal, 160));
+    };
+    const bool blocks = block_circulant(s), rows = n <= 128 || (blocks ? n <= 192 || d <= 40LL * 32 * 160 : used());
     if (blocks) {
       first_block_row(s, poly);
     } else if (n > 128 && rows) {
@@ -656,6 +684,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
     }
     if ((n <= 96 && (n > 64 || d > 32LL * 32 * 100)) || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
     if (rows) detag::rows_polynomial(n, poly, blocks, s->split, s->rows);
+    if (n > 128 && !blocks && !used()) s->rows = detag::SplitPoly{};
   }
   s->map_cache.reserve(8);
   // the workspace's tables as they are uploaded, the cleared status block in front

@@ -1046,6 +1046,7 @@ void rows_polynomial(int n, const std::vector<double>& poly, bool circulant, con
     made.guard = other.guard;
     made.guard_size = other.guard_size;
     made.guard_tau = other.guard_tau;
+    made.unequal = other.unequal;
   }
   if (rows_plan(n, kModeDetag, static_cast<int>(made.guard.size())).bytes == 0) return;
   unsigned used[2] = {0, 0};
