@@ -148,6 +148,7 @@ inline RowsPlan rows_plan(int n, int mode, int guard_entries) {
   constexpr int two[2][3] = {{2, 1, 1}, {1, 1, 1}};
   if (n <= kPRows) {
     for (const auto& t : one) {
+      if (n <= 64 && t[2] < 2) continue;  // two sets of warps take stages in turn
       const RowsPlan s = plan_for(n, mode, guard_entries, t[0], t[1], t[2], 0, 0);
       if (static_cast<size_t>(s.bytes) <= kPSmemLimit) return s;
     }
