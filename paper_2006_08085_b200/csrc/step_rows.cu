@@ -963,7 +963,8 @@ template <int kRows, bool kAtStart>
 RowsKernel pick_rows(const StepParams& p, bool wide) {
   if (p.mode == kModeDpsgd)
     return wide ? step_rows_kernel<kModeDpsgd, true, kRows, kAtStart> : step_rows_kernel<kModeDpsgd, false, kRows, kAtStart>;
-  return wide ? step_rows_kernel<kModeDetag, true, kRows, kAtStart> : step_rows_kernel<kModeDetag, false, kRows, kAtStart>;
+  // up to 64 workers the DeTAG step never goes by the rounds' name (resolve_variant)
+  return wide && kRows > 64 ? step_rows_kernel<kModeDetag, (kRows > 64), kRows, kAtStart> : step_rows_kernel<kModeDetag, false, kRows, kAtStart>;
 }
 
 template <int kRows>

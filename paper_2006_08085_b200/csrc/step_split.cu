@@ -99,7 +99,7 @@ constexpr int kTmemColumns = 512, kPAccColumns = kPDigits * kPChunk;
 __host__ __device__ constexpr int digit_buffers(int nb) { return nb <= 2 ? 2 : 1; }
 __host__ __device__ constexpr int accumulators(bool big) { return big ? 1 : 2; }
 static_assert(digit_buffers(2) * 40 * 2 + accumulators(false) * kPAccColumns <= kTmemColumns &&
-                  digit_buffers(4) * 40 * 4 + accumulators(false) * kPAccColumns <= kTmemColumns &&
+                  digit_buffers(3) * 40 * 3 + accumulators(false) * kPAccColumns <= kTmemColumns &&
                   digit_buffers(8) * 40 * 8 + accumulators(true) * kPAccColumns <= kTmemColumns,
               "tensor memory plan");
 constexpr size_t kPCtrlBytes = 640, kPSmemLimit = 232448;
@@ -316,7 +316,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
   tmem_fence_before();
   __syncthreads();
   tmem_fence_after();
-  if (p.beside == 0) chain_wait();
+  chain_wait();
   chain_next();
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at address 0
   if (tid == 0 && *tmem_slot != 0) atomicExch(p.status, 2);
@@ -792,7 +792,6 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
     }
     __syncwarp();
   }
-  if (p.beside != 0) chain_wait();
   tmem_fence_before();
   __syncthreads();
   if (warp == kMmaWarp) {
