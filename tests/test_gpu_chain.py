@@ -15,7 +15,16 @@ CASES = [  # n, d, K, graph, variant, mode
     (48, 30_001, 3, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (64, 20_010, 4, "torus", B.DETAG_VARIANT_AUTO, "detag"),
     (100, 30_002, 4, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (256, 3_003, 9, "torus", B.DETAG_VARIANT_AUTO, "detag"),
     (96, 40_005, 4, "ring", B.DETAG_VARIANT_AUTO, "detag"),  # band kernel, its last columns in a launch of their own
-    (60, 5_003, 3, "regular4", B.DETAG_VARIANT_CSR, "detag")]
+    (60, 5_003, 3, "regular4", B.DETAG_VARIANT_CSR, "detag"),
+    (90, 20_003, 4, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (60, 160_010, 4, "regular4", B.DETAG_VARIANT_AUTO, "detag"),  # step_split
+    (256, 6_003, 2, "torus", B.DETAG_VARIANT_AUTO, "dpsgd"), (160, 6_002, 2, "torus", B.DETAG_VARIANT_AUTO, "detag"),
+    (144, 20_003, 8, "regular4", B.DETAG_VARIANT_AUTO, "detag"), (100, 20_003, 6, "regular4", B.DETAG_VARIANT_AUTO, "external"),  # step_rows
+    (160, 20_003, 40, "ring", B.DETAG_VARIANT_AUTO, "external"),
+    (256, 20_005, 4, "ring", B.DETAG_VARIANT_AUTO, "detag"), (96, 20_005, 9, "ring", B.DETAG_VARIANT_RING, "dpsgd")]  # band, rounds beside it
+
+KERNELS = {(8, "ring"): "step_small", (16, "ring"): "step_small", (24, "regular4"): "step_dense", (30, "regular4"): "step_mma", (48, "regular4"): "step_dense",
+           (64, "torus"): "step_torus", (96, "ring"): "step_ring", (90, "regular4"): "step_split", (256, "torus"): ("step_rows", "step_split"),
+           (160, "torus"): "step_split", (144, "regular4"): "step_rows", (100, "regular4"): "step_rows", (160, "ring"): "step_rows", (256, "ring"): "step_ring"}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -27,14 +36,15 @@ def _session(n, d, K, graph, variant, mode):
     m = inputs.metropolis_weights(inputs.ring_graph(n) if graph == "ring" else inputs.torus_graph(n // 8, 8)
                                   if graph == "torus" else inputs.random_regular4_graph(n, n))
     rng = np.random.default_rng(n + d)
-    s = Session(m, d, K, 0.2, 0.02, sigma=0.1, seed=5, variant=variant, external_gradient=mode == "external")
+    s = Session(m, d, K, 0.2, 0.02, sigma=0.1, seed=5, variant=variant, external_gradient=mode == "external",
+                algorithm=B.DETAG_ALGORITHM_DPSGD if mode == "dpsgd" else B.DETAG_ALGORITHM_DETAG)
     for k in ("x", "y", "g", "a", "c") + (("g_new",) if mode == "external" else ()):
         s.upload(k, rng.standard_normal((n, d)).astype(np.float32))
     B.detag_set_step(s.state, 0)
     return s
 
 
-@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[0]}-{c[3]}-{c[5]}")
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[0]}-{c[3]}-{c[5]}-{c[1]}")
 def test_back_to_back_as_with_the_device_idle_between(case):
     import torch
 
@@ -65,6 +75,7 @@ def test_back_to_back_as_with_the_device_idle_between(case):
                     steps(6)
             stream.synchronize()
             s.status()
+            assert B.detag_debug_kernel(s.state) in KERNELS.get(case[::3][:2], ("step_split", "step_csr"))  # 60 workers: by length, by name
             got.append({k: s.download(k) for k in ("x", "y", "g")})
     for other in got[1:]:
         for k in ("x", "y", "g"):

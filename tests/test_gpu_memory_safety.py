@@ -25,9 +25,9 @@ def _built():
     build.build()
 
 
-def _guarded_state(torch, m, d, ld, K, eta, observe, variant, where):
+def _guarded_state(torch, m, d, ld, K, eta, observe, variant, where, external=False):
     n = m.n
-    names = ["x", "y", "g", "a", "c"] + (["obs"] if observe else [])
+    names = ["x", "y", "g", "a", "c"] + (["obs"] if observe else []) + (["new"] if external else [])
     span = n * ld + 2 * GUARD
     span += (-span) % 4  # keep every array 16-byte aligned
     pool = torch.full((span * len(names),), CANARY, dtype=torch.float32, device="cuda:0")
@@ -44,6 +44,8 @@ def _guarded_state(torch, m, d, ld, K, eta, observe, variant, where):
     B.detag_set_gradient_point(st, where)
     if observe:
         B.detag_observe_gossiped_tracker(st, views["obs"])
+    if external:
+        B.detag_set_gradient_source(st, B.DETAG_GRADIENT_EXTERNAL, views["new"])
     return st, pool, views, names, span, ws
 
 
@@ -85,6 +87,43 @@ def test_nothing_outside_the_arrays_is_written(n, d, ld, K, variant):
                     assert bool(torch.isfinite(views[name][:, :d]).all())
             finally:
                 B.detag_destroy(st)
+
+
+# kernels that only some lengths and numbers of rounds lead to
+@pytest.mark.parametrize("n,d,ld,K,graph,mode,ran", [
+    (72, 4_003, 4_008, 3, "regular4", "detag", "step_split"), (60, 151_603, 151_604, 2, "regular4", "start", "step_split"),
+    (160, 4_771, 4_776, 20, "ring", "detag", "step_split"), (256, 4_771, 4_772, 2, "torus", "dpsgd", "step_rows"), (256, 19_007, 19_008, 2, "torus", "dpsgd", "step_split"),
+    (150, 67, 68, 20, "regular4", "start", "step_rows"), (255, 4_771, 4_772, 12, "regular4", "detag", "step_rows"),
+    (50, 33, 36, 16, "regular4", "external", "step_rows"), (70, 67, 72, 30, "ring", "external", "step_rows"), (100, 4_771, 4_780, 6, "regular4", "external", "step_rows"),
+    (130, 35, 36, 14, "regular4", "external", "step_rows"), (192, 97, 100, 16, "regular4", "external", "step_rows"), (193, 97, 100, 16, "regular4", "external", "step_csr")])
+def test_nothing_outside_the_arrays_is_written_by_this_kernel(n, d, ld, K, graph, mode, ran):
+    import torch
+
+    rng = np.random.default_rng(n * 7 + d)
+    m = inputs.metropolis_weights(inputs.torus_graph(n // 16, 16) if graph == "torus" else inputs.ring_graph(n) if graph == "ring"
+                                  else inputs.random_regular4_graph(n, n))
+    external = mode == "external"
+    st, pool, views, names, span, ws = _guarded_state(torch, m, d, ld, K, 0.2, mode != "dpsgd", B.DETAG_VARIANT_AUTO, int(mode == "start"), external)
+    try:
+        if mode == "dpsgd":
+            B.detag_set_algorithm(st, B.DETAG_ALGORITHM_DPSGD)
+        for name in ("a", "c", "x") + (("new",) if external else ()):
+            views[name][:, :d] = torch.from_numpy(rng.uniform(0.5, 2.0, (n, d)).astype(np.float32))
+        B.detag_init(st)
+        for _ in range(3):
+            B.detag_step(st)
+            assert B.detag_debug_kernel(st) == ran
+        B.detag_status(st)
+        torch.cuda.synchronize()
+        for k, name in enumerate(names):
+            lo = pool[k * span: k * span + GUARD]
+            hi = pool[k * span + GUARD + n * ld: (k + 1) * span]
+            assert bool((lo == CANARY).all()) and bool((hi == CANARY).all()), name
+            assert bool((views[name][:, d:] == CANARY).all()), (name, "padding columns")
+        for name in ("x", "y", "g"):
+            assert bool(torch.isfinite(views[name][:, :d]).all())
+    finally:
+        B.detag_destroy(st)
 
 
 @pytest.mark.parametrize("n,d,K", [(16, 5_003, 4), (64, 700, 3), (128, 130, 2), (90, 203, 3)])

@@ -18,6 +18,20 @@ def _built():
     build.build()
 
 
+@pytest.fixture
+def kernels(monkeypatch):
+    """Names of the kernels that the steps before every status() ran on."""
+    from paper_2006_08085_b200 import binding as B
+    seen, plain = set(), Session.status
+
+    def status(self):
+        seen.add(B.detag_debug_kernel(self.state))
+        plain(self)
+
+    monkeypatch.setattr(Session, "status", status)
+    return seen
+
+
 # below, at and beyond a chunk, one and several per block and (beyond 16 per block) chunks in pairs; odd numbers of chunks
 @pytest.mark.parametrize("n,d,K,kind,at_start", [
     (49, 31, 3, "regular4", False), (64, 33, 4, "ring", True), (64, 17 * CHUNKS + 33, 3, "regular4", False), (65, 3 * CHUNKS + 5, 3, "path", False),
@@ -26,6 +40,57 @@ def _built():
     (200, 63, 12, "regular4", False), (255, 2 * CHUNKS + 3, 9, "ring", True), (256, 17 * CHUNKS + 66, 5, "regular4", False)])
 def test_one_step(n, d, K, kind, at_start):
     one_step(n, d, K, kind, at_start)
+
+
+# ... of them those whose dispatch chooses other kernels, at numbers of rounds and lengths where it chooses this one
+@pytest.mark.parametrize("n,d,K,kind,at_start", [
+    (65, 3 * CHUNKS // 4, 3, "path", False), (96, 31, 9, "regular4", True), (130, 31, 20, "regular4", False), (161, 130, 24, "regular4", True), (200, 63, 20, "regular4", False),
+    (256, 1, 20, "regular4", True), (181, 150, 40, "ring", False), (160, 33, 40, "ring", True), (256, CHUNKS + 66, 9, "torus", False)])
+def test_one_step_of_this_kernel(n, d, K, kind, at_start, kernels):
+    one_step(n, d, K, kind, at_start)
+    assert kernels == {"step_rows"}
+
+
+@pytest.mark.parametrize("kind,n,K", [("regular4", 144, 16), ("ring", 181, 60), ("regular4", 256, 16), ("ring", 192, 40)])
+def test_precision_of_this_kernel_beyond_128_workers(kind, n, K, kernels):
+    precision(kind, n, K)
+    assert kernels == {"step_rows"}
+
+
+@pytest.mark.parametrize("n,d,K", [(144, 130, 16), (171, 131, 24), (256, 5 * CHUNKS + 9, 12)])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_dpsgd_and_what_is_not_finite_beyond_128_workers(n, d, K, bad, kernels):
+    """D-PSGD, and DeTAG's tracker: dense polynomials, so what is not finite reaches everyone - in its own column and array."""
+    from paper_2006_08085_b200 import binding as B
+    m, eta, alpha = _graph("regular4", n), 0.2, 0.05
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(n)
+    x, y, g = (rng.standard_normal((n, d), dtype=np.float32) for _ in range(3))
+    x[9, 40] = bad
+    y[n - 1, 70] = bad
+    zero = np.zeros((n, d), np.float32)
+    cols = np.unique(np.concatenate([np.arange(130), np.arange(d - 100, d)]))
+    fine = x[:, cols].astype(np.float64), y[:, cols].astype(np.float64), g[:, cols].astype(np.float64)
+    for algorithm in (B.DETAG_ALGORITHM_DPSGD, B.DETAG_ALGORITHM_DETAG):
+        with Session(m, d, K, eta, alpha, zero, zero, x, algorithm=algorithm, observe_gossip=algorithm == B.DETAG_ALGORITHM_DETAG) as s:
+            s.upload("y", y)
+            s.upload("g", g)
+            s.step()
+            s.status()
+            got = s.download("x")[:, cols]
+            yt = s.download("y_gossip")[:, cols] if algorithm == B.DETAG_ALGORITHM_DETAG else None
+        with np.errstate(invalid="ignore"):
+            want = P @ fine[0] - alpha * (fine[2] if yt is None else P @ fine[1])
+        at = np.isin(cols, [40, 70] if yt is not None else [40])
+        assert not np.isfinite(got[:, at]).any()
+        assert (np.abs(got[:, ~at] - want[:, ~at]) <= 1e-5 * (1.0 + np.abs(want[:, ~at]))).all()
+        if yt is not None:
+            at = cols == 70
+            assert not np.isfinite(yt[:, at]).any()
+            with np.errstate(invalid="ignore"):
+                want = P @ fine[1]
+            assert (np.abs(yt[:, ~at] - want[:, ~at]) <= 1e-5 * (1.0 + np.abs(want[:, ~at]))).all()
+    assert kernels == {"step_rows"}
 
 
 @pytest.mark.parametrize("kind,n", [("regular4", 144), ("ring", 181), ("regular4", 256)])
@@ -73,8 +138,8 @@ def test_caller_written_gradients(n, d, K, kind):
 
 
 @pytest.mark.parametrize("n,kind", [(60, "regular4"), (90, "regular4"), (128, "regular4"), (160, "ring"), (192, "regular4")])
-@pytest.mark.parametrize("K", [1, 2, 6])
-def test_caller_written_gradients_whose_fold_cancels(n, kind, K):
+@pytest.mark.parametrize("K", [1, 2, 6, 16])
+def test_caller_written_gradients_whose_fold_cancels(n, kind, K, kernels):
     """y + g_new - g far below its parts: the first step after detag_init (y = g) where gradients have fallen.  The bound knows the sum z
     alone: half an ulp of what is stored and as much again of the magnitudes read, nothing of the three parts (of which float64 itself
     loses 2^-53, here some 2^-28 of the sum)."""
@@ -122,10 +187,25 @@ def test_caller_written_gradients_whose_fold_cancels(n, kind, K):
     assert max(worst) <= 1.0, [round(v, 2) for v in worst]
     assert (np.abs(got["x"] - xt) <= of_x).all()
     assert np.array_equal(got["g"], gn[:, cols])
+    assert K < 16 or kernels == {"step_rows"}  # fewer rounds run as such, some of them
 
 
-def test_caller_written_gradients_that_are_not_finite():
-    n, d, K, eta = 70, 40, 2, 0.2
+# one worker beyond a block, whole blocks, one beyond the first half; below, at and beyond a chunk
+@pytest.mark.parametrize("n,d,K,kind", [(49, 1, 16, "regular4"), (50, 35, 30, "ring"), (64, 33, 12, "regular4"), (70, 97, 30, "ring"), (96, 31, 12, "regular4"),
+                                        (97, CHUNKS + 34, 12, "regular4"), (129, 35, 14, "regular4"), (160, 3 * CHUNKS + 2, 16, "regular4"), (192, 31, 16, "regular4")])
+def test_caller_written_gradients_of_this_kernel(n, d, K, kind, kernels):
+    test_caller_written_gradients(n, d, K, kind)
+    assert kernels == {"step_rows"}
+
+
+@pytest.mark.parametrize("n,K", [(70, 30), (56, 30), (160, 40)])
+def test_caller_written_gradients_of_this_kernel_that_are_not_finite(n, K, kernels):
+    test_caller_written_gradients_that_are_not_finite(n, K)
+    assert kernels == {"step_rows"}
+
+
+def test_caller_written_gradients_that_are_not_finite(n=70, K=2):
+    d, eta = 40, 0.2
     m = _graph("ring", n)
     P = _polynomial(m, K, eta)
     rng = np.random.default_rng(7)

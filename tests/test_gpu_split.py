@@ -239,3 +239,85 @@ def test_dpsgd(n, d):
         p = oracle_problem(m, K, eta, alpha, a[:, lo:hi], c[:, lo:hi], 0.1, 3, lo)
         assert worst_ratio(g[:, lo:hi], orc.stochastic_gradient(p, want[:, lo:hi], 1)) <= 1.0
     assert np.array_equal(y, a)  # no tracker: untouched
+
+
+# What the dispatch leaves to step_split.cu: the DeTAG step of 65 to 96 workers and D-PSGD of sparse ones at length, long vectors of 49 to 64
+# (two slabs' digits), block-circulant matrices beyond 128 workers with more than one (D-PSGD four, dense polynomials forty) chunk per block
+KEPT = [(72, "regular4", 4_003, 2, "detag"), (90, "path", 4_003, 6, "start"), (96, "regular4", SLABS + 33, 16, "detag"), (81, "regular4", 3_600, 1, "detag"),
+        (49, "path", 152_001, 2, "detag"), (60, "regular4", 160_003, 6, "start"), (60, "ring", 160_001, 3, "dpsgd"), (90, "regular4", 303_202, 2, "dpsgd"),
+        (160, "ring", 5_003, 20, "detag"), (224, "ring", 5_001, 17, "start"), (256, "ring", 190_002, 34, "detag"), (256, "torus", 5_003, 2, "detag"),
+        (256, "torus", 19_001, 3, "dpsgd"), (256, "torus", 190_001, 16, "detag")]
+
+
+@pytest.mark.parametrize("n,kind,d,K,mode", KEPT)
+def test_every_result_is_as_precise_as_what_it_reads_at_lengths_that_this_kernel_keeps(n, kind, d, K, mode):
+    """As above, every column of the model and of the tracker; an infinity in one column and a NaN in another reach as far as the polynomial."""
+    eta, wide = 0.2, 1997
+    m = _graph(kind, n)
+    P = _polynomial(m, K, eta)
+    rng = np.random.default_rng(n + d)
+    patterns = ["alike", "one larger", "every eighth", "all but the last", "sorted", "log-uniform", "one alone", "consensus"]
+    # a block of columns over and over: patterns side by side, so that one slab holds coordinates of both kinds
+    blocks = {}
+    for shift, name in enumerate(("x", "y")):
+        z = np.empty((n, wide), np.float32)
+        for k, pattern in enumerate(patterns):
+            at = (np.arange(wide) + 3 * shift) % 8 == k
+            z[:, at] = _unequal(pattern, n, int(at.sum()), rng)
+        blocks[name] = z
+    state = {k: np.ascontiguousarray(np.tile(z, -(-d // wide))[:, :d]) for k, z in blocks.items()}
+    bad = {"x": (d // 2 + 1, np.inf), "y": (d - 2, np.nan)}
+    for name, (col, v) in bad.items():
+        state[name][9, col] = v
+    zero = np.zeros((n, d), np.float32)
+    with Session(m, d, K, eta, 0.0, zero, zero, zero, gradient_point=int(mode == "start"), algorithm=int(mode == "dpsgd")) as s:
+        for name, v in state.items():
+            s.upload(name, v)
+        s.step()
+        s.status()
+        assert B.detag_debug_kernel(s.state) == "step_split"
+        got = {k: s.download(k) for k in ("x", "y")}
+    reached = P[:, 9] != 0.0
+    if mode == "dpsgd":
+        assert np.array_equal(got.pop("y"), state["y"], equal_nan=True)  # no tracker: untouched
+    for name, have in got.items():
+        z = blocks[name].astype(np.float64)
+        want = P @ z
+        bound = 2.0 ** -24 * (np.abs(want) + np.abs(P) @ np.abs(z)) + 1e-45
+        for lo in range(0, d, wide):
+            cut = have[:, lo:lo + wide].astype(np.float64)
+            keep = np.ones(cut.shape, bool)
+            for other, (col, _) in bad.items():
+                if lo <= col < lo + wide:  # x' = P x - 0 * P y, y' = P y + 0 * x'
+                    assert other != name or not np.isfinite(cut[reached, col - lo]).any()
+                    keep[reached, col - lo] = False
+            w = cut.shape[1]
+            assert ((np.abs(cut - want[:, :w]) <= bound[:, :w]) | ~keep).all(), (name, lo)
+
+
+@pytest.mark.parametrize("n,kind,d,K,mode", [(72, "regular4", 2 * SLABS + 5, 3, "detag"), (60, "regular4", 17 * SLABS + 5, 3, "start"),
+                                             (90, "regular4", 303_202, 2, "dpsgd"), (256, "torus", 2 * SLABS + 5, 2, "start"), (256, "torus", 2 * SLABS + 5, 2, "dpsgd")])
+def test_loads_that_stop_time_out_and_the_state_recovers(n, kind, d, K, mode):
+    from test_gpu_failure_detection import _rebind
+    m = _graph(kind, n)
+    rng = np.random.default_rng(n)
+    state = {k: rng.standard_normal((n, d), dtype=np.float32) for k in ("x", "y", "g", "a", "c")}
+    got = []
+    for stalled in (False, True):
+        with Session(m, d, K, 0.2, 0.01, sigma=0.1, seed=5, gradient_point=int(mode == "start"), algorithm=int(mode == "dpsgd")) as s:
+            if stalled:
+                B.detag_debug_inject_stall(s.state, 1, 2048)
+                s.step()
+                with pytest.raises(B.DetagError) as e:
+                    s.status()
+                assert e.value.code == B.DETAG_ERR_TIMEOUT
+                B.detag_debug_inject_stall(s.state, -1, 0)
+                _rebind(s)
+            for k, v in state.items():
+                s.upload(k, v)
+            B.detag_set_step(s.state, 0)
+            s.step()
+            s.status()
+            assert B.detag_debug_kernel(s.state) == "step_split"
+            got.append({k: s.download(k) for k in ("x", "y", "g")})
+    assert all(np.array_equal(got[0][k], got[1][k]) for k in got[0])
