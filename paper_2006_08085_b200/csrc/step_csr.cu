@@ -28,6 +28,8 @@
 // mode only the model is gossiped and x' = x~ - alpha g.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "chain.cuh"
 #include "detag_internal.h"
 #include "noise.cuh"
@@ -81,7 +83,8 @@ __device__ __forceinline__ void store4(float* base, long long off, long long j, 
 
 // kTables: the CSR arrays are read from shared memory (they fit) instead of global memory.
 // kSwap: fewer than eight coordinate groups, the pairs of a row swap places by a bit of the row index.
-template <bool kTables, bool kSwap>
+// kBeside: p.beside.
+template <bool kTables, bool kSwap, bool kBeside>
 __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // S coordinates per slab in p.csr_sub independent pieces of W = S / p.csr_sub coordinates (each with its own rows
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepPara
     cols = s_col;
     __syncthreads();  // the tables are read right below
   }
-  if (p.beside == 0) chain_wait();
+  if (!kBeside) chain_wait();
   chain_next();
   // item = ((row quad * 4 + row within quad) * groups + coordinate group): a row's threads side by side, the four
   // rows of a Philox call `groups` lanes apart in one warp (groups is a power of two, at most 8)
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(kCsrThreads, 1) step_csr_kernel(const StepPara
       }
     }
   }
-  if (p.beside != 0) chain_wait();
+  if (kBeside) chain_wait();
 }
 
 }  // namespace
@@ -310,8 +313,12 @@ int launch_step_csr(const StepParams& p, int sm_count, cudaStream_t stream) {
   const bool tables = p.log2S > 0;
   const size_t smem = csr_smem_bytes(p.n, p.nnz, p.S, tables);
   const bool swap = p.S / p.csr_sub < kCsrMaxS;
-  auto kernel = tables ? (swap ? step_csr_kernel<true, true> : step_csr_kernel<true, false>)
-                       : (swap ? step_csr_kernel<false, true> : step_csr_kernel<false, false>);
+  auto pick = [&](auto beside) {
+    constexpr bool kBeside = decltype(beside)::value;
+    return tables ? (swap ? step_csr_kernel<true, true, kBeside> : step_csr_kernel<true, false, kBeside>)
+                  : (swap ? step_csr_kernel<false, true, kBeside> : step_csr_kernel<false, false, kBeside>);
+  };
+  const auto kernel = p.beside != 0 ? pick(std::true_type()) : pick(std::false_type());
   const int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), static_cast<int>(smem));
   if (rc != 0) return rc;
   const long long ctas = static_cast<long long>(sm_count) * (kCsrThreads / p.csr_threads);
