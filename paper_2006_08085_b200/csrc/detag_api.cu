@@ -500,25 +500,25 @@ bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
 }
 
 // Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0,
-// 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7; D-PSGD of 96, 10 k 17.5 -> 14.5, 1 M 707 -> 639, but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
+// 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7; D-PSGD of 96, 10 k 17.5 -> 14.5, 1 M 707 -> 639 (but, where operands spread over four decades go to
+// float64, 90, K = 2, d = 100 k 273 -> 420), but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
 // 8 k 12.4 -> 14.4, 300 k 224 -> 234, only the shortest of these better (96, 3000 11.7 -> 10.9, K = 1, 700 12.8 -> 11.4); 64, 10 k 12.9 -> 11.0,
 // 100 k 55.4 -> 54.4, but 300 k 150 -> 160 (rows in pieces of 128 bytes): up to 64 workers therefore calls whose blocks have at most 32 chunks of
 // 32 coordinates to do.  What would run as rounds otherwise runs here if rows_beat_rounds says so.  Block-circulant
-// matrices beyond 160 workers come here while P is dense and calls are not the longest (lanes as coordinates -> here: 256-ring, K = 40, d = 4 k
-// 34.6 -> 21.9, 60 k 285 -> 207, 16 x 16 torus, 19 k 88.5 -> 77.2, but K = 196, 200 k 577 -> 594, D-PSGD, 300 k 694 -> 775; torus, K = 2, 500 k 1152 -> 1202),
-// all with a chunk per block at most.
+// matrices beyond 160 workers come here while P is dense and calls are not long (lanes as coordinates -> here: 256-ring, K = 40, d = 4 k
+// 34.6 -> 21.9, 60 k 263 -> 233, 16 x 16 torus, K = 9, 10 k 65 -> 49, 60 k 197 -> 186, but 100 k 303 -> 310, 189 k 554 -> 600; 224, 60 k 171 -> 166, but 75 k 195 -> 205;
+// 192, 19 k 62 -> 58, but 60 k 134 -> 145; D-PSGD, 14 k 56 -> 46, but 18 k 57 -> 58), all with a chunk per block at most.
 bool rows_ok(const detag_state* s, const StepParams& p) {
   if (s->rows.weights.empty()) return false;
   if (p.mode == detag::kModeExternal) return detag::rows_take_external(s->rows) && rows_beat_rounds(s, p.mode, s->sm_count);
   const double turns = std::ceil(static_cast<double>(s->d) / (32.0 * s->sm_count));
-  const bool sparse = s->rows.guard.size() > static_cast<size_t>(s->n);
   if (p.n <= 64) return turns <= 32.0 || s->split.weights.empty();
-  if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd ? turns <= 64.0 || !sparse : s->d <= 24LL * s->sm_count);
+  if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd ? turns <= 1.0 || s->rows.unequal < 0.5f : s->d <= 24LL * s->sm_count);
   if (s->split.weights.empty()) return rows_beat_rounds(s, p.mode, s->sm_count);
   const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
   // two chunks a block are one slab of 64 coordinates there (12 x 16 torus, d = 4863 24.0 against 27.5, but 256-ring, K = 40, d = 9 k 85 -> 38)
   if (p.n <= 192 && turns > 1.0 && turns <= 2.0) return false;
-  return turns <= (p.n <= 160 ? 1.0 : p.mode == detag::kModeDpsgd ? 4.0 : dense ? 40.0 : 1.0);
+  return turns <= (p.n <= 160 || !dense ? 1.0 : p.mode == detag::kModeDpsgd ? 3.0 : p.n <= 192 ? 6.0 : 13.0);
 }
 
 // Up to 16 workers the step runs in registers, without staging.  us per step, tensor-path kernel with its stages and barriers
@@ -676,7 +676,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
       return rows_beat_rounds(s, detag::kModeDetag, 160) || rows_beat_rounds(s, detag::kModeDpsgd, 160) ||
              (n <= 192 && rows_beat_rounds(s, detag::kModeExternal, 160));
     };
-    const bool blocks = block_circulant(s), rows = n <= 128 || (blocks ? n <= 192 || d <= 40LL * 32 * 160 : used());
+    const bool blocks = block_circulant(s), rows = n <= 128 || (blocks ? n <= 192 || d <= 13LL * 32 * 160 : used());
     if (blocks) {
       first_block_row(s, poly);
     } else if (n > 128 && rows) {

@@ -241,8 +241,8 @@ def test_dpsgd(n, d):
     assert np.array_equal(y, a)  # no tracker: untouched
 
 
-# What the dispatch leaves to step_split.cu: the DeTAG step of 65 to 96 workers and D-PSGD of sparse ones at length, long vectors of 49 to 64
-# (two slabs' digits), block-circulant matrices beyond 128 workers with more than one (D-PSGD four, dense polynomials forty) chunk per block
+# What the dispatch leaves to step_split.cu: the DeTAG step of 65 to 96 workers and D-PSGD of sparse polynomials, not the shortest, long vectors of 49 to 64
+# (two slabs' digits), block-circulant matrices beyond 128 workers with more than one (dense polynomials: thirteen, D-PSGD three) chunk per block
 KEPT = [(72, "regular4", 4_003, 2, "detag"), (90, "path", 4_003, 6, "start"), (96, "regular4", SLABS + 33, 16, "detag"), (81, "regular4", 3_600, 1, "detag"),
         (49, "path", 152_001, 2, "detag"), (60, "regular4", 160_003, 6, "start"), (60, "ring", 160_001, 3, "dpsgd"), (90, "regular4", 303_202, 2, "dpsgd"),
         (160, "ring", 5_003, 20, "detag"), (224, "ring", 5_001, 17, "start"), (256, "ring", 190_002, 34, "detag"), (256, "torus", 5_003, 2, "detag"),
