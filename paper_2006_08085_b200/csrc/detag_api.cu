@@ -499,6 +499,11 @@ bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
   return here < rounds && here + unequal * d / (32.0 * sms) < 1.1 * rounds;
 }
 
+// Of 97 to 128 workers, calls in which reading the model a second time, in pieces of 32 bytes, costs the printed timing more than
+// step_rows.cu gains: step_split.cu -> there, n = 98, d = 1 M 1021 -> 990, 2 M 2040 -> 2082; 112, 600 k 647 -> 614, 1 M 1077 -> 1087, 2 M 2143 -> 2333; 128, 600 k
+// 703 -> 662, 1 M 1167 -> 1218, 2 M 2318 -> 2616.
+bool long_calls(const detag_state* s, int sms) { return s->n * std::ceil(static_cast<double>(s->d) / (32.0 * sms)) > 24000.0; }
+
 // Which of its two kernels.  us per step, lanes as coordinates -> as output workers: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0,
 // 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7; D-PSGD of 96, 10 k 17.5 -> 14.5, 1 M 707 -> 639 (but, where operands spread over four decades go to
 // float64, 90, K = 2, d = 100 k 273 -> 420), but the DeTAG step of 80, 20 k 23.1 -> 24.0, of 96,
@@ -513,7 +518,8 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
   if (p.mode == detag::kModeExternal) return detag::rows_take_external(s->rows) && rows_beat_rounds(s, p.mode, s->sm_count);
   const double turns = std::ceil(static_cast<double>(s->d) / (32.0 * s->sm_count));
   if (p.n <= 64) return turns <= 32.0 || s->split.weights.empty();
-  if (p.n <= 128) return p.n > 96 || (p.mode == detag::kModeDpsgd ? turns <= 1.0 || s->rows.unequal < 0.5f : s->d <= 24LL * s->sm_count);
+  if (p.n > 96 && p.n <= 128) return !(p.mode == detag::kModeDetag && p.grad_at_start != 0 && long_calls(s, s->sm_count) && !s->split.weights.empty());
+  if (p.n <= 128) return p.mode == detag::kModeDpsgd ? turns <= 1.0 || s->rows.unequal < 0.5f : s->d <= 24LL * s->sm_count;
   if (s->split.weights.empty()) return rows_beat_rounds(s, p.mode, s->sm_count);
   const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
   // two chunks a block are one slab of 64 coordinates there (12 x 16 torus, d = 4863 24.0 against 27.5, but 256-ring, K = 40, d = 9 k 85 -> 38)
@@ -682,7 +688,7 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
     } else if (n > 128 && rows) {
       gossip_polynomial(s, poly);
     }
-    if ((n <= 96 && (n > 64 || d > 32LL * 32 * 100)) || (n > 128 && blocks)) detag::split_polynomial(n, poly, blocks, s->split);
+    if (n <= 64 ? d > 32LL * 32 * 100 : n <= 96 || (n <= 128 ? long_calls(s, 100) : blocks)) detag::split_polynomial(n, poly, blocks, s->split);
     if (rows) detag::rows_polynomial(n, poly, blocks, s->split, s->rows);
     if (n > 128 && !blocks && !used()) s->rows = detag::SplitPoly{};
   }

@@ -1,7 +1,7 @@
 // DeTAG step with the polynomial P = P_K(M) applied on the fifth-generation tensor cores in exact integer arithmetic,
 // for gossip matrices with 48 < n <= 256 whose distinct 32 x 32 blocks of P fit in shared memory.  Its other kernel, step_rows.cu,
-// takes the others and what it is faster at (rows_ok in detag_api.cu): left here are the DeTAG step of 65 to 96 workers, long vectors up
-// to 64, long vectors of block-circulant matrices beyond 128.
+// takes the others and what it is faster at (rows_ok in detag_api.cu): left here are the DeTAG step of 65 to 96 workers and D-PSGD of theirs
+// with sparse polynomials, long vectors up to 64, the longest of 97 to 128 with the printed timing, long ones of block-circulant matrices beyond 128.
 //
 // AG_K(z) = P z.  The float64 tensor path (mma m8n8k4) bounds this product at 64 multiply-adds per clock and SM, which
 // for n = 100 is 3.3 times and for a dense n = 256 eight times the time of the step's HBM traffic.  Here both operands
@@ -99,7 +99,7 @@ constexpr int kTmemColumns = 512, kPAccColumns = kPDigits * kPChunk;
 __host__ __device__ constexpr int digit_buffers(int nb) { return nb <= 2 ? 2 : 1; }
 __host__ __device__ constexpr int accumulators(bool big) { return big ? 1 : 2; }
 static_assert(digit_buffers(2) * 40 * 2 + accumulators(false) * kPAccColumns <= kTmemColumns &&
-                  digit_buffers(3) * 40 * 3 + accumulators(false) * kPAccColumns <= kTmemColumns &&
+                  digit_buffers(4) * 40 * 4 + accumulators(false) * kPAccColumns <= kTmemColumns &&
                   digit_buffers(8) * 40 * 8 + accumulators(true) * kPAccColumns <= kTmemColumns,
               "tensor memory plan");
 constexpr size_t kPCtrlBytes = 640, kPSmemLimit = 232448;
