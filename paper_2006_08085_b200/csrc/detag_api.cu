@@ -143,6 +143,29 @@ void first_block_row(const detag_state* s, std::vector<double>& out) {
   }
 }
 
+// Of the 32 x 32 blocks of P_K(M), those per 32 rows whose workers hear from one another in K rounds (n <= 256).
+double reached_blocks(const detag_state* s) {
+  const int n = s->n, nb = (n + 31) / 32;
+  std::vector<uint32_t> from(static_cast<size_t>(n) * nb, 0), next;
+  for (int i = 0; i < n; ++i) from[static_cast<size_t>(i) * nb + i / 32] = 1u << (i % 32);
+  for (int r = 0; r < s->K; ++r) {
+    next = from;
+    for (int i = 0; i < n; ++i)
+      for (int k = s->row_ptr[i]; k < s->row_ptr[i + 1]; ++k)
+        for (int b = 0; b < nb; ++b) next[static_cast<size_t>(i) * nb + b] |= from[static_cast<size_t>(s->col_idx[k]) * nb + b];
+    if (next == from) break;
+    from.swap(next);
+  }
+  int count = 0;
+  for (int c = 0; c < nb; ++c)
+    for (int b = 0; b < nb; ++b) {
+      uint32_t any = 0;
+      for (int i = 32 * c; i < n && i < 32 * c + 32; ++i) any |= from[static_cast<size_t>(i) * nb + b];
+      count += any != 0 ? 1 : 0;
+    }
+  return static_cast<double>(count) / nb;
+}
+
 // Circulant M (row i = row 0 shifted by i): then P_K(M) is circulant too; its row 0 is computed with the
 // recursion of Algorithm 3 on a single row and stored as a band around the diagonal.
 void analyse_circulant(detag_state* s) {
@@ -461,7 +484,7 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
 }
 
 // Whether step_rows.cu takes less than the rounds: caller-written gradients up to 192 workers, beyond 128 matrices without block
-// structure.  Estimates of both in us (`sms`: as if on that many SMs; before the tables are made with their best case).  Rounds -> there, operands alike: caller-written,
+// structure.  Estimates of both in us (`sms`: as if on that many SMs).  Rounds -> there, operands alike: caller-written,
 // 100 workers, K = 6, d = 1 M 3177 -> 862, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 984,
 // 256, K = 12, d = 200 k 3830 -> 750, ring of 144, K = 4, d = 8931 35.6 against 48.1.  On short vectors rounds take their latency, one after the other:
 // caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
@@ -475,23 +498,31 @@ bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
   const double n = s->n, d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * sms));
   const double products = s->K * static_cast<double>(s->col_idx.size());
   const bool sparse = t.guard.size() > static_cast<size_t>(s->n);
-  int reach = 0;  // 32 x 32 blocks that the float64 path goes through, per 32 outputs
-  for (unsigned char r : t.reach) reach += __builtin_popcount(r);
-  const double blocks = reach / std::ceil(n / 32.0);
+  // share of the work that is float64 then, and the 32 x 32 blocks which that goes through per 32 outputs.  Before the tables are made: all of
+  // it while the walks of K steps, degree - 1 onwards at each, are fewer than three per worker (random graphs of degree 4, 8 and 16: from four
+  // on is the first that is less)
+  double share = t.unequal, blocks = s->reach;
+  if (t.guard.empty()) {
+    share = std::pow(std::fmax(products / s->K / n - 2.0, 0.0), s->K) < 3.0 * n ? 1.0 : 0.0;
+  } else {
+    int reach = 0;
+    for (unsigned char r : t.reach) reach += __builtin_popcount(r);
+    blocks = reach / std::ceil(n / 32.0);
+  }
   double here, unequal, rounds, latency;
   if (mode == detag::kModeExternal) {
     here = n > 128 ? 10.0 + 0.065 * n * turns * (sparse ? 1.5 : 1.0)
                    : 9.0 + turns * (1.0 + 0.031 * n) * (sparse && n > 64 && n <= 96 ? 2.2 : 1.0);  // six warps for the test
-    unequal = t.unequal * (n > 128 ? 20.0 + 2.4 * blocks : 5.5 * blocks);
+    unequal = share * (n > 128 ? 20.0 + 2.4 * blocks : 5.5 * blocks);
     rounds = 6.0 + (n > 128 ? 1.2 + 0.003 * n + 0.00105 * products : 0.0021 * n + 0.00099 * products) * d / 1000.0;
     latency = 6.0 + 0.0155 * n * s->K;
   } else {
     here = sparse ? 14.0 + 0.098 * n * turns : 10.0 + 0.065 * n * turns;
-    unequal = t.unequal * (3.5 + 7.2 * blocks);
+    unequal = share * (3.5 + 7.2 * blocks);
     rounds = (1.35 + 0.004 * n + 0.0011 * products) * d / 1000.0;
     latency = 6.0 + 0.0068 * n * s->K;
     if (mode == detag::kModeDpsgd) {  // one array
-      unequal = (1.0 - std::sqrt(1.0 - t.unequal)) * 0.75 * (3.5 + 7.2 * blocks);
+      unequal = (1.0 - std::sqrt(1.0 - share)) * 0.75 * (3.5 + 7.2 * blocks);
       rounds *= 0.64;
     }
   }
@@ -676,13 +707,15 @@ int detag_create(detag_state** out, int n, int64_t d, const int32_t* row_ptr, co
   analyse_torus(s);
   if (n > detag::kMaxDenseStepWorkers && n <= detag::kMaxSplitWorkers) {
     // tables for whichever of the two kernels may be asked (rows_ok); those of step_rows.cu take 1 .. 3 ms to make beyond 128 workers
-    // and are left out where no call would use them on a device of up to 160 SMs (detag_create of 254 workers, K = 3, d = 374 3.4 ms -> 0.02
-    // and 0.85 MB less of workspace)
+    // and are left out where no call would use them on a device of up to 160 SMs (256 workers, K = 4, d = 200 k 3.5 ms -> 0.05 and 0.85 MB less of
+    // workspace)
     auto used = [&]() {
       return rows_beat_rounds(s, detag::kModeDetag, 160) || rows_beat_rounds(s, detag::kModeDpsgd, 160) ||
              (n <= 192 && rows_beat_rounds(s, detag::kModeExternal, 160));
     };
-    const bool blocks = block_circulant(s), rows = n <= 128 || (blocks ? n <= 192 || d <= 13LL * 32 * 160 : used());
+    const bool blocks = block_circulant(s);
+    if (n > 128 && !blocks) s->reach = reached_blocks(s);
+    const bool rows = n <= 128 || (blocks ? n <= 192 || d <= 13LL * 32 * 160 : used());
     if (blocks) {
       first_block_row(s, poly);
     } else if (n > 128 && rows) {

@@ -175,6 +175,7 @@ struct detag_state {
   bool torus = false;
   std::vector<double> torus_frag;
   detag::SplitPoly split, rows;   // 48 < n <= 256: P_K(M) for the integer tensor path's two kernels (empty: not taken)
+  double reach = 0.0;             // of unstructured matrices beyond 128 workers: blocks of P_K(M) reached per 32 rows
   std::vector<unsigned char> image;  // the workspace up to the partial sums, as it is uploaded
   int variant_forced = DETAG_VARIANT_AUTO;
   int gradient_point = DETAG_GRADIENT_AT_NEW_MODEL;
