@@ -1,10 +1,11 @@
-// What the two kernels of the integer tensor path share: how operands are scaled and split.
+// What the two kernels of the integer tensor path share: how operands are tested, scaled and split, how the sums are joined.
 #ifndef DETAG_DIGITS_CUH
 #define DETAG_DIGITS_CUH
 
 #include <cstdint>
 
 #include "packed.cuh"
+#include "pipeline.cuh"
 
 namespace detag {
 
@@ -81,6 +82,45 @@ __device__ __forceinline__ void four_fold_digits(const float* src, int array, in
     }
   }
   digits_of<true>(x, rest, scale, d);
+}
+
+// Smallest of the largest magnitudes of groups first, first + step, ... of `size` inputs (2, or a multiple of 4), read as Four and Two.
+template <typename Four, typename Two, typename Value, typename Index>
+__device__ __forceinline__ float group_low(Value value, const Index* guard, int groups, int size, int first, int step) {
+  float low = __uint_as_float(0x7f800000u);
+  if (size == 2) {
+#pragma unroll 4
+    for (int q = first; q < groups; q += step) {
+      const Two at = *reinterpret_cast<const Two*>(guard + 2 * q);
+      low = fminf(low, max_abs3(value(at.x), value(at.y), 0.f));
+    }
+    return low;
+  }
+  for (int q = first; q < groups; q += step) {
+    float m = 0.f;
+#pragma unroll 2
+    for (int i = 0; i < size; i += 4) {
+      const Four at = *reinterpret_cast<const Four*>(guard + q * size + i);
+      m = max_abs3(max_abs3(m, value(at.x), value(at.y)), value(at.z), value(at.w));
+    }
+    low = fminf(low, m);
+  }
+  return low;
+}
+
+// Integer sums of the five weights -> one float64, exact but for the rounding of the lowest: a 64-bit integer below 2^51, in units
+// of 256^5, added to the bits of 1.5 * 2^52 with the coordinate's scale in its exponent field (`magic_hi`: the upper word; `magic`:
+// that number), which is then subtracted.  `hi` = s8 * 256 + s7, `low` = s5 + s4 / 256, rounded.  Up to 128 workers (not kBig) the rest
+// fits 32 bits (3 * 128 * 2^14 * 256 < 2^31).
+template <bool kBig>
+__device__ __forceinline__ double join_sums(int hi, int s6, int low, int magic_hi, double magic) {
+  if (kBig) {
+    const long long lo = static_cast<long long>(s6) * 256 + (low + (static_cast<long long>(magic_hi) << 32));
+    return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - magic;
+  }
+  const int lo = s6 * 256 + low;
+  const unsigned long long upper = static_cast<uint32_t>(magic_hi + (lo >> 31));
+  return __longlong_as_double(static_cast<long long>(hi) * 65536 + static_cast<long long>(upper << 32 | static_cast<uint32_t>(lo))) - magic;
 }
 
 }  // namespace

@@ -170,22 +170,6 @@ __device__ __forceinline__ void bytes_load(void* dst, const void* src, unsigned 
                : "memory");
 }
 
-// Integer sums of the five weights -> one float64, exact but for the rounding of the lowest: a 64-bit integer below 2^51, in units
-// of 256^5, added to the bits of 1.5 * 2^52 with the coordinate's scale in its exponent field (`magic_hi`: the upper word; `magic`:
-// that number), which is then subtracted.  `hi` = s8 * 256 + s7.  Up to 128 workers the rest fits 32 bits
-// (3 * 128 * 2^14 * 256 < 2^31).
-template <bool kTwo>
-__device__ __forceinline__ double join_sums(int hi, int s6, int low, int magic_hi) {
-  const double magic = __hiloint2double(magic_hi, 0);
-  if (kTwo) {
-    const long long lo = static_cast<long long>(s6) * 256 + (low + (static_cast<long long>(magic_hi) << 32));
-    return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - magic;
-  }
-  const int lo = s6 * 256 + low;
-  const unsigned long long upper = static_cast<uint32_t>(magic_hi + (lo >> 31));
-  return __longlong_as_double(static_cast<long long>(hi) * 65536 + static_cast<long long>(upper << 32 | static_cast<uint32_t>(lo))) - magic;
-}
-
 // Joined sums of this thread's output worker from the accumulators at `acc` on (whole warp): its eight
 // coordinates, model or tracker.  `magic_hi`: of these; `row_power`: the row's exponent in the same place.
 template <bool kTwo>
@@ -212,36 +196,14 @@ __device__ __forceinline__ void take_sums(uint32_t acc, const int* magic_hi, int
   tmem_wait_load();
 #pragma unroll
   for (int u = 0; u < kCount; u += 4) {
-    const int4 m = *reinterpret_cast<const int4*>(magic_hi + u);
-    out[u] = join_sums<kTwo>(hi[u], s6[u], low[u], m.x + row_power);
-    out[u + 1] = join_sums<kTwo>(hi[u + 1], s6[u + 1], low[u + 1], m.y + row_power);
-    out[u + 2] = join_sums<kTwo>(hi[u + 2], s6[u + 2], low[u + 2], m.z + row_power);
-    out[u + 3] = join_sums<kTwo>(hi[u + 3], s6[u + 3], low[u + 3], m.w + row_power);
-  }
-}
-
-// Smallest of the largest magnitudes of groups first, first + step, ... of `size` inputs (2, or a multiple of 4).
-template <typename Value>
-__device__ __forceinline__ float group_low(Value value, const uint8_t* guard, int groups, int size, int first, int step) {
-  float low = __uint_as_float(0x7f800000u);
-  if (size == 2) {
-#pragma unroll 4
-    for (int q = first; q < groups; q += step) {
-      const uchar2 at = *reinterpret_cast<const uchar2*>(guard + 2 * q);
-      low = fminf(low, max_abs3(value(at.x), value(at.y), 0.f));
+    const int4 four = *reinterpret_cast<const int4*>(magic_hi + u);
+    const int m[4] = {four.x, four.y, four.z, four.w};
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int magic = m[v] + row_power;
+      out[u + v] = join_sums<kTwo>(hi[u + v], s6[u + v], low[u + v], magic, __hiloint2double(magic, 0));
     }
-    return low;
   }
-  for (int q = first; q < groups; q += step) {
-    float m = 0.f;
-#pragma unroll 2
-    for (int i = 0; i < size; i += 4) {
-      const uchar4 at = *reinterpret_cast<const uchar4*>(guard + q * size + i);
-      m = max_abs3(max_abs3(m, value(at.x), value(at.y)), value(at.z), value(at.w));
-    }
-    low = fminf(low, m);
-  }
-  return low;
 }
 
 // A warp's 32 output workers x 8 coordinates in float64, from the operands themselves: of the model where one of bits 0 .. 7 of
@@ -500,7 +462,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
             for (int u = 0; u < 4; ++u) v[u] = at[u * kPS];
           });
         }
-        low_f = group_low(value, guard, tb.guard_groups, tb.guard_size, part, kParts);
+        low_f = group_low<uchar4, uchar2>(value, guard, tb.guard_groups, tb.guard_size, part, kParts);
         // These sums lack what their two roundings leave out, 2^-24 of the difference and of themselves: below 2^-18 of the largest of
         // them while that is 2^-5 of the largest difference.  Else every warp looks anew, below.
         if (fold && change * 0x1p-5f > top_f) low_f = -1.f;
@@ -523,7 +485,7 @@ step_rows_kernel(const StepParams p, const __grid_constant__ RowsMaps maps, cons
         top_f = 0.f;
 #pragma unroll 2
         for (int w = 0; w < 16 * halves; w += 2) top_f = max_abs3(sum(w), sum(w + 1), top_f);
-        low_f = group_low(sum, guard, tb.guard_groups, tb.guard_size, 0, 1);
+        low_f = group_low<uchar4, uchar2>(sum, guard, tb.guard_groups, tb.guard_size, 0, 1);
       }
       const unsigned top = __float_as_uint(top_f);
       // as float bits: not finite, too small for the scale; an output may read nothing near the largest operand

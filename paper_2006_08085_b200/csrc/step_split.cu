@@ -158,22 +158,6 @@ inline SplitPlan split_plan(int nb, int num_blocks, int guard_entries) {
   return SplitPlan{};
 }
 
-// Integer sums of the five weights -> one float64, exact but for the rounding of the lowest: a 64-bit integer below 2^51, in units
-// of 256^5, added to the bits of 1.5 * 2^52 with the coordinate's scale in its exponent field (`magic_hi`: the upper word; `magic`:
-// that number), which is then subtracted.  `hi` = s8 * 256 + s7.  Up to 128 workers the rest fits 32 bits
-// (3 * 128 * 2^14 * 256 < 2^31).
-template <bool kBig>
-__device__ __forceinline__ double join_sums(int hi, int s6, int s5, int s4, int magic_hi, double magic) {
-  const int low = s5 + ((s4 + 128) >> 8);
-  if (kBig) {
-    const long long lo = static_cast<long long>(s6) * 256 + (low + (static_cast<long long>(magic_hi) << 32));
-    return __longlong_as_double(static_cast<long long>(hi) * 65536 + lo) - magic;
-  }
-  const int lo = s6 * 256 + low;
-  const unsigned long long upper = static_cast<uint32_t>(magic_hi + (lo >> 31));
-  return __longlong_as_double(static_cast<long long>(hi) * 65536 + static_cast<long long>(upper << 32 | static_cast<uint32_t>(lo))) - magic;
-}
-
 // Eight joined sums of this thread's coordinate from the accumulators at `acc` (whole warp).
 template <bool kBig>
 __device__ __forceinline__ void take_sums(uint32_t acc, int magic_hi, double magic, double (&out)[8]) {
@@ -191,7 +175,7 @@ __device__ __forceinline__ void take_sums(uint32_t acc, int magic_hi, double mag
   tmem_load8(acc + 4 * kPChunk, s4);
   tmem_wait_load();
 #pragma unroll
-  for (int u = 0; u < 8; ++u) out[u] = join_sums<kBig>(hi[u], s6[u], s5[u], s4[u], magic_hi, magic);
+  for (int u = 0; u < 8; ++u) out[u] = join_sums<kBig>(hi[u], s6[u], s5[u] + ((s4[u] + 128) >> 8), magic_hi, magic);
 }
 
 // Largest magnitude of a block's 32 staged rows (those beyond n are zeros), with what came before.
@@ -204,29 +188,6 @@ __device__ __forceinline__ float block_max(const float* src, float top) {
     top = max_abs3(top, m, m);
   }
   return top;
-}
-
-// Smallest of the largest magnitudes of groups first, first + step, ... of `size` inputs (2, or a multiple of 4).
-__device__ __forceinline__ float group_low(const float* col, const int* guard, int groups, int size, int first, int step) {
-  float low = __uint_as_float(0x7f800000u);
-  if (size == 2) {
-#pragma unroll 4
-    for (int q = first; q < groups; q += step) {
-      const int2 at = *reinterpret_cast<const int2*>(guard + 2 * q);
-      low = fminf(low, max_abs3(col[at.x], col[at.y], 0.f));
-    }
-    return low;
-  }
-  for (int q = first; q < groups; q += step) {
-    float m = 0.f;
-#pragma unroll 2
-    for (int i = 0; i < size; i += 4) {
-      const int4 at = *reinterpret_cast<const int4*>(guard + q * size + i);
-      m = max_abs3(max_abs3(m, col[at.x], col[at.y]), col[at.z], col[at.w]);
-    }
-    low = fminf(low, m);
-  }
-  return low;
 }
 
 // Digits of a block's 32 workers (zeros beyond n): digit 0 in w0, digit k in words 8 (k - 1) .. 8 k - 1 of w.  No test per row:
@@ -365,7 +326,7 @@ step_split_kernel(const StepParams p, const __grid_constant__ SplitMaps maps, co
         for (int b = first; b < last; ++b) {
           top_f = block_max(col + b * (2 * kPTileFloats), top_f);
         }
-        low_f = group_low(col, guard, tb.guard_groups, tb.guard_size, kBig ? 0 : part, kBig ? 1 : 2);
+        low_f = group_low<int4, int2>([&](int at) { return col[at]; }, guard, tb.guard_groups, tb.guard_size, kBig ? 0 : part, kBig ? 1 : 2);
       }
       if (!kBig) {  // the other group's blocks
         float2* const mx = maxima + (k & 1) * 256 + row;  // read again two slabs later, behind the next hand-over
