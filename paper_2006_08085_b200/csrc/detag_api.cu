@@ -488,7 +488,7 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
 // 100 workers, K = 6, d = 1 M 3177 -> 862, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 984,
 // 256, K = 12, d = 200 k 3830 -> 750, ring of 144, K = 4, d = 8931 35.6 against 48.1.  On short vectors rounds take their latency, one after the other:
 // caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
-// The rounds do not care how operands differ, and there what cannot share a scale is summed in float64 at up to five times the time (22 us more
+// The rounds do not care how operands differ, and there what cannot share a scale is summed in float64 at up to five times the time (15 us more
 // per turn of the SMs at 100 workers, 61 at 256).  So the estimate is for operands spread over four decades (a tenth is allowed): few rounds on sparse graphs
 // then stay rounds, which alike would gain.  Alike / spread over four / over eight decades against rounds: caller-written, 100, d = 1 M, K = 2
 // 1323 / 5380 / 6348 against 1638, K = 4 1118 / 3392 / 4972 against 2402, but K = 6 923 / 1265 / 3321 against 3175; 144, d = 500 k, K = 6 894 / 2580 / 4251
@@ -513,7 +513,7 @@ bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
   if (mode == detag::kModeExternal) {
     here = n > 128 ? 10.0 + 0.065 * n * turns * (sparse ? 1.5 : 1.0)
                    : 9.0 + turns * (1.0 + 0.031 * n) * (sparse && n > 64 && n <= 96 ? 2.2 : 1.0);  // six warps for the test
-    unequal = share * (n > 128 ? 20.0 + 2.4 * blocks : 5.5 * blocks);
+    unequal = share * (n > 128 ? 20.0 + 2.4 * blocks : (n <= 96 ? 5.5 : 3.7) * blocks);
     rounds = 6.0 + (n > 128 ? 1.2 + 0.003 * n + 0.00105 * products : 0.0021 * n + 0.00099 * products) * d / 1000.0;
     latency = 6.0 + 0.0155 * n * s->K;
   } else {
