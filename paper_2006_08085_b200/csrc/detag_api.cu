@@ -499,11 +499,11 @@ bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
   const double products = s->K * static_cast<double>(s->col_idx.size());
   const bool sparse = t.guard.size() > static_cast<size_t>(s->n);
   // share of the work that is float64 then, and the 32 x 32 blocks which that goes through per 32 outputs.  Before the tables are made: all of
-  // it while the walks of K steps, degree - 1 onwards at each, are fewer than three per worker (random graphs of degree 4, 8 and 16: from four
-  // on is the first that is less)
+  // it while the walks of K steps, degree - 1 onwards at each, are fewer than 2.5 per worker (random graphs of degree 4, 8 and 16: the first that
+  // come here have 2.8)
   double share = t.unequal, blocks = s->reach;
   if (t.guard.empty()) {
-    share = std::pow(std::fmax(products / s->K / n - 2.0, 0.0), s->K) < 3.0 * n ? 1.0 : 0.0;
+    share = std::pow(std::fmax(products / s->K / n - 2.0, 0.0), s->K) < 2.5 * n ? 1.0 : 0.0;
   } else {
     int reach = 0;
     for (unsigned char r : t.reach) reach += __builtin_popcount(r);
@@ -518,7 +518,7 @@ bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
     latency = 6.0 + 0.0155 * n * s->K;
   } else {
     here = sparse ? 14.0 + 0.098 * n * turns : 10.0 + 0.065 * n * turns;
-    unequal = share * (3.5 + 7.2 * blocks);
+    unequal = share * (share < 0.999 ? 0.62 : 1.0) * (3.5 + 7.2 * blocks);  // single columns of both arrays together
     rounds = (1.35 + 0.004 * n + 0.0011 * products) * d / 1000.0;
     latency = 6.0 + 0.0068 * n * s->K;
     if (mode == detag::kModeDpsgd) {  // one array

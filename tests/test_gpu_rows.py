@@ -5,7 +5,7 @@ import pytest
 
 from paper_2006_08085_b200 import build, inputs
 from paper_2006_08085_b200.session import Session
-from test_gpu_split import (_graph, _polynomial, _unequal, test_dpsgd as dpsgd, test_every_result_is_as_precise_as_what_it_reads as precision,
+from test_gpu_split import (_graph, _polynomial, _unequal, patterns_side_by_side, test_dpsgd as dpsgd, test_every_result_is_as_precise_as_what_it_reads as precision,
                             test_one_step_against_the_oracle as one_step, test_what_is_not_finite_stays_in_reach as not_finite)
 
 pytestmark = pytest.mark.gpu
@@ -55,6 +55,15 @@ def test_one_step_of_this_kernel(n, d, K, kind, at_start, kernels):
 def test_precision_of_this_kernel_beyond_128_workers(kind, n, K, kernels):
     precision(kind, n, K)
     assert kernels == {"step_rows"}
+
+
+# from one to all of eight coordinates of either array in float64, or of both; chunks with and without them in turn
+@pytest.mark.parametrize("n,kind,d,K,mode", [(60, "regular4", 2_003, 2, "detag"), (50, "path", 3 * CHUNKS + 1, 6, "dpsgd"), (80, "regular4", 3_001, 2, "start"),
+                                             (70, "ring", 1_999, 4, "dpsgd"), (100, "path", 2 * CHUNKS + 3, 3, "detag"), (128, "regular4", 18 * CHUNKS + 1, 6, "start"),
+                                             (112, "regular4", 2_001, 1, "dpsgd"), (144, "regular4", 2_003, 16, "detag"), (160, "ring", 4_003, 20, "start"),
+                                             (256, "regular4", 3 * CHUNKS, 12, "detag"), (256, "torus", 2 * CHUNKS + 1, 9, "dpsgd")])
+def test_float64_columns_beside_split_ones(n, kind, d, K, mode):
+    patterns_side_by_side(n, kind, d, K, mode, "step_rows")
 
 
 @pytest.mark.parametrize("n,d,K", [(144, 130, 16), (171, 131, 24), (256, 5 * CHUNKS + 9, 12)])
@@ -303,7 +312,7 @@ def test_the_gradient_beyond_128_workers_is_the_rounds(n, mode):
 @pytest.mark.parametrize("n,d,K,kind,mode,ran", [
     (100, 1_000_000, 2, "regular4", "external", "step_csr"), (100, 100_000, 4, "regular4", "external", "step_csr"), (100, 100_000, 6, "regular4", "external", "step_rows"),
     (144, 500_000, 3, "regular4", "external", "step_csr"), (160, 100_000, 16, "ring", "external", "step_rows"), (192, 100_000, 6, "regular4", "external", "step_rows"),
-    (144, 400_000, 4, "regular4", "detag", "step_csr"), (144, 100_000, 8, "regular4", "detag", "step_rows"), (256, 200_000, 6, "regular4", "detag", "step_csr"),
+    (144, 400_000, 4, "regular4", "detag", "step_csr"), (144, 100_000, 8, "regular4", "detag", "step_rows"), (256, 200_000, 4, "regular4", "detag", "step_csr"), (256, 200_000, 6, "regular4", "detag", "step_rows"),
     (256, 200_000, 3, "regular4", "dpsgd", "step_csr"), (256, 100_000, 12, "regular4", "detag", "step_rows")])
 def test_few_rounds_on_sparse_graphs_stay_rounds(n, d, K, kind, mode, ran):
     """Operands that differ by four decades would send most coordinates of these to float64 on the integer path, at two to three times the

@@ -251,6 +251,10 @@ KEPT = [(72, "regular4", 4_003, 2, "detag"), (90, "path", 4_003, 6, "start"), (9
 
 @pytest.mark.parametrize("n,kind,d,K,mode", KEPT)
 def test_every_result_is_as_precise_as_what_it_reads_at_lengths_that_this_kernel_keeps(n, kind, d, K, mode):
+    patterns_side_by_side(n, kind, d, K, mode, "step_split")
+
+
+def patterns_side_by_side(n, kind, d, K, mode, kernel):
     """As above, every column of the model and of the tracker; an infinity in one column and a NaN in another reach as far as the polynomial."""
     eta, wide = 0.2, 1997
     m = _graph(kind, n)
@@ -275,7 +279,7 @@ def test_every_result_is_as_precise_as_what_it_reads_at_lengths_that_this_kernel
             s.upload(name, v)
         s.step()
         s.status()
-        assert B.detag_debug_kernel(s.state) == "step_split"
+        assert B.detag_debug_kernel(s.state) == kernel
         got = {k: s.download(k) for k in ("x", "y")}
     reached = P[:, 9] != 0.0
     if mode == "dpsgd":
