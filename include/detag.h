@@ -54,21 +54,27 @@ enum {
   DETAG_ERR_SPECTRUM = -9        /* lambda >= 1: disconnected or bipartite graph, no valid eta */
 };
 
-/* Kernel variants of the gossip part of the step; all compute the same result.  Up to 48 workers the polynomial variants run in
-   float64 throughout.  Those of 48 < n <= 256 run on the integer tensor path where its shared-memory plan holds P_K(M) (any matrix up to n = 128, beyond that
-   matrices whose 32 x 32 blocks depend on their distance only); coordinates in which an output may read operands far below
-   the largest are summed in float64 instead, which takes up to five times as long when it concerns all of them (one or two
-   rounds on sparse graphs, workers of very different magnitude).  Circulant bands run in float64 throughout.  What neither
-   takes runs as rounds. */
+/* Kernel variants of the gossip part of the step; all compute the same result.
+   In float64 throughout: the polynomial up to 48 workers, the rounds, the torus transform, and circulant bands (K * bandwidth <= 16) - where the
+   choice is the library's but for a band's last d % 64 coordinates up to n = 128 and for ragged calls short enough for one launch.
+   On the integer tensor path (fixed point of 39 bits, exact sums): the other polynomials of 49 to 128 workers and those of matrices up to 256 whose
+   32 x 32 blocks depend on their distance only; and, where the choice is the library's and an estimate says that the rounds take longer, the other
+   matrices up to 256 and caller-written gradients up to 192.  The error of a sum there is below 2^-24 of sum_j |P_ij z_j|
+   (some 1e-11 of it on operands of like magnitude); coordinates in which an output may read only operands far below the largest are summed in
+   float64, at up to five times the time when it concerns all of them (few rounds on sparse graphs, workers of very different magnitude).
+   Which of them runs depends on d too, so that beyond 48 workers a shard of the coordinates need not give the bits of the whole; the rounds,
+   chosen by name, do.  What none takes runs as rounds. */
 enum {
   DETAG_VARIANT_AUTO = 0,  /* host cost model picks */
   DETAG_VARIANT_CSR = 1,   /* K rounds of neighbour-indexed sums over the CSR rows, slab staged on chip: any graph, n <= 1024.
                               Where AUTO resolves to it, the library still applies the rounds as one product with their
-                              polynomial up to n = 48 or if the integer tensor path takes it; forced, the rounds run as such */
+                              polynomial up to n = 48 or if the integer tensor path takes it; forced, the rounds run as such, in
+                              float64 */
   DETAG_VARIANT_DENSE = 2, /* one product with the host-precomputed polynomial P_K(M), n <= 128 (any M) */
   DETAG_VARIANT_RING = 3,  /* circulant M (rings), n % 32 == 0, 64 <= n <= 1024: the circulant polynomial P_K(M), a band
                               while K * bandwidth <= 16, or any (n <= 256), e.g. at Theorem 3's phase length; a band's last
-                              d % 64 coordinates run through another kernel in the same call */
+                              d % 64 coordinates run through another kernel in the same call.  Forced, a band and its last
+                              coordinates run in float64 */
   DETAG_VARIANT_TORUS = 4  /* block-circulant M with 8-worker blocks, symmetric in the block distance (R x 8 tori, n = 32 or 64):
                               Fourier transform along the block axis, one 8 x 8 polynomial block per frequency, transform back */
 };

@@ -342,7 +342,7 @@ bool dense_ok(const detag_state* s) {
 // Host cost model.  The product with the polynomial beats the sparse rounds wherever a kernel takes it: K rounds cost
 // K * (nnz per row) shared-memory gathers of 16 bytes per element and array and two barriers each.  Tori of 8-worker blocks
 // take the transform kernel (24 multiply-adds per element and array).  Caller-written gradients run on the dense kernels
-// for n <= 48 (under the rounds' name beyond 32) and on the rounds kernel otherwise.
+// for n <= 48 (under the rounds' name beyond 32), beyond on step_rows.cu (to 192) or as rounds (rows_beat_rounds).
 bool variant_runs_mode(const detag_state* s, int variant) {
   if (step_mode(s) == detag::kModeDetag) return true;
   if (variant == DETAG_VARIANT_RING) return step_mode(s) == detag::kModeDpsgd;
@@ -441,7 +441,7 @@ int launch_split(detag_state* s, const StepParams& p, bool rows, bool wide, cuda
 }
 
 // The columns from `first` on, which the circulant kernel leaves (it takes whole 64-coordinate slabs), in the same call, beside
-// it (64-ring, K = 4, d = 14001 21.3 -> 14.6 us in one launch, 256, d = 60001 188 -> 168 in two): through the integer tensor path up to
+// it (64-ring, K = 4, d = 14001 21.3 -> 14.6 us in one launch, 256, d = 60001 188 -> 143 in two): through the integer tensor path up to
 // 128 workers (one chunk or two 8 .. 11 us), beyond as rounds, whose latency is the smaller one (256 workers 6 us and 1.7 a round,
 // step_split.cu's slab 38), and so where the caller asked for the circulant kernel, which runs in float64 throughout.
 int launch_tail_columns(detag_state* s, const StepParams& p, long long first, cudaStream_t stream) {

@@ -24,11 +24,11 @@
 // Caller-written gradients: y + (g_new - g) is split as the float32 sum and what it rounds off, normalised where the three cancel (a loop of
 // its own for each: with the choice inside the unrolled one 100 workers, d = 1 M 862 -> 930 us); g' = g_new is stored from the staged rows.
 //
-// Bound by issue slots and latency of the finishing warps (137 instructions per worker-coordinate of 128 lanes, 0.6 of the slots), by
+// Bound by issue slots and latency of the finishing warps (136 instructions per worker-coordinate of 128 lanes, 0.6 of the slots), by
 // the power cap (1.5 .. 1.7 GHz on long vectors), and beyond a row pitch of 2 MB by rows travelling in pieces of 128 bytes: loads
 // and stores alone then reach 0.68 of the copy rate (0.85 below that pitch), where 256-byte pieces reach 0.84.  us per step,
 // step_split.cu -> here: 100 workers, d = 2 k 13.0 -> 9.4, 20 k 31.8 -> 26.0, 300 k 283 -> 262, 1 M 938 -> 859; 128, 40 k 53.2 -> 42.7, 1 M 1063 -> 1044;
-// D-PSGD of 128, 1 M 966 -> 828; 256-ring, K = 40, d = 4 k 34.6 -> 21.9, 60 k 285 -> 207; rounds -> here: 144, K = 6, d = 500 k 3396 -> 984, 256
+// D-PSGD of 128, 1 M 966 -> 828; 256-ring, K = 40, d = 4 k 34.6 -> 21.9, 60 k 263 -> 233; rounds -> here: 144, K = 6, d = 500 k 3396 -> 984, 256
 // 5327 -> 1680 (waiting for P; all of it at hand would be 1250); caller-written gradients, 100 workers, d = 1 M 3177 -> 862, 20 k 76 -> 27.
 //
 // Measured without gain: asking for 256-byte pieces in L2 ahead of the loads 917 -> 1200 us (128 workers, loads and stores alone); sums
