@@ -52,9 +52,9 @@ MEASURED_TRAFFIC = {
     ("dense", "product"): ("1d4428cc1d4b78f9", 31.21),  # cfg5 shape at d = 2 M: 1.2801 + 0.7177 GB / 64 M wc
     ("torus", "torus8"): ("194904bdd0cabfdc", 31.23),  # cfg3 shape at d = 1 M: 1.2802 + 0.7185 GB / 64 M wc
     ("ring", "band"): ("72c17745930c7df4", 31.09),  # cfg4 shape at d = 200 k: 1.0277 + 0.5641 GB / 51.2 M wc
-    ("split", "digits"): ("feb6f88094eb2145", 31.05),  # 16 x 16 torus at d = 200 k: 1.0200 + 0.5698 GB / 51.2 M wc
-    ("rows", "digits"): ("6ddfc9a5b7574d81", 30.80),  # 100-worker random graph at d = 400 k: 0.8007 + 0.4312 GB / 40 M wc
-    ("csr", "rounds"): ("57f2704a52f61fcf", 30.61),  # 300-worker random graph at d = 100 k: 0.6017 + 0.3165 GB / 30 M wc
+    ("split", "digits"): ("adecf464e2c4f133", 31.01),  # 16 x 16 torus at d = 200 k: 1.0200 + 0.5678 GB / 51.2 M wc
+    ("rows", "digits"): ("652707a08d767b36", 30.79),  # 100-worker random graph at d = 400 k: 0.8003 + 0.4312 GB / 40 M wc
+    ("csr", "rounds"): ("9562d0977f62cdfa", 30.62),  # 300-worker random graph at d = 100 k: 0.6017 + 0.3169 GB / 30 M wc
 }
 
 # Float64 multiply-adds per worker-coordinate on the FP64 pipe (both contractions, padded shapes; the dense product by its

@@ -210,12 +210,85 @@ __device__ __forceinline__ void take_sums(uint32_t acc, const int* magic_hi, int
 // tracker (kFold: with the caller's gradients, y + g_new - g) for bits 8 .. 15.  z: [array][input worker][32] at
 // the first of the coordinates.  poly: rows of P of these workers (circulant: of the first 32, block `b` of whose columns is block
 // (b + c) mod nb here).  Products on the float64 tensor path: four tiles of eight output workers (M) by eight columns (N), either the bits
-// that are set, of both arrays, or all eight coordinates of both (100 workers, K = 6, d = 300 k, spread over six decades 729 -> 577 us, 256, K = 8,
-// 200 k, over four 1787 -> 1423; not with the caller's gradients, where the callee's registers cost the splitting warps 263 -> 277, 100 workers, d = 300 k).  Rare, and so out of the way of the main path's registers, on which its own tell all the same: with sixteen
-// entries of P in flight instead of eight the main path took 1824 us for 1651 (100 workers, d = 2 M).  Bound by the latency of P from L2: with
-// every coordinate here 100 workers, K = 2, d = 1 M 888 -> 3900 us (with an array at a time a third more).
+// that are set, of both arrays (exact_columns), or all eight coordinates of both (100 workers, K = 6, d = 300 k, spread over six decades
+// 729 -> 577 us, 256, K = 8, 200 k, over four 1787 -> 1423; not with the caller's gradients, where it costs the splitting warps 263 -> 277, 100
+// workers, d = 300 k).
+// Rare, and so out of the way of the main path's registers, on which its own tell all the same: with sixteen entries of P in flight
+// instead of eight the main path took 1824 us for 1651 (100 workers, d = 2 M), with the columns in the same function 1656 for 1645, in one to
+// choose from 1678, with what the two share in functions of its own 1673.  Bound by the latency of P from L2: with every coordinate here 100
+// workers, K = 2, d = 1 M 888 -> 3900 us (with an array at a time a third more).
+__device__ __noinline__ void exact_columns(const float* z, const double* poly, unsigned which, int circulant, int c, int nb, unsigned reach, double* out) {
+  const int lane = threadIdx.x & 31, pitch = nb * kPBlock;
+  const int stride = nb * kPBlock * kPS;
+  auto weights = [&](int b) {  // this lane's entry of the first tile and k-step
+    const int pb = !circulant ? b : b >= c ? b - c : b - c + nb;
+    return poly + static_cast<size_t>(lane >> 2) * pitch + kPBlock * pb + (lane & 3);
+  };
+  bool finite = true;
+  // lane l has tiles' rows l / 4, columns 2 (l % 4) + e; it wants row l, i.e. row l % 8 of tile l / 8
+  auto hand_over = [&](const double (&sum)[4][2], int column, double* to) {
+    double mine = 0.0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const double v = __shfl_sync(0xffffffffu, (column & 1) != 0 ? sum[t][1] : sum[t][0], 4 * (lane & 7) + (column >> 1));
+      if ((lane >> 3) == t) mine = v;
+    }
+    finite = finite && (__double2hiint(mine) & 0x7ff00000) != 0x7ff00000;
+    *to = mine;
+  };
+  const bool model = (which & 0xffu) != 0, tracker = which >> 8 != 0;
+  unsigned left = which;
+  for (int i = 0; i < (lane >> 2) && (left & (left - 1)) != 0; ++i) left &= left - 1;  // columns beyond the last repeat it
+  const int mine = __ffs(left) - 1, array = mine >> 3;
+  const float* const column = z + array * stride + (mine & 7) + (lane & 3) * kPS;
+  double sum[4][2];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sum[i >> 1][i & 1] = 0.0;
+  for (int b = 0; b < nb; ++b) {
+    if ((reach >> b & 1) == 0) continue;  // a zero block of P
+    const double* const pw = weights(b);
+    const float* const zb = column + kPBlock * b * kPS;
+#pragma unroll 1
+    for (int h = 0; h < kPBlock; h += 16) {
+#pragma unroll 2
+      for (int s = 0; s < 4; ++s) {
+        double w[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) w[t] = __ldg(pw + static_cast<size_t>(8 * t) * pitch + h + 4 * s);
+        const double v = static_cast<double>(zb[(h + 4 * s) * kPS]);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) dmma(sum[t], w[t], v);
+      }
+    }
+  }
+  left = which;
+  for (int q = 0; left != 0; ++q, left &= left - 1) hand_over(sum, q, out + __ffs(left) - 1);
+  if (__any_sync(0xffffffffu, !finite)) {
+    // Infinities or NaN among the operands: a lane sums its own worker, without the zeros of P, which the products above turn
+    // into NaN.
+#pragma unroll 1
+    for (int u = 0; u < 16; ++u) {
+      if (!(u < 8 ? model : tracker)) continue;
+      const int array = u >> 3;
+      double own = 0.0;
+      for (int b = 0; b < nb; ++b) {
+        if ((reach >> b & 1) == 0) continue;
+        const int pb = !circulant ? b : b >= c ? b - c : b - c + nb;
+        const double* const pw = poly + static_cast<size_t>(lane) * pitch + kPBlock * pb;
+        for (int w = 0; w < kPBlock; ++w)
+          if (pw[w] != 0.0) own = fma(pw[w], static_cast<double>(z[array * stride + (kPBlock * b + w) * kPS + (u & 7)]), own);
+      }
+      out[u] = own;
+    }
+  }
+}
+
 template <bool kFold>
 __device__ __noinline__ void exact_sums(const float* z, const double* poly, unsigned which, int circulant, int c, int nb, unsigned reach, double* out) {
+  if (!kFold && __popc(which) <= 8) {
+    exact_columns(z, poly, which, circulant, c, nb, reach, out);
+    return;
+  }
   const int lane = threadIdx.x & 31, pitch = nb * kPBlock;
   const int stride = nb * kPBlock * kPS;
   auto value = [&](int array, const float* at) {
@@ -240,73 +313,44 @@ __device__ __noinline__ void exact_sums(const float* z, const double* poly, unsi
     *to = mine;
   };
   const bool model = (which & 0xffu) != 0, tracker = which >> 8 != 0;
-  if (!kFold && __popc(which) <= 8) {
-    unsigned left = which;
-    for (int i = 0; i < (lane >> 2) && (left & (left - 1)) != 0; ++i) left &= left - 1;  // columns beyond the last repeat it
-    const int mine = __ffs(left) - 1, array = mine >> 3;
-    const float* const column = z + array * stride + (mine & 7) + (lane & 3) * kPS;
-    double sum[4][2];
+  double sum[2][4][2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) sum[i >> 1][i & 1] = 0.0;
-    for (int b = 0; b < nb; ++b) {
-      if ((reach >> b & 1) == 0) continue;  // a zero block of P
-      const double* const pw = weights(b);
-      const float* const zb = column + kPBlock * b * kPS;
+  for (int i = 0; i < 16; ++i) sum[i >> 3][i >> 1 & 3][i & 1] = 0.0;
+  for (int b = 0; b < nb; ++b) {
+    if ((reach >> b & 1) == 0) continue;
+    const double* const pw = weights(b);
+    const float* const zb = z + (kPBlock * b + (lane & 3)) * kPS + (lane >> 2);
 #pragma unroll 1
-      for (int h = 0; h < kPBlock; h += 16) {
+    for (int h = 0; h < kPBlock; h += 16) {
 #pragma unroll 2
-        for (int s = 0; s < 4; ++s) {
-          double w[4];
+      for (int s = 0; s < 4; ++s) {
+        const float* const at = zb + (h + 4 * s) * kPS;
+        double w[4];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) w[t] = __ldg(pw + static_cast<size_t>(8 * t) * pitch + h + 4 * s);
-          const double v = value(array, zb + (h + 4 * s) * kPS);
+        for (int t = 0; t < 4; ++t) w[t] = __ldg(pw + static_cast<size_t>(8 * t) * pitch + h + 4 * s);
+        if (!kFold) {
+          const double v = value(0, at), u = value(1, at + stride);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) dmma(sum[t], w[t], v);
+          for (int t = 0; t < 4; ++t) dmma(sum[0][t], w[t], v);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) dmma(sum[1][t], w[t], u);
+          continue;
+        }
+        if (model) {
+          const double v = value(0, at);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) dmma(sum[0][t], w[t], v);
+        }
+        if (tracker) {
+          const double v = value(1, at + stride);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) dmma(sum[1][t], w[t], v);
         }
       }
     }
-    left = which;
-    for (int q = 0; left != 0; ++q, left &= left - 1) hand_over(sum, q, out + __ffs(left) - 1);
-  } else {
-    double sum[2][4][2];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) sum[i >> 3][i >> 1 & 3][i & 1] = 0.0;
-    for (int b = 0; b < nb; ++b) {
-      if ((reach >> b & 1) == 0) continue;
-      const double* const pw = weights(b);
-      const float* const zb = z + (kPBlock * b + (lane & 3)) * kPS + (lane >> 2);
-#pragma unroll 1
-      for (int h = 0; h < kPBlock; h += 16) {
-#pragma unroll 2
-        for (int s = 0; s < 4; ++s) {
-          const float* const at = zb + (h + 4 * s) * kPS;
-          double w[4];
-#pragma unroll
-          for (int t = 0; t < 4; ++t) w[t] = __ldg(pw + static_cast<size_t>(8 * t) * pitch + h + 4 * s);
-          if (!kFold) {
-            const double v = value(0, at), u = value(1, at + stride);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) dmma(sum[0][t], w[t], v);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) dmma(sum[1][t], w[t], u);
-            continue;
-          }
-          if (model) {
-            const double v = value(0, at);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) dmma(sum[0][t], w[t], v);
-          }
-          if (tracker) {
-            const double v = value(1, at + stride);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) dmma(sum[1][t], w[t], v);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 16; ++u) hand_over(sum[u >> 3], u & 7, out + u);
   }
+#pragma unroll
+  for (int u = 0; u < 16; ++u) hand_over(sum[u >> 3], u & 7, out + u);
   if (__any_sync(0xffffffffu, !finite)) {
     // Infinities or NaN among the operands: a lane sums its own worker, without the zeros of P, which the products above turn
     // into NaN.
