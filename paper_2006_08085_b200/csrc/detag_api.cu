@@ -490,9 +490,10 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
 // caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
 // The rounds do not care how operands differ, and there what cannot share a scale is summed in float64 at up to five times the time (15 us more
 // per turn of the SMs at 100 workers, 61 at 256).  So the estimate is for operands spread over four decades (a tenth is allowed): few rounds on sparse graphs
-// then stay rounds, which alike would gain.  Alike / spread over four / over eight decades against rounds: caller-written, 100, d = 1 M, K = 2
-// 1323 / 5380 / 6348 against 1638, K = 4 1118 / 3392 / 4972 against 2402, but K = 6 923 / 1265 / 3321 against 3175; 144, d = 500 k, K = 6 894 / 2580 / 4251
-// against 3100; 256, d = 200 k, K = 4 719 / 3335 / 3338 against 1591, K = 6 731 / 2767 / 3215 against 2137, but K = 12 745 / 1157 / 2724 against 3827.
+// then stay rounds, which alike would gain.  Alike / spread over four / over eight decades there, against rounds: caller-written, 100 workers, d = 1 M, K = 2
+// 1323 / 5380 / 6348 against 1638, K = 4 1118 / 3392 / 4972 against 2402, but K = 5 1028 / 1255 / 2167 against 2797, K = 6 870 / 1153 / 2383 against 3187;
+// 144, d = 500 k, K = 6 839 / 2542 / 4217 against 3091; 256, d = 200 k, K = 4 719 / 3335 / 3338 against 1591, but K = 6 700 / 2175 / 2914 against 2134, K = 12
+// 726 / 996 / 2127 against 3815.
 bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
   const detag::SplitPoly& t = s->rows;
   const double n = s->n, d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * sms));
