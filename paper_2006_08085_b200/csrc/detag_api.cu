@@ -488,47 +488,55 @@ bool split_ok(const detag_state* s, const StepParams& p, int variant) {
 // 100 workers, K = 6, d = 1 M 3177 -> 862, 20 k 76 -> 27, ring of 54, K = 1, d = 27 k 13.9 against 24.1; 144, K = 6, d = 500 k 3396 -> 984,
 // 256, K = 12, d = 200 k 3830 -> 750, ring of 144, K = 4, d = 8931 35.6 against 48.1.  On short vectors rounds take their latency, one after the other:
 // caller-written, 124 workers, K = 12, d = 785 31.7 us; 226, K = 16, d = 246 32.5.
-// The rounds do not care how operands differ, and there what cannot share a scale is summed in float64 at up to five times the time (15 us more
-// per turn of the SMs at 100 workers, 61 at 256).  So the estimate is for operands spread over four decades (a tenth is allowed): few rounds on sparse graphs
-// then stay rounds, which alike would gain.  Alike / spread over four / over eight decades there, against rounds: caller-written, 100 workers, d = 1 M, K = 2
-// 1323 / 5380 / 6348 against 1638, K = 4 1118 / 3392 / 4972 against 2402, but K = 5 1028 / 1255 / 2167 against 2797, K = 6 870 / 1153 / 2383 against 3187;
-// 144, d = 500 k, K = 6 839 / 2542 / 4217 against 3091; 256, d = 200 k, K = 4 719 / 3335 / 3338 against 1591, but K = 6 700 / 2175 / 2914 against 2134, K = 12
-// 726 / 996 / 2127 against 3815.
+// The rounds do not care how operands differ, and there what cannot share a scale is summed in float64 at up to five times the time (14 us more
+// per turn of the SMs at 100 workers, 55 at 250).  So the estimate is for operands spread over four decades: few rounds on sparse graphs
+// then stay rounds, which alike would gain.  Of passes of eight coordinates the share that is held up goes with the fourth root of the coordinates'
+// (0.2 at 0.003, 0.36 at 0.015, 0.6 at 0.12, 0.8 at 0.45, measured).  A limit of 1.1 for caller-written gradients, 1.35 for the others, for which the
+// estimate is the more careful one: where it says 0.74 of the rounds' speed or more 0.8 is the least that was measured.  Rounds' time / time there, operands alike, spread over two, over four
+// decades, d = 150 k: caller-written, 100 workers, K = 3 1.7, 1.3, 0.59, K = 5 2.5, 2.1, 1.8; 128, K = 4 2.4, 1.9, 0.98; 160, K = 5 2.9, 0.98, 0.63; 192, K = 5 2.4, 1.7, 0.68; DeTAG, 140, K = 3 1.9, 1.2, 0.53,
+// K = 4 2.3, 1.7, 0.75, K = 6 3.1, 2.9, 1.7; 215, K = 5 3.1, 1.6, 0.78, K = 6 3.6, 1.2, 0.91; 250, K = 4 2.1, 0.94, 0.52; D-PSGD, 180, K = 5 2.3, 0.75, 0.57; 155-ring, K = 6 2.4, 2.1, 0.77, K = 10 3.3,
+// 2.8, 1.2; 14 x 13 torus, K = 3 1.9, 1.7, 0.50, K = 6 2.7, 2.5, 0.87.
 bool rows_beat_rounds(const detag_state* s, int mode, int sms) {
   const detag::SplitPoly& t = s->rows;
-  const double n = s->n, d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * sms));
+  const double n = s->n, d = static_cast<double>(s->d), turns = std::ceil(d / (32.0 * sms)), nb = std::ceil(n / 32.0);
   const double products = s->K * static_cast<double>(s->col_idx.size());
   const bool sparse = t.guard.size() > static_cast<size_t>(s->n);
-  // share of the work that is float64 then, and the 32 x 32 blocks which that goes through per 32 outputs.  Before the tables are made: all of
-  // it while the walks of K steps, degree - 1 onwards at each, are fewer than 2.5 per worker (random graphs of degree 4, 8 and 16: the first that
-  // come here have 2.8)
+  // The 32 x 32 blocks that the float64 sums go through per 32 outputs.  Before the tables are made the share is the least that was found
+  // for graphs with fewer than 2.5 walks of K steps, degree - 1 onwards at each, per worker, and none beyond.
   double share = t.unequal, blocks = s->reach;
   if (t.guard.empty()) {
-    share = std::pow(std::fmax(products / s->K / n - 2.0, 0.0), s->K) < 2.5 * n ? 1.0 : 0.0;
+    share = std::pow(std::fmax(products / s->K / n - 2.0, 0.0), s->K) < 2.5 * n ? 0.15 : 0.0;
   } else {
     int reach = 0;
     for (unsigned char r : t.reach) reach += __builtin_popcount(r);
-    blocks = reach / std::ceil(n / 32.0);
+    blocks = reach / nb;
   }
-  double here, unequal, rounds, latency;
+  double here, unequal, rounds, latency, limit = 1.35;
   if (mode == detag::kModeExternal) {
-    here = n > 128 ? 10.0 + 0.065 * n * turns * (sparse ? 1.5 : 1.0)
-                   : 9.0 + turns * (1.0 + 0.031 * n) * (sparse && n > 64 && n <= 96 ? 2.2 : 1.0);  // six warps for the test
-    unequal = share * (n > 128 ? 20.0 + 2.4 * blocks : (n <= 96 ? 5.5 : 3.7) * blocks);
-    rounds = 6.0 + (n > 128 ? 1.2 + 0.003 * n + 0.00105 * products : 0.0021 * n + 0.00099 * products) * d / 1000.0;
+    limit = 1.1;
+    if (n > 128) {
+      here = 10.0 + 0.065 * n * turns * (sparse ? 1.05 : 1.0);
+      unequal = 2.0 + 8.0 * blocks;
+      rounds = 6.0 + (1.2 + 0.003 * n + 0.00105 * products) * d / 1000.0;
+    } else {  // of 65 to 96 workers six warps for the test of the operands
+      here = 8.0 + turns * (n <= 64 ? 0.6 + 0.036 * n : n <= 96 ? 0.063 * n * (sparse ? 1.3 : 1.0) : (3.4 + 0.009 * n) * (sparse ? 1.2 : 1.0));
+      unequal = (n <= 64 ? 2.5 : n <= 96 ? 5.5 : 3.5) * blocks;
+      rounds = 6.0 + (0.0085 * n + 0.00078 * products) * (n <= 64 ? 0.86 : 1.0) * d / 1000.0;
+    }
     latency = 6.0 + 0.0155 * n * s->K;
   } else {
-    here = sparse ? 14.0 + 0.098 * n * turns : 10.0 + 0.065 * n * turns;
-    unequal = share * (share < 0.999 ? 0.62 : 1.0) * (3.5 + 7.2 * blocks);  // single columns of both arrays together
+    here = 10.0 + 0.065 * n * turns * (sparse ? 1.07 : 1.0);
+    unequal = 3.0 + 1.2 * nb + 5.0 * blocks;
     rounds = (1.35 + 0.004 * n + 0.0011 * products) * d / 1000.0;
     latency = 6.0 + 0.0068 * n * s->K;
     if (mode == detag::kModeDpsgd) {  // one array
-      unequal = (1.0 - std::sqrt(1.0 - share)) * 0.75 * (3.5 + 7.2 * blocks);
-      rounds *= 0.64;
+      here *= 0.88;
+      unequal *= 0.85;
+      rounds *= 0.68;
     }
   }
   rounds = std::fmax(std::fmax(rounds, latency), 8.0);
-  return here < rounds && here + unequal * d / (32.0 * sms) < 1.1 * rounds;
+  return here < rounds && here + std::sqrt(std::sqrt(share)) * unequal * d / (32.0 * sms) < limit * rounds;
 }
 
 // Of 97 to 128 workers, calls in which reading the model a second time, in pieces of 32 bytes, costs the printed timing more than
@@ -551,7 +559,7 @@ bool rows_ok(const detag_state* s, const StepParams& p) {
   const double turns = std::ceil(static_cast<double>(s->d) / (32.0 * s->sm_count));
   if (p.n <= 64) return turns <= 32.0 || s->split.weights.empty();
   if (p.n > 96 && p.n <= 128) return !(p.mode == detag::kModeDetag && p.grad_at_start != 0 && long_calls(s, s->sm_count) && !s->split.weights.empty());
-  if (p.n <= 128) return p.mode == detag::kModeDpsgd ? turns <= 1.0 || s->rows.unequal < 0.5f : s->d <= 24LL * s->sm_count;
+  if (p.n <= 128) return p.mode == detag::kModeDpsgd ? turns <= 1.0 || s->rows.unequal < 0.04f : s->d <= 24LL * s->sm_count;
   if (s->split.weights.empty()) return rows_beat_rounds(s, p.mode, s->sm_count);
   const bool dense = s->rows.use.count[0] + s->rows.use.count[1] == 2 * ((p.n + 31) / 32);
   // two chunks a block are one slab of 64 coordinates there (12 x 16 torus, d = 4863 24.0 against 27.5, but 256-ring, K = 40, d = 9 k 85 -> 38)

@@ -91,7 +91,7 @@ struct SplitPoly {
   std::vector<double> poly;  // in float64, padded; step_split.cu: transposed
   std::vector<uint8_t> guard;  // groups of guard_size inputs
   int guard_size;
-  float unequal;           // share of its passes that hold a coordinate in float64 when operands are spread over four decades
+  float unequal;           // share of coordinates (a bound) that stay in float64 when operands are spread over four decades
   float guard_tau;         // each group's largest operand must be at least this share of the coordinate's largest
   bool circulant;          // the 32 x 32 blocks depend on their distance only: `poly` holds output workers 0 .. 31
   unsigned char id[64];    // step_split.cu: [output block][input block] -> distinct block, 255: no digit of it is set

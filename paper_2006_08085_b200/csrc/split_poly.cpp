@@ -123,11 +123,9 @@ void split_guard(int n, const std::vector<double>& poly, int rows, SplitPoly& ou
     out.guard_tau = 2.f;
   }
   // Magnitudes spread evenly over four decades, times a normal: the largest of many is some 2 10^2, and an operand is below tau of it with
-  // a probability of 1 - (log10(1 / tau) - 0.6) / 4.  A pass has eight coordinates of two arrays.  (Measured by what such steps take longer,
-  // estimate -> share: 100 workers, K = 4 0.86 -> 0.58, K = 6 0.08 -> 0.07; 144, K = 6 0.44 -> 0.50; 256, K = 6 0.97 -> 0.82.)
+  // a probability of 1 - (log10(1 / tau) - 0.6) / 4.
   const double below = std::fmin(std::fmax(1.0 - (-std::log10(std::fmin(out.guard_tau, 1.f)) - 0.6) / 4.0, 0.0), 1.0);
-  const double groups_fail = std::fmin(static_cast<double>(out.guard.size()) / out.guard_size * std::pow(below, out.guard_size), 1.0);
-  out.unequal = static_cast<float>(1.0 - std::pow(1.0 - groups_fail, 16));
+  out.unequal = static_cast<float>(std::fmin(static_cast<double>(out.guard.size()) / out.guard_size * std::pow(below, out.guard_size), 1.0));
 }
 
 // Digits of the `rows` given rows of the n x n matrix, as bytes of 64-bit integers (`wide` per row, zeros beyond n), and the exponent

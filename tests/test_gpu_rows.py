@@ -312,7 +312,7 @@ def test_the_gradient_beyond_128_workers_is_the_rounds(n, mode):
 @pytest.mark.parametrize("n,d,K,kind,mode,ran", [
     (100, 1_000_000, 2, "regular4", "external", "step_csr"), (100, 100_000, 4, "regular4", "external", "step_csr"), (100, 100_000, 6, "regular4", "external", "step_rows"),
     (144, 500_000, 3, "regular4", "external", "step_csr"), (160, 100_000, 16, "ring", "external", "step_rows"), (192, 100_000, 6, "regular4", "external", "step_rows"),
-    (144, 400_000, 4, "regular4", "detag", "step_csr"), (144, 100_000, 8, "regular4", "detag", "step_rows"), (256, 200_000, 4, "regular4", "detag", "step_csr"), (256, 200_000, 6, "regular4", "detag", "step_rows"),
+    (144, 400_000, 4, "regular4", "detag", "step_csr"), (215, 143_473, 6, "regular4", "detag", "step_rows"), (144, 100_000, 8, "regular4", "detag", "step_rows"), (256, 200_000, 4, "regular4", "detag", "step_csr"), (256, 200_000, 6, "regular4", "detag", "step_rows"),
     (256, 200_000, 3, "regular4", "dpsgd", "step_csr"), (256, 100_000, 12, "regular4", "detag", "step_rows")])
 def test_few_rounds_on_sparse_graphs_stay_rounds(n, d, K, kind, mode, ran):
     """Operands that differ by four decades would send most coordinates of these to float64 on the integer path, at two to three times the
